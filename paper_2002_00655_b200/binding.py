@@ -138,8 +138,16 @@ def _hptr(t, dtype=None):
     return t.data_ptr()
 
 
+# The current stream's handle, as torch.cuda.current_stream().cuda_stream gives it, without building a Stream object for
+# every call (3.3 us against 0.2 us, as much as the launch of a kernel).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_raw_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream():
-    return torch.cuda.current_stream().cuda_stream
+    if _raw_stream is None or _raw_device is None or not torch.cuda.is_initialized():
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(_raw_device())
 
 
 _U32 = (torch.int32, torch.uint32)

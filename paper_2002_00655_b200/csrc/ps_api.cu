@@ -200,6 +200,13 @@ static ps_status_t release_set(SortSet* ss, cudaStream_t s) {
     return cuda_ok(cudaGetLastError());
 }
 
+// A step without a sort: everything on the caller's stream, which already waits for a batch still on its way from the
+// host.  It takes neither a buffer set nor a call number (a bad index leaves its mark in the keys).
+static uint32_t* begin_small(ps_store* ps) {
+    ps->batch_ready = nullptr;
+    return small_keys(ps);
+}
+
 static void next_epoch(ps_store* ps) {
     ps->epoch++;
     if (ps->epoch == 0) ps->epoch = 1;
@@ -419,6 +426,10 @@ ps_status_t ps_push(ps_store_t* ps, const uint64_t* d_keys, uint64_t n, const fl
         return release_set(ss, s);
     }
     if (n > ps->max_keys) return PS_ERR_WORKSPACE;
+    if (small_call(n)) {
+        run_small_push_keys(ps, d_keys, (uint32_t)n, d_updates, s);
+        return after_launch();
+    }
     SortSet* ss = next_set(ps);
     if (!fork_side(ps, ss, s)) return PS_ERR_CUDA;         // the keys are sorted beside earlier calls' kernels
     const int which = radix_sort_keys64(ps, d_keys, (uint32_t)n, ps->side, ps->starter_count,
@@ -511,6 +522,11 @@ ps_status_t ps_step_mf(ps_store_t* ps, const uint32_t* d_i, const uint32_t* d_j,
     if (!d_i || !d_j || !d_v) return PS_ERR_INVALID_ARG;
     if (2 * n > ps->max_keys) return PS_ERR_WORKSPACE;
     if (col_key_base > ps->cfg.num_keys) return PS_ERR_INVALID_ARG;
+    if (small_call(2 * n) && ps->mf_path == PS_MF_AUTO) {
+        const uint32_t lb = launch_step_mf(ps, d_i, d_j, d_v, n, col_key_base, lr, lambda, begin_small(ps), s);
+        run_small_reduce(ps, (uint32_t)(2 * n), d_loss_accum, d_loss_accum ? lb : 0, s);
+        return after_launch();
+    }
     SortSet* ss = next_set(ps);
     alternate_side(ps);
     if (!fork_side(ps, ss, s, true)) return PS_ERR_CUDA;
@@ -536,7 +552,7 @@ ps_status_t ps_step_mf(ps_store_t* ps, const uint32_t* d_i, const uint32_t* d_j,
                      ps->row_map_ok && ps->mf_path != PS_MF_SYMMETRIC_ROW_COPIES);
         return release_set(ss, s);
     }
-    const uint32_t lb = launch_step_mf(ps, d_i, d_j, d_v, n, col_key_base, lr, lambda, s);
+    const uint32_t lb = launch_step_mf(ps, d_i, d_j, d_v, n, col_key_base, lr, lambda, nullptr, s);
     if (!join_side(ps, s)) return PS_ERR_CUDA;
     run_push_reduce(ps, (uint32_t)(2 * n), which, ps->upd, d_loss_accum, d_loss_accum ? lb : 0, s);
     return release_set(ss, s);
@@ -554,6 +570,14 @@ ps_status_t ps_step_kge(ps_store_t* ps, const uint32_t* d_s, const uint32_t* d_r
     if ((3 + (uint64_t)n_neg) * n > ps->max_keys) return PS_ERR_WORKSPACE;
     if (rel_key_base > ps->cfg.num_keys) return PS_ERR_INVALID_ARG;
     const uint32_t occ = (uint32_t)((3 + (uint64_t)n_neg) * n);
+    if (small_call(occ)) {
+        const bool grad_only = dim_complex % 2 == 0;
+        const uint32_t lb = launch_step_kge(ps, d_s, d_r, d_o, d_neg_ent, d_neg_side, n, n_neg, rel_key_base, dim_complex,
+                                            lr, eps, grad_only, begin_small(ps), s);
+        if (grad_only) run_small_adagrad(ps, occ, lr, eps, d_loss_accum, d_loss_accum ? lb : 0, s);
+        else run_small_reduce(ps, occ, d_loss_accum, d_loss_accum ? lb : 0, s);
+        return after_launch();
+    }
     SortSet* ss = next_set(ps);
     if (!fork_side(ps, ss, s)) return PS_ERR_CUDA;
     launch_keys_kge(ps, d_s, d_r, d_o, d_neg_ent, n, n_neg, rel_key_base, ps->side);
@@ -562,7 +586,7 @@ ps_status_t ps_step_kge(ps_store_t* ps, const uint32_t* d_s, const uint32_t* d_r
     // gradient rows + AdaGrad inside the reduction where a gradient row is whole float4s and fits the reduction's staging
     const bool grad_only = dim_complex % 2 == 0 && dim_complex <= 128;
     const uint32_t lb = launch_step_kge(ps, d_s, d_r, d_o, d_neg_ent, d_neg_side, n, n_neg, rel_key_base, dim_complex,
-                                        lr, eps, grad_only, s);
+                                        lr, eps, grad_only, nullptr, s);
     if (!join_side(ps, s)) return PS_ERR_CUDA;
     if (grad_only) run_kge_reduce(ps, occ, which, dim_complex, lr, eps, d_loss_accum, d_loss_accum ? lb : 0, s);
     else run_push_reduce(ps, occ, which, ps->upd, d_loss_accum, d_loss_accum ? lb : 0, s);
@@ -581,6 +605,12 @@ ps_status_t ps_step_rescal(ps_store_t* ps, const uint32_t* d_s, const uint32_t* 
     if ((2 + (uint64_t)n_neg + dim) * n > ps->max_keys) return PS_ERR_WORKSPACE;
     if (rel_key_base > ps->cfg.num_keys) return PS_ERR_INVALID_ARG;
     const uint32_t occ = (uint32_t)((2 + (uint64_t)n_neg + dim) * n);
+    if (small_call(occ)) {
+        const uint32_t lb = launch_grad_rescal(ps, d_s, d_r, d_o, d_neg_ent, d_neg_side, n, n_neg, rel_key_base, dim,
+                                               begin_small(ps), s);
+        run_small_adagrad(ps, occ, lr, eps, d_loss_accum, d_loss_accum ? lb : 0, s);
+        return after_launch();
+    }
     SortSet* ss = next_set(ps);
     if (!fork_side(ps, ss, s)) return PS_ERR_CUDA;
     launch_keys_rescal(ps, d_s, d_r, d_o, d_neg_ent, n, n_neg, rel_key_base, dim, ps->side);
@@ -588,7 +618,7 @@ ps_status_t ps_step_rescal(ps_store_t* ps, const uint32_t* d_s, const uint32_t* 
     if (!sorted_keys_at(ps, ss, which, occ)) return PS_ERR_CUDA;
     // gradient rows of dim values per occurrence; AdaGrad inside the reduction, to which a row [dim | dim] is what
     // [Re Im | G_Re G_Im] of dim / 2 complex dimensions is
-    const uint32_t lb = launch_grad_rescal(ps, d_s, d_r, d_o, d_neg_ent, d_neg_side, n, n_neg, rel_key_base, dim, s);
+    const uint32_t lb = launch_grad_rescal(ps, d_s, d_r, d_o, d_neg_ent, d_neg_side, n, n_neg, rel_key_base, dim, nullptr, s);
     if (!join_side(ps, s)) return PS_ERR_CUDA;
     run_kge_reduce(ps, occ, which, dim / 2, lr, eps, d_loss_accum, d_loss_accum ? lb : 0, s);
     return release_set(ss, s);
@@ -684,6 +714,15 @@ static ps_status_t sgns_checks(ps_store_t* ps, uint64_t first_pos, uint64_t n_ce
     return PS_OK;
 }
 
+static void sgns_small(ps_store_t* ps, const uint32_t* d_tokens, uint64_t tok_first, uint64_t first_pos,
+                       uint64_t n_centers, uint64_t corpus_len, uint32_t window, const uint32_t* d_negs, uint32_t n_neg,
+                       uint64_t out_key_base, float lr, uint64_t occ, double* d_loss_accum, cudaStream_t s) {
+    const uint32_t lb = launch_step_sgns(ps, d_tokens, tok_first, first_pos, n_centers, corpus_len, window, d_negs, n_neg,
+                                         out_key_base, lr, begin_small(ps), s);
+    run_small_reduce(ps, (uint32_t)occ, d_loss_accum, d_loss_accum ? lb : 0, s, sgns_scales(ps, n_centers),
+                     (uint32_t)(occ / n_centers));
+}
+
 ps_status_t ps_step_sgns(ps_store_t* ps, const uint32_t* d_tokens, uint64_t first_pos, uint64_t n_centers,
                          uint64_t corpus_len, uint32_t window, const uint32_t* d_negs, uint32_t n_neg,
                          uint64_t out_key_base, float lr, double* d_loss_accum, void* stream) {
@@ -693,13 +732,18 @@ ps_status_t ps_step_sgns(ps_store_t* ps, const uint32_t* d_tokens, uint64_t firs
     uint64_t occ;
     const ps_status_t c = sgns_checks(ps, first_pos, n_centers, corpus_len, window, n_neg, out_key_base, &occ);
     if (c != PS_OK) return c;
+    if (small_call(occ)) {
+        sgns_small(ps, d_tokens, 0, first_pos, n_centers, corpus_len, window, d_negs, n_neg, out_key_base, lr, occ,
+                   d_loss_accum, s);
+        return after_launch();
+    }
     SortSet* ss = next_set(ps);
     if (!fork_side(ps, ss, s)) return PS_ERR_CUDA;
     launch_keys_sgns(ps, d_tokens, 0, first_pos, n_centers, corpus_len, window, d_negs, n_neg, out_key_base, ps->side);
     const int which = run_push_sort(ps, (uint32_t)occ, ps->side);
     if (!sorted_keys_at(ps, ss, which, (uint32_t)occ)) return PS_ERR_CUDA;
     const uint32_t lb = launch_step_sgns(ps, d_tokens, 0, first_pos, n_centers, corpus_len, window, d_negs, n_neg,
-                                         out_key_base, lr, s);
+                                         out_key_base, lr, nullptr, s);
     if (!join_side(ps, s)) return PS_ERR_CUDA;
     run_push_reduce(ps, (uint32_t)occ, which, ps->upd, d_loss_accum, d_loss_accum ? lb : 0, s,
                     sgns_scales(ps, n_centers), (uint32_t)(occ / n_centers));
@@ -836,6 +880,12 @@ ps_status_t ps_step_sgns_host(ps_store_t* ps, const uint32_t* h_tokens, uint64_t
     if (n_negs && cudaMemcpyAsync(d_negs, h_negs, n_negs * 4, cudaMemcpyHostToDevice, hb.cs) != cudaSuccess)
         return PS_ERR_CUDA;
     if (!host_batch_copied(ps, s, hb)) return PS_ERR_CUDA;
+    if (small_call(occ)) {
+        sgns_small(ps, d_tok, tok_first, first_pos, n_centers, corpus_len, window, d_negs, n_neg, out_key_base, lr, occ,
+                   d_loss_accum, s);
+        c = after_launch();
+        return c != PS_OK ? c : finish_host_step(ps, hb, d_loss_accum, h_loss, s);
+    }
     SortSet* ss = next_set(ps);
     if (hb.slot >= 0) {
         if (!fork_side(ps, ss, s)) return PS_ERR_CUDA;      // waits for the copy; pipelined or ordered as the handle is set
@@ -846,7 +896,7 @@ ps_status_t ps_step_sgns_host(ps_store_t* ps, const uint32_t* h_tokens, uint64_t
                      ps->side);
     const int which = run_push_sort(ps, (uint32_t)occ, ps->side);
     const uint32_t lb = launch_step_sgns(ps, d_tok, tok_first, first_pos, n_centers, corpus_len, window, d_negs, n_neg,
-                                         out_key_base, lr, s);
+                                         out_key_base, lr, nullptr, s);
     if (!join_side(ps, s)) return PS_ERR_CUDA;
     run_push_reduce(ps, (uint32_t)occ, which, ps->upd, d_loss_accum, d_loss_accum ? lb : 0, s,
                     sgns_scales(ps, n_centers), (uint32_t)(occ / n_centers));

@@ -22,6 +22,7 @@ constexpr int kSortCtlWords = kMaxSortPasses * kRadix + kMaxSortPasses;   // dig
 constexpr int kReduceTile = 32;                  // sorted occurrences per warp in the segmented reduction
 constexpr int kGroupSpan = 64 * kReduceTile;      // sorted positions whose parked parts are pre-added together
 constexpr int kMaxLossBlocks = 4096;
+constexpr uint32_t kSmallOcc = 4096;             // calls of at most this many key occurrences are reduced without a sort (small.cu)
 constexpr int kHostStages = 3;                   // staging areas for batches that arrive from host memory
 constexpr int kSortSets = 4;                     // calls whose key sort may be in flight at once (see SortSet)
 constexpr int kSideStreams = 3;                  // internal streams that calls with a long sort take in turn
@@ -235,6 +236,18 @@ void run_mf_col(ps_store* ps, uint32_t n_cells, int which, float lr, float lambd
 void run_kge_reduce(ps_store* ps, uint32_t n, int which, uint32_t dim, float lr, float eps, double* d_loss_accum,
                     uint32_t loss_blocks, cudaStream_t s);
 
+// ---- small.cu ----
+// Calls of at most kSmallOcc key occurrences, all on the caller's stream, no sort.  The step's gradient kernel leaves the
+// slots' keys in small_keys (num_keys: no key; kSentinelPad: index out of range) and its rows in ps->upd, as for the
+// sorted reductions.
+inline bool small_call(uint64_t n_occ) { return n_occ <= kSmallOcc; }
+uint32_t* small_keys(ps_store* ps);
+void run_small_push_keys(ps_store* ps, const uint64_t* d_keys, uint32_t n, const float* d_upd, cudaStream_t s);
+void run_small_reduce(ps_store* ps, uint32_t n, double* d_loss_accum, uint32_t loss_blocks, cudaStream_t s,
+                      const float* d_scales = nullptr, uint32_t slots = 0);
+void run_small_adagrad(ps_store* ps, uint32_t n, float lr, float eps, double* d_loss_accum, uint32_t loss_blocks,
+                       cudaStream_t s);
+
 // ---- localize.cu ----
 // busy_keys: sorted keys of a call that may run beside this relocation (null: none); moving keys among them keep
 // table entry and row until run_localize_deferred, which the caller enqueues once that call is through.
@@ -246,29 +259,31 @@ void run_localize_deferred(ps_store* ps, uint32_t worker, uint32_t n, cudaStream
 // launch_keys_* write the keys of a batch's occurrence slots to keysA (they depend on the batch
 // only, so they and the sort can run beside the gradient kernel); launch_step_* write the slots'
 // update rows to `upd` (launch_step_sgns: two source rows per center and one factor per slot, to be
-// reduced with run_push_reduce's d_scales) and return the number of per-block loss partials they wrote.
+// reduced with run_push_reduce's d_scales) and return the number of per-block loss partials they wrote.  With keys_out
+// (calls without a sort, small.cu) they write the slots' keys there themselves and latch errors for no call number.
 // ---- rescal.cu ----
 void launch_keys_rescal(ps_store* ps, const uint32_t* d_s, const uint32_t* d_r, const uint32_t* d_o,
                         const uint32_t* d_neg_ent, uint64_t n, uint32_t n_neg, uint64_t rel_key_base, uint32_t dim,
                         cudaStream_t s);
 uint32_t launch_grad_rescal(ps_store* ps, const uint32_t* d_s, const uint32_t* d_r, const uint32_t* d_o,
                             const uint32_t* d_neg_ent, const uint8_t* d_neg_side, uint64_t n, uint32_t n_neg,
-                            uint64_t rel_key_base, uint32_t dim, cudaStream_t s);
+                            uint64_t rel_key_base, uint32_t dim, uint32_t* keys_out, cudaStream_t s);
 void launch_keys_kge(ps_store* ps, const uint32_t* d_s, const uint32_t* d_r, const uint32_t* d_o,
                      const uint32_t* d_neg_ent, uint64_t n, uint32_t n_neg, uint64_t rel_key_base, cudaStream_t s);
 void launch_keys_sgns(ps_store* ps, const uint32_t* d_tokens, uint64_t tok_first, uint64_t first_pos,
                       uint64_t n_centers, uint64_t corpus_len, uint32_t window, const uint32_t* d_negs, uint32_t n_neg,
                       uint64_t out_key_base, cudaStream_t s);
 uint32_t launch_step_mf(ps_store* ps, const uint32_t* d_i, const uint32_t* d_j, const float* d_v, uint64_t n,
-                        uint64_t col_key_base, float lr, float lambda, cudaStream_t s);
+                        uint64_t col_key_base, float lr, float lambda, uint32_t* keys_out, cudaStream_t s);
 // grad_only: the update rows hold gradients (2 dim values each), to be reduced with run_kge_reduce
 uint32_t launch_step_kge(ps_store* ps, const uint32_t* d_s, const uint32_t* d_r, const uint32_t* d_o,
                          const uint32_t* d_neg_ent, const uint8_t* d_neg_side, uint64_t n, uint32_t n_neg,
-                         uint64_t rel_key_base, uint32_t dim, float lr, float eps, bool grad_only, cudaStream_t s);
+                         uint64_t rel_key_base, uint32_t dim, float lr, float eps, bool grad_only, uint32_t* keys_out,
+                         cudaStream_t s);
 float* sgns_scales(ps_store* ps, uint64_t n_centers);     // where launch_step_sgns puts the per-slot factors
 uint32_t launch_step_sgns(ps_store* ps, const uint32_t* d_tokens, uint64_t tok_first, uint64_t first_pos,
                           uint64_t n_centers, uint64_t corpus_len, uint32_t window, const uint32_t* d_negs,
-                          uint32_t n_neg, uint64_t out_key_base, float lr, cudaStream_t s);
+                          uint32_t n_neg, uint64_t out_key_base, float lr, uint32_t* keys_out, cudaStream_t s);
 
 // ---- device helpers ----
 #ifdef __CUDACC__

@@ -53,7 +53,7 @@ rescal_grad_kernel(const uint32_t* __restrict__ ts, const uint32_t* __restrict__
                    const uint32_t* __restrict__ neg_ent, const uint8_t* __restrict__ neg_side, uint64_t n,
                    uint32_t n_neg, uint64_t rel_base, uint32_t d, const float* __restrict__ store,
                    const uint2* __restrict__ table, uint64_t S, uint64_t K, float* __restrict__ grad,
-                   double* __restrict__ loss_partial) {
+                   uint32_t* __restrict__ keys_out, double* __restrict__ loss_partial, DevStatus* st) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double s_wl[kRescalThreads / 32];
     constexpr int kWarps = kRescalThreads / 32;
@@ -72,11 +72,21 @@ rescal_grad_kernel(const uint32_t* __restrict__ ts, const uint32_t* __restrict__
         if (lane < (int)n_ent) key = lane == 0 ? ts[t] : (lane == 1 ? to[t] : neg_ent[t * n_neg + (lane - 2)]);
         const uint32_t side = (lane >= 2 && lane < (int)n_ent) ? neg_side[t * n_neg + (lane - 2)] : 0u;
         const uint64_t rk = rel_base + (uint64_t)tr[t] * d; // key of row 0 of the matrix
-        if (__ballot_sync(full, lane < (int)n_ent && key >= rel_base) != 0u || rk + d > K) continue;   // (latched by the key kernel)
+        if (__ballot_sync(full, lane < (int)n_ent && key >= rel_base) != 0u || rk + d > K) {
+            if (keys_out) {                                 // (a call with a sort: latched by its key kernel)
+                if (lane == 0) latch_error(st, 0u, PS_ERR_KEY_RANGE);
+                for (uint32_t u = lane; u < n_slots; u += 32) keys_out[t * n_slots + u] = kSentinelPad;
+            }
+            continue;
+        }
         int rep = lane;                                     // first slot that holds the same key
         for (int z = 0; z < (int)n_ent; ++z) {
             const uint32_t kz = __shfl_sync(full, key, z);
             if (lane < (int)n_ent && kz == key && z < rep) rep = z;
+        }
+        if (keys_out) {
+            if (lane < (int)n_ent) keys_out[t * n_slots + lane] = rep == lane ? key : (uint32_t)K;
+            for (uint32_t a = lane; a < d; a += 32) keys_out[t * n_slots + n_ent + a] = (uint32_t)(rk + a);
         }
         uint64_t erow = 0;
         if (lane < (int)n_ent) erow = phys_row(table[key], S);
@@ -306,7 +316,7 @@ void launch_keys_rescal(ps_store* ps, const uint32_t* d_s, const uint32_t* d_r, 
 
 uint32_t launch_grad_rescal(ps_store* ps, const uint32_t* d_s, const uint32_t* d_r, const uint32_t* d_o,
                             const uint32_t* d_neg_ent, const uint8_t* d_neg_side, uint64_t n, uint32_t n_neg,
-                            uint64_t rel_key_base, uint32_t dim, cudaStream_t s) {
+                            uint64_t rel_key_base, uint32_t dim, uint32_t* keys_out, cudaStream_t s) {
     const size_t smem = rescal_smem(dim);
     (void)n_neg;
     // two blocks per SM, a warp per data point at a time
@@ -320,7 +330,7 @@ uint32_t launch_grad_rescal(ps_store* ps, const uint32_t* d_s, const uint32_t* d
         if (ps->prof) prof_before(ps, "rescal_grad_kernel<" #kE ">", s);                                            \
         rescal_grad_kernel<kE><<<grid, kRescalThreads, smem, s>>>(                                                  \
             d_s, d_r, d_o, d_neg_ent, d_neg_side, n, n_neg, rel_key_base, dim, (const float*)ps->store, ps->table,  \
-            ps->cfg.slots_per_part, ps->cfg.num_keys, (float*)ps->upd, ps->loss_partial);                          \
+            ps->cfg.slots_per_part, ps->cfg.num_keys, (float*)ps->upd, keys_out, ps->loss_partial, ps->status);    \
     } while (0)
     if (dim <= 32) RESCAL_LAUNCH(1);
     else if (dim <= 64) RESCAL_LAUNCH(2);

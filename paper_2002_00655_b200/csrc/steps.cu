@@ -56,7 +56,8 @@ __global__ void __launch_bounds__(256)
 mf_step_kernel(const uint32_t* __restrict__ ci, const uint32_t* __restrict__ cj, const float* __restrict__ cv,
                uint64_t n, uint64_t col_base, float lr, float lam, const float4* __restrict__ store,
                const uint2* __restrict__ table, uint64_t S, uint64_t K, uint32_t L4,
-               float4* __restrict__ upd, double* __restrict__ loss_partial, DevStatus* st, unsigned int epoch) {
+               float4* __restrict__ upd, uint32_t* __restrict__ keys_out, double* __restrict__ loss_partial,
+               DevStatus* st, unsigned int epoch) {
     const int lane = threadIdx.x & 31;
     const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint64_t n_warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
@@ -66,7 +67,9 @@ mf_step_kernel(const uint32_t* __restrict__ ci, const uint32_t* __restrict__ cj,
         const uint32_t i = ci[t], j = cj[t];
         const float v = cv[t];
         const uint64_t kw = i, kh = col_base + j;
-        if (kw >= col_base || kh >= K) {
+        const bool bad = kw >= col_base || kh >= K;
+        if (keys_out && lane < 2) keys_out[2 * t + lane] = bad ? kSentinelPad : (uint32_t)(lane ? kh : kw);
+        if (bad) {
             if (lane == 0) latch_error(st, epoch, PS_ERR_KEY_RANGE);
             continue;
         }
@@ -132,8 +135,8 @@ __global__ void __launch_bounds__(256)
 mf_step_small_kernel(const uint32_t* __restrict__ ci, const uint32_t* __restrict__ cj, const float* __restrict__ cv,
                      uint64_t n, uint64_t col_base, float lr, float lam, const float4* __restrict__ store,
                      const uint2* __restrict__ table, uint64_t S, uint64_t K, uint32_t L4,
-                     float4* __restrict__ upd, double* __restrict__ loss_partial, DevStatus* st,
-                     unsigned int epoch) {
+                     float4* __restrict__ upd, uint32_t* __restrict__ keys_out, double* __restrict__ loss_partial,
+                     DevStatus* st, unsigned int epoch) {
     const int lane = threadIdx.x & 31;
     const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint64_t n_warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
@@ -150,7 +153,9 @@ mf_step_small_kernel(const uint32_t* __restrict__ ci, const uint32_t* __restrict
             kw[c] = ok[c] ? ci[t] : 0;
             kh[c] = ok[c] ? col_base + cj[t] : 0;
             v[c] = ok[c] ? cv[t] : 0.f;
-            if (ok[c] && (kw[c] >= col_base || kh[c] >= K)) {
+            const bool bad = ok[c] && (kw[c] >= col_base || kh[c] >= K);
+            if (keys_out && ok[c] && lane < 2) keys_out[2 * t + lane] = bad ? kSentinelPad : (uint32_t)(lane ? kh[c] : kw[c]);
+            if (bad) {
                 if (lane == 0) latch_error(st, epoch, PS_ERR_KEY_RANGE);
                 ok[c] = false;
             }
@@ -195,13 +200,16 @@ mf_step_small_kernel(const uint32_t* __restrict__ ci, const uint32_t* __restrict
 }
 
 uint32_t launch_step_mf(ps_store* ps, const uint32_t* d_i, const uint32_t* d_j, const float* d_v, uint64_t n,
-                        uint64_t col_key_base, float lr, float lambda, cudaStream_t s) {
+                        uint64_t col_key_base, float lr, float lambda, uint32_t* keys_out, cudaStream_t s) {
     const uint32_t L4 = ps->cfg.row_len / 4;
     const uint32_t grid = step_grid(ps, n);
+    const uint32_t epoch = keys_out ? 0u : ps->epoch;
 #define MF_ARGS d_i, d_j, d_v, n, col_key_base, lr, lambda, (const float4*)ps->store, ps->table,                 \
-                ps->cfg.slots_per_part, ps->cfg.num_keys, L4, (float4*)ps->upd, ps->loss_partial,              \
-                ps->status, ps->epoch
-    if (L4 <= 32) PS_LAUNCH(ps, mf_step_small_kernel<4>, grid, 256, s, MF_ARGS);
+                ps->cfg.slots_per_part, ps->cfg.num_keys, L4, (float4*)ps->upd, keys_out, ps->loss_partial,    \
+                ps->status, epoch
+    // (a warp per cell for the calls without a sort: they do not fill the chip with four cells a warp)
+    if (L4 <= 32 && keys_out) PS_LAUNCH(ps, mf_step_small_kernel<1>, grid, 256, s, MF_ARGS);
+    else if (L4 <= 32) PS_LAUNCH(ps, mf_step_small_kernel<4>, grid, 256, s, MF_ARGS);
     else if (L4 <= 64) PS_LAUNCH(ps, mf_step_kernel<2>, grid, 256, s, MF_ARGS);
     else if (L4 <= 128) PS_LAUNCH(ps, mf_step_kernel<4>, grid, 256, s, MF_ARGS);
     else PS_LAUNCH(ps, mf_step_kernel<0>, grid, 256, s, MF_ARGS);
@@ -235,7 +243,7 @@ kge_step_kernel(const uint32_t* __restrict__ ts, const uint32_t* __restrict__ tr
                 const uint32_t* __restrict__ neg_ent, const uint8_t* __restrict__ neg_side, uint64_t n,
                 uint32_t n_neg_arg, uint64_t rel_base, uint32_t d_arg, float lr, float eps, const float* __restrict__ store,
                 const uint2* __restrict__ table, uint64_t S, uint64_t K, float* __restrict__ upd,
-                double* __restrict__ loss_partial, DevStatus* st, unsigned int epoch) {
+                uint32_t* __restrict__ keys_out, double* __restrict__ loss_partial, DevStatus* st, unsigned int epoch) {
     const int lane = threadIdx.x & 31;
     const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint64_t n_warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
@@ -263,6 +271,7 @@ kge_step_kernel(const uint32_t* __restrict__ ts, const uint32_t* __restrict__ tr
         }
         if (__any_sync(full, bad)) {
             if (lane == 0) latch_error(st, epoch, PS_ERR_KEY_RANGE);
+            if (keys_out && lane < n_slots) keys_out[t * n_slots + lane] = kSentinelPad;
             continue;
         }
         uint64_t off = 0;
@@ -272,6 +281,7 @@ kge_step_kernel(const uint32_t* __restrict__ ts, const uint32_t* __restrict__ tr
             const uint64_t kz = __shfl_sync(full, key, z);
             if (z < lane && kz == key) rep = z;
         }
+        if (keys_out && lane < n_slots) keys_out[t * n_slots + lane] = rep == lane ? (uint32_t)key : (uint32_t)K;
         const float* Srow = store + __shfl_sync(full, off, 0);
         const float* Rrow = store + __shfl_sync(full, off, 1);
         const float* Orow = store + __shfl_sync(full, off, 2);
@@ -455,11 +465,13 @@ kge_keys_kernel(const uint32_t* __restrict__ ts, const uint32_t* __restrict__ tr
 
 uint32_t launch_step_kge(ps_store* ps, const uint32_t* d_s, const uint32_t* d_r, const uint32_t* d_o,
                          const uint32_t* d_neg_ent, const uint8_t* d_neg_side, uint64_t n, uint32_t n_neg,
-                         uint64_t rel_key_base, uint32_t dim, float lr, float eps, bool grad_only, cudaStream_t s) {
+                         uint64_t rel_key_base, uint32_t dim, float lr, float eps, bool grad_only, uint32_t* keys_out,
+                         cudaStream_t s) {
     const uint32_t grid = step_grid(ps, n);
+    const uint32_t epoch = keys_out ? 0u : ps->epoch;
 #define KGE_ARGS d_s, d_r, d_o, d_neg_ent, d_neg_side, n, n_neg, rel_key_base, dim, lr, eps,                     \
                  (const float*)ps->store, ps->table, ps->cfg.slots_per_part, ps->cfg.num_keys, ps->upd,         \
-                 ps->loss_partial, ps->status, ps->epoch
+                 keys_out, ps->loss_partial, ps->status, epoch
 #define KGE_LAUNCH(kMaxNeg, kDim, kExact, kGrad)                                                                 \
     do {                                                                                                         \
         if (ps->prof) prof_before(ps, "kge_step_kernel<" #kMaxNeg ">", s);                                       \
@@ -518,8 +530,8 @@ __global__ void __launch_bounds__(256, 2)
 sgns_step_kernel(const uint32_t* __restrict__ tokens, uint64_t tok_first, uint64_t first_pos, uint64_t n_centers,
                  uint64_t T, uint32_t window_arg, const uint32_t* __restrict__ negs, uint32_t n_neg_arg, uint64_t out_base,
                  float lr, const float4* __restrict__ store, const uint2* __restrict__ table, uint64_t S, uint64_t K,
-                 uint32_t L4_arg, float4* __restrict__ upd, float* __restrict__ scales, double* __restrict__ loss_partial,
-                 DevStatus* st, unsigned int epoch) {
+                 uint32_t L4_arg, float4* __restrict__ upd, float* __restrict__ scales, uint32_t* __restrict__ keys_out,
+                 double* __restrict__ loss_partial, DevStatus* st, unsigned int epoch) {
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -542,6 +554,10 @@ sgns_step_kernel(const uint32_t* __restrict__ tokens, uint64_t tok_first, uint64
         float4* U = upd + cidx * 2 * L4;
         float* F = scales + cidx * slots;
         const uint32_t wtok = tokens[p - tok_first];
+        if (keys_out) {                                         // (slots of contexts cut off at the stream's ends: no key)
+            if (lane == 0) keys_out[cidx * slots] = wtok < out_base ? wtok : kSentinelPad;
+            for (uint32_t t = n_out + lane; t + 1 < slots; t += 32) keys_out[cidx * slots + 1 + t] = (uint32_t)K;
+        }
         if (wtok >= out_base) {
             if (lane == 0) latch_error(st, epoch, PS_ERR_KEY_RANGE);
             continue;
@@ -572,6 +588,7 @@ sgns_step_kernel(const uint32_t* __restrict__ tokens, uint64_t tok_first, uint64
                 } else {
                     bad = true;
                 }
+                if (keys_out) keys_out[cidx * slots + 1 + t] = my_ok ? (uint32_t)ku : kSentinelPad;
             }
             const unsigned ok_mask = __ballot_sync(full, my_ok);
             const uint32_t in_round = tmin<uint32_t>(32u, n_out - t0);
@@ -684,12 +701,13 @@ float* sgns_scales(ps_store* ps, uint64_t n_centers) { return ps->upd + n_center
 
 uint32_t launch_step_sgns(ps_store* ps, const uint32_t* d_tokens, uint64_t tok_first, uint64_t first_pos,
                           uint64_t n_centers, uint64_t corpus_len, uint32_t window, const uint32_t* d_negs,
-                          uint32_t n_neg, uint64_t out_key_base, float lr, cudaStream_t s) {
+                          uint32_t n_neg, uint64_t out_key_base, float lr, uint32_t* keys_out, cudaStream_t s) {
     const uint32_t L4 = ps->cfg.row_len / 4;
+    const uint32_t epoch = keys_out ? 0u : ps->epoch;
     const uint32_t grid = step_grid(ps, n_centers, 2);      // the kernels are bounded to two blocks per SM
 #define SG_ARGS d_tokens, tok_first, first_pos, n_centers, corpus_len, window, d_negs, n_neg, out_key_base, lr,   \
                 (const float4*)ps->store, ps->table, ps->cfg.slots_per_part, ps->cfg.num_keys, L4,              \
-                (float4*)ps->upd, sgns_scales(ps, n_centers), ps->loss_partial, ps->status, ps->epoch
+                (float4*)ps->upd, sgns_scales(ps, n_centers), keys_out, ps->loss_partial, ps->status, epoch
 #define SG_LAUNCH(kCh, kL4, kW, kN)                                                                                  \
     do {                                                                                                             \
         if (ps->prof) prof_before(ps, "sgns_step_kernel<" #kCh ">", s);                                              \
