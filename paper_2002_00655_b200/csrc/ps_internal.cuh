@@ -22,7 +22,7 @@ constexpr int kSortCtlWords = kMaxSortPasses * kRadix + kMaxSortPasses;   // dig
 constexpr int kReduceTile = 32;                  // sorted occurrences per warp in the segmented reduction
 constexpr int kGroupSpan = 64 * kReduceTile;      // sorted positions whose parked parts are pre-added together
 constexpr int kMaxLossBlocks = 4096;
-constexpr uint32_t kSmallOcc = 4096;             // calls of at most this many key occurrences are reduced without a sort (small.cu)
+constexpr uint32_t kSmallOcc = 8192;             // calls of at most this many key occurrences are reduced without a sort (small.cu)
 constexpr int kHostStages = 3;                   // staging areas for batches that arrive from host memory
 constexpr int kSortSets = 4;                     // calls whose key sort may be in flight at once (see SortSet)
 constexpr int kSideStreams = 3;                  // internal streams that calls with a long sort take in turn
@@ -253,6 +253,9 @@ void run_small_adagrad(ps_store* ps, uint32_t n, float lr, float eps, double* d_
 // table entry and row until run_localize_deferred, which the caller enqueues once that call is through.
 void run_localize(ps_store* ps, uint32_t worker, uint32_t n, int which, cudaStream_t s,
                   const uint32_t* busy_keys = nullptr, uint32_t n_busy = 0);
+// Few keys: the whole call, without a sort, in one launch on the caller's stream.
+bool localize_is_small(const ps_store* ps, uint64_t n);
+void run_localize_small(ps_store* ps, uint32_t worker, const uint64_t* d_keys, uint32_t n, cudaStream_t s);
 void run_localize_deferred(ps_store* ps, uint32_t worker, uint32_t n, cudaStream_t s);
 
 // ---- steps.cu ----

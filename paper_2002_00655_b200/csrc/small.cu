@@ -1,14 +1,15 @@
 // Calls of few key occurrences (kSmallOcc at most): the cumulative push without a sort.
 //
 // A push of a few thousand rows is a microsecond or two of memory traffic; sorted, it is a fork to another stream, a
-// cooperative sort with a grid barrier per pass, a reduction and a fix-up launch, 27 us of which the host spends 20
-// (push of 13 rows).  Here ONE launch does it: every block reads all keys of the call into shared memory (16 KB at
-// most), a warp takes one occurrence, compares its key with all the others (32 x 4 keys per instruction) and is done if
-// an earlier occurrence has the same key; otherwise the occurrence is the first of its key and the warp adds the rows of
-// all of them, in the order of the call, in fp64, and rounds once, as the sorted reduction does.  The comparison costs n^2 / 128
-// warp instructions in all, a microsecond at 4,096 keys, and twice the keys would cost four times that: the limit.
-// A key with more than kShortRun occurrences is shared by the block's warps (a range of the keys each, partial sums
-// added in range order), so one hot key costs n / 16 rows of latency and not n.
+// cooperative sort with a grid barrier per pass, a reduction and a fix-up launch: 27 us for 13 rows, of which the host
+// spends 20.  Here ONE launch does it.  Every block reads all keys of the call and keeps those of its hash bucket (a
+// dozen or two, in the order of the call: lane masks of the warps' shares, no sort), finds the first occurrence and the
+// number of occurrences of each in a table in shared memory, and a warp per distinct key adds its occurrences' rows in
+// the order of the call, in fp64, and rounds once, as the sorted reduction does.  A key with more than kShortRun
+// occurrences is shared by the block's warps (a range of the list each, partial sums added in range order).
+// What grows with the call is the reading of all keys by every block: kSmallOcc is where the sort takes over.
+// (A first form compared every occurrence with all others, 128 keys per instruction: 1,200 to 1,800 warp instructions
+// per occurrence, 11 us at 2,048 and 27 us at 3,328 occurrences of AdaGrad.)
 //
 // Training steps take the same launch after their gradient kernel, which leaves the key of every occurrence slot in
 // a buffer (num_keys: no key; all ones: an index out of range, the whole call is a no-op).
@@ -22,8 +23,14 @@ namespace {
 
 constexpr int kThreads = 512;
 constexpr int kWarps = kThreads / 32;
-constexpr uint32_t kShortRun = 64;              // occurrences of one key that a warp adds alone
-constexpr uint32_t kRange = kSmallOcc / kWarps; // keys per warp in the shared walk
+constexpr uint32_t kShortRun = 8;               // occurrences of one key that a warp adds alone
+constexpr int kTableBits = 10, kTable = 1 << kTableBits;
+static_assert(kSmallOcc <= 32 * kThreads, "a lane per round of the bucket's selection");
+
+// which of the blocks takes a key: a multiplicative hash, so that neighbouring keys (the frequent ones) are spread
+__device__ __forceinline__ uint32_t bucket_of(uint32_t key, uint32_t n_buckets) {
+    return (((key * 0x9e3779b1u) >> 16) * n_buckets) >> 16;
+}
 
 struct acc4 {
     double x, y, z, w;
@@ -51,36 +58,51 @@ struct SmallArgs {
 
 // kCh: float4 per lane; blockIdx.y counts stretches of 32 kCh float4 of the row
 template <int kMode, int kCh>
-__global__ void __launch_bounds__(kThreads) small_push_kernel(const SmallArgs A) {
-    __shared__ __align__(16) uint32_t s_key[kSmallOcc];
-    __shared__ uint16_t s_list[kWarps][kRange];
-    __shared__ uint32_t s_long[kWarps];         // the warp's occurrence starts a long run
+__global__ void __launch_bounds__(kThreads, kCh == 1 ? 2 : 1) small_push_kernel(const SmallArgs A) {
+    extern __shared__ __align__(16) uint32_t s_dyn[];
+    uint32_t* const s_key = s_dyn;                          // the bucket: keys of its occurrences, in the order of the call
+    uint16_t* const s_pos = reinterpret_cast<uint16_t*>(s_dyn + A.n);      // ... and their numbers
+    __shared__ uint32_t t_key[kTable], t_first[kTable], t_count[kTable];
+    __shared__ uint16_t s_firsts[kTable];
+    __shared__ uint32_t s_cnt[kWarps], s_n_firsts, s_over;
     __shared__ acc4 s_part[kWarps][32];
     constexpr int kHalves = kMode == kAdaGrad ? 2 : 1;      // AdaGrad: sums for the parameters and for their accumulators
+    constexpr int kFly = kCh == 1 ? 4 : (kCh == 2 && kMode != kAdaGrad ? 4 : 2) / (kCh == 4 ? 2 : 1);      // update rows a warp has in flight
     const unsigned full = 0xffffffffu;
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    const uint32_t n = A.n, K = A.K;
-    const uint32_t n_pad = (n + 127) & ~127u;
-    int bad = 0;
-    for (uint32_t i = tid; i < n_pad; i += kThreads) {
-        uint32_t k = K;
-        if (i < n) {
-            if (A.keys64) {
-                const uint64_t k64 = A.keys64[i];
-                bad |= k64 >= K;
-                k = (uint32_t)k64;
-            } else {
-                k = A.keys32[i];
-                bad |= k == kSentinelPad;
-            }
+    const uint32_t n = A.n, K = A.K, n_buckets = gridDim.x - 1, bucket = blockIdx.x;
+    auto key_at = [&](uint32_t i) -> uint32_t {             // kSentinelPad: out of range
+        if (A.keys64) {
+            const uint64_t k = A.keys64[i];
+            return k < K ? (uint32_t)k : kSentinelPad;
         }
-        s_key[i] = k;
+        return A.keys32[i];
+    };
+    // ---- the occurrences whose keys fall into this block's bucket; warp w looks at its 16th of the call ----
+    const uint32_t rounds = (n + kThreads - 1) / kThreads;  // at most 32: lane r keeps the bucket's lanes of round r
+    const uint32_t w0 = w * rounds * 32;
+    uint32_t mask_of = 0, cnt_w = 0;
+    int bad = 0;
+#pragma unroll 4
+    for (uint32_t r = 0; r < rounds; ++r) {
+        const uint32_t i = w0 + r * 32 + lane;
+        const uint32_t k = i < n ? key_at(i) : K;
+        bad |= k == kSentinelPad;
+        const unsigned m = __ballot_sync(full, k < K && bucket_of(k, n_buckets) == bucket);
+        if (lane == (int)r) mask_of = m;
+        cnt_w += __popc(m);
     }
+    if (lane == 0) s_cnt[w] = cnt_w;
+    for (int i = tid; i < kTable; i += kThreads) {
+        t_key[i] = t_first[i] = kSentinelPad;
+        t_count[i] = 0;
+    }
+    if (tid == 0) s_n_firsts = s_over = 0;
     if (__syncthreads_or(bad)) {                // the same decision in every block: nothing has been written yet
-        if (A.keys64 && blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) latch_error(A.st, 0u, PS_ERR_KEY_RANGE);
+        if (A.keys64 && bucket == 0 && blockIdx.y == 0 && tid == 0) latch_error(A.st, 0u, PS_ERR_KEY_RANGE);
         return;
     }
-    if (blockIdx.x == gridDim.x - 1) {          // the last block adds the loss partials: strided per thread, then a tree
+    if (bucket == n_buckets) {                  // the last block adds the loss partials: strided per thread, then a tree
         if (blockIdx.y != 0 || !A.loss_accum) return;
         double* ws = reinterpret_cast<double*>(s_part);
         double t = 0;
@@ -95,10 +117,53 @@ __global__ void __launch_bounds__(kThreads) small_push_kernel(const SmallArgs A)
         }
         return;
     }
+    uint32_t at = 0, m = 0;                     // where the warp's part of the list begins; the length of the list
+#pragma unroll
+    for (int i = 0; i < kWarps; ++i) {
+        if (i < w) at += s_cnt[i];
+        m += s_cnt[i];
+    }
+    if (m == 0) return;
+    if (cnt_w) {
+        for (unsigned some = __ballot_sync(full, mask_of != 0); some; some &= some - 1) {
+            const int r = __ffs(some) - 1;
+            const unsigned mk = __shfl_sync(full, mask_of, r);
+            if ((mk >> lane) & 1u) {
+                const uint32_t i = w0 + r * 32 + lane, to = at + __popc(mk & ((1u << lane) - 1u));
+                s_key[to] = key_at(i);
+                s_pos[to] = (uint16_t)i;
+            }
+            at += __popc(mk);
+        }
+    }
+    __syncthreads();
+    // ---- first occurrence and number of occurrences of every key of the bucket ----
+    auto probe = [&](uint32_t k) -> uint32_t { return (k * 0x85ebca6bu) >> (32 - kTableBits); };
+    for (uint32_t i = tid; i < m; i += kThreads) {
+        const uint32_t k = s_key[i];
+        uint32_t s = probe(k), tries = 0;
+        for (; tries < kTable; ++tries, s = (s + 1) & (kTable - 1)) {
+            const uint32_t was = atomicCAS(&t_key[s], kSentinelPad, k);
+            if (was == kSentinelPad || was == k) break;
+        }
+        if (tries == kTable) {
+            s_over = 1;
+        } else {
+            atomicMin(&t_first[s], i);
+            atomicAdd(&t_count[s], 1u);
+        }
+    }
+    __syncthreads();
+    const bool over = s_over != 0;              // more keys than the table has room for: a warp compares for itself, below
+    for (uint32_t i = tid; i < m && !over; i += kThreads) {
+        const uint32_t k = s_key[i];
+        uint32_t s = probe(k);
+        while (t_key[s] != k) s = (s + 1) & (kTable - 1);
+        if (t_first[s] == i) s_firsts[atomicAdd(&s_n_firsts, 1u)] = (uint16_t)s;
+    }
+    __syncthreads();
+    // ---- sums ----
     const uint32_t f0 = blockIdx.y * (32 * kCh) + lane;
-    const uint32_t t = blockIdx.x * kWarps + w;
-    const uint32_t my = t < n ? s_key[t] : K;
-    const bool usable = my < K;
     // one occurrence's update row: where it is, and what it is multiplied by
     auto source = [&](uint32_t o, float& sc) -> const float4* {
         sc = 1.f;
@@ -108,56 +173,6 @@ __global__ void __launch_bounds__(kThreads) small_push_kernel(const SmallArgs A)
             return A.upd + (uint64_t)(2u * e + (o != e * A.slots ? 1u : 0u)) * A.F4;
         }
         return A.upd + (uint64_t)o * A.F4;
-    };
-    // Asked for before the keys are compared, used after: the target row and this occurrence's own update.
-    float4 row[kHalves][kCh], own[kCh];
-    float own_sc = 1.f;
-    float4* target = A.store;
-    if (usable) {
-        target = A.store + phys_row(A.table[my], A.S) * A.L4;
-        const float4* u = source(t, own_sc);
-#pragma unroll
-        for (int c = 0; c < kCh; ++c) {
-            const uint32_t f = f0 + 32 * c;
-            own[c] = f < A.F4 ? u[f] : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-            for (int h = 0; h < kHalves; ++h)
-                row[h][c] = f < A.F4 ? target[h * A.F4 + f] : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-    }
-    bool earlier = false;
-    uint32_t same = 0;
-    const uint4* k4 = reinterpret_cast<const uint4*>(s_key);
-#pragma unroll 4
-    for (uint32_t b = 0; b < n_pad; b += 128) {
-        const uint4 q = k4[b / 4 + lane];
-        const uint32_t i = b + 4 * lane;
-        same += (q.x == my) + (q.y == my) + (q.z == my) + (q.w == my);
-        earlier |= (q.x == my && i < t) || (q.y == my && i + 1 < t) || (q.z == my && i + 2 < t) || (q.w == my && i + 3 < t);
-    }
-    same = __reduce_add_sync(full, same);
-    const bool first = usable && !__any_sync(full, earlier);
-    const bool is_long = first && same > kShortRun;
-    if (lane == 0) s_long[w] = is_long;
-    // positions of a key's occurrences among keys [lo, hi), ascending, into the warp's list; how many
-    auto find = [&](uint32_t key, uint32_t lo, uint32_t hi) -> uint32_t {
-        const unsigned lt = (1u << lane) - 1u;
-        uint32_t cnt = 0;
-        for (uint32_t b = lo; b < hi; b += 128) {
-            const uint32_t i = b + 4 * lane;
-            const uint4 q = i < hi ? k4[i / 4] : make_uint4(kSentinelPad, kSentinelPad, kSentinelPad, kSentinelPad);
-            const bool m0 = q.x == key, m1 = q.y == key, m2 = q.z == key, m3 = q.w == key;
-            const unsigned b0 = __ballot_sync(full, m0), b1 = __ballot_sync(full, m1), b2 = __ballot_sync(full, m2),
-                           b3 = __ballot_sync(full, m3);
-            uint32_t at = cnt + __popc(b0 & lt) + __popc(b1 & lt) + __popc(b2 & lt) + __popc(b3 & lt);
-            if (m0) s_list[w][at++] = (uint16_t)i;
-            if (m1) s_list[w][at++] = (uint16_t)(i + 1);
-            if (m2) s_list[w][at++] = (uint16_t)(i + 2);
-            if (m3) s_list[w][at++] = (uint16_t)(i + 3);
-            cnt += __popc(b0) + __popc(b1) + __popc(b2) + __popc(b3);
-        }
-        __syncwarp();
-        return cnt;
     };
     auto add = [&](acc4& a, const float4& u, double d) {
         if (kMode == kScaled) {
@@ -176,39 +191,83 @@ __global__ void __launch_bounds__(kThreads) small_push_kernel(const SmallArgs A)
         r.z = (float)((double)r.z + a.z); r.w = (float)((double)r.w + a.w);
         return r;
     };
-    // the warp's list summed into a[][], several occurrences' rows in flight; G: the accumulators before the call
-    auto sum_list = [&](uint32_t cnt, acc4 (*a)[kCh], const float4* G, int n_ch, uint32_t fa) {
-        constexpr int kFly = kCh == 4 ? 2 : 4;
-        for (uint32_t j = 0; j < cnt; j += kFly) {
-            float4 u[kFly][kCh];
-            float sc[kFly];
+    auto load_row = [&](const float4* target, float4 (*row)[kCh]) {
 #pragma unroll
-            for (int k = 0; k < kFly; ++k) {
-                const float4* p = source(s_list[w][j + k < cnt ? j + k : j], sc[k]);
+        for (int c = 0; c < kCh; ++c)
 #pragma unroll
-                for (int c = 0; c < kCh; ++c)
-                    u[k][c] = (c < n_ch && fa + 32 * c < A.F4) ? p[fa + 32 * c] : make_float4(0.f, 0.f, 0.f, 0.f);
-            }
+            for (int h = 0; h < kHalves; ++h)
+                row[h][c] = f0 + 32 * c < A.F4 ? target[h * A.F4 + f0 + 32 * c] : make_float4(0.f, 0.f, 0.f, 0.f);
+    };
+    // the occurrences of key k among list entries [lo, hi), in order, kFly rows in flight; G: the accumulators before the call
+    auto sum_range = [&](uint32_t k, uint32_t lo, uint32_t hi, acc4 (*a)[kCh], const float4* G) {
 #pragma unroll
-            for (int k = 0; k < kFly; ++k) {
-                if (j + k >= cnt) break;
-                const double d = (double)sc[k];
+        for (int h = 0; h < kHalves; ++h)
 #pragma unroll
-                for (int c = 0; c < kCh; ++c) {
-                    if (c >= n_ch) break;
-                    if (kMode == kAdaGrad) {
-                        float4 step, q;
-                        ada(u[k][c], G[c], step, q);
-                        add(a[0][c], step, d);
-                        add(a[kHalves - 1][c], q, d);
-                    } else {
-                        add(a[0][c], u[k][c], d);
+            for (int c = 0; c < kCh; ++c) a[h][c] = acc4{0.0, 0.0, 0.0, 0.0};
+        for (uint32_t b = lo; b < hi; b += 32) {
+            const uint32_t e = b + lane;
+            const bool hit = e < hi && s_key[e] == k;
+            const uint32_t mine = hit ? s_pos[e] : 0u;
+            unsigned todo = __ballot_sync(full, hit);
+            while (todo) {
+                float4 u[kFly][kCh];
+                float sc[kFly];
+                int got = 0;
+#pragma unroll
+                for (int q = 0; q < kFly; ++q) {
+                    const int src = todo ? __ffs(todo) - 1 : 0;
+                    if (todo) got = q + 1;
+                    todo &= todo - 1;                       // 0 stays 0
+                    const uint32_t o = __shfl_sync(full, mine, src);
+                    if (q < got) {
+                        const float4* p = source(o, sc[q]);
+#pragma unroll
+                        for (int c = 0; c < kCh; ++c)
+                            u[q][c] = f0 + 32 * c < A.F4 ? p[f0 + 32 * c] : make_float4(0.f, 0.f, 0.f, 0.f);
+                    }
+                }
+#pragma unroll
+                for (int q = 0; q < kFly; ++q) {
+                    if (q >= got) break;
+                    const double d = (double)sc[q];
+#pragma unroll
+                    for (int c = 0; c < kCh; ++c) {
+                        if (kMode == kAdaGrad) {
+                            float4 step, sq;
+                            ada(u[q][c], G[c], step, sq);
+                            add(a[0][c], step, d);
+                            add(a[kHalves - 1][c], sq, d);
+                        } else {
+                            add(a[0][c], u[q][c], d);
+                        }
                     }
                 }
             }
         }
     };
-    if (first && same == 1) {                   // most keys: the exact sum is rounded once in fp32
+    // a key whose occurrences one warp adds alone: entry i of the list is the first of `count`
+    auto one_key = [&](uint32_t i, uint32_t count) {
+        const uint32_t k = s_key[i];
+        float4* target = A.store + phys_row(A.table[k], A.S) * A.L4;
+        float4 row[kHalves][kCh];
+        if (count > 1) {
+            acc4 a[kHalves][kCh];
+            load_row(target, row);
+            sum_range(k, i & ~31u, m, a, row[kHalves - 1]);
+#pragma unroll
+            for (int c = 0; c < kCh; ++c)
+#pragma unroll
+                for (int h = 0; h < kHalves; ++h)
+                    if (f0 + 32 * c < A.F4) target[h * A.F4 + f0 + 32 * c] = finish(row[h][c], a[h][c]);
+            return;
+        }
+        // one occurrence (most keys): the exact sum is rounded once in fp32
+        float sc;
+        const float4* p = source(s_pos[i], sc);
+        float4 own[kCh];
+#pragma unroll
+        for (int c = 0; c < kCh; ++c) own[c] = f0 + 32 * c < A.F4 ? p[f0 + 32 * c] : make_float4(0.f, 0.f, 0.f, 0.f);
+        load_row(target, row);
 #pragma unroll
         for (int c = 0; c < kCh; ++c) {
             const uint32_t f = f0 + 32 * c;
@@ -222,75 +281,85 @@ __global__ void __launch_bounds__(kThreads) small_push_kernel(const SmallArgs A)
                 G.x += q.x; G.y += q.y; G.z += q.z; G.w += q.w;
                 target[A.F4 + f] = G;
             } else if (kMode == kScaled) {
-                r.x = fmaf(own_sc, u.x, r.x); r.y = fmaf(own_sc, u.y, r.y);
-                r.z = fmaf(own_sc, u.z, r.z); r.w = fmaf(own_sc, u.w, r.w);
+                r.x = fmaf(sc, u.x, r.x); r.y = fmaf(sc, u.y, r.y); r.z = fmaf(sc, u.z, r.z); r.w = fmaf(sc, u.w, r.w);
             } else {
                 r.x += u.x; r.y += u.y; r.z += u.z; r.w += u.w;
             }
             target[f] = r;
         }
-    } else if (first && !is_long) {
-        const uint32_t cnt = find(my, t & ~127u, n_pad);
+    };
+    if (over) {
+        for (uint32_t i = w; i < m; i += kWarps) {
+            const uint32_t k = s_key[i];
+            uint32_t before = 0, count = 0;
+            for (uint32_t e = lane; e < m; e += 32) {
+                before += s_key[e] == k && e < i;
+                count += s_key[e] == k;
+            }
+            if (!__any_sync(full, before != 0)) one_key(i, __reduce_add_sync(full, count));
+        }
+        return;
+    }
+    const uint32_t n_firsts = s_n_firsts;
+    bool any_long = false;
+    for (uint32_t j = 0; j < n_firsts; ++j) {
+        const uint32_t s = s_firsts[j], count = t_count[s];
+        if (count > kShortRun) any_long = true;
+        else if (j % kWarps == (uint32_t)w) one_key(t_first[s], count);
+    }
+    if (!any_long) return;                      // the same decision in every warp
+    // ---- keys with many occurrences: the whole block on one at a time, a range of the list per warp ----
+    const uint32_t per = (m + kWarps - 1) / kWarps, lo = tmin<uint32_t>(w * per, m), hi = tmin<uint32_t>(lo + per, m);
+    for (uint32_t j = 0; j < n_firsts; ++j) {
+        const uint32_t s = s_firsts[j];
+        if (t_count[s] <= kShortRun) continue;
+        const uint32_t k = t_key[s];
+        float4* target = A.store + phys_row(A.table[k], A.S) * A.L4;
+        float4 row[kHalves][kCh];
         acc4 a[kHalves][kCh];
+        load_row(target, row);
+        sum_range(k, lo, hi, a, row[kHalves - 1]);
 #pragma unroll
         for (int h = 0; h < kHalves; ++h)
 #pragma unroll
-            for (int c = 0; c < kCh; ++c) a[h][c] = acc4{0.0, 0.0, 0.0, 0.0};
-        sum_list(cnt, a, row[kHalves - 1], kCh, f0);
-#pragma unroll
-        for (int c = 0; c < kCh; ++c) {
-            const uint32_t f = f0 + 32 * c;
-            if (f >= A.F4) continue;
-#pragma unroll
-            for (int h = 0; h < kHalves; ++h) target[h * A.F4 + f] = finish(row[h][c], a[h][c]);
-        }
-    }
-    __syncthreads();
-    for (int j = 0; j < kWarps; ++j) {          // long runs: the whole block on one key at a time
-        if (!s_long[j]) continue;               // the same decision in every warp
-        const uint32_t key = s_key[blockIdx.x * kWarps + j];
-        float4* dst = A.store + phys_row(A.table[key], A.S) * A.L4;
-        const uint32_t lo = tmin<uint32_t>(w * kRange, n_pad), hi = tmin<uint32_t>(lo + kRange, n_pad);
-        const uint32_t cnt = find(key, lo, hi);
-        for (int c = 0; c < kCh; ++c) {
-            const uint32_t f = f0 + 32 * c;
-            float4 r[kHalves];
-#pragma unroll
-            for (int h = 0; h < kHalves; ++h) r[h] = f < A.F4 ? dst[h * A.F4 + f] : make_float4(0.f, 0.f, 0.f, 0.f);
-            acc4 a[kHalves][kCh];
-#pragma unroll
-            for (int h = 0; h < kHalves; ++h) a[h][0] = acc4{0.0, 0.0, 0.0, 0.0};
-            sum_list(cnt, a, r + kHalves - 1, 1, f);
-#pragma unroll
-            for (int h = 0; h < kHalves; ++h) {
-                s_part[w][lane] = a[h][0];
+            for (int c = 0; c < kCh; ++c) {
+                s_part[w][lane] = a[h][c];
                 __syncthreads();                // (every warp has read the row by now)
-                if (w == 0 && f < A.F4) {
+                if (w == 0 && f0 + 32 * c < A.F4) {
                     acc4 tot = s_part[0][lane];
 #pragma unroll
                     for (int i = 1; i < kWarps; ++i) {
                         tot.x += s_part[i][lane].x; tot.y += s_part[i][lane].y;
                         tot.z += s_part[i][lane].z; tot.w += s_part[i][lane].w;
                     }
-                    dst[h * A.F4 + f] = finish(r[h], tot);
+                    target[h * A.F4 + f0 + 32 * c] = finish(row[h][c], tot);
                 }
                 __syncthreads();
             }
-        }
     }
 }
 
+template <int kMode, int kCh>
+void launch_as(ps_store* ps, const SmallArgs& a, uint32_t strips, cudaStream_t s) {
+    // about a dozen occurrences per block of 16 warps, two blocks per SM at most (more would only read the keys again)
+    const uint32_t buckets = tmax<uint32_t>(1u, tmin<uint32_t>(div_up_u32(a.n, 12), (uint32_t)ps->sm_count * 2 - 1));
+    const size_t smem = ((size_t)a.n * 6 + 15) & ~(size_t)15;
+    static std::atomic<unsigned long long> smem_set{0};
+    opt_in_smem((const void*)small_push_kernel<kMode, kCh>, (size_t)kSmallOcc * 6, &smem_set);
+    if (ps->prof) prof_before(ps, kMode == kAdaGrad ? "small_push_kernel<adagrad>" : kMode == kScaled ? "small_push_kernel<scaled>" : "small_push_kernel", s);
+    small_push_kernel<kMode, kCh><<<dim3(buckets + 1, div_up_u32(strips, kCh)), kThreads, smem, s>>>(a);
+    if (ps->prof) prof_after(ps, s);
+    ps->launches++;
+}
 template <int kMode>
 void launch(ps_store* ps, const SmallArgs& a, cudaStream_t s) {
     const uint32_t strips = div_up_u32(a.F4, 32);
-    const uint32_t bx = div_up_u32(a.n, kWarps) + 1;
     // Few rows: a warp per 32 float4, for latency.  Once that is more than about two waves of warps the
-    // comparison of the keys, done anew for every stretch of columns, should serve more of the row.
+    // selection of the bucket, done anew for every stretch of columns, should serve more of the row.
     const bool narrow = strips == 1 || (uint64_t)a.n * strips <= (uint64_t)ps->sm_count * kWarps * 4;
-    if (narrow) PS_LAUNCH(ps, (small_push_kernel<kMode, 1>), dim3(bx, strips), kThreads, s, a);
-    else if (strips == 2) PS_LAUNCH(ps, (small_push_kernel<kMode, 2>), dim3(bx, 1), kThreads, s, a);
-    else if (kMode == kAdaGrad) PS_LAUNCH(ps, (small_push_kernel<kMode, 2>), dim3(bx, div_up_u32(strips, 2)), kThreads, s, a);
-    else PS_LAUNCH(ps, (small_push_kernel<kMode, kMode == kAdaGrad ? 2 : 4>), dim3(bx, div_up_u32(strips, 4)), kThreads, s, a);
+    if (narrow) launch_as<kMode, 1>(ps, a, strips, s);
+    else if (kMode == kAdaGrad || strips == 2) launch_as<kMode, 2>(ps, a, strips, s);
+    else launch_as<kMode, kMode == kAdaGrad ? 2 : 4>(ps, a, strips, s);
 }
 
 SmallArgs common(ps_store* ps, uint32_t n, double* d_loss_accum, uint32_t loss_blocks) {

@@ -1,0 +1,96 @@
+"""GPU parity of the calls that are reduced without a sort (few key occurrences): sizes around the limits of that path,
+hot keys that a whole block adds up, rows of one to many stretches of columns, bad indexes."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2002_00655_b200 as ps
+from synth import workloads as W
+from tests.util import close, compare_state, dev, make_pair
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("L", [4, 100, 132, 512, 520, 4100])
+@pytest.mark.parametrize("n,hot", [(1, 0.0), (12, 0.0), (13, 1.0), (513, 0.3), (4096, 0.05), (8191, 0.9), (8192, 0.0), (8193, 0.0)])
+def test_small_push_is_exact_on_integers(n, hot, L):
+    K = 5000 if L < 500 else 700
+    g, o = make_pair(K, L, 3, max_batch_keys=n)
+    rng = np.random.default_rng(n + L)
+    rows = rng.integers(-100, 100, size=(K, L)).astype(np.float32)
+    g.set_all_rows(torch.from_numpy(rows))
+    o.set_rows(np.arange(K), rows)
+    keys = rng.integers(0, K, size=n)
+    keys[rng.random(n) < hot] = K // 2
+    keys[-1] = K - 1
+    upd = rng.integers(-4, 5, size=(n, L)).astype(np.float32)     # integers: sums are exact in any order
+    g.push(dev(keys), dev(upd))
+    o.push(keys, upd)
+    g.sync()
+    compare_state(g, o, exact_rows=True, what="small push")
+    if n > 1:
+        keys[n // 2] = K                                           # one bad key: the call changes nothing
+        g.push(dev(keys), dev(upd))
+        assert g.sync(check=False) == ps.PS_ERR_KEY_RANGE
+        compare_state(g, o, exact_rows=True, what="small push with a bad key")
+
+
+def test_small_push_with_more_keys_in_one_bucket_than_its_table_holds():
+    """Keys whose hash puts them all into the same block: the table overflows and warps compare for themselves."""
+    K, L, n = 2_000_000, 4, 8000
+    k = np.arange(K, dtype=np.uint64)
+    h = ((k * 0x9E3779B1) & 0xFFFFFFFF) >> 16
+    keys = k[h < 0x10000 // 400].astype(np.int64)[:n - 500]        # the lowest 1/400 of the hash range: one block of 295
+    assert len(keys) > 3000
+    g, o = make_pair(K, L, 1, max_batch_keys=n)
+    rng = np.random.default_rng(5)
+    keys = np.concatenate([keys, keys[rng.integers(0, len(keys), size=500)]])
+    rng.shuffle(keys)
+    upd = rng.integers(-4, 5, size=(len(keys), L)).astype(np.float32)
+    g.push(dev(keys), dev(upd))
+    o.push(keys, upd)
+    g.sync()
+    compare_state(g, o, exact_rows=True, what="overflowing bucket")
+
+
+@pytest.mark.parametrize("n,dim,n_neg", [(1, 1, 1), (40, 7, 3), (64, 100, 10), (300, 12, 20), (20, 132, 4), (9, 1000, 29)])
+def test_small_complex_steps(n, dim, n_neg):
+    cfg = W.scaled(W.KGE_TINY, entities=300, dim=dim, n_neg=n_neg, batch=n, n_triples=4 * n)
+    rows = W.kge_init_rows(cfg, 0, cfg.num_keys, "cpu")
+    rows[:, 2 * dim:] = rows[:, :2 * dim].square() + 0.01           # accumulators some way into training
+    g, o = make_pair(cfg.num_keys, cfg.row_len, 2, rows=rows, max_batch_keys=(3 + n_neg) * n)
+    for b in range(3):
+        s, r, ob, ne, ns = W.kge_triples(cfg, b * n, n, "cpu")
+        args = (cfg.rel_key_base, dim, cfg.lr, cfg.eps)
+        ps.ps_step_kge(g.h, s.cuda(), r.cuda(), ob.cuda(), ne.cuda(), ns.cuda(), n_neg, *args, g.loss)
+        o.step_kge(s, r, ob, ne, ns, *args)
+    g.sync()
+    compare_state(g, o, what="small complex steps")
+    assert close(float(g.loss.cpu()[0]), o.loss[0])
+    ne[0, 0] = cfg.entities                                         # out of range: a no-op, loss included
+    before = float(g.loss.cpu()[0])
+    ps.ps_step_kge(g.h, s.cuda(), r.cuda(), ob.cuda(), ne.cuda(), ns.cuda(), n_neg, *args, g.loss)
+    assert g.sync(check=False) == ps.PS_ERR_KEY_RANGE
+    compare_state(g, o, what="small complex step with a bad index")
+    assert float(g.loss.cpu()[0]) == before
+
+
+@pytest.mark.parametrize("N,L,counts", [(8, 128, (1, 7, 600, 2047, 2048, 2049)), (1500, 4, (5, 700, 2048, 2500, 4000)),
+                                        (3, 256, (2048, 1, 2049, 1025))])
+def test_localize_around_the_limit_of_the_single_launch(N, L, counts):
+    K = 30_000
+    g, o = make_pair(K, L, N, 2 * -(-K // N) + 4200, max_batch_keys=4000)
+    rng = np.random.default_rng(N)
+    for it, m in enumerate(counts * 2):
+        w = int(rng.integers(0, N))
+        keys = (rng.zipf(1.2, size=m) - 1) % K if it % 2 else rng.integers(0, K, size=m)
+        g.localize(w, dev(keys))
+        o.localize(w, keys)
+        g.sync()
+        compare_state(g, o, exact_rows=True, what=f"localize of {m}")
+        upd = rng.integers(-2, 3, size=(m, L)).astype(np.float32)
+        g.push(dev(keys), dev(upd))
+        o.push(keys, upd)
+    g.localize(0, dev(np.array([3, K])))
+    assert g.sync(check=False) == ps.PS_ERR_KEY_RANGE
+    compare_state(g, o, exact_rows=True, what="bad key")
