@@ -467,6 +467,156 @@ loc_fused_kernel(const uint32_t* __restrict__ sk, uint32_t n, uint32_t span, uin
     grid_leave(bar, G);
 }
 
+// ------------------------------------------------------------------------------------------------
+// Few keys (kLocSmallKeys at most, kLocSmallBytes of rows): the whole call, sort included, as ONE launch of one cluster
+// of eight blocks.  With the cooperative sort and the launch above, 600 keys took 30 us of which nearly all was grid
+// barriers and launches; here the blocks meet once, at the cluster's own barrier.
+// Every block reads all keys, drops repeats with a hash table in shared memory and looks the others up; no order is needed
+// beyond what counting gives: a moving key's place among the moving keys (= its slot from the top of the requester's
+// stack) is the number of smaller moving keys, its place on its old owner's stack the number of smaller ones
+// with that owner.  A block counts for its eighth of the keys, kLocSmallThreads / (n / 8) threads per key; the n^2 / 8
+// comparisons per block are what kLocSmallKeys limits (a microsecond at 1,024 keys, six at 2,048).
+// Nothing is written before every block has read what it needs (cluster barrier), and each block then moves its own keys.
+constexpr int kLocSmallThreads = 1024;
+constexpr uint32_t kLocSmallBlocks = 8;
+constexpr uint32_t kLocSmallKeys = 2048;
+constexpr uint64_t kLocSmallBytes = 2u << 20;       // eight SMs move this in about 4 us; more is better spread over the chip
+constexpr int kLocTableBits = 12;
+constexpr size_t kLocSmallSmem = ((size_t)kLocSmallKeys * 2 + ((size_t)2 << kLocTableBits)) * 4;
+
+__global__ void __cluster_dims__(kLocSmallBlocks, 1, 1) __launch_bounds__(kLocSmallThreads)
+loc_small_kernel(const uint64_t* __restrict__ keys, uint32_t n, uint2* table, uint32_t worker, uint64_t S, uint32_t K,
+                 unsigned long long* tops, uint32_t* stacks, float4* store, uint32_t L4, uint32_t part_size, DevStatus* st) {
+    constexpr uint32_t kSlots = 1u << kLocTableBits, kPer = kLocSmallKeys / kLocSmallThreads;
+    extern __shared__ __align__(16) uint32_t loc_dyn[];
+    uint32_t* const s_key = loc_dyn;                        // per position of the call: the key if it moves, else kSentinelPad
+    uint32_t* const s_own = s_key + kLocSmallKeys;          // ... and its old owner
+    uint32_t* const t_key = s_own + kLocSmallKeys;
+    uint32_t* const t_first = t_key + kSlots;
+    __shared__ uint32_t s_src[kLocSmallKeys / kLocSmallBlocks][2], s_dst[kLocSmallKeys / kLocSmallBlocks];
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const uint32_t b = blockIdx.x;
+    const unsigned long long top_w = tops[worker];
+    uint32_t key[kPer], slot_of[kPer];
+    int bad = 0;
+#pragma unroll
+    for (uint32_t q = 0; q < kPer; ++q) {
+        const uint32_t i = q * kLocSmallThreads + tid;
+        const uint64_t k = i < n ? keys[i] : (uint64_t)kSentinelPad;
+        bad |= i < n && k >= K;
+        key[q] = i < n ? (uint32_t)k : kSentinelPad;
+    }
+    for (uint32_t i = tid; i < kSlots; i += kLocSmallThreads) t_key[i] = t_first[i] = kSentinelPad;
+    if (__syncthreads_or(bad)) {                            // the same decision in every block: nothing has been written
+        if (b == 0 && tid == 0) latch_error(st, 0u, PS_ERR_KEY_RANGE);
+        return;
+    }
+#pragma unroll
+    for (uint32_t q = 0; q < kPer; ++q) {
+        const uint32_t i = q * kLocSmallThreads + tid;
+        if (i >= n) continue;
+        uint32_t s = (key[q] * 0x85ebca6bu) >> (32 - kLocTableBits);
+        for (uint32_t tries = 0; tries < kSlots; ++tries, s = (s + 1) & (kSlots - 1)) {    // (half the slots stay empty)
+            const uint32_t was = atomicCAS(&t_key[s], kSentinelPad, key[q]);
+            if (was == kSentinelPad || was == key[q]) break;
+        }
+        atomicMin(&t_first[s], i);
+        slot_of[q] = s;
+    }
+    __syncthreads();
+    uint32_t total = 0, local = 0;
+#pragma unroll
+    for (uint32_t q = 0; q < kPer; ++q) {
+        const uint32_t i = q * kLocSmallThreads + tid;
+        const bool first = i < n && t_first[slot_of[q]] == i;
+        const uint32_t own = first ? table[key[q]].x : kSentinelPad;
+        const bool moves = first && own != worker;
+        s_key[i] = moves ? key[q] : kSentinelPad;
+        s_own[i] = moves ? own : kSentinelPad;
+        total += (uint32_t)__syncthreads_count(moves);
+        local += (uint32_t)__syncthreads_count(first && !moves);
+    }
+    if ((unsigned long long)total > top_w) {                // the same decision in every block
+        if (b == 0 && tid == 0) latch_error(st, 0u, PS_ERR_CAPACITY);
+        return;
+    }
+    // ---- the block's eighth of the positions, T neighbouring lanes per position ----
+    const uint32_t share = (n + kLocSmallBlocks - 1) / kLocSmallBlocks;
+    uint32_t T = 1;
+    while (T < 32 && share * T * 2 <= kLocSmallThreads) T <<= 1;
+    const uint32_t mine = tid / T, sub = tid % T, i = b * share + mine;
+    const bool have = mine < share && i < n;
+    const uint32_t k = have ? s_key[i] : kSentinelPad, o = have ? s_own[i] : kSentinelPad;
+    const bool moves = k != kSentinelPad;
+    uint32_t m = 0, r = 0, c = 0;                           // smaller moving keys; those of the same owner; all of that owner
+    if (moves) {
+        const uint4* k4 = reinterpret_cast<const uint4*>(s_key);
+        const uint4* o4 = reinterpret_cast<const uint4*>(s_own);
+        for (uint32_t j = sub; j < (n + 3) / 4; j += T) {
+            const uint4 a = k4[j], p = o4[j];
+            const uint32_t l0 = a.x < k, l1 = a.y < k, l2 = a.z < k, l3 = a.w < k;
+            const uint32_t e0 = p.x == o, e1 = p.y == o, e2 = p.z == o, e3 = p.w == o;
+            m += l0 + l1 + l2 + l3;
+            c += e0 + e1 + e2 + e3;
+            r += (l0 & e0) + (l1 & e1) + (l2 & e2) + (l3 & e3);
+        }
+    }
+    for (uint32_t d = T / 2; d; d >>= 1) {
+        m += __shfl_xor_sync(0xffffffffu, m, d);
+        r += __shfl_xor_sync(0xffffffffu, r, d);
+        c += __shfl_xor_sync(0xffffffffu, c, d);
+    }
+    const bool lead = moves && sub == 0;
+    uint32_t new_slot = 0, old_slot = 0;
+    unsigned long long top_o = 0;
+    if (lead) {
+        new_slot = stacks[(uint64_t)worker * S + (top_w - 1 - m)];
+        old_slot = table[k].y;
+        top_o = tops[o];
+        s_src[mine][0] = o;
+        s_src[mine][1] = old_slot;
+        s_dst[mine] = new_slot;
+    } else if (sub == 0 && mine < share) {
+        s_dst[mine] = kSentinelPad;
+    }
+    const uint32_t again = (uint32_t)__syncthreads_count(lead && o != k / part_size);      // it had left its initial partition before
+    asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+    if (lead) {
+        table[k] = make_uint2(worker, new_slot);
+        stacks[(uint64_t)o * S + top_o + r] = old_slot;
+        if (r + 1 == c) tops[o] = top_o + c;                // one thread per old owner; never the requester
+    }
+    if (tid == 0) {
+        if (again) atomicAdd(&st->loc_moved_again, (unsigned long long)again);
+        if (b == 0) {
+            tops[worker] = top_w - total;
+            st->moved_total = total;
+            st->deferred_now = 0u;
+            st->rows_moved += total;
+            st->loc_requested += n;
+            st->loc_already_local += local;
+        }
+    }
+    for (uint32_t e = w; e < share; e += kLocSmallThreads / 32) {
+        if (s_dst[e] == kSentinelPad) continue;
+        const float4* src = store + ((uint64_t)s_src[e][0] * S + s_src[e][1]) * L4;
+        float4* dst = store + ((uint64_t)worker * S + s_dst[e]) * L4;
+        for (uint32_t f = lane; f < L4; f += 32) dst[f] = src[f];
+    }
+}
+
+bool localize_is_small(const ps_store* ps, uint64_t n) {
+    return n <= kLocSmallKeys && n * ps->cfg.row_len * 4 <= kLocSmallBytes;
+}
+
+void run_localize_small(ps_store* ps, uint32_t worker, const uint64_t* d_keys, uint32_t n, cudaStream_t s) {
+    static std::atomic<unsigned long long> smem_set{0};
+    opt_in_smem((const void*)loc_small_kernel, kLocSmallSmem, &smem_set);
+    PS_LAUNCH_SMEM(ps, loc_small_kernel, kLocSmallBlocks, kLocSmallThreads, kLocSmallSmem, s, d_keys, n, ps->table, worker,
+                   ps->cfg.slots_per_part, (uint32_t)ps->cfg.num_keys, ps->tops, ps->stacks, (float4*)ps->store,
+                   ps->cfg.row_len / 4, div_up_u32(ps->cfg.num_keys, ps->cfg.num_workers), ps->status);
+}
+
 // Second half of a relocation that ran beside another call: the moving keys that call touched (flag[m] = 1) get
 // their rows moved and their table entries rewritten now that it is through.
 __global__ void __launch_bounds__(256)

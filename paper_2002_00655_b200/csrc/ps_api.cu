@@ -150,6 +150,17 @@ static void alternate_side(ps_store* ps) {
 // Ordered mode: the side stream starts after everything already enqueued on the caller's stream.
 // Pipelined mode: it starts as soon as the buffer set's previous user is done, i.e. beside the previous
 // step's kernels; the batch arrays must then be complete when the call is made.
+// A new graph capture (or the end of one): events recorded on the other side of that border cannot be waited on.
+static bool note_capture(ps_store* ps, cudaStream_t s, unsigned long long* id) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamGetCaptureInfo(s, &cs, id) != cudaSuccess) return false;
+    if (cs != cudaStreamCaptureStatusActive) *id = 0;
+    if (*id != ps->capture_id) {
+        ps->capture_id = *id;
+        for (int b = 0; b < kSortSets; ++b) ps->sets[b].used = false;
+    }
+    return true;
+}
 static bool fork_side(ps_store* ps, SortSet* ss, cudaStream_t s, bool reads_table = false) {
     // for a relocation that may be asked to run beside this call (ps_localize_beside): everything earlier ends here
     ss->sorted_which = -1;
@@ -166,14 +177,8 @@ static bool fork_side(ps_store* ps, SortSet* ss, cudaStream_t s, bool reads_tabl
         ps->batch_ready = nullptr;
         if (cudaStreamWaitEvent(ps->side, ev, 0) != cudaSuccess) return false;
     }
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     unsigned long long id = 0;
-    if (cudaStreamGetCaptureInfo(s, &cs, &id) != cudaSuccess) return false;
-    if (cs != cudaStreamCaptureStatusActive) id = 0;
-    if (id != ps->capture_id) {
-        ps->capture_id = id;
-        for (int b = 0; b < kSortSets; ++b) ps->sets[b].used = false;
-    }
+    if (!note_capture(ps, s, &id)) return false;
     const bool crossed = id != ps->side_capture_id[ps->side_idx];       // this side stream is still on the other side
     ps->side_capture_id[ps->side_idx] = id;
     // a sort that reads the location table (the matrix-factorization records) must come after a call that rewrote it
@@ -186,12 +191,26 @@ static bool fork_side(ps_store* ps, SortSet* ss, cudaStream_t s, bool reads_tabl
 static bool join_side(ps_store* ps, cudaStream_t s) {
     return cudaEventRecord(ps->ev_join, ps->side) == cudaSuccess && cudaStreamWaitEvent(s, ps->ev_join, 0) == cudaSuccess;
 }
-// after the call's sort has been enqueued on the side stream: where its sorted keys are, for ps_localize_beside
-static bool sorted_keys_at(ps_store* ps, SortSet* ss, int which, uint32_t n) {
+// Where the sort of a call runs that has nothing to do beside it (push, localize, the matrix-factorization step): on a
+// side stream in pipelined mode, on the caller's own stream in ordered mode.  There it would only wait for that stream
+// and be waited for: four event calls on the host and two hops between streams on the device for nothing.
+static bool begin_sort(ps_store* ps, SortSet* ss, cudaStream_t s, bool reads_table, cudaStream_t* where) {
+    *where = ps->side;
+    if (ps->pipelined) return fork_side(ps, ss, s, reads_table);
+    *where = s;
+    ss->sorted_which = -1;
+    ss->loc_reader = false;                         // (s waits for every earlier relocation, and for a batch still being copied)
+    ps->batch_ready = nullptr;
+    unsigned long long id = 0;
+    return cudaEventRecord(ps->ev_before, s) == cudaSuccess && note_capture(ps, s, &id);
+}
+static bool end_sort(ps_store* ps, cudaStream_t s, cudaStream_t where) { return where == s || join_side(ps, s); }
+// after the call's sort has been enqueued: where its sorted keys are, for ps_localize_beside
+static bool sorted_keys_at(ps_store* ps, SortSet* ss, int which, uint32_t n, cudaStream_t where) {
     ss->sorted_which = which;
     ss->sorted_n = n;
     ps->last_set = ss;
-    return cudaEventRecord(ps->ev_sorted, ps->side) == cudaSuccess;
+    return cudaEventRecord(ps->ev_sorted, where) == cudaSuccess;
 }
 // after the last kernel of a call that used the set
 static ps_status_t release_set(SortSet* ss, cudaStream_t s) {
@@ -431,10 +450,10 @@ ps_status_t ps_push(ps_store_t* ps, const uint64_t* d_keys, uint64_t n, const fl
         return after_launch();
     }
     SortSet* ss = next_set(ps);
-    if (!fork_side(ps, ss, s)) return PS_ERR_CUDA;         // the keys are sorted beside earlier calls' kernels
-    const int which = radix_sort_keys64(ps, d_keys, (uint32_t)n, ps->side, ps->starter_count,
-                                        div_up_u32(n, kGroupSpan));
-    if (!sorted_keys_at(ps, ss, which, (uint32_t)n) || !join_side(ps, s)) return PS_ERR_CUDA;
+    cudaStream_t q;
+    if (!begin_sort(ps, ss, s, false, &q)) return PS_ERR_CUDA;  // pipelined: the keys are sorted beside earlier calls' kernels
+    const int which = radix_sort_keys64(ps, d_keys, (uint32_t)n, q, ps->starter_count, div_up_u32(n, kGroupSpan));
+    if (!sorted_keys_at(ps, ss, which, (uint32_t)n, q) || !end_sort(ps, s, q)) return PS_ERR_CUDA;
     run_push_reduce(ps, (uint32_t)n, which, d_updates, nullptr, 0, s);
     return release_set(ss, s);
 }
@@ -445,12 +464,18 @@ ps_status_t ps_localize(ps_store_t* ps, uint32_t worker, const uint64_t* d_keys,
     if (n == 0) return PS_OK;
     if (!d_keys) return PS_ERR_INVALID_ARG;
     if (n > ps->max_keys) return PS_ERR_WORKSPACE;
+    if (localize_is_small(ps, n)) {
+        run_localize_small(ps, worker, d_keys, (uint32_t)n, s);
+        for (int b = 0; b < kSideStreams; ++b) ps->table_dirty[b] = true;
+        return after_launch();
+    }
     // stores of more than 1024 partitions: one block scans the call's per-chunk counts in shared memory
     if (n > (1u << 20) && ps->cfg.num_workers > 1024) return PS_ERR_UNSUPPORTED;
     SortSet* ss = next_set(ps);
-    if (!fork_side(ps, ss, s)) return PS_ERR_CUDA;
-    const int which = radix_sort_keys64(ps, d_keys, (uint32_t)n, ps->side, nullptr, 0);
-    if (!join_side(ps, s)) return PS_ERR_CUDA;
+    cudaStream_t q;
+    if (!begin_sort(ps, ss, s, false, &q)) return PS_ERR_CUDA;
+    const int which = radix_sort_keys64(ps, d_keys, (uint32_t)n, q, nullptr, 0);
+    if (!end_sort(ps, s, q)) return PS_ERR_CUDA;
     run_localize(ps, worker, (uint32_t)n, which, s);
     for (int b = 0; b < kSideStreams; ++b) ps->table_dirty[b] = true;
     return release_set(ss, s);
@@ -529,25 +554,26 @@ ps_status_t ps_step_mf(ps_store_t* ps, const uint32_t* d_i, const uint32_t* d_j,
     }
     SortSet* ss = next_set(ps);
     alternate_side(ps);
-    if (!fork_side(ps, ss, s, true)) return PS_ERR_CUDA;
     // rows short enough to be staged whole, and row numbers that fit the 32-bit fields of the sort's records
     const bool fused = ps->cfg.row_len <= 128 && (uint64_t)ps->cfg.num_workers * ps->cfg.slots_per_part < (1ull << 32);
     // The one-launch form over the column side is taken on request only: on the 10M x 1M matrix it runs at 49 us
     // per step against 45 for the symmetric form (its launch takes 35 to 41 us, the two of the symmetric form 42,
     // but it adds a kernel to the internal stream, whose sort is what bounds the step).
     const bool by_column = fused && ps->mf_path == 1;
-    const int which = radix_sort_mf(ps, d_i, d_j, d_v, (uint32_t)n, col_key_base, fused, ps->side, ps->starter_count,
+    cudaStream_t q = ps->side;                      // (rows of more than 128 values: the sort runs beside the gradient kernel)
+    if (fused ? !begin_sort(ps, ss, s, true, &q) : !fork_side(ps, ss, s, true)) return PS_ERR_CUDA;
+    const int which = radix_sort_mf(ps, d_i, d_j, d_v, (uint32_t)n, col_key_base, fused, q, ps->starter_count,
                                     div_up_u32(2 * n, fused ? 64 * 8 : kGroupSpan));
-    if (!sorted_keys_at(ps, ss, which, (uint32_t)(2 * n))) return PS_ERR_CUDA;
+    if (!sorted_keys_at(ps, ss, which, (uint32_t)(2 * n), q)) return PS_ERR_CUDA;
     if (by_column) {
-        launch_mf_plan(ps, (uint32_t)n, which, ps->side);
-        if (!join_side(ps, s)) return PS_ERR_CUDA;
+        launch_mf_plan(ps, (uint32_t)n, which, q);
+        if (!end_sort(ps, s, q)) return PS_ERR_CUDA;
         run_mf_col(ps, (uint32_t)n, which, lr, lambda, d_loss_accum, s);
         return release_set(ss, s);
     }
     if (fused) {
         // gradient and reduction in one kernel over the sorted occurrences: no update rows
-        if (!join_side(ps, s)) return PS_ERR_CUDA;
+        if (!end_sort(ps, s, q)) return PS_ERR_CUDA;
         run_mf_fused(ps, (uint32_t)n, which, col_key_base, lr, lambda, d_loss_accum, s,
                      ps->row_map_ok && ps->mf_path != PS_MF_SYMMETRIC_ROW_COPIES);
         return release_set(ss, s);
@@ -582,7 +608,7 @@ ps_status_t ps_step_kge(ps_store_t* ps, const uint32_t* d_s, const uint32_t* d_r
     if (!fork_side(ps, ss, s)) return PS_ERR_CUDA;
     launch_keys_kge(ps, d_s, d_r, d_o, d_neg_ent, n, n_neg, rel_key_base, ps->side);
     const int which = run_push_sort(ps, occ, ps->side);
-    if (!sorted_keys_at(ps, ss, which, occ)) return PS_ERR_CUDA;
+    if (!sorted_keys_at(ps, ss, which, occ, ps->side)) return PS_ERR_CUDA;
     // gradient rows + AdaGrad inside the reduction where a gradient row is whole float4s and fits the reduction's staging
     const bool grad_only = dim_complex % 2 == 0 && dim_complex <= 128;
     const uint32_t lb = launch_step_kge(ps, d_s, d_r, d_o, d_neg_ent, d_neg_side, n, n_neg, rel_key_base, dim_complex,
@@ -615,7 +641,7 @@ ps_status_t ps_step_rescal(ps_store_t* ps, const uint32_t* d_s, const uint32_t* 
     if (!fork_side(ps, ss, s)) return PS_ERR_CUDA;
     launch_keys_rescal(ps, d_s, d_r, d_o, d_neg_ent, n, n_neg, rel_key_base, dim, ps->side);
     const int which = run_push_sort(ps, occ, ps->side);
-    if (!sorted_keys_at(ps, ss, which, occ)) return PS_ERR_CUDA;
+    if (!sorted_keys_at(ps, ss, which, occ, ps->side)) return PS_ERR_CUDA;
     // gradient rows of dim values per occurrence; AdaGrad inside the reduction, to which a row [dim | dim] is what
     // [Re Im | G_Re G_Im] of dim / 2 complex dimensions is
     const uint32_t lb = launch_grad_rescal(ps, d_s, d_r, d_o, d_neg_ent, d_neg_side, n, n_neg, rel_key_base, dim, nullptr, s);
@@ -741,7 +767,7 @@ ps_status_t ps_step_sgns(ps_store_t* ps, const uint32_t* d_tokens, uint64_t firs
     if (!fork_side(ps, ss, s)) return PS_ERR_CUDA;
     launch_keys_sgns(ps, d_tokens, 0, first_pos, n_centers, corpus_len, window, d_negs, n_neg, out_key_base, ps->side);
     const int which = run_push_sort(ps, (uint32_t)occ, ps->side);
-    if (!sorted_keys_at(ps, ss, which, (uint32_t)occ)) return PS_ERR_CUDA;
+    if (!sorted_keys_at(ps, ss, which, (uint32_t)occ, ps->side)) return PS_ERR_CUDA;
     const uint32_t lb = launch_step_sgns(ps, d_tokens, 0, first_pos, n_centers, corpus_len, window, d_negs, n_neg,
                                          out_key_base, lr, nullptr, s);
     if (!join_side(ps, s)) return PS_ERR_CUDA;
