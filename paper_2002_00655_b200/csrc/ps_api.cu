@@ -36,7 +36,7 @@ WsLayout ws_layout(const ps_config_t& cfg, uint64_t max_keys) {
         l.valsA[b] = take(mk * 4);
         l.valsB[b] = take(mk * 4);
         l.tile_state[b] = take((size_t)kMaxSortPasses * sort_tiles * kRadix * 4);
-        l.sort_ctl[b] = take(((size_t)kSortCtlWords + groups) * 4);
+        l.sort_ctl[b] = take(((size_t)kSortCtlWords + groups + kSegCounters) * 4);
         l.rec[b] = take(mk * 16);
         l.cellpos[b] = take(mk * 4);
         l.mf_dup[b] = take((mk / 2 + 1 + mk / 512 + 2) * 16);      // per column position, then per block of 256 of them
@@ -630,23 +630,26 @@ ps_status_t ps_step_rescal(ps_store_t* ps, const uint32_t* d_s, const uint32_t* 
     if (ps->cfg.row_len != 2 * (uint64_t)dim) return PS_ERR_INVALID_ARG;
     if ((2 + (uint64_t)n_neg + dim) * n > ps->max_keys) return PS_ERR_WORKSPACE;
     if (rel_key_base > ps->cfg.num_keys) return PS_ERR_INVALID_ARG;
-    const uint32_t occ = (uint32_t)((2 + (uint64_t)n_neg + dim) * n);
-    if (small_call(occ)) {
-        const uint32_t lb = launch_grad_rescal(ps, d_s, d_r, d_o, d_neg_ent, d_neg_side, n, n_neg, rel_key_base, dim,
-                                               begin_small(ps), s);
-        run_small_adagrad(ps, occ, lr, eps, d_loss_accum, d_loss_accum ? lb : 0, s);
+    const RescalBatch B = {d_s, d_r, d_o, d_neg_ent, d_neg_side, n, n_neg, rel_key_base, dim, lr, eps};
+    const uint32_t n_loss = d_loss_accum ? (uint32_t)n : 0u;
+    const uint64_t all = (2 + (uint64_t)n_neg + dim) * n;
+    if (small_call(all)) {
+        const double* loss_terms = run_rescal_small(ps, B, begin_small(ps), s);
+        run_small_adagrad(ps, (uint32_t)all, lr, eps, d_loss_accum, n_loss, s, loss_terms);
         return after_launch();
     }
+    // entity slots and one slot per data point for its relation are sorted; the matrices' rows follow from the latter
+    // (so the sorted keys do not list them, and a relocation is not run beside this call)
+    const uint32_t occ = (uint32_t)((3 + (uint64_t)n_neg) * n);
     SortSet* ss = next_set(ps);
-    if (!fork_side(ps, ss, s)) return PS_ERR_CUDA;
-    launch_keys_rescal(ps, d_s, d_r, d_o, d_neg_ent, n, n_neg, rel_key_base, dim, ps->side);
-    const int which = run_push_sort(ps, occ, ps->side);
-    if (!sorted_keys_at(ps, ss, which, occ, ps->side)) return PS_ERR_CUDA;
-    // gradient rows of dim values per occurrence; AdaGrad inside the reduction, to which a row [dim | dim] is what
-    // [Re Im | G_Re G_Im] of dim / 2 complex dimensions is
-    const uint32_t lb = launch_grad_rescal(ps, d_s, d_r, d_o, d_neg_ent, d_neg_side, n, n_neg, rel_key_base, dim, nullptr, s);
-    if (!join_side(ps, s)) return PS_ERR_CUDA;
-    run_kge_reduce(ps, occ, which, dim / 2, lr, eps, d_loss_accum, d_loss_accum ? lb : 0, s);
+    cudaStream_t q;
+    if (!begin_sort(ps, ss, s, false, &q)) return PS_ERR_CUDA;
+    launch_keys_rescal(ps, B, q);
+    const int which = run_segment_sort(ps, occ, q);
+    launch_segments(ps, occ, which, dim, rel_key_base, q);
+    if (!end_sort(ps, s, q)) return PS_ERR_CUDA;
+    const double* loss_terms = run_rescal_sorted(ps, B, which, s);
+    run_segment_adagrad(ps, occ, which, dim, lr, eps, loss_terms, n_loss, d_loss_accum, s);
     return release_set(ss, s);
 }
 

@@ -216,6 +216,7 @@ void run_push_pipeline(ps_store* ps, uint32_t n, const float* d_upd, double* d_l
 // With d_scales, occurrence o contributes d_scales[o] times a shared source row of d_upd: row 2e for slot 0
 // of example e = o / slots, row 2e + 1 for its other slots.
 int run_push_sort(ps_store* ps, uint32_t n, cudaStream_t s);
+int run_segment_sort(ps_store* ps, uint32_t n, cudaStream_t s);     // the same; also clears the counters of seg_lists
 void run_push_reduce(ps_store* ps, uint32_t n, int which, const float* d_upd, double* d_loss_accum,
                      uint32_t loss_blocks, cudaStream_t s, const float* d_scales = nullptr, uint32_t slots = 0);
 
@@ -246,7 +247,43 @@ void run_small_push_keys(ps_store* ps, const uint64_t* d_keys, uint32_t n, const
 void run_small_reduce(ps_store* ps, uint32_t n, double* d_loss_accum, uint32_t loss_blocks, cudaStream_t s,
                       const float* d_scales = nullptr, uint32_t slots = 0);
 void run_small_adagrad(ps_store* ps, uint32_t n, float lr, float eps, double* d_loss_accum, uint32_t loss_blocks,
-                       cudaStream_t s);
+                       cudaStream_t s, const double* loss_terms = nullptr);     // null: ps->loss_partial
+
+// ---- segments.cu ----
+constexpr uint32_t kRelPiece = 8;                // data points of one relation that a block of rescal_points_kernel takes
+constexpr uint32_t kRelChunk = 64;               // ... that a block of rescal_matrix_kernel sums before parking
+constexpr uint32_t kRelTickets = 16;             // ticket words per chunk of a relation of several chunks
+struct SegLists {
+    unsigned int* counts;           // entries of shorts, longs, pieces, chunks; partial sums parked
+    uint8_t* single;                // per occurrence
+    uint2 *shorts, *pieces;         // {first position, length}
+    uint4 *longs, *chunks;          // {first position, length, the segment's first parked sum, piece | pieces << 16}
+    unsigned int *tickets, *long_tickets;
+    uint32_t strips;                // long_tickets per parked sum
+};
+constexpr uint32_t kSegCounters = 6;
+SegLists seg_lists(ps_store* ps);   // of the current buffer set
+// after the sort, on its stream; keys from rel_key_base on are RESCAL's relations (num_keys: none)
+void launch_segments(ps_store* ps, uint32_t n, int which, uint32_t half_row, uint64_t rel_key_base, cudaStream_t s);
+// gradient rows (half_row values per occurrence, in ps->upd) of the keys that occur several times -> AdaGrad; loss terms
+void run_segment_adagrad(ps_store* ps, uint32_t n, int which, uint32_t half_row, float lr, float eps,
+                         const double* loss_terms, uint32_t n_loss, double* d_loss_accum, cudaStream_t s);
+
+// ---- rescal.cu ----
+struct RescalBatch {
+    const uint32_t *s, *r, *o, *neg_ent;
+    const uint8_t* neg_side;
+    uint64_t n;
+    uint32_t n_neg;
+    uint64_t rel_key_base;
+    uint32_t dim;
+    float lr, eps;
+};
+void launch_keys_rescal(ps_store* ps, const RescalBatch& B, cudaStream_t s);    // 3 + n_neg slots per data point
+// Return where the data points' loss terms are.  small: gradient rows and keys of all 2 + n_neg + dim slots; sorted:
+// matrices and keys that occur once are updated, gradient rows of the other entity slots written.
+const double* run_rescal_small(ps_store* ps, const RescalBatch& B, uint32_t* keys_out, cudaStream_t s);
+const double* run_rescal_sorted(ps_store* ps, const RescalBatch& B, int which, cudaStream_t s);
 
 // ---- localize.cu ----
 // busy_keys: sorted keys of a call that may run beside this relocation (null: none); moving keys among them keep
@@ -264,13 +301,6 @@ void run_localize_deferred(ps_store* ps, uint32_t worker, uint32_t n, cudaStream
 // update rows to `upd` (launch_step_sgns: two source rows per center and one factor per slot, to be
 // reduced with run_push_reduce's d_scales) and return the number of per-block loss partials they wrote.  With keys_out
 // (calls without a sort, small.cu) they write the slots' keys there themselves and latch errors for no call number.
-// ---- rescal.cu ----
-void launch_keys_rescal(ps_store* ps, const uint32_t* d_s, const uint32_t* d_r, const uint32_t* d_o,
-                        const uint32_t* d_neg_ent, uint64_t n, uint32_t n_neg, uint64_t rel_key_base, uint32_t dim,
-                        cudaStream_t s);
-uint32_t launch_grad_rescal(ps_store* ps, const uint32_t* d_s, const uint32_t* d_r, const uint32_t* d_o,
-                            const uint32_t* d_neg_ent, const uint8_t* d_neg_side, uint64_t n, uint32_t n_neg,
-                            uint64_t rel_key_base, uint32_t dim, uint32_t* keys_out, cudaStream_t s);
 void launch_keys_kge(ps_store* ps, const uint32_t* d_s, const uint32_t* d_r, const uint32_t* d_o,
                      const uint32_t* d_neg_ent, uint64_t n, uint32_t n_neg, uint64_t rel_key_base, cudaStream_t s);
 void launch_keys_sgns(ps_store* ps, const uint32_t* d_tokens, uint64_t tok_first, uint64_t first_pos,
@@ -314,6 +344,46 @@ __device__ __forceinline__ uint64_t phys_row(uint2 e, uint64_t S) { return (uint
 __device__ __forceinline__ float adagrad_step(float g, float x, float lr, float eps) {
     const float root = x > 0.f ? x * rsqrtf(x) : 0.f;
     return __fdividef(-lr * g, root + eps);
+}
+// The same for N values at a time.  Once sqrt(x) is thousands of times eps, which is all but the very first steps of a
+// parameter, 1 / (sqrt(x) + eps) = r (1 - eps r) with r = 1 / sqrt(x), to within (eps r)^2 < 4e-8: one operation of the
+// special-function unit instead of two, and that unit (16 lanes per clock and SM, conversions to and from fp64 included)
+// is what bounds the reductions with AdaGrad.  One test for all N values, so that their chains interleave.  True if that
+// form was taken, which it is not where a value is not finite.
+template <int N>
+__device__ __forceinline__ bool adagrad_steps(const float (&g)[N], const float (&x)[N], float lr, float eps, float (&step)[N]) {
+    float er[N], worst = 0.f, top = 0.f;
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        float r;
+        asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x[i]));      // (zero or denormal: infinite, the other form)
+        er[i] = eps * r;
+        step[i] = (-lr * g[i]) * (r - er[i] * r);
+        worst = fmaxf(worst, er[i]);
+        top = fmaxf(top, x[i]);
+    }
+    bool fine = worst < 2e-4f && top < 3e38f;
+#pragma unroll
+    for (int i = 0; i < N; ++i) fine = fine && x[i] == x[i];            // (fmaxf passes over a NaN)
+    if (fine) return true;
+#pragma unroll
+    for (int i = 0; i < N; ++i) step[i] = adagrad_step(g[i], x[i], lr, eps);
+    return false;
+}
+__device__ __forceinline__ void adagrad_steps4(const float4& g, const float4& x, float lr, float eps, float4& step) {
+    const float gv[4] = {g.x, g.y, g.z, g.w}, xv[4] = {x.x, x.y, x.z, x.w};
+    float sv[4];
+    adagrad_steps<4>(gv, xv, lr, eps, sv);
+    step = make_float4(sv[0], sv[1], sv[2], sv[3]);
+}
+// A finite fp32 value times 2^-896 as fp64, exactly, by integer operations: fp32's exponent and mantissa put into fp64's
+// fields without a change of bias (denormals included).  Sums of such terms are the sums of the terms times 2^-896, with
+// the same roundings; kUnscale takes the factor out again.  For sums whose conversions would queue for the
+// special-function unit; the integer pipe has room there.
+constexpr double kUnscale = 0x1p896, kScale = 0x1p-896;
+__device__ __forceinline__ double widen_scaled(float v) {
+    const int b = __float_as_int(v);
+    return __hiloint2double((b >> 3) & 0x8fffffff, b << 29);
 }
 
 constexpr unsigned kBarrierSpins = 1u << 21;     // x ~100 ns: gives up after about a fifth of a second
@@ -372,6 +442,9 @@ __device__ __forceinline__ void mbar_init(uint64_t* bar, unsigned count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_addr(bar)), "r"(count) : "memory");
 }
 __device__ __forceinline__ void mbar_init_fence() { asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory"); }
+__device__ __forceinline__ void mbar_inval(uint64_t* bar) {
+    asm volatile("mbarrier.inval.shared::cta.b64 [%0];\n" ::"r"(smem_addr(bar)) : "memory");
+}
 // one arrival that also announces `bytes` of copies
 __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, unsigned bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_addr(bar)), "r"(bytes) : "memory");

@@ -1303,6 +1303,10 @@ int run_push_sort(ps_store* ps, uint32_t n, cudaStream_t s) {
     return radix_sort_pairs(ps, n, nullptr, ps->key_bits, s, 0, ps->starter_count, div_up_u32(n, kGroupSpan));
 }
 
+int run_segment_sort(ps_store* ps, uint32_t n, cudaStream_t s) {
+    return radix_sort_pairs(ps, n, nullptr, ps->key_bits, s, 0, nullptr, kSegCounters);
+}
+
 // The launch that follows a reduction: finishes the border-crossing segments (tiles of tile_len positions), adds the
 // loss partials and, for calls that staged new rows instead of writing them, moves the rows staged at
 // positions apply_lo .. n into the store.

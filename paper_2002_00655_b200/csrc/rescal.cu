@@ -1,6 +1,6 @@
 // RESCAL (Section 4.1 of the paper names the model; Table 4: entity dimension d, relation dimension d * d): the
-// gradient kernel of one minibatch.  Rows of the store have one length, so a relation's d x d matrix is d keys, one
-// per matrix row:  key e < rel_base: entity e, row [x | G];  key rel_base + r d + a: row a of R_r, row [R_r[a][.] | G]
+// gradient kernels of one minibatch.  Rows of the store have one length, so a relation's d x d matrix is d keys, one per
+// matrix row:  key e < rel_base: entity e, row [x | G];  key rel_base + r d + a: row a of R_r, row [R_r[a][.] | G]
 // (G: element-wise AdaGrad accumulators, row_len = 2 d).  Score  phi(s, r, o) = x_s^T R_r x_o.
 //
 // A data point is a positive triple and its negatives (each replaces the subject or the object).  With c_q the
@@ -12,278 +12,522 @@
 //   subject slot: R b      object slot: R^T a      subject-negative k: c_k u      object-negative k: c_k w
 //   matrix row alpha:  a[alpha] x_o + x_s[alpha] b'
 // Slots that hold the same entity are folded into the first of them before anything is written (AdaGrad is taken on
-// the gradient with respect to each DISTINCT key), as the key kernel marks the later ones "no key".
+// the gradient with respect to each DISTINCT key), as the key kernel marks the later ones "no key": the gradient of an
+// entity slot is c1 (R b) + c2 (R^T a) + c3 u + c4 w with four numbers per slot, and folding adds the numbers.
 //
-// One WARP works on one data point at a time, with no block-wide synchronisation (a block of eight warps per data
-// point, the matrix in shared memory or in registers, spent its time in a dozen dependent phases: 660-700 us per
-// step of 8,192 data points).  Lane l holds elements l, l + 32, l + 64, l + 96 of every vector, in fp64.  A pass over
-// the matrix goes row by row, coalesced (a lane reads its columns of the row, the loads of eight rows are issued
-// before the first is used) and gives two products at once: the row's dot product with a vector (the lanes' shares go
-// through a 32 x 33 tile of the warp and one lane adds a row's shares in lane order) and the product of the transpose
-// with another vector (a lane accumulates its columns).  Two passes per data point.
-// The gradient of an entity slot is c1 (R b) + c2 (R^T a) + c3 u + c4 w with four numbers per slot, so slots that
-// hold the same entity are folded by adding their numbers, and no gradient is stored before it is final.  Written per
-// occurrence slot (2 + n_neg entity slots, then d matrix rows): the gradient row of d values; the ComplEx path's
-// reduction (kge_reduce_kernel: AdaGrad inside the segmented reduction of gradient rows) does the rest, a row of
-// [d | d] values being to it what [Re Im | G_Re G_Im] of d / 2 complex dimensions is.
+// The data points of a batch that share a relation share its matrix, so the batch is worked on by relation: a data point
+// has 2 + n_neg entity slots and ONE slot for its relation in the key sort, the relations' runs of sorted positions are
+// its groups (segments.cu), and
+//   rescal_points_kernel  takes up to eight data points of one relation per block.  The matrix goes to shared memory once
+//                         for all of them and the four products are matrix products on the fp64 tensor instructions
+//                         (DMMA, m8n8k4); scores, coefficients and the entities' gradients follow in the same block.
+//                         An entity whose key occurs once in the batch is updated in place, the others' gradients go to
+//                         the segmented reduction.  Per data point it leaves the vectors a, b', x_o, x_s.
+//   rescal_matrix_kernel  updates the matrices: a thread holds a few elements of R and G in registers and walks over
+//                         the relation's data points, forming each one's gradient a[alpha] x_o + x_s[alpha] b' from those
+//                         vectors (staged in shared memory) and AdaGrad's step from it; sums in fp64, one rounding.
+// The d * d gradients of a data point never go through memory (335 MB per 8,192 data points of dimension 100 did, with
+// a sort of 112 keys per data point where 13 do now), and a relation's rows are read and written once per batch.
+// Before: a warp per data point with two passes over the matrix in L2, 292 us, and the matrix rows through the sorted
+// reduction, 278 us, of 577 us per step of 8,192 data points of dimension 100; now 125 + 108 + 33 us, 273 us per step.
+// rescal_points_kernel is bound by the latency of its phases (16 warps per SM, issue slots 40 % used, tensor pipe 27 %),
+// rescal_matrix_kernel by instruction issue and the special-function unit.
+#include <string.h>
+
 #include "ps_internal.cuh"
 
 namespace psb {
 
-__device__ __forceinline__ double rescal_softplus(double z) { return fmax(z, 0.0) + log1p(exp(-fabs(z))); }
-__device__ __forceinline__ double rescal_sigmoid(double z) {
-    if (z >= 0.0) return 1.0 / (1.0 + exp(-z));
-    const double e = exp(z);
-    return e / (1.0 + e);
+namespace {
+
+constexpr int kPoints = 8;                      // data points of one relation per block at a time: a warp each, the columns of one tile
+constexpr int kPointThreads = 32 * kPoints;
+constexpr int kMatThreads = 256;                // eight matrix elements each
+constexpr int kMatStage = 8;                    // data points whose vectors are staged together
+
+// Row stride of the matrix and of the vectors in shared memory: 4 mod 8 elements, so that the eight rows x four columns a
+// warp reads for one tensor instruction fall into different banks (two-way for the transposed read).
+__host__ __device__ constexpr uint32_t pad_ld(uint32_t d) { return d % 8 == 4 ? d : d + 4; }
+
+struct RescalArgs {
+    const uint32_t *ts, *tr, *to, *neg_ent;
+    const uint8_t* neg_side;
+    uint32_t n, n_neg, d, K;
+    uint64_t rel_base;
+    float lr, eps;
+    float* store;
+    const uint2* table;
+    uint64_t S;
+    float* grad;                    // a row of d values per slot (2 + n_neg + n_mat per data point)
+    double* vec;                    // per data point: a, b', x_o, x_s
+    double* loss_of;                // per data point
+    const uint32_t *sk, *sv;        // sorted keys and occurrences (null: calls without a sort)
+    SegLists L;
+    uint32_t* keys_out;             // calls without a sort: keys of all slots, the d matrix rows among them
+    DevStatus* st;
+    unsigned int epoch;
+};
+
+// D += A B, fp64: A 8x4 (lane: row lane / 4, column lane % 4), B 4x8 (row lane % 4, column lane / 4), D 8x8 (row lane / 4,
+// columns 2 (lane % 4) and the next)
+__device__ __forceinline__ void dmma(double (&c)[2], double a, double b) {
+    asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};"
+                 : "+d"(c[0]), "+d"(c[1]) : "d"(a), "d"(b));
+}
+__device__ __forceinline__ double sum8(double v) {          // over the eight lanes of a group
+    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    v += __shfl_xor_sync(0xffffffffu, v, 2);
+    return v + __shfl_xor_sync(0xffffffffu, v, 4);
 }
 
-constexpr int kRescalThreads = 256;
-constexpr int kRescalMaxNeg = 29;
-constexpr int kBatch = 8;             // matrix rows whose loads a warp has in flight together
-
-// shared memory of a warp, fp64: x_s and a (read as broadcasts by the lanes), and a 32 x 33 tile
-__host__ __device__ inline size_t rescal_smem(uint32_t d) {
-    return (size_t)(kRescalThreads / 32) * (2 * d + 32 * 33) * sizeof(double);
-}
-
-// kE: elements of a vector per lane, d <= 32 kE
-template <int kE>
-__global__ void __launch_bounds__(kRescalThreads, 2)
-rescal_grad_kernel(const uint32_t* __restrict__ ts, const uint32_t* __restrict__ tr, const uint32_t* __restrict__ to,
-                   const uint32_t* __restrict__ neg_ent, const uint8_t* __restrict__ neg_side, uint64_t n,
-                   uint32_t n_neg, uint64_t rel_base, uint32_t d, const float* __restrict__ store,
-                   const uint2* __restrict__ table, uint64_t S, uint64_t K, float* __restrict__ grad,
-                   uint32_t* __restrict__ keys_out, double* __restrict__ loss_partial, DevStatus* st) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ double s_wl[kRescalThreads / 32];
-    constexpr int kWarps = kRescalThreads / 32;
+// kSorted: the blocks take the pieces segment_kernel listed.  Otherwise (calls without a sort): data points one by one,
+// every gradient row written (the d matrix rows' too) together with the slots' keys.
+// All rows a block needs (the matrix, the points' entities) are asked for at once as bulk copies into shared memory and
+// waited for once; with plain loads phase by phase the block's time was a chain of memory latencies (248 us a step).
+template <bool kSorted>
+__global__ void __launch_bounds__(kPointThreads, 2) rescal_points_kernel(const RescalArgs A) {
+    extern __shared__ __align__(128) unsigned char dyn[];
+    __shared__ __align__(8) uint64_t bar;
+    __shared__ uint32_t s_t[kPoints];
     const unsigned full = 0xffffffffu;
-    const uint32_t L = 2 * d;
-    const uint32_t n_ent = 2 + n_neg, n_slots = n_ent + d;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    double* sxs = reinterpret_cast<double*>(smem_raw) + (size_t)warp * (2 * d + 32 * 33);
-    double* sA = sxs + d;
-    double* tile = sA + d;                                  // [32][33]
-    const uint64_t n_warps = (uint64_t)gridDim.x * kWarps;
-    double loss = 0;                                        // lane 0's
-    for (uint64_t t = (uint64_t)blockIdx.x * kWarps + warp; t < n; t += n_warps) {
-        // entity slots: subject, object, negatives (lane u holds slot u)
-        uint32_t key = 0;
-        if (lane < (int)n_ent) key = lane == 0 ? ts[t] : (lane == 1 ? to[t] : neg_ent[t * n_neg + (lane - 2)]);
-        const uint32_t side = (lane >= 2 && lane < (int)n_ent) ? neg_side[t * n_neg + (lane - 2)] : 0u;
-        const uint64_t rk = rel_base + (uint64_t)tr[t] * d; // key of row 0 of the matrix
-        if (__ballot_sync(full, lane < (int)n_ent && key >= rel_base) != 0u || rk + d > K) {
-            if (keys_out) {                                 // (a call with a sort: latched by its key kernel)
-                if (lane == 0) latch_error(st, 0u, PS_ERR_KEY_RANGE);
-                for (uint32_t u = lane; u < n_slots; u += 32) keys_out[t * n_slots + u] = kSentinelPad;
-            }
-            continue;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const uint32_t d = A.d, d4 = d / 4, ld = pad_ld(d), n_neg = A.n_neg, n_ent = 2 + n_neg;
+    const uint32_t n_slots = n_ent + (kSorted ? 1u : d);
+    const bool slot = lane < (int)n_ent, act = (uint32_t)lane < d4;
+    double* const Y = reinterpret_cast<double*>(dyn);           // [8][ld]: x_o, then b, then R b
+    double* const X = Y + kPoints * ld;                         // x_s, then a, then R^T a
+    double* const U = X + kPoints * ld;                         // R x_o
+    double* const W = U + kPoints * ld;                         // R^T x_s
+    float* const R = reinterpret_cast<float*>(W + kPoints * ld);        // [d][ld]
+    float* const E = R + d * ld;                                // [points][n_ent][d]: the entities' rows
+    if (kSorted && call_failed(A.st, A.epoch)) return;
+    if (tid == 0) mbar_init(&bar, 1);
+    mbar_init_fence();
+    const uint64_t L = 2 * (uint64_t)d;
+    const uint32_t row_bytes = d * 4;
+    const uint32_t n_items = kSorted ? A.L.counts[2] : A.n;
+    const uint32_t m_tiles = (d + 7) / 8;
+    unsigned parity = 0;
+    // Both products of a pass, R Y and R^T X: warp w takes the tiles w, w + 8, w + 16, w + 24 of the 2 m_tiles together
+    // (four independent chains of tensor instructions).
+    double acc[4][2];
+    auto products = [&]() {
+        const float* a[4];
+        uint32_t step[4];
+        bool tr[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const uint32_t job = tmin<uint32_t>(w + 8 * j, 2 * m_tiles - 1);    // (past the last: computed, not stored)
+            tr[j] = job >= m_tiles;
+            const uint32_t row = tmin<uint32_t>((tr[j] ? job - m_tiles : job) * 8 + lane / 4, d - 1);
+            a[j] = tr[j] ? R + (lane % 4) * ld + row : R + row * ld + lane % 4;
+            step[j] = tr[j] ? 4 * ld : 4;
+            acc[j][0] = acc[j][1] = 0.0;
         }
-        int rep = lane;                                     // first slot that holds the same key
-        for (int z = 0; z < (int)n_ent; ++z) {
-            const uint32_t kz = __shfl_sync(full, key, z);
-            if (lane < (int)n_ent && kz == key && z < rep) rep = z;
+        const double* by = Y + (lane / 4) * ld + lane % 4;
+        const double* bx = X + (lane / 4) * ld + lane % 4;
+#pragma unroll 2
+        for (uint32_t k = 0; k < d4; ++k) {
+            const double y = by[4 * k], x = bx[4 * k];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) dmma(acc[j], (double)a[j][k * step[j]], tr[j] ? x : y);
         }
-        if (keys_out) {
-            if (lane < (int)n_ent) keys_out[t * n_slots + lane] = rep == lane ? key : (uint32_t)K;
-            for (uint32_t a = lane; a < d; a += 32) keys_out[t * n_slots + n_ent + a] = (uint32_t)(rk + a);
+    };
+    auto store_products = [&](double* u, double* wt, uint32_t len) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const uint32_t job = w + 8 * j;
+            const bool tr = job >= m_tiles;
+            const uint32_t row = (tr ? job - m_tiles : job) * 8 + lane / 4, col = 2 * (lane % 4);
+            if (job >= 2 * m_tiles || row >= d) continue;
+            double* o = (tr ? wt : u) + col * ld + row;
+            if (col < len) o[0] = acc[j][0];
+            if (col + 1 < len) o[ld] = acc[j][1];
         }
+    };
+    for (uint32_t item = blockIdx.x; item < n_items; item += gridDim.x) {
+        uint32_t len = 1, pos = 0;
+        uint64_t rk;
+        if (kSorted) {
+            const uint2 it = A.L.pieces[item];
+            pos = it.x;
+            len = it.y;
+            rk = A.sk[pos];
+            if (tid < (int)len) s_t[tid] = A.sv[pos + tid] / n_slots;
+        } else {
+            rk = A.rel_base + (uint64_t)A.tr[item] * d;
+            if (tid == 0) s_t[0] = item;
+        }
+        if (tid == 0) mbar_expect_tx(&bar, (d + len * n_ent) * row_bytes);
+        fence_async_smem();                     // (the rows of the item before have been read)
+        __syncthreads();
+        // ---- the slots of the warp's data point: lane u holds slot u (subject, object, negatives) ----
+        const bool mine = w < (int)len;
+        const uint64_t t = mine ? s_t[w] : 0;
+        uint32_t key = 0, side = 0;
+        int rep = lane;
+        bool once = false, bad = !kSorted && rk + d > A.K;
         uint64_t erow = 0;
-        if (lane < (int)n_ent) erow = phys_row(table[key], S);
-        // rows of the matrix this lane owns, and its elements of x_s and x_o
-        const float* rowp[kE];
-        double xs[kE], xo[kE];
-        const float* ps_ = store + __shfl_sync(full, erow, 0) * L;
-        const float* po_ = store + __shfl_sync(full, erow, 1) * L;
+        if (mine) {
+            if (slot) key = lane == 0 ? A.ts[t] : (lane == 1 ? A.to[t] : A.neg_ent[t * n_neg + (lane - 2)]);
+            if (slot && lane >= 2) side = A.neg_side[t * n_neg + (lane - 2)];
+            if (!kSorted) bad |= slot && key >= A.rel_base;
+            const unsigned same = __match_any_sync(full, slot ? key : kSentinelPad);
+            if (slot) rep = __ffs(same) - 1;
+            if (kSorted && slot) once = rep == lane && A.L.single[t * n_slots + lane] != 0;
+        }
+        if (!kSorted) {                         // (a call with a sort: checked and latched by its key kernel)
+            uint32_t* ko = A.keys_out + (uint64_t)item * n_slots;
+            if (__syncthreads_or(bad)) {
+                if (tid == 0) {
+                    latch_error(A.st, 0u, PS_ERR_KEY_RANGE);
+                    // nothing is copied for this item: the announced bytes are taken back by starting the barrier anew
+                    mbar_inval(&bar);
+                    mbar_init(&bar, 1);
+                }
+                mbar_init_fence();
+                parity = 0;
+                for (uint32_t u = tid; u < n_slots; u += kPointThreads) ko[u] = kSentinelPad;
+                __syncthreads();
+                continue;
+            }
+            if (w == 0 && slot) ko[lane] = rep == lane ? key : A.K;
+            for (uint32_t a = tid; a < d; a += kPointThreads) ko[n_ent + a] = (uint32_t)(rk + a);
+        }
+        if (mine && slot) {
+            erow = phys_row(A.table[key], A.S);
+            bulk_g2s(E + (w * n_ent + lane) * d, A.store + erow * L, row_bytes, &bar);
+            if (once)                           // its accumulators are wanted at the end
+                for (uint32_t o = 0; o < row_bytes; o += 128)
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"((const char*)(A.store + erow * L + d) + o));
+        }
+        if (tid < (int)d) bulk_g2s(R + tid * ld, A.store + phys_row(A.table[rk + tid], A.S) * L, row_bytes, &bar);
+        const bool ok = mbar_wait(&bar, parity) || mbar_wait(&bar, parity);
+        if (__syncthreads_or(!ok)) {
+            if (tid == 0) latch_error(A.st, A.epoch, PS_ERR_CUDA);
+            return;                             // a copy that does not arrive: give the call up
+        }
+        parity ^= 1;
+        const float4* const e4 = reinterpret_cast<const float4*>(E + w * n_ent * d);    // row z of the warp's point: e4 + z d4
+        float4 x_s = make_float4(0.f, 0.f, 0.f, 0.f), x_o = x_s;
+        if (act) {
+            if (mine) {
+                x_s = e4[lane];
+                x_o = e4[d4 + lane];
+            }
+            double* y = Y + w * ld + 4 * lane;
+            double* x = X + w * ld + 4 * lane;
+            y[0] = x_o.x; y[1] = x_o.y; y[2] = x_o.z; y[3] = x_o.w;
+            x[0] = x_s.x; x[1] = x_s.y; x[2] = x_s.z; x[3] = x_s.w;
+        }
+        __syncthreads();
+        products();
+        store_products(U, W, len);
+        __syncthreads();
+        // ---- scores, coefficients, a and b ----
+        double coef = 0;                        // lane 1: the positive's, lane 2 + q: negative q's
+        if (mine) {
+            const double *x = X + w * ld, *u = U + w * ld, *wv = W + w * ld;
+            const int g = lane >> 3, l8 = lane & 7;
+            double phi = 0;
+            // eight lanes per triple; slot 1 stands for the positive, u . x_s
+            for (uint32_t z0 = 1; z0 < n_ent; z0 += 4) {
+                const uint32_t z = z0 + g;
+                const uint32_t sd = __shfl_sync(full, side, z & 31);
+                double s = 0;
+                if (z < n_ent) {
+                    const double* m = (z == 1 || sd == 0) ? u : wv;
+                    const float4* row = e4 + (z == 1 ? 0 : z * d4);
+#pragma unroll 4
+                    for (uint32_t e = l8; e < d4; e += 8) {
+                        const float4 v = row[e];
+                        s += (double)v.x * m[4 * e] + (double)v.y * m[4 * e + 1] + (double)v.z * m[4 * e + 2] + (double)v.w * m[4 * e + 3];
+                    }
+                }
+                s = sum8(s);
+                const double got = __shfl_sync(full, s, ((lane - z0) & 3) * 8);
+                if ((uint32_t)lane >= z0 && (uint32_t)lane < z0 + 4) phi = got;
+            }
+            double loss = 0;
+            if (lane >= 1 && slot) {
+                const double yl = lane == 1 ? 1.0 : -1.0, z = -yl * phi, e = exp(-fabs(z));
+                coef = -yl * ((z >= 0.0 ? 1.0 : e) / (1.0 + e));
+                loss = fmax(z, 0.0) + log1p(e);
+            }
+            loss = warp_sum_d(loss);
+            if (lane == 0) A.loss_of[t] = loss;
+            const double c_pos = __shfl_sync(full, coef, 1);
+            double a[4] = {c_pos * (double)x_s.x, c_pos * (double)x_s.y, c_pos * (double)x_s.z, c_pos * (double)x_s.w};
+            double b[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 2
+            for (uint32_t z = 2; z < n_ent; ++z) {
+                const double c = __shfl_sync(full, coef, z);
+                const uint32_t sd = __shfl_sync(full, side, z);
+                const double ca = sd == 0 ? c : 0.0, cb = sd == 0 ? 0.0 : c;
+                const float4 v = act ? e4[z * d4 + lane] : make_float4(0.f, 0.f, 0.f, 0.f);
+                const double vv[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-        for (int k = 0; k < kE; ++k) {
-            const uint32_t e = lane + 32 * k;
-            rowp[k] = store;
-            xs[k] = xo[k] = 0;
-            if (e < d) {
-                rowp[k] = store + phys_row(table[rk + e], S) * L;
-                xs[k] = (double)ps_[e];
-                xo[k] = (double)po_[e];
+                for (int i = 0; i < 4; ++i) {
+                    a[i] += ca * vv[i];
+                    b[i] += cb * vv[i];
+                }
+            }
+            if (act) {
+                const double o[4] = {x_o.x, x_o.y, x_o.z, x_o.w}, sx[4] = {x_s.x, x_s.y, x_s.z, x_s.w};
+                // for the matrices: a, b', x_o, x_s (calls without a sort: in columns of U that one data point leaves free)
+                double* v = kSorted ? A.vec + t * d * 4 : U + ld;
+                const uint32_t vs = kSorted ? d : ld;
+#pragma unroll
+                for (int i = 0; i < 4; i += 2) {
+                    *reinterpret_cast<double2*>(v + 4 * lane + i) = make_double2(a[i], a[i + 1]);
+                    *reinterpret_cast<double2*>(v + vs + 4 * lane + i) = make_double2(b[i], b[i + 1]);
+                    *reinterpret_cast<double2*>(v + 2 * vs + 4 * lane + i) = make_double2(o[i], o[i + 1]);
+                    *reinterpret_cast<double2*>(v + 3 * vs + 4 * lane + i) = make_double2(sx[i], sx[i + 1]);
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    X[w * ld + 4 * lane + i] = a[i];
+                    Y[w * ld + 4 * lane + i] = c_pos * o[i] + b[i];
+                }
             }
         }
-        __syncwarp();                                       // the data point before is done with the warp's shared memory
+        __syncthreads();
+        products();
+        __syncthreads();
+        store_products(Y, X, len);              // R b, R^T a
+        __syncthreads();
+        // ---- the entities' gradients, folded into the first slot of each key ----
+        if (mine) {
+            double c1 = 0, c2 = 0, c3 = 0, c4 = 0;      // lane v: the numbers of slot v
+            for (int z = 0; z < (int)n_ent; ++z) {
+                const int rz = __shfl_sync(full, rep, z);
+                const double cz = __shfl_sync(full, coef, z);
+                const uint32_t sz = __shfl_sync(full, side, z);
+                if (rz != lane) continue;
+                if (z == 0) c1 += 1.0;
+                else if (z == 1) c2 += 1.0;
+                else if (sz == 0u) c3 += cz;
+                else c4 += cz;
+            }
+            double gs[4], go[4], u[4], wv[4];
 #pragma unroll
-        for (int k = 0; k < kE; ++k) {
-            const uint32_t e = lane + 32 * k;
-            if (e < d) sxs[e] = xs[k];
+            for (int i = 0; i < 4; ++i) {
+                const uint32_t e = w * ld + 4 * lane + i;
+                gs[i] = act ? Y[e] : 0.0;
+                go[i] = act ? X[e] : 0.0;
+                u[i] = act ? U[e] : 0.0;
+                wv[i] = act ? W[e] : 0.0;
+            }
+            float* out = A.grad + t * n_slots * d;
+            const unsigned reps = __ballot_sync(full, slot && rep == lane), in_place = __ballot_sync(full, once);
+            for (uint32_t v0 = 0; v0 < n_ent; v0 += 4) {        // four slots' accumulators asked for at a time
+                float4 G[4];
+                float* rows[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    rows[i] = A.store + __shfl_sync(full, erow, (v0 + i) & 31) * L + 4 * lane;
+                    if (kSorted && act && ((in_place >> (v0 + i)) & 1u)) G[i] = *reinterpret_cast<const float4*>(rows[i] + d);
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int v = v0 + i;
+                    const double f1 = __shfl_sync(full, c1, v & 31), f2 = __shfl_sync(full, c2, v & 31);
+                    const double f3 = __shfl_sync(full, c3, v & 31), f4 = __shfl_sync(full, c4, v & 31);
+                    if (v >= (int)n_ent || !((reps >> v) & 1u) || !act) continue;
+                    float4 g;
+                    g.x = (float)(f1 * gs[0] + f2 * go[0] + f3 * u[0] + f4 * wv[0]);
+                    g.y = (float)(f1 * gs[1] + f2 * go[1] + f3 * u[1] + f4 * wv[1]);
+                    g.z = (float)(f1 * gs[2] + f2 * go[2] + f3 * u[2] + f4 * wv[2]);
+                    g.w = (float)(f1 * gs[3] + f2 * go[3] + f3 * u[3] + f4 * wv[3]);
+                    if (kSorted && ((in_place >> v) & 1u)) {
+                        const float4 s2 = make_float4(g.x * g.x, g.y * g.y, g.z * g.z, g.w * g.w);
+                        float4 th = e4[v * d4 + lane], c = G[i];
+                        c.x += s2.x; c.y += s2.y; c.z += s2.z; c.w += s2.w;
+                        float4 step;
+                        adagrad_steps4(g, c, A.lr, A.eps, step);
+                        th.x += step.x; th.y += step.y; th.z += step.z; th.w += step.w;
+                        *reinterpret_cast<float4*>(rows[i]) = th;
+                        *reinterpret_cast<float4*>(rows[i] + d) = c;
+                    } else {
+                        *reinterpret_cast<float4*>(out + (size_t)v * d + 4 * lane) = g;
+                    }
+                }
+            }
         }
-        __syncwarp();
-        // v = R y and z = R^T s in one pass over the matrix, row by row (coalesced: a lane reads its columns of the
-        // row).  The lane's columns' share of the row's dot product with y goes to a 32 x 32 tile of the warp, and
-        // after 32 rows lane j adds up row j's shares, in lane order.  y: the lanes' elements; s: in shared memory.
-        auto products = [&](const double (&y)[kE], const double* ss, double (&v)[kE], double (&z)[kE]) {
-#pragma unroll
-            for (int k = 0; k < kE; ++k) v[k] = z[k] = 0;
-#pragma unroll
-            for (int kk = 0; kk < kE; ++kk) {
-                const uint32_t a0 = 32u * kk;               // the rows a0 .. a0 + 31 are the lanes' rows number kk
-                if (a0 >= d) break;
-                const uint32_t cnt = d - a0 < 32u ? d - a0 : 32u;
-                // kBatch rows at a time: all their loads are issued before the first is used
-                for (uint32_t j0 = 0; j0 < cnt; j0 += kBatch) {
-                    const float* ra[kBatch];
-                    float r[kBatch][kE];
-#pragma unroll
-                    for (int i = 0; i < kBatch; ++i) {
-                        const uint32_t j = j0 + i < cnt ? j0 + i : cnt - 1;
-                        ra[i] = reinterpret_cast<const float*>(__shfl_sync(full, (unsigned long long)rowp[kk], j));
-                    }
-#pragma unroll
-                    for (int i = 0; i < kBatch; ++i)
-#pragma unroll
-                        for (int k = 0; k < kE; ++k) r[i][k] = (uint32_t)(lane + 32 * k) < d ? __ldg(ra[i] + lane + 32 * k) : 0.f;
-#pragma unroll
-                    for (int i = 0; i < kBatch; ++i) {
-                        if (j0 + i >= cnt) break;
-                        const double sa = ss[a0 + j0 + i];
-                        double p = 0;
-#pragma unroll
-                        for (int k = 0; k < kE; ++k) {
-                            const double rv = (double)r[i][k];
-                            z[k] += sa * rv;
-                            p += rv * y[k];
-                        }
-                        tile[(j0 + i) * 33 + lane] = p;
-                    }
-                }
-                __syncwarp();
-                if ((uint32_t)lane < cnt) {
-                    double acc = 0;
-#pragma unroll 8
-                    for (int l = 0; l < 32; ++l) acc += tile[lane * 33 + l];
-                    v[kk] = acc;
-                }
-                __syncwarp();
+        if (!kSorted) {                         // matrix rows: a[alpha] x_o + x_s[alpha] b'
+            const double *a = U + ld, *b = a + ld, *xo = b + ld, *xs = xo + ld;
+            float* out = A.grad + ((uint64_t)item * n_slots + n_ent) * d;
+            for (uint32_t x = tid; x < d * d4; x += kPointThreads) {
+                const uint32_t al = x / d4, e = 4 * (x - al * d4);
+                const double aa = a[al], sa = xs[al];
+                float4 g;
+                g.x = (float)(aa * xo[e] + sa * b[e]);
+                g.y = (float)(aa * xo[e + 1] + sa * b[e + 1]);
+                g.z = (float)(aa * xo[e + 2] + sa * b[e + 2]);
+                g.w = (float)(aa * xo[e + 3] + sa * b[e + 3]);
+                *reinterpret_cast<float4*>(out + (size_t)al * d + e) = g;
+            }
+        }
+        __syncthreads();
+    }
+}
+
+// The matrices' update.  blockIdx.y: which 2,048 (kMatThreads x 8) of a matrix's d * d elements; blocks of one y loop over
+// the chunks of at most kRelChunk data points that segment_kernel listed.  Per element and data point: two fp64
+// multiply-adds, a rounding to fp32, a reciprocal square root, two fp64 sums.  Bound by the unit that does roundings,
+// widenings and roots (16 lanes per clock and SM: each such operation per element is 18 us of a step of 8,192 data points
+// of dimension 100), so the vectors are staged in fp64 (widened once per data point, not once per element), the squares
+// are summed as fp64 products and the steps widened by integer operations.  A relation of several chunks
+// leaves fp64 partial sums of each; the last of its chunks to finish (a ticket) adds them in chunk order.
+__global__ void __launch_bounds__(kMatThreads, 3) rescal_matrix_kernel(const RescalArgs A, double* __restrict__ parked) {
+    extern __shared__ __align__(128) unsigned char dyn[];
+    __shared__ __align__(8) uint64_t bars[2];
+    __shared__ uint32_t s_t[kRelChunk];
+    __shared__ uint32_t s_ticket;
+    if (call_failed(A.st, A.epoch)) return;
+    const int tid = threadIdx.x;
+    if (tid < 2) mbar_init(&bars[tid], 1);
+    mbar_init_fence();
+    unsigned uses = 0;                          // parity of each stage's barrier
+    const uint32_t d = A.d, d4 = d / 4, quads = d * d4, n_slots = 3 + A.n_neg;
+    const uint64_t L = 2 * (uint64_t)d;
+    const uint32_t n_items = A.L.counts[3];
+    for (uint32_t item = blockIdx.x; item < n_items; item += gridDim.x) {
+        const uint4 it = A.L.chunks[item];
+        const uint32_t pos = it.x, len = it.y, nc = it.w >> 16, chunk = it.w & 0xffffu;
+        const uint32_t rk = A.sk[pos];
+        if (tid < (int)len) s_t[tid] = A.sv[pos + tid] / n_slots;
+        __syncthreads();
+        // the vectors of the data points p0 .. p0 + kMatStage: one bulk copy per data point
+        auto issue = [&](uint32_t p0) {
+            if (p0 >= len) return;
+            const uint32_t cnt = tmin<uint32_t>(kMatStage, len - p0), stage = p0 / kMatStage & 1;
+            if (tid == 0) {
+                mbar_expect_tx(&bars[stage], cnt * 32 * d);
+                for (uint32_t p = 0; p < cnt; ++p)
+                    bulk_g2s(dyn + (size_t)(stage * kMatStage + p) * 32 * d, A.vec + (uint64_t)s_t[p0 + p] * 4 * d, 32 * d, &bars[stage]);
             }
         };
-        double u[kE], w[kE];
-        products(xo, sxs, u, w);
-        // scores: lane 1 keeps the positive's, lane 2 + q negative q's; then every lane forms its triple's coefficient
-        // and loss term (the exponentials once per data point, not once per triple); then a and b'
-        double phi_mine = 0;
-        {
-            double p = 0;
+        issue(0);
+        bool dead = false;                      // a copy that does not arrive
+        // a thread's two quads are the same four columns of two neighbouring rows
+        const uint32_t x = blockIdx.y * kMatThreads + tid;
+        const bool act = x < quads / 2;
+        const uint32_t al = act ? 2 * (x / d4) : 0u, e = act ? 4 * (x % d4) : 0u;
+        float* row[2];
+        float4 G[2];
+        double at[2][4], ag[2][4];
 #pragma unroll
-            for (int k = 0; k < kE; ++k) p += xs[k] * u[k];
-            p = warp_sum_d(p);
-            if (lane == 1) phi_mine = p;
+        for (int i = 0; i < 2; ++i) {
+            row[i] = A.store + phys_row(A.table[rk + al + i], A.S) * L + e;
+            G[i] = *reinterpret_cast<const float4*>(row[i] + d);
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(row[i]));     // (the parameters: read at the end)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) at[i][k] = ag[i][k] = 0.0;
         }
-        for (uint32_t q = 0; q < n_neg; ++q) {
-            const float* pk = store + __shfl_sync(full, erow, 2 + q) * L;
-            const bool subj = __shfl_sync(full, side, 2 + q) == 0u;
-            double p = 0;
+        for (uint32_t p0 = 0; p0 < len; p0 += kMatStage) {
+            const uint32_t cnt = tmin<uint32_t>(kMatStage, len - p0), stage = p0 / kMatStage & 1;
+            issue(p0 + kMatStage);              // (the stage's readers have met at the end of the round before)
+            const bool ok = mbar_wait(&bars[stage], (uses >> stage) & 1u) || mbar_wait(&bars[stage], (uses >> stage) & 1u);
+            uses ^= 1u << stage;
+            if (!ok) dead = true;
+#pragma unroll 1
+            for (uint32_t p = 0; p < cnt; ++p) {
+                const double* a = reinterpret_cast<const double*>(dyn) + (stage * kMatStage + p) * 4 * d;
+                const double2 aa = *reinterpret_cast<const double2*>(a + al), sa = *reinterpret_cast<const double2*>(a + 3 * d + al);
+                const double2 b0 = *reinterpret_cast<const double2*>(a + d + e), b1 = *reinterpret_cast<const double2*>(a + d + e + 2);
+                const double2 o0 = *reinterpret_cast<const double2*>(a + 2 * d + e), o1 = *reinterpret_cast<const double2*>(a + 2 * d + e + 2);
+                const double ov[4] = {o0.x, o0.y, o1.x, o1.y}, bv[4] = {b0.x, b0.y, b1.x, b1.y};
+                float gf[8], xf[8];
 #pragma unroll
-            for (int k = 0; k < kE; ++k) {
-                const uint32_t e = lane + 32 * k;
-                if (e < d) p += (double)pk[e] * (subj ? u[k] : w[k]);
+                for (int i = 0; i < 2; ++i) {
+                    const double ai = i ? aa.y : aa.x, si = i ? sa.y : sa.x;
+                    const float gv[4] = {G[i].x, G[i].y, G[i].z, G[i].w};
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const double g = ai * ov[k] + si * bv[k];
+                        gf[4 * i + k] = (float)g;
+                        xf[4 * i + k] = fmaf(gf[4 * i + k], gf[4 * i + k], gv[k]);
+                        ag[i][k] += g * g;
+                    }
+                }
+                float step[8];
+                const bool fine = adagrad_steps<8>(gf, xf, A.lr, A.eps, step);
+                if (fine) {
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) at[k / 4][k % 4] += widen_scaled(step[k]);
+                } else {
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) at[k / 4][k % 4] += kScale * (double)step[k];
+                }
             }
-            p = warp_sum_d(p);
-            if (lane == (int)(2 + q)) phi_mine = p;
+            __syncthreads();
         }
-        double my_coef = 0, my_loss = 0;                    // d loss / d phi and the loss term of this lane's triple
-        if (lane >= 1 && lane < (int)n_ent) {
-            const double y = lane == 1 ? 1.0 : -1.0;
-            my_coef = -y * rescal_sigmoid(-y * phi_mine);
-            my_loss = rescal_softplus(-y * phi_mine);
+        if (__syncthreads_or(dead)) {
+            if (tid == 0) latch_error(A.st, A.epoch, PS_ERR_CUDA);
+            return;
         }
-        const double lsum = warp_sum_d(my_loss);
-        const double c_pos = __shfl_sync(full, my_coef, 1);
-        double av[kE], bp[kE];
 #pragma unroll
-        for (int k = 0; k < kE; ++k) { av[k] = c_pos * xs[k]; bp[k] = 0; }
-        for (uint32_t q = 0; q < n_neg; ++q) {
-            const float* pk = store + __shfl_sync(full, erow, 2 + q) * L;
-            const bool subj = __shfl_sync(full, side, 2 + q) == 0u;
-            const double cq = __shfl_sync(full, my_coef, 2 + q);
+        for (int i = 0; i < 2; ++i)
 #pragma unroll
-            for (int k = 0; k < kE; ++k) {
-                const uint32_t e = lane + 32 * k;
-                const double xk = e < d ? (double)pk[e] : 0.0;
-                if (subj) av[k] += cq * xk;
-                else bp[k] += cq * xk;
-            }
-        }
-        if (lane == 0) loss += lsum;
-        double bv[kE];
+            for (int k = 0; k < 4; ++k) at[i][k] *= kUnscale;
+        bool finish = true;
+        if (nc > 1) {
+            // laid out [chunk][value of the thread's eight][thread]: coalesced either way
+            double2* mine = reinterpret_cast<double2*>(parked) + (uint64_t)(it.z + chunk) * quads * 4;
+            if (act)
 #pragma unroll
-        for (int k = 0; k < kE; ++k) {
-            const uint32_t e = lane + 32 * k;
-            bv[k] = c_pos * xo[k] + bp[k];
-            if (e < d) sA[e] = av[k];
-        }
-        __syncwarp();
-        double gs[kE], go[kE];
-        products(bv, sA, gs, go);                           // R b, R^T a
-        // the four numbers of every slot, folded into the first slot of its key (lane v: the numbers of slot v)
-        double c1 = 0, c2 = 0, c3 = 0, c4 = 0;
-        for (int z = 0; z < (int)n_ent; ++z) {
-            const int rz = __shfl_sync(full, rep, z);
-            const double cz = __shfl_sync(full, my_coef, z);
-            const uint32_t sz = __shfl_sync(full, side, z);
-            if (rz != lane) continue;
-            if (z == 0) c1 += 1.0;
-            else if (z == 1) c2 += 1.0;
-            else if (sz == 0u) c3 += cz;
-            else c4 += cz;
-        }
-        float* out = grad + (uint64_t)t * n_slots * d;
-        for (int v = 0; v < (int)n_ent; ++v) {
-            if (__shfl_sync(full, rep, v) != v) continue;   // a later slot of a key: marked "no key", never read
-            const double f1 = __shfl_sync(full, c1, v), f2 = __shfl_sync(full, c2, v);
-            const double f3 = __shfl_sync(full, c3, v), f4 = __shfl_sync(full, c4, v);
+                for (int i = 0; i < 2; ++i)
 #pragma unroll
-            for (int k = 0; k < kE; ++k) {
-                const uint32_t e = lane + 32 * k;
-                if (e < d) out[(size_t)v * d + e] = (float)(f1 * gs[k] + f2 * go[k] + f3 * u[k] + f4 * w[k]);
-            }
-        }
-        // matrix rows: a[alpha] x_o + x_s[alpha] b', written as float4: x_o and b' go through the tile so that a lane
-        // holds four consecutive columns
-        float* outR = out + (uint64_t)n_ent * d;
-        __syncwarp();
+                    for (int k = 0; k < 4; ++k) mine[(uint64_t)(4 * i + k) * (quads / 2) + x] = make_double2(at[i][k], ag[i][k]);
+            __threadfence();
+            __syncthreads();
+            if (tid == 0) s_ticket = atomicAdd(&A.L.tickets[it.z * kRelTickets + blockIdx.y], 1u);
+            __syncthreads();
+            finish = s_ticket == nc - 1;
+            if (finish) {
+                __threadfence();
 #pragma unroll
-        for (int k = 0; k < kE; ++k) {
-            const uint32_t e = lane + 32 * k;
-            if (e < d) { tile[e] = xo[k]; tile[d + e] = bp[k]; }
-        }
-        __syncwarp();
-        if ((uint32_t)lane < d / 4) {
-            const double o0 = tile[4 * lane], o1 = tile[4 * lane + 1], o2 = tile[4 * lane + 2], o3 = tile[4 * lane + 3];
-            const double b0 = tile[d + 4 * lane], b1 = tile[d + 4 * lane + 1], b2 = tile[d + 4 * lane + 2], b3 = tile[d + 4 * lane + 3];
-#pragma unroll 4
-            for (uint32_t al = 0; al < d; ++al) {
-                const double aa = sA[al], sa = sxs[al];
-                float4 g;
-                g.x = (float)(aa * o0 + sa * b0);
-                g.y = (float)(aa * o1 + sa * b1);
-                g.z = (float)(aa * o2 + sa * b2);
-                g.w = (float)(aa * o3 + sa * b3);
-                *reinterpret_cast<float4*>(outR + (size_t)al * d + 4 * lane) = g;
+                for (int i = 0; i < 2; ++i)
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) at[i][k] = ag[i][k] = 0.0;
+                for (uint32_t c = 0; c < nc && act; ++c) {
+                    const double2* from = reinterpret_cast<const double2*>(parked) + (uint64_t)(it.z + c) * quads * 4;
+#pragma unroll
+                    for (int i = 0; i < 2; ++i)
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            const double2 v = __ldcg(from + (uint64_t)(4 * i + k) * (quads / 2) + x);
+                            at[i][k] += v.x;
+                            ag[i][k] += v.y;
+                        }
+                }
             }
         }
-    }
-    if (lane == 0) s_wl[warp] = loss;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double tot = 0;
-        for (int i = 0; i < kWarps; ++i) tot += s_wl[i];
-        loss_partial[blockIdx.x] = tot;
+        if (finish && act) {
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                float4 t = *reinterpret_cast<const float4*>(row[i]), g = G[i];
+                t.x = (float)((double)t.x + at[i][0]); t.y = (float)((double)t.y + at[i][1]);
+                t.z = (float)((double)t.z + at[i][2]); t.w = (float)((double)t.w + at[i][3]);
+                g.x = (float)((double)g.x + ag[i][0]); g.y = (float)((double)g.y + ag[i][1]);
+                g.z = (float)((double)g.z + ag[i][2]); g.w = (float)((double)g.w + ag[i][3]);
+                *reinterpret_cast<float4*>(row[i]) = t;
+                *reinterpret_cast<float4*>(row[i] + d) = g;
+            }
+        }
     }
 }
 
-// Keys of the occurrence slots: 2 + n_neg entity slots (a slot that repeats an earlier slot's key gets the "no key"
-// mark K), then the d rows of the relation's matrix; every slot of a data point with an index out of range gets K.
+// Keys of the occurrence slots of each data point: 2 + n_neg entity slots (a slot that repeats an earlier slot's key gets the
+// "no key" mark K), then one slot for the relation (the key of its matrix's row 0); every slot of a data point with an
+// index out of range gets K.
 __global__ void __launch_bounds__(256)
 rescal_keys_kernel(const uint32_t* __restrict__ ts, const uint32_t* __restrict__ tr, const uint32_t* __restrict__ to,
                    const uint32_t* __restrict__ neg_ent, uint64_t n, uint32_t n_neg, uint64_t rel_base, uint32_t d,
                    uint64_t K, uint32_t* __restrict__ keys_out, DevStatus* st, unsigned int epoch) {
     const uint64_t idx = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const uint32_t n_ent = 2 + n_neg, n_slots = n_ent + d;
+    const uint32_t n_ent = 2 + n_neg, n_slots = n_ent + 1;
     if (idx >= n * n_slots) return;
     const uint64_t t = idx / n_slots;
     const uint32_t u = (uint32_t)(idx - t * n_slots);
@@ -295,8 +539,8 @@ rescal_keys_kernel(const uint32_t* __restrict__ ts, const uint32_t* __restrict__
         keys_out[idx] = (uint32_t)K;
         return;
     }
-    if (u >= n_ent) {
-        keys_out[idx] = (uint32_t)(rk + (u - n_ent));
+    if (u == n_ent) {
+        keys_out[idx] = (uint32_t)rk;
         return;
     }
     auto key_of = [&](uint32_t z) { return z == 0 ? ts[t] : (z == 1 ? to[t] : neg_ent[t * n_neg + (z - 2)]); };
@@ -306,39 +550,66 @@ rescal_keys_kernel(const uint32_t* __restrict__ ts, const uint32_t* __restrict__
     keys_out[idx] = first ? mine : (uint32_t)K;
 }
 
-void launch_keys_rescal(ps_store* ps, const uint32_t* d_s, const uint32_t* d_r, const uint32_t* d_o,
-                        const uint32_t* d_neg_ent, uint64_t n, uint32_t n_neg, uint64_t rel_key_base, uint32_t dim,
-                        cudaStream_t s) {
-    const uint64_t occ = n * (2 + (uint64_t)n_neg + dim);
-    PS_LAUNCH(ps, rescal_keys_kernel, div_up_u32(occ, 256), 256, s, d_s, d_r, d_o, d_neg_ent, n, n_neg, rel_key_base,
-              dim, ps->cfg.num_keys, ps->keysA, ps->status, ps->epoch);
+RescalArgs rescal_args(ps_store* ps, const RescalBatch& B, uint32_t rows_per_point) {
+    RescalArgs A;
+    memset(&A, 0, sizeof A);
+    A.ts = B.s; A.tr = B.r; A.to = B.o; A.neg_ent = B.neg_ent; A.neg_side = B.neg_side;
+    A.n = (uint32_t)B.n; A.n_neg = B.n_neg; A.d = B.dim; A.K = (uint32_t)ps->cfg.num_keys;
+    A.rel_base = B.rel_key_base;
+    A.lr = B.lr; A.eps = B.eps;
+    A.store = ps->store;
+    A.table = ps->table;
+    A.S = ps->cfg.slots_per_part;
+    // the update rows' region (2 dim values for every one of the call's (2 + n_neg + dim) n key occurrences): gradient
+    // rows, then the data points' vectors, then their loss terms
+    A.grad = ps->upd;
+    A.vec = (double*)(ps->upd + B.n * rows_per_point * B.dim);
+    A.loss_of = A.vec + B.n * B.dim * 4;
+    A.st = ps->status;
+    A.epoch = ps->epoch;
+    return A;
 }
 
-uint32_t launch_grad_rescal(ps_store* ps, const uint32_t* d_s, const uint32_t* d_r, const uint32_t* d_o,
-                            const uint32_t* d_neg_ent, const uint8_t* d_neg_side, uint64_t n, uint32_t n_neg,
-                            uint64_t rel_key_base, uint32_t dim, uint32_t* keys_out, cudaStream_t s) {
-    const size_t smem = rescal_smem(dim);
-    (void)n_neg;
-    // two blocks per SM, a warp per data point at a time
-    uint64_t g = tmin<uint64_t>((n + 7) / 8, (uint64_t)ps->sm_count * 2);
-    if (g > kMaxLossBlocks) g = kMaxLossBlocks;
-    const uint32_t grid = (uint32_t)g;
-#define RESCAL_LAUNCH(kE)                                                                                           \
-    do {                                                                                                            \
-        static std::atomic<unsigned long long> smem_set{0};                                                         \
-        opt_in_smem((const void*)rescal_grad_kernel<kE>, rescal_smem(128), &smem_set);                              \
-        if (ps->prof) prof_before(ps, "rescal_grad_kernel<" #kE ">", s);                                            \
-        rescal_grad_kernel<kE><<<grid, kRescalThreads, smem, s>>>(                                                  \
-            d_s, d_r, d_o, d_neg_ent, d_neg_side, n, n_neg, rel_key_base, dim, (const float*)ps->store, ps->table,  \
-            ps->cfg.slots_per_part, ps->cfg.num_keys, (float*)ps->upd, keys_out, ps->loss_partial, ps->status);    \
-    } while (0)
-    if (dim <= 32) RESCAL_LAUNCH(1);
-    else if (dim <= 64) RESCAL_LAUNCH(2);
-    else RESCAL_LAUNCH(4);
-#undef RESCAL_LAUNCH
-    if (ps->prof) prof_after(ps, s);
-    ps->launches++;
-    return grid;
+constexpr size_t points_smem(uint32_t d, uint32_t n_neg, int points) {
+    return (size_t)4 * kPoints * pad_ld(d) * 8 + (size_t)d * pad_ld(d) * 4 + (size_t)points * (2 + n_neg) * d * 4;
+}
+constexpr size_t kMaxSmem = points_smem(128, 29, kPoints);
+static_assert(kMaxSmem + 1024 <= 227 * 1024, "a block's shared memory");
+
+}  // namespace
+
+void launch_keys_rescal(ps_store* ps, const RescalBatch& B, cudaStream_t s) {
+    PS_LAUNCH(ps, rescal_keys_kernel, div_up_u32(B.n * (3 + (uint64_t)B.n_neg), 256), 256, s, B.s, B.r, B.o, B.neg_ent, B.n, B.n_neg,
+              B.rel_key_base, B.dim, ps->cfg.num_keys, ps->keysA, ps->status, ps->epoch);
+}
+
+const double* run_rescal_small(ps_store* ps, const RescalBatch& B, uint32_t* keys_out, cudaStream_t s) {
+    RescalArgs A = rescal_args(ps, B, 2 + B.n_neg + B.dim);
+    A.keys_out = keys_out;
+    A.loss_of = ps->loss_partial;               // (kSmallOcc key occurrences are fewer data points than it has room for)
+    static std::atomic<unsigned long long> smem_set{0};
+    opt_in_smem((const void*)rescal_points_kernel<false>, kMaxSmem, &smem_set);
+    PS_LAUNCH_SMEM(ps, rescal_points_kernel<false>, (uint32_t)tmin<uint64_t>(B.n, (uint64_t)ps->sm_count * 2), kPointThreads,
+                   points_smem(B.dim, B.n_neg, 1), s, A);
+    return A.loss_of;
+}
+
+const double* run_rescal_sorted(ps_store* ps, const RescalBatch& B, int which, cudaStream_t s) {
+    RescalArgs A = rescal_args(ps, B, 3 + B.n_neg);
+    A.sk = which ? ps->keysB : ps->keysA;
+    A.sv = which ? ps->valsB : ps->valsA;
+    A.L = seg_lists(ps);
+    static std::atomic<unsigned long long> smem_set{0}, smem_set2{0};
+    opt_in_smem((const void*)rescal_points_kernel<true>, kMaxSmem, &smem_set);
+    PS_LAUNCH_SMEM(ps, rescal_points_kernel<true>, (uint32_t)tmin<uint64_t>(B.n, (uint64_t)ps->sm_count * 2), kPointThreads,
+                   points_smem(B.dim, B.n_neg, kPoints), s, A);
+    const uint32_t strips = div_up_u32((uint64_t)B.dim * B.dim / 8, kMatThreads);
+    static_assert(128 * 128 / 8 / kMatThreads <= (int)kRelTickets, "a ticket per strip of a matrix");
+    const size_t smem = (size_t)2 * kMatStage * B.dim * 32;
+    opt_in_smem((const void*)rescal_matrix_kernel, (size_t)2 * kMatStage * 128 * 32, &smem_set2);
+    PS_LAUNCH_SMEM(ps, rescal_matrix_kernel, dim3((uint32_t)tmin<uint64_t>(B.n, tmax(1, ps->sm_count * 3 / (int)strips)), strips),
+                   kMatThreads, smem, s, A, ps->carry);
+    return A.loss_of;
 }
 
 }  // namespace psb

@@ -1,0 +1,337 @@
+// Reduction of gradient rows key by key, for the steps with AdaGrad (ComplEx, RESCAL).
+//
+// Most keys of a batch occur once.  Such a key's row is read by one data point only, so that data point's gradient
+// kernel, which has the gradient in registers, updates the row in place; its gradient never goes through memory.  What
+// is left for a reduction are the keys that occur several times, as runs (segments) of the sorted occurrences.
+//
+// segment_kernel (on the stream of the sort, right after it) looks at every sorted position and writes
+//   single[occurrence]     1 iff the occurrence's key occurs once
+//   shorts                 {first position, length} of the other segments of fewer than kLongRun occurrences
+//   longs                  the longer ones, cut into pieces of about kLongPiece
+//   pieces, chunks         RESCAL only: the relations' segments (any length), cut into pieces for its two kernels
+// The lists' order is the hardware's, the sums' is not: a segment is summed in position order whoever takes it.
+#include "ps_internal.cuh"
+
+namespace psb {
+
+namespace {
+constexpr uint32_t kLongRun = 24;               // occurrences from which on a block, not a warp, adds a segment
+constexpr uint32_t kLongPiece = 96;             // ... and about as many as one block adds of it
+constexpr uint32_t kMaxStrips = 64;             // (wider rows, of 16,384 values and more, are not cut: the tickets' room)
+}  // namespace
+
+__global__ void __launch_bounds__(256)
+segment_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restrict__ sv, uint32_t n, uint32_t K, uint32_t rel_base,
+               uint32_t long_piece, SegLists L, const DevStatus* st, unsigned int epoch) {
+    if (call_failed(st, epoch)) return;
+    const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= n) return;
+    const uint32_t key = sk[p];
+    if (key >= K) return;
+    const uint32_t prev = p ? sk[p - 1] : kSentinelPad, next = p + 1 < n ? sk[p + 1] : kSentinelPad;
+    const bool head = key != prev, rel = key >= rel_base;
+    L.single[sv[p]] = head && key != next && !rel;
+    if (!head || (key != next && !rel)) return;
+    // the end of the segment: doubling steps, then bisection
+    uint32_t lo = p, step = 1;                  // sk[lo] == key
+    while (lo + step < n && sk[lo + step] == key) {
+        lo += step;
+        step <<= 1;
+    }
+    uint32_t hi = lo + step < n ? lo + step : n;        // sk[hi] != key, or the end
+    while (hi - lo > 1) {
+        const uint32_t mid = (lo + hi) >> 1;
+        if (sk[mid] == key) lo = mid; else hi = mid;
+    }
+    const uint32_t len = hi - p;
+    if (!rel) {
+        if (len < kLongRun) {
+            L.shorts[atomicAdd(L.counts, 1u)] = make_uint2(p, len);
+            return;
+        }
+        const uint32_t np = tmin<uint32_t>((uint32_t)(((uint64_t)len + long_piece - 1) / long_piece), 0xffffu);
+        const uint32_t at = atomicAdd(L.counts + 1, np);
+        const uint32_t park = np > 1 ? atomicAdd(L.counts + 5, np) : 0u;   // where its pieces leave their partial sums
+        if (np > 1)
+            for (uint32_t i = 0; i < L.strips; ++i) L.long_tickets[(uint64_t)park * L.strips + i] = 0u;
+        for (uint32_t i = 0; i < np; ++i) {
+            const uint32_t a = (uint32_t)((uint64_t)len * i / np), b = (uint32_t)((uint64_t)len * (i + 1) / np);
+            L.longs[at + i] = make_uint4(p + a, b - a, park, i | np << 16);
+        }
+        return;
+    }
+    const uint32_t np = (len + kRelPiece - 1) / kRelPiece;
+    uint32_t at = atomicAdd(L.counts + 2, np);
+    for (uint32_t i = 0; i < np; ++i) {         // pieces of nearly equal length
+        const uint32_t a = (uint32_t)((uint64_t)len * i / np), b = (uint32_t)((uint64_t)len * (i + 1) / np);
+        L.pieces[at + i] = make_uint2(p + a, b - a);
+    }
+    const uint32_t nc = (len + kRelChunk - 1) / kRelChunk;
+    at = atomicAdd(L.counts + 3, nc);
+    const uint32_t park = nc > 1 ? atomicAdd(L.counts + 4, nc) : 0u;    // where its chunks leave their partial sums
+    if (nc > 1)
+        for (uint32_t i = 0; i < kRelTickets; ++i) L.tickets[park * kRelTickets + i] = 0u;
+    for (uint32_t i = 0; i < nc; ++i) {
+        const uint32_t a = (uint32_t)((uint64_t)len * i / nc), b = (uint32_t)((uint64_t)len * (i + 1) / nc);
+        L.chunks[at + i] = make_uint4(p + a, b - a, park, i | nc << 16);
+    }
+}
+
+SegLists seg_lists(ps_store* ps) {
+    SegLists L;
+    L.counts = ps->group_done;                  // (zeroed by the sort)
+    L.single = (uint8_t*)ps->cellpos;
+    // the records of the matrix-factorization step (16 bytes per key occurrence) are not in use
+    L.longs = ps->rec;
+    L.shorts = (uint2*)(L.longs + ps->max_keys / kLongRun + 2);
+    L.pieces = L.shorts + ps->max_keys / 2 + 1;
+    L.long_tickets = (unsigned int*)(L.pieces + ps->max_keys / 6 + 1);     // at least six slots per data point of RESCAL
+    L.chunks = ps->mf_dup;
+    L.tickets = ps->mf_tickets;
+    L.strips = 1;
+    return L;
+}
+
+// stretches of a half row's columns that blocks take separately (blockIdx.y of segment_adagrad_kernel)
+static uint32_t seg_strips(uint32_t half_row) {
+    const bool quads = half_row % 4 == 0;
+    const uint32_t vec = quads ? 4 : 2, ch = half_row <= (quads ? 128u : 64u) ? 1 : 2;
+    return div_up_u32(half_row, 32 * vec * ch);
+}
+
+void launch_segments(ps_store* ps, uint32_t n, int which, uint32_t half_row, uint64_t rel_key_base, cudaStream_t s) {
+    const uint32_t* sk = which ? ps->keysB : ps->keysA;
+    const uint32_t* sv = which ? ps->valsB : ps->valsA;
+    SegLists L = seg_lists(ps);
+    L.strips = seg_strips(half_row);
+    PS_LAUNCH(ps, segment_kernel, div_up_u32(n, 256), 256, s, sk, sv, n, (uint32_t)ps->cfg.num_keys, (uint32_t)rel_key_base,
+              L.strips <= kMaxStrips ? kLongPiece : kSentinelPad, L, ps->status, ps->epoch);
+}
+
+// The segments' sums: AdaGrad per occurrence from the row [parameters | accumulators] as it was before the batch (the
+// expression of the gradient kernels), steps and squared gradients added in fp64 in position order, one rounding.  A warp
+// takes a short segment, kFly gradient rows in flight; a long one is shared by the block's warps (a stretch of it
+// each, partial sums added in order), and one of several pieces leaves each piece's fp64 sum in memory for the block
+// that draws its last ticket, which adds them in piece order.  What bounds it is the unit for square roots and
+// conversions, four operations per value: the hottest entity of a batch (1,200 of 16,384 subjects and objects on
+// Zipf(1) triples) took one block 40 us.  V: float4, or float2 for rows whose halves are not whole float4s; blockIdx.y counts
+// stretches of 32 kCh vectors.  Conversions go through the integer pipe (widen_scaled).  The last block adds the loss terms, strided per thread, then a tree.
+template <class V> struct Vec;
+template <> struct Vec<float4> {
+    static constexpr int kN = 4;
+    __device__ static float get(const float4& v, int i) { return i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w; }
+    __device__ static void set(float4& v, int i, float f) { if (i == 0) v.x = f; else if (i == 1) v.y = f; else if (i == 2) v.z = f; else v.w = f; }
+};
+template <> struct Vec<float2> {
+    static constexpr int kN = 2;
+    __device__ static float get(const float2& v, int i) { return i == 0 ? v.x : v.y; }
+    __device__ static void set(float2& v, int i, float f) { if (i == 0) v.x = f; else v.y = f; }
+};
+
+template <class V, int kCh>
+__global__ void __launch_bounds__(256, 2)
+segment_adagrad_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restrict__ sv, const V* __restrict__ grad,
+                       V* __restrict__ store, const uint2* __restrict__ table, uint64_t S, uint32_t GV, float lr, float eps,
+                       SegLists L, double* __restrict__ parked, const double* __restrict__ loss_terms, uint32_t n_loss,
+                       double* loss_accum, const DevStatus* st, unsigned int epoch) {
+    constexpr int kN = Vec<V>::kN, kWarps = 8;
+    constexpr int kFly = kCh * kN >= 8 ? 4 : 8;
+    __shared__ double s_part[kWarps][32 * kN];
+    if (call_failed(st, epoch)) return;
+    const unsigned full = 0xffffffffu;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    if (blockIdx.x == gridDim.x - 1) {
+        if (blockIdx.y != 0 || !loss_accum) return;
+        double t = 0;
+        for (uint32_t i = tid; i < n_loss; i += 256) t += loss_terms[i];
+        t = warp_sum_d(t);
+        if (lane == 0) s_part[0][w] = t;
+        __syncthreads();
+        if (tid == 0) {
+            double tot = 0;
+            for (int i = 0; i < kWarps; ++i) tot += s_part[0][i];
+            *loss_accum += tot;
+        }
+        return;
+    }
+    const uint32_t f0 = blockIdx.y * (32 * kCh) + lane;
+    V th[kCh], G[kCh];
+    double a_t[kCh][kN], a_g[kCh][kN];
+    auto load_row = [&](const V* row) {
+#pragma unroll
+        for (int c = 0; c < kCh; ++c)
+            if (f0 + 32 * c < GV) {
+                th[c] = row[f0 + 32 * c];
+                G[c] = row[GV + f0 + 32 * c];
+            }
+    };
+    // occurrences at positions lo .. lo + cnt of one segment
+    auto sum = [&](uint32_t lo, uint32_t cnt) {
+#pragma unroll
+        for (int c = 0; c < kCh; ++c)
+#pragma unroll
+            for (int i = 0; i < kN; ++i) a_t[c][i] = a_g[c][i] = 0.0;       // (times 2^-896: widen_scaled)
+        for (uint32_t j0 = 0; j0 < cnt; j0 += 32) {
+            const uint32_t in = cnt - j0 < 32u ? cnt - j0 : 32u;
+            const uint32_t occ = (uint32_t)lane < in ? sv[lo + j0 + lane] : 0u;
+            for (uint32_t j = 0; j < in; j += kFly) {
+                V u[kFly][kCh];
+#pragma unroll
+                for (int q = 0; q < kFly; ++q) {
+                    const uint32_t o = __shfl_sync(full, occ, (j + q) & 31);
+#pragma unroll
+                    for (int c = 0; c < kCh; ++c)
+                        if (j + q < in && f0 + 32 * c < GV) u[q][c] = __ldg(grad + (uint64_t)o * GV + f0 + 32 * c);
+                }
+#pragma unroll
+                for (int q = 0; q < kFly; ++q) {
+                    if (j + q >= in) break;
+#pragma unroll
+                    for (int c = 0; c < kCh; ++c) {
+                        if (f0 + 32 * c >= GV) continue;
+                        float g[kN], g2[kN], x[kN], step[kN];
+#pragma unroll
+                        for (int i = 0; i < kN; ++i) {
+                            g[i] = Vec<V>::get(u[q][c], i);
+                            g2[i] = g[i] * g[i];
+                            x[i] = Vec<V>::get(G[c], i) + g2[i];
+                        }
+                        const bool fine = adagrad_steps<kN>(g, x, lr, eps, step);
+#pragma unroll
+                        for (int i = 0; i < kN; ++i) {
+                            a_t[c][i] += fine ? widen_scaled(step[i]) : kScale * (double)step[i];
+                            a_g[c][i] += fine ? widen_scaled(g2[i]) : kScale * (double)g2[i];
+                        }
+                    }
+                }
+            }
+        }
+    };
+    auto unscale = [&]() {
+#pragma unroll
+        for (int c = 0; c < kCh; ++c)
+#pragma unroll
+            for (int i = 0; i < kN; ++i) {
+                a_t[c][i] *= kUnscale;
+                a_g[c][i] *= kUnscale;
+            }
+    };
+    auto finish = [&](V* row) {
+#pragma unroll
+        for (int c = 0; c < kCh; ++c)
+            if (f0 + 32 * c < GV) {
+#pragma unroll
+                for (int i = 0; i < kN; ++i) {
+                    Vec<V>::set(th[c], i, (float)((double)Vec<V>::get(th[c], i) + a_t[c][i]));
+                    Vec<V>::set(G[c], i, (float)((double)Vec<V>::get(G[c], i) + a_g[c][i]));
+                }
+                row[f0 + 32 * c] = th[c];
+                row[GV + f0 + 32 * c] = G[c];
+            }
+    };
+    const uint32_t n_work = gridDim.x - 1;
+    const uint32_t n_longs = L.counts[1], n_shorts = L.counts[0];
+    for (uint32_t j = blockIdx.x; j < n_longs; j += n_work) {
+        const uint4 seg = L.longs[j];
+        V* row = store + phys_row(table[sk[seg.x]], S) * (2 * GV);
+        load_row(row);
+        const uint32_t a = (uint32_t)((uint64_t)seg.y * w / kWarps), b = (uint32_t)((uint64_t)seg.y * (w + 1) / kWarps);
+        sum(seg.x + a, b - a);
+        unscale();
+#pragma unroll
+        for (int c = 0; c < kCh; ++c)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                __syncthreads();                // (every warp has read the row; the sums before are taken)
+#pragma unroll
+                for (int i = 0; i < kN; ++i) s_part[w][i * 32 + lane] = h ? a_g[c][i] : a_t[c][i];
+                __syncthreads();
+                if (w == 0) {
+#pragma unroll
+                    for (int i = 0; i < kN; ++i) {
+                        double tot = s_part[0][i * 32 + lane];
+#pragma unroll
+                        for (int k = 1; k < kWarps; ++k) tot += s_part[k][i * 32 + lane];
+                        if (h) a_g[c][i] = tot; else a_t[c][i] = tot;
+                    }
+                }
+            }
+        const uint32_t np = seg.w >> 16, piece = seg.w & 0xffffu;
+        if (np > 1) {
+            if (w == 0) {
+                double* p = parked + (uint64_t)(seg.z + piece) * (2 * GV * kN);
+#pragma unroll
+                for (int c = 0; c < kCh; ++c)
+                    if (f0 + 32 * c < GV)
+#pragma unroll
+                        for (int i = 0; i < kN; ++i) {
+                            p[(f0 + 32 * c) * kN + i] = a_t[c][i];
+                            p[(GV + f0 + 32 * c) * kN + i] = a_g[c][i];
+                        }
+                __threadfence();
+                __syncwarp();
+                uint32_t ticket = 0;
+                if (lane == 0) ticket = atomicAdd(&L.long_tickets[(uint64_t)seg.z * gridDim.y + blockIdx.y], 1u);
+                ticket = __shfl_sync(full, ticket, 0);
+                if (ticket != np - 1) continue;
+                __threadfence();
+#pragma unroll
+                for (int c = 0; c < kCh; ++c)
+#pragma unroll
+                    for (int i = 0; i < kN; ++i) a_t[c][i] = a_g[c][i] = 0.0;
+                for (uint32_t k = 0; k < np; ++k) {
+                    const double* q = parked + (uint64_t)(seg.z + k) * (2 * GV * kN);
+#pragma unroll
+                    for (int c = 0; c < kCh; ++c)
+                        if (f0 + 32 * c < GV)
+#pragma unroll
+                            for (int i = 0; i < kN; ++i) {
+                                a_t[c][i] += __ldcg(q + (f0 + 32 * c) * kN + i);
+                                a_g[c][i] += __ldcg(q + (GV + f0 + 32 * c) * kN + i);
+                            }
+                }
+                finish(row);
+            }
+            continue;
+        }
+        if (w == 0) finish(row);
+    }
+    for (uint32_t j = blockIdx.x * kWarps + w; j < n_shorts; j += n_work * kWarps) {
+        const uint2 seg = L.shorts[j];
+        V* row = store + phys_row(table[sk[seg.x]], S) * (2 * GV);
+        load_row(row);
+        sum(seg.x, seg.y);
+        unscale();
+        finish(row);
+    }
+}
+
+void run_segment_adagrad(ps_store* ps, uint32_t n, int which, uint32_t half_row, float lr, float eps,
+                         const double* loss_terms, uint32_t n_loss, double* d_loss_accum, cudaStream_t s) {
+    const uint32_t* sk = which ? ps->keysB : ps->keysA;
+    const uint32_t* sv = which ? ps->valsB : ps->valsA;
+    const SegLists L = seg_lists(ps);
+    if (!n_loss) d_loss_accum = nullptr;
+#define SEG_LAUNCH(V, kCh)                                                                                              \
+    do {                                                                                                                \
+        const uint32_t GV = half_row / Vec<V>::kN, strips = seg_strips(half_row);                                       \
+        /* two waves of blocks at most over all stretches of columns; the warps loop over the lists */                  \
+        const uint32_t gx = tmax<uint32_t>(1u, tmin<uint32_t>(div_up_u32(n, 32), (uint32_t)ps->sm_count * 4 / strips)); \
+        if (ps->prof) prof_before(ps, "segment_adagrad_kernel", s);                                                     \
+        segment_adagrad_kernel<V, kCh><<<dim3(gx + 1, strips), 256, 0, s>>>(                                            \
+            sk, sv, (const V*)ps->upd, (V*)ps->store, ps->table, ps->cfg.slots_per_part, GV, lr, eps, L, ps->carry,     \
+            loss_terms, n_loss, d_loss_accum, ps->status, ps->epoch);                                                               \
+        if (ps->prof) prof_after(ps, s);                                                                                \
+        ps->launches++;                                                                                                 \
+    } while (0)
+    if (half_row % 4 == 0) {
+        if (half_row <= 128) SEG_LAUNCH(float4, 1);
+        else SEG_LAUNCH(float4, 2);
+    } else {
+        if (half_row <= 64) SEG_LAUNCH(float2, 1);
+        else SEG_LAUNCH(float2, 2);
+    }
+#undef SEG_LAUNCH
+}
+
+}  // namespace psb

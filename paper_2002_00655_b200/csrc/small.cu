@@ -402,8 +402,9 @@ void run_small_reduce(ps_store* ps, uint32_t n, double* d_loss_accum, uint32_t l
 }
 
 void run_small_adagrad(ps_store* ps, uint32_t n, float lr, float eps, double* d_loss_accum, uint32_t loss_blocks,
-                       cudaStream_t s) {
+                       cudaStream_t s, const double* loss_terms) {
     SmallArgs a = common(ps, n, d_loss_accum, loss_blocks);
+    if (loss_terms) a.loss_partial = loss_terms;
     a.F4 /= 2;
     a.lr = lr;
     a.eps = eps;
