@@ -596,26 +596,30 @@ ps_status_t ps_step_kge(ps_store_t* ps, const uint32_t* d_s, const uint32_t* d_r
     if ((3 + (uint64_t)n_neg) * n > ps->max_keys) return PS_ERR_WORKSPACE;
     if (rel_key_base > ps->cfg.num_keys) return PS_ERR_INVALID_ARG;
     const uint32_t occ = (uint32_t)((3 + (uint64_t)n_neg) * n);
+    const KgeBatch B = {d_s, d_r, d_o, d_neg_ent, d_neg_side, n, n_neg, rel_key_base, dim_complex, lr, eps};
     if (small_call(occ)) {
-        const bool grad_only = dim_complex % 2 == 0;
-        const uint32_t lb = launch_step_kge(ps, d_s, d_r, d_o, d_neg_ent, d_neg_side, n, n_neg, rel_key_base, dim_complex,
-                                            lr, eps, grad_only, begin_small(ps), s);
-        if (grad_only) run_small_adagrad(ps, occ, lr, eps, d_loss_accum, d_loss_accum ? lb : 0, s);
-        else run_small_reduce(ps, occ, d_loss_accum, d_loss_accum ? lb : 0, s);
+        // (the reduction without a sort works on whole float4s: gradient rows where the halves of a row are)
+        const bool finished = dim_complex % 2 != 0;
+        const uint32_t lb = launch_points_kge(ps, B, nullptr, finished, begin_small(ps), s);
+        if (finished) run_small_reduce(ps, occ, d_loss_accum, d_loss_accum ? lb : 0, s);
+        else run_small_adagrad(ps, occ, lr, eps, d_loss_accum, d_loss_accum ? lb : 0, s);
         return after_launch();
     }
     SortSet* ss = next_set(ps);
-    if (!fork_side(ps, ss, s)) return PS_ERR_CUDA;
-    launch_keys_kge(ps, d_s, d_r, d_o, d_neg_ent, n, n_neg, rel_key_base, ps->side);
-    const int which = run_push_sort(ps, occ, ps->side);
-    if (!sorted_keys_at(ps, ss, which, occ, ps->side)) return PS_ERR_CUDA;
-    // gradient rows + AdaGrad inside the reduction where a gradient row is whole float4s and fits the reduction's staging
-    const bool grad_only = dim_complex % 2 == 0 && dim_complex <= 128;
-    const uint32_t lb = launch_step_kge(ps, d_s, d_r, d_o, d_neg_ent, d_neg_side, n, n_neg, rel_key_base, dim_complex,
-                                        lr, eps, grad_only, nullptr, s);
-    if (!join_side(ps, s)) return PS_ERR_CUDA;
-    if (grad_only) run_kge_reduce(ps, occ, which, dim_complex, lr, eps, d_loss_accum, d_loss_accum ? lb : 0, s);
-    else run_push_reduce(ps, occ, which, ps->upd, d_loss_accum, d_loss_accum ? lb : 0, s);
+    // Long rows: keys that occur once are updated by the gradient kernel, which therefore comes after the sort.  Short
+    // rows: all gradients go to the reduction, and the gradient kernel runs beside the sort.
+    const bool in_place = dim_complex > 128;
+    cudaStream_t q = ps->side;
+    if (in_place ? !begin_sort(ps, ss, s, false, &q) : !fork_side(ps, ss, s)) return PS_ERR_CUDA;
+    launch_keys_kge(ps, B, q);
+    const int which = run_segment_sort(ps, occ, q);
+    if (!sorted_keys_at(ps, ss, which, occ, q)) return PS_ERR_CUDA;
+    launch_segments(ps, occ, which, 2 * dim_complex, ps->cfg.num_keys, q);
+    uint32_t lb = 0;
+    if (!in_place) lb = launch_points_kge(ps, B, nullptr, false, nullptr, s);
+    if (!end_sort(ps, s, q)) return PS_ERR_CUDA;
+    if (in_place) lb = launch_points_kge(ps, B, seg_lists(ps).single, false, nullptr, s);
+    run_segment_adagrad(ps, occ, which, 2 * dim_complex, !in_place, lr, eps, ps->loss_partial, d_loss_accum ? lb : 0, d_loss_accum, s);
     return release_set(ss, s);
 }
 
@@ -649,7 +653,7 @@ ps_status_t ps_step_rescal(ps_store_t* ps, const uint32_t* d_s, const uint32_t* 
     launch_segments(ps, occ, which, dim, rel_key_base, q);
     if (!end_sort(ps, s, q)) return PS_ERR_CUDA;
     const double* loss_terms = run_rescal_sorted(ps, B, which, s);
-    run_segment_adagrad(ps, occ, which, dim, lr, eps, loss_terms, n_loss, d_loss_accum, s);
+    run_segment_adagrad(ps, occ, which, dim, false, lr, eps, loss_terms, n_loss, d_loss_accum, s);
     return release_set(ss, s);
 }
 

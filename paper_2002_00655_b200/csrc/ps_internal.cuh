@@ -233,10 +233,6 @@ void run_mf_fused(ps_store* ps, uint32_t n_cells, int which, uint64_t col_key_ba
 void launch_mf_plan(ps_store* ps, uint32_t n_cells, int which, cudaStream_t side);
 void run_mf_col(ps_store* ps, uint32_t n_cells, int which, float lr, float lambda, double* d_loss_accum, cudaStream_t s);
 
-// ComplEx: reduce GRADIENT rows (2 dim values per occurrence, in ps->upd) into AdaGrad steps per key; dim even, <= 128
-void run_kge_reduce(ps_store* ps, uint32_t n, int which, uint32_t dim, float lr, float eps, double* d_loss_accum,
-                    uint32_t loss_blocks, cudaStream_t s);
-
 // ---- small.cu ----
 // Calls of at most kSmallOcc key occurrences, all on the caller's stream, no sort.  The step's gradient kernel leaves the
 // slots' keys in small_keys (num_keys: no key; kSentinelPad: index out of range) and its rows in ps->upd, as for the
@@ -261,13 +257,29 @@ struct SegLists {
     unsigned int *tickets, *long_tickets;
     uint32_t strips;                // long_tickets per parked sum
 };
-constexpr uint32_t kSegCounters = 6;
+constexpr uint32_t kSegCounters = 8;             // (rows whose single keys are reduced have at most two stretches of columns)
 SegLists seg_lists(ps_store* ps);   // of the current buffer set
 // after the sort, on its stream; keys from rel_key_base on are RESCAL's relations (num_keys: none)
 void launch_segments(ps_store* ps, uint32_t n, int which, uint32_t half_row, uint64_t rel_key_base, cudaStream_t s);
-// gradient rows (half_row values per occurrence, in ps->upd) of the keys that occur several times -> AdaGrad; loss terms
-void run_segment_adagrad(ps_store* ps, uint32_t n, int which, uint32_t half_row, float lr, float eps,
+// gradient rows (half_row values per occurrence, in ps->upd) -> AdaGrad, of the keys that occur several times and, with
+// singles, of those that occur once; loss terms
+void run_segment_adagrad(ps_store* ps, uint32_t n, int which, uint32_t half_row, bool singles, float lr, float eps,
                          const double* loss_terms, uint32_t n_loss, double* d_loss_accum, cudaStream_t s);
+
+// ---- complex.cu ----
+struct KgeBatch {
+    const uint32_t *s, *r, *o, *neg_ent;
+    const uint8_t* neg_side;
+    uint64_t n;
+    uint32_t n_neg;
+    uint64_t rel_key_base;
+    uint32_t dim;
+    float lr, eps;
+};
+void launch_keys_kge(ps_store* ps, const KgeBatch& B, cudaStream_t s);
+// single: per slot, does its key occur once in the batch (such rows are updated in place).  Gradient rows of 2 dim values
+// per slot in ps->upd (finished: rows of 4 dim values, step and squared gradient).  Returns the number of loss partials.
+uint32_t launch_points_kge(ps_store* ps, const KgeBatch& B, const uint8_t* single, bool finished, uint32_t* keys_out, cudaStream_t s);
 
 // ---- rescal.cu ----
 struct RescalBatch {
@@ -301,18 +313,11 @@ void run_localize_deferred(ps_store* ps, uint32_t worker, uint32_t n, cudaStream
 // update rows to `upd` (launch_step_sgns: two source rows per center and one factor per slot, to be
 // reduced with run_push_reduce's d_scales) and return the number of per-block loss partials they wrote.  With keys_out
 // (calls without a sort, small.cu) they write the slots' keys there themselves and latch errors for no call number.
-void launch_keys_kge(ps_store* ps, const uint32_t* d_s, const uint32_t* d_r, const uint32_t* d_o,
-                     const uint32_t* d_neg_ent, uint64_t n, uint32_t n_neg, uint64_t rel_key_base, cudaStream_t s);
 void launch_keys_sgns(ps_store* ps, const uint32_t* d_tokens, uint64_t tok_first, uint64_t first_pos,
                       uint64_t n_centers, uint64_t corpus_len, uint32_t window, const uint32_t* d_negs, uint32_t n_neg,
                       uint64_t out_key_base, cudaStream_t s);
 uint32_t launch_step_mf(ps_store* ps, const uint32_t* d_i, const uint32_t* d_j, const float* d_v, uint64_t n,
                         uint64_t col_key_base, float lr, float lambda, uint32_t* keys_out, cudaStream_t s);
-// grad_only: the update rows hold gradients (2 dim values each), to be reduced with run_kge_reduce
-uint32_t launch_step_kge(ps_store* ps, const uint32_t* d_s, const uint32_t* d_r, const uint32_t* d_o,
-                         const uint32_t* d_neg_ent, const uint8_t* d_neg_side, uint64_t n, uint32_t n_neg,
-                         uint64_t rel_key_base, uint32_t dim, float lr, float eps, bool grad_only, uint32_t* keys_out,
-                         cudaStream_t s);
 float* sgns_scales(ps_store* ps, uint64_t n_centers);     // where launch_step_sgns puts the per-slot factors
 uint32_t launch_step_sgns(ps_store* ps, const uint32_t* d_tokens, uint64_t tok_first, uint64_t first_pos,
                           uint64_t n_centers, uint64_t corpus_len, uint32_t window, const uint32_t* d_negs,

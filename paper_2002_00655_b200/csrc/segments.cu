@@ -1,8 +1,11 @@
 // Reduction of gradient rows key by key, for the steps with AdaGrad (ComplEx, RESCAL).
 //
 // Most keys of a batch occur once.  Such a key's row is read by one data point only, so that data point's gradient
-// kernel, which has the gradient in registers, updates the row in place; its gradient never goes through memory.  What
-// is left for a reduction are the keys that occur several times, as runs (segments) of the sorted occurrences.
+// kernel, which has the gradient in registers, can update the row in place; its gradient then never goes through memory.
+// RESCAL and ComplEx on rows of more than 512 values do that (the gradients of long rows do not stay in L2 between two
+// kernels); for shorter ComplEx rows it was no gain (gradient kernel 64 -> 113 us for 85 MB of gradients less, reduction
+// 73 -> 45), and single keys are a case of the reduction here.  The keys that occur several times are runs (segments) of
+// the sorted occurrences.
 //
 // segment_kernel (on the stream of the sort, right after it) looks at every sorted position and writes
 //   single[occurrence]     1 iff the occurrence's key occurs once
@@ -131,11 +134,12 @@ template <> struct Vec<float2> {
 template <class V, int kCh>
 __global__ void __launch_bounds__(256, 2)
 segment_adagrad_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restrict__ sv, const V* __restrict__ grad,
-                       V* __restrict__ store, const uint2* __restrict__ table, uint64_t S, uint32_t GV, float lr, float eps,
+                       V* __restrict__ store, const uint2* __restrict__ table, uint64_t S, uint32_t K, uint32_t n_singles,
+                       uint32_t GV, float lr, float eps,
                        SegLists L, double* __restrict__ parked, const double* __restrict__ loss_terms, uint32_t n_loss,
                        double* loss_accum, const DevStatus* st, unsigned int epoch) {
     constexpr int kN = Vec<V>::kN, kWarps = 8;
-    constexpr int kFly = kCh * kN >= 8 ? 4 : 8;
+    constexpr int kFly = 4;                     // gradient rows a warp has in flight
     __shared__ double s_part[kWarps][32 * kN];
     if (call_failed(st, epoch)) return;
     const unsigned full = 0xffffffffu;
@@ -304,9 +308,67 @@ segment_adagrad_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restri
         unscale();
         finish(row);
     }
+    // Keys that occur once, 32 sorted positions per warp at a time: all look-ups together, then kPair rows in flight; row
+    // + step in fp32 rounds the exact sum once.
+    // They come last and the warps draw them, so that blocks which had long segments take fewer.
+    auto draw = [&]() {
+        uint32_t v = 0;
+        if (lane == 0) v = atomicAdd(L.counts + 6 + blockIdx.y, 1u);
+        return __shfl_sync(full, v, 0) * 32;
+    };
+    for (uint32_t p0 = n_singles ? draw() : 0; p0 < n_singles;) {
+        const uint32_t p = p0 + lane;
+        p0 = draw();
+        const uint32_t key = p < n_singles ? sk[p] : K;
+        const bool mine = key < K && (p == 0 || sk[p - 1] != key) && (p + 1 == n_singles || sk[p + 1] != key);
+        const uint32_t occ = mine ? sv[p] : 0u;
+        const uint64_t row_of = mine ? phys_row(table[key], S) : 0;
+        unsigned todo = __ballot_sync(full, mine);
+        constexpr int kPair = kCh * kN >= 8 ? 3 : 4;
+        while (todo) {
+            V u[kPair][kCh], t1[kPair][kCh], g1[kPair][kCh];
+            V* row[kPair];
+            bool have[kPair];
+#pragma unroll
+            for (int q = 0; q < kPair; ++q) {
+                have[q] = todo != 0;
+                const int src = todo ? __ffs(todo) - 1 : 0;
+                todo &= todo - 1;                   // 0 stays 0
+                const V* g = grad + (uint64_t)__shfl_sync(full, occ, src) * GV;
+                row[q] = store + __shfl_sync(full, row_of, src) * (2 * GV);
+#pragma unroll
+                for (int c = 0; c < kCh; ++c)
+                    if (have[q] && f0 + 32 * c < GV) {
+                        u[q][c] = __ldg(g + f0 + 32 * c);
+                        t1[q][c] = row[q][f0 + 32 * c];
+                        g1[q][c] = row[q][GV + f0 + 32 * c];
+                    }
+            }
+#pragma unroll
+            for (int q = 0; q < kPair; ++q)
+#pragma unroll
+                for (int c = 0; c < kCh; ++c) {
+                    if (!have[q] || f0 + 32 * c >= GV) continue;
+                    float g[kN], x[kN], step[kN];
+#pragma unroll
+                    for (int i = 0; i < kN; ++i) {
+                        g[i] = Vec<V>::get(u[q][c], i);
+                        x[i] = Vec<V>::get(g1[q][c], i) + g[i] * g[i];
+                    }
+                    adagrad_steps<kN>(g, x, lr, eps, step);
+#pragma unroll
+                    for (int i = 0; i < kN; ++i) {
+                        Vec<V>::set(t1[q][c], i, Vec<V>::get(t1[q][c], i) + step[i]);
+                        Vec<V>::set(g1[q][c], i, x[i]);
+                    }
+                    row[q][f0 + 32 * c] = t1[q][c];
+                    row[q][GV + f0 + 32 * c] = g1[q][c];
+                }
+        }
+    }
 }
 
-void run_segment_adagrad(ps_store* ps, uint32_t n, int which, uint32_t half_row, float lr, float eps,
+void run_segment_adagrad(ps_store* ps, uint32_t n, int which, uint32_t half_row, bool singles, float lr, float eps,
                          const double* loss_terms, uint32_t n_loss, double* d_loss_accum, cudaStream_t s) {
     const uint32_t* sk = which ? ps->keysB : ps->keysA;
     const uint32_t* sv = which ? ps->valsB : ps->valsA;
@@ -315,11 +377,12 @@ void run_segment_adagrad(ps_store* ps, uint32_t n, int which, uint32_t half_row,
 #define SEG_LAUNCH(V, kCh)                                                                                              \
     do {                                                                                                                \
         const uint32_t GV = half_row / Vec<V>::kN, strips = seg_strips(half_row);                                       \
-        /* two waves of blocks at most over all stretches of columns; the warps loop over the lists */                  \
-        const uint32_t gx = tmax<uint32_t>(1u, tmin<uint32_t>(div_up_u32(n, 32), (uint32_t)ps->sm_count * 4 / strips)); \
+        /* as many blocks as are resident over all stretches of columns; the warps loop over the lists */               \
+        const uint32_t gx = tmax<uint32_t>(1u, tmin<uint32_t>(div_up_u32(n, 32), (uint32_t)ps->sm_count * 2 / strips)); \
         if (ps->prof) prof_before(ps, "segment_adagrad_kernel", s);                                                     \
         segment_adagrad_kernel<V, kCh><<<dim3(gx + 1, strips), 256, 0, s>>>(                                            \
-            sk, sv, (const V*)ps->upd, (V*)ps->store, ps->table, ps->cfg.slots_per_part, GV, lr, eps, L, ps->carry,     \
+            sk, sv, (const V*)ps->upd, (V*)ps->store, ps->table, ps->cfg.slots_per_part, (uint32_t)ps->cfg.num_keys,   \
+            singles ? n : 0u, GV, lr, eps, L, ps->carry,                                                                \
             loss_terms, n_loss, d_loss_accum, ps->status, ps->epoch);                                                               \
         if (ps->prof) prof_after(ps, s);                                                                                \
         ps->launches++;                                                                                                 \

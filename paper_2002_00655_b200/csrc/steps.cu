@@ -1,6 +1,6 @@
-// Fused pull -> per-example gradient kernels of the three training tasks of
-// Section 4.1 / Appendix A of the paper.  One warp handles one example (a
-// matrix cell, a knowledge-graph data point with its negatives, a skip-gram
+// Fused pull -> per-example gradient kernels of the matrix-factorization and
+// skip-gram tasks of Section 4.1 / Appendix A of the paper (ComplEx: complex.cu,
+// RESCAL: rescal.cu).  One warp handles one example (a matrix cell, a skip-gram
 // center word with its window): it looks the example's keys up in the location
 // table, gathers their rows with coalesced loads, forms dot products with warp
 // shuffles, and writes one additive update row per key occurrence plus that
@@ -17,13 +17,6 @@ __device__ __forceinline__ float sigmoidf(float z) {
     const float e = expf(z);
     return e / (1.f + e);
 }
-__device__ __forceinline__ double softplus_d(double z) { return fmax(z, 0.0) + log1p(exp(-fabs(z))); }
-__device__ __forceinline__ double sigmoid_d(double z) {
-    if (z >= 0.0) return 1.0 / (1.0 + exp(-z));
-    const double e = exp(z);
-    return e / (1.0 + e);
-}
-
 // Sum of the warps' loss terms -> loss_partial[blockIdx.x]; fixed order.
 __device__ __forceinline__ void block_loss_out(double loss, double* __restrict__ loss_partial) {
     __shared__ double wl[8];
@@ -215,289 +208,6 @@ uint32_t launch_step_mf(ps_store* ps, const uint32_t* d_i, const uint32_t* d_j, 
     else PS_LAUNCH(ps, mf_step_kernel<0>, grid, 256, s, MF_ARGS);
 #undef MF_ARGS
     return grid;
-}
-
-// ------------------------------------------------------------- ComplEx ----
-// Slots of a data point: 0 = subject, 1 = relation, 2 = object, 3 + q = the
-// q-th negative entity.  Lane u holds slot u's key and row offset.  Slots that
-// repeat an earlier slot's key emit no update (key mark K): their gradient is
-// folded into the first slot with that key, so that AdaGrad sees the gradient
-// of the data point's loss with respect to each DISTINCT key.
-//
-// Scores and gradient sums are formed in fp64 from the fp32 rows.  With a zero
-// accumulator AdaGrad's step is -lr * g / (|g| + eps), which near g = 0 turns
-// rounding noise of g into a visible change of the parameter; fp64 sums keep
-// that noise far below the fp32 resolution of the result.  The final AdaGrad
-// expression is evaluated in fp32 on the rounded gradient.
-// kMaxNeg bounds n_neg at compile time so that a data point's values live in registers: for every block
-// of 32 complex dimensions the Re and Im of all its rows are requested together, before any is used.
-// kDim / kExactNeg: the complex dimension and "n_neg equals kMaxNeg" known at compile time (0 / false: taken from
-// the arguments).  With both fixed the offsets of the four quarters of a row become immediates and the tests on
-// the number of negatives fold away; the kernel spends more issue slots on integer bookkeeping than on fp64.
-// kGradOnly: the update row of a slot is the GRADIENT of the data point's loss with respect to the slot's key
-// (2 d values, Re then Im), and the reduction turns it into the AdaGrad step from the accumulators it finds in the
-// target row (kge_reduce_kernel); otherwise the row is the finished pair (step, squared gradient) of 4 d values.
-template <int kMaxNeg, int kDim, bool kExactNeg, bool kGradOnly>
-__global__ void __launch_bounds__(256, kMaxNeg <= 10 ? 2 : 1)
-kge_step_kernel(const uint32_t* __restrict__ ts, const uint32_t* __restrict__ tr, const uint32_t* __restrict__ to,
-                const uint32_t* __restrict__ neg_ent, const uint8_t* __restrict__ neg_side, uint64_t n,
-                uint32_t n_neg_arg, uint64_t rel_base, uint32_t d_arg, float lr, float eps, const float* __restrict__ store,
-                const uint2* __restrict__ table, uint64_t S, uint64_t K, float* __restrict__ upd,
-                uint32_t* __restrict__ keys_out, double* __restrict__ loss_partial, DevStatus* st, unsigned int epoch) {
-    const int lane = threadIdx.x & 31;
-    const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const uint64_t n_warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-    const uint32_t d = kDim ? (uint32_t)kDim : d_arg;
-    const uint32_t n_neg = kExactNeg ? (uint32_t)kMaxNeg : n_neg_arg;
-    const int n_slots = 3 + (int)n_neg;
-    const uint32_t L = 4 * d;
-    const unsigned full = 0xffffffffu;
-    double loss = 0;
-    for (uint64_t t = warp; t < n; t += n_warps) {
-        // ---- keys, validity, row offsets, first-slot-with-same-key (lane u holds slot u) ----
-        uint64_t key = K;
-        int side = 0;
-        bool bad = false;
-        if (lane < n_slots) {
-            if (lane == 1) {
-                key = rel_base + tr[t];
-                bad = key >= K;
-            } else {
-                const uint32_t e = lane == 0 ? ts[t] : (lane == 2 ? to[t] : neg_ent[t * n_neg + (lane - 3)]);
-                key = e;
-                bad = e >= rel_base;
-                if (lane >= 3) side = neg_side[t * n_neg + (lane - 3)] != 0;
-            }
-        }
-        if (__any_sync(full, bad)) {
-            if (lane == 0) latch_error(st, epoch, PS_ERR_KEY_RANGE);
-            if (keys_out && lane < n_slots) keys_out[t * n_slots + lane] = kSentinelPad;
-            continue;
-        }
-        uint64_t off = 0;
-        if (lane < n_slots) off = phys_row(table[key], S) * L;
-        int rep = lane;
-        for (int z = n_slots - 1; z >= 0; --z) {
-            const uint64_t kz = __shfl_sync(full, key, z);
-            if (z < lane && kz == key) rep = z;
-        }
-        if (keys_out && lane < n_slots) keys_out[t * n_slots + lane] = rep == lane ? (uint32_t)key : (uint32_t)K;
-        const float* Srow = store + __shfl_sync(full, off, 0);
-        const float* Rrow = store + __shfl_sync(full, off, 1);
-        const float* Orow = store + __shfl_sync(full, off, 2);
-        const float* Nrow[kMaxNeg];
-#pragma unroll
-        for (int q = 0; q < kMaxNeg; ++q) Nrow[q] = store + __shfl_sync(full, off, (3 + q) & 31);
-        // bit q: negative q stands in the subject's place / is the first slot with its key
-        const unsigned subj_mask = __ballot_sync(full, lane >= 3 && lane < n_slots && side == 0) >> 3;
-        const unsigned nrep_mask = __ballot_sync(full, lane >= 3 && lane < n_slots && rep == lane) >> 3;
-
-        // ---- pass A: partial scores of the 1 + n_neg triples over this lane's dimensions ----
-        double part[kMaxNeg + 1];
-#pragma unroll
-        for (int q = 0; q <= kMaxNeg; ++q) part[q] = 0.0;
-        for (uint32_t c = lane; c < d; c += 32) {
-            const float a_f = Srow[c], b_f = Srow[d + c], cr_f = Rrow[c], ci_f = Rrow[d + c];
-            const float e_f = Orow[c], f_f = Orow[d + c];
-            float na_f[kMaxNeg], nb_f[kMaxNeg];
-#pragma unroll
-            for (int q = 0; q < kMaxNeg; ++q) {
-                na_f[q] = q < (int)n_neg ? Nrow[q][c] : 0.f;
-                nb_f[q] = q < (int)n_neg ? Nrow[q][d + c] : 0.f;
-            }
-            const double a = a_f, b = b_f, cr = cr_f, ci = ci_f, e = e_f, f = f_f;
-            part[0] += cr * (a * e + b * f) + ci * (a * f - b * e);
-            // (n, r, o): cr (na e + nb f) + ci (na f - nb e);   (s, r, n): cr (a na + b nb) + ci (a nb - b na)
-            const double re_o = cr * e + ci * f, im_o = cr * f - ci * e;        // multiplies (na, nb) for side 0
-            const double re_s = cr * a - ci * b, im_s = cr * b + ci * a;        // multiplies (na, nb) for side 1
-#pragma unroll
-            for (int q = 0; q < kMaxNeg; ++q) {
-                const double na = na_f[q], nb = nb_f[q];
-                part[q + 1] += ((subj_mask >> q) & 1u) ? (na * re_o + nb * im_o) : (na * re_s + nb * im_s);
-            }
-        }
-        // lane q keeps triple q's score
-        double phi_mine = 0;
-#pragma unroll
-        for (int q = 0; q <= kMaxNeg; ++q) {
-            if (q <= (int)n_neg) {
-                const double phi = warp_sum_d(part[q]);
-                if (lane == q) phi_mine = phi;
-            }
-        }
-        // lane q: loss term and d loss / d phi of triple q (label +1 for the positive, -1 for negatives)
-        double coef = 0, loss_q = 0;
-        if (lane <= (int)n_neg) {
-            const double y = lane == 0 ? 1.0 : -1.0;
-            loss_q = softplus_d(-y * phi_mine);
-            coef = -y * sigmoid_d(-y * phi_mine);
-        }
-        loss += warp_sum_d(loss_q);
-
-        // ---- weights with which each entity slot receives the two "negative role" directions ----
-        // A negative with side 0 stands in the subject's place: its gradient is coef * dphi/dS(r, o).
-        // With side 1 it stands in the object's place: coef * dphi/dO(s, r).  Summed over the
-        // negatives whose key's first slot is this lane.
-        double wS = 0, wO = 0;
-#pragma unroll
-        for (int q = 0; q < kMaxNeg; ++q) {
-            const int rq = __shfl_sync(full, rep, (3 + q) & 31);
-            const double cfq = __shfl_sync(full, coef, (q + 1) & 31);
-            if (q < (int)n_neg && rq == lane) {
-                if ((subj_mask >> q) & 1u) wS += cfq; else wO += cfq;
-            }
-        }
-        const double cf0 = __shfl_sync(full, coef, 0);
-        const int rep_o = __shfl_sync(full, rep, 2);            // 0 if object == subject
-        const double wS0 = __shfl_sync(full, wS, 0), wO0 = __shfl_sync(full, wO, 0);
-        const double wS2 = __shfl_sync(full, wS, 2), wO2 = __shfl_sync(full, wO, 2);
-
-        // ---- pass B: gradients per block of 32 complex dimensions, AdaGrad, update rows ----
-        const uint32_t LU = kGradOnly ? 2 * d : L;        // values per update row
-        float* U = upd + (t * n_slots) * LU;
-        // -lr g / (sqrt(G + g^2) + eps) with the hardware reciprocal square root and reciprocal (each within
-        // 2 ulp, far inside the fp32 tolerance of the result); x = 0 is kept away from 0 * inf
-        auto adagrad_out = [&](float* Uu, uint32_t c, double gd_re, double gd_im, float G_re, float G_im) {
-            const float g_re = (float)gd_re, g_im = (float)gd_im;
-            if (kGradOnly) {
-                Uu[c] = g_re;
-                Uu[d + c] = g_im;
-                return;
-            }
-            const float g2_re = g_re * g_re, g2_im = g_im * g_im;
-            Uu[c] = adagrad_step(g_re, G_re + g2_re, lr, eps);
-            Uu[d + c] = adagrad_step(g_im, G_im + g2_im, lr, eps);
-            Uu[2 * d + c] = g2_re;
-            Uu[3 * d + c] = g2_im;
-        };
-        for (uint32_t c0 = 0; c0 < d; c0 += 32) {
-            const uint32_t c = c0 + lane;
-            const bool act = c < d;
-            const uint32_t cl = act ? c : 0;                 // idle lanes read (and discard) dimension 0
-            // every value this block of dimensions needs, requested before the first use
-            const float a_f = Srow[cl], b_f = Srow[d + cl], cr_f = Rrow[cl], ci_f = Rrow[d + cl];
-            const float e_f = Orow[cl], f_f = Orow[d + cl];
-            float GS_re = 0.f, GS_im = 0.f, GR_re = 0.f, GR_im = 0.f, GO_re = 0.f, GO_im = 0.f;
-            if (!kGradOnly) {
-                GS_re = Srow[2 * d + cl]; GS_im = Srow[3 * d + cl];
-                GR_re = Rrow[2 * d + cl]; GR_im = Rrow[3 * d + cl];
-                GO_re = Orow[2 * d + cl]; GO_im = Orow[3 * d + cl];
-            }
-            float na_f[kMaxNeg], nb_f[kMaxNeg], GN_re[kMaxNeg], GN_im[kMaxNeg];
-#pragma unroll
-            for (int q = 0; q < kMaxNeg; ++q) {
-                const bool live = q < (int)n_neg;
-                na_f[q] = live ? Nrow[q][cl] : 0.f;
-                nb_f[q] = live ? Nrow[q][d + cl] : 0.f;
-                GN_re[q] = (!kGradOnly && ((nrep_mask >> q) & 1u)) ? Nrow[q][2 * d + cl] : 0.f;
-                GN_im[q] = (!kGradOnly && ((nrep_mask >> q) & 1u)) ? Nrow[q][3 * d + cl] : 0.f;
-            }
-            const double a = a_f, b = b_f, cr = cr_f, ci = ci_f, e = e_f, f = f_f;
-            // directions that do not depend on the negative
-            const double dS_re = cr * e + ci * f, dS_im = cr * f - ci * e;      // d phi / d subject, object = o
-            const double dO_re = cr * a - ci * b, dO_im = cr * b + ci * a;      // d phi / d object, subject = s
-            double gs_re = cf0 * dS_re, gs_im = cf0 * dS_im;
-            double go_re = cf0 * dO_re, go_im = cf0 * dO_im;
-            double gr_re = cf0 * (a * e + b * f), gr_im = cf0 * (a * f - b * e);
-            // The negatives enter the gradients of subject, relation and object only through their weighted sums:
-            // (A0, B0) over those in the subject's place (triples (n, r, o)), (A1, B1) over those in the object's
-            // place (triples (s, r, n)).  Two multiply-adds per negative instead of twelve.
-            double A0 = 0.0, B0 = 0.0, A1 = 0.0, B1 = 0.0;
-#pragma unroll
-            for (int q = 0; q < kMaxNeg; ++q) {
-                const double na = na_f[q], nb = nb_f[q];
-                const double w = __shfl_sync(full, coef, (q + 1) & 31);
-                const bool in_subject_place = (subj_mask >> q) & 1u;
-                const double w0 = in_subject_place ? w : 0.0, w1 = in_subject_place ? 0.0 : w;
-                A0 += w0 * na; B0 += w0 * nb;
-                A1 += w1 * na; B1 += w1 * nb;
-            }
-            gr_re += (A0 * e + B0 * f) + (a * A1 + b * B1); gr_im += (A0 * f - B0 * e) + (a * B1 - b * A1);
-            go_re += cr * A0 - ci * B0; go_im += cr * B0 + ci * A0;
-            gs_re += cr * A1 + ci * B1; gs_im += cr * B1 - ci * A1;
-            // negatives that coincide with the subject or the object
-            gs_re += wS0 * dS_re + wO0 * dO_re; gs_im += wS0 * dS_im + wO0 * dO_im;
-            go_re += wS2 * dS_re + wO2 * dO_re; go_im += wS2 * dS_im + wO2 * dO_im;
-            if (rep_o == 0) { gs_re += go_re; gs_im += go_im; }
-            if (act) {
-                adagrad_out(U, c, gs_re, gs_im, GS_re, GS_im);
-                adagrad_out(U + LU, c, gr_re, gr_im, GR_re, GR_im);
-                if (rep_o == 2) adagrad_out(U + 2 * (uint64_t)LU, c, go_re, go_im, GO_re, GO_im);
-            }
-#pragma unroll
-            for (int q = 0; q < kMaxNeg; ++q) {
-                const double wSq = __shfl_sync(full, wS, (3 + q) & 31), wOq = __shfl_sync(full, wO, (3 + q) & 31);
-                if (act && ((nrep_mask >> q) & 1u))
-                    adagrad_out(U + (uint64_t)(3 + q) * LU, c, wSq * dS_re + wOq * dO_re, wSq * dS_im + wOq * dO_im,
-                                GN_re[q], GN_im[q]);
-            }
-        }
-    }
-    block_loss_out(loss, loss_partial);
-}
-
-// Keys of the occurrence slots of each data point; a slot that repeats an earlier slot's key, and every
-// slot of a data point with an index out of range, gets the "no key" mark K.
-__global__ void __launch_bounds__(256)
-kge_keys_kernel(const uint32_t* __restrict__ ts, const uint32_t* __restrict__ tr, const uint32_t* __restrict__ to,
-                const uint32_t* __restrict__ neg_ent, uint64_t n, uint32_t n_neg, uint64_t rel_base, uint64_t K,
-                uint32_t* __restrict__ keys_out, DevStatus* st, unsigned int epoch) {
-    const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= n) return;
-    const int n_slots = 3 + (int)n_neg;
-    uint64_t key[32];
-    key[0] = ts[t];
-    key[1] = rel_base + tr[t];
-    key[2] = to[t];
-    bool bad = key[0] >= rel_base || key[2] >= rel_base || key[1] >= K;
-    for (int q = 0; q < (int)n_neg; ++q) {
-        key[3 + q] = neg_ent[t * n_neg + q];
-        bad |= key[3 + q] >= rel_base;
-    }
-    if (bad) latch_error(st, epoch, PS_ERR_KEY_RANGE);
-    uint32_t* kout = keys_out + t * n_slots;
-    for (int u = 0; u < n_slots; ++u) {
-        bool first = true;
-        for (int z = 0; z < u; ++z) first &= key[z] != key[u];
-        kout[u] = (first && !bad) ? (uint32_t)key[u] : (uint32_t)K;
-    }
-}
-
-uint32_t launch_step_kge(ps_store* ps, const uint32_t* d_s, const uint32_t* d_r, const uint32_t* d_o,
-                         const uint32_t* d_neg_ent, const uint8_t* d_neg_side, uint64_t n, uint32_t n_neg,
-                         uint64_t rel_key_base, uint32_t dim, float lr, float eps, bool grad_only, uint32_t* keys_out,
-                         cudaStream_t s) {
-    const uint32_t grid = step_grid(ps, n);
-    const uint32_t epoch = keys_out ? 0u : ps->epoch;
-#define KGE_ARGS d_s, d_r, d_o, d_neg_ent, d_neg_side, n, n_neg, rel_key_base, dim, lr, eps,                     \
-                 (const float*)ps->store, ps->table, ps->cfg.slots_per_part, ps->cfg.num_keys, ps->upd,         \
-                 keys_out, ps->loss_partial, ps->status, epoch
-#define KGE_LAUNCH(kMaxNeg, kDim, kExact, kGrad)                                                                 \
-    do {                                                                                                         \
-        if (ps->prof) prof_before(ps, "kge_step_kernel<" #kMaxNeg ">", s);                                       \
-        kge_step_kernel<kMaxNeg, kDim, kExact, kGrad><<<grid, 256, 0, s>>>(KGE_ARGS);                            \
-        if (ps->prof) prof_after(ps, s);                                                                         \
-        ps->launches++;                                                                                          \
-    } while (0)
-    if (grad_only) {
-        if (n_neg == 10 && dim == 100) KGE_LAUNCH(10, 100, true, true);
-        else if (n_neg <= 4) KGE_LAUNCH(4, 0, false, true);
-        else if (n_neg <= 10) KGE_LAUNCH(10, 0, false, true);
-        else KGE_LAUNCH(29, 0, false, true);
-    } else {
-        if (n_neg <= 4) KGE_LAUNCH(4, 0, false, false);
-        else if (n_neg <= 10) KGE_LAUNCH(10, 0, false, false);
-        else KGE_LAUNCH(29, 0, false, false);
-    }
-#undef KGE_LAUNCH
-#undef KGE_ARGS
-    return grid;
-}
-
-void launch_keys_kge(ps_store* ps, const uint32_t* d_s, const uint32_t* d_r, const uint32_t* d_o,
-                     const uint32_t* d_neg_ent, uint64_t n, uint32_t n_neg, uint64_t rel_key_base, cudaStream_t s) {
-    PS_LAUNCH(ps, kge_keys_kernel, div_up_u32(n, 256), 256, s, d_s, d_r, d_o, d_neg_ent, n, n_neg, rel_key_base,
-              ps->cfg.num_keys, ps->keysA, ps->status, ps->epoch);
 }
 
 // ---------------------------------------------------------------- SGNS ----
