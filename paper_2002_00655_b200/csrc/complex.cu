@@ -61,6 +61,8 @@ __global__ void __launch_bounds__(256, kMaxNeg <= 10 ? 2 : 1) kge_points_kernel(
     const uint32_t n_neg = kExact ? (uint32_t)kMaxNeg : A.n_neg;
     const int n_slots = 3 + (int)n_neg;
     const uint64_t L = 4 * (uint64_t)d, K = A.K;
+    pdl_trigger();
+    pdl_wait();
     if (A.single && call_failed(A.st, A.epoch)) return;
     double loss = 0;
     for (uint64_t t = (uint64_t)blockIdx.x * kGroups + group; t < A.n; t += (uint64_t)gridDim.x * kGroups) {
@@ -304,9 +306,11 @@ __global__ void __launch_bounds__(256, 2) kge_wide_kernel(const KgeArgs A) {
     const int n_slots = 3 + (int)n_neg;
     const bool slot = lane < n_slots;
     const uint64_t L = 4 * (uint64_t)d, K = A.K;
-    if (A.single && call_failed(A.st, A.epoch)) return;
     if (tid < 2) mbar_init(&bars[tid], 1);
     mbar_init_fence();
+    pdl_trigger();
+    pdl_wait();
+    if (A.single && call_failed(A.st, A.epoch)) return;
     __syncthreads();
     const uint32_t n_str = (d + kStretch - 1) / kStretch;
     double loss = 0;
@@ -562,7 +566,8 @@ uint32_t launch_points_kge(ps_store* ps, const KgeBatch& B, const uint8_t* singl
             static std::atomic<unsigned long long> smem_set{0};                                                  \
             const size_t smem = (size_t)2 * (3 + kMaxNeg) * 4 * kStretchPad * sizeof(float);                     \
             opt_in_smem((const void*)kge_wide_kernel<kMaxNeg>, smem, &smem_set);                                 \
-            PS_LAUNCH_SMEM(ps, kge_wide_kernel<kMaxNeg>, grid, 256, smem, s, A);                                 \
+            if (keys_out) PS_LAUNCH_PDL(ps, "kge_wide_kernel<" #kMaxNeg ">", kge_wide_kernel<kMaxNeg>, dim3(grid), dim3(256), smem, s, A); \
+            else PS_LAUNCH_SMEM(ps, kge_wide_kernel<kMaxNeg>, grid, 256, smem, s, A);                            \
         } while (0)
         if (B.n_neg <= 4) KGE_WIDE(4);
         else KGE_WIDE(10);
@@ -574,10 +579,15 @@ uint32_t launch_points_kge(ps_store* ps, const KgeBatch& B, const uint8_t* singl
     const uint32_t grid = (uint32_t)g;
 #define KGE_LAUNCH(kMaxNeg, kDim, kExact, kW, kAcc)                                                                   \
     do {                                                                                                         \
-        if (ps->prof) prof_before(ps, kW > 1 ? "kge_points_kernel<wide>" : "kge_points_kernel", s);              \
-        kge_points_kernel<kMaxNeg, kDim, kExact, kW, kAcc><<<grid, 256, 0, s>>>(A);                              \
-        if (ps->prof) prof_after(ps, s);                                                                         \
-        ps->launches++;                                                                                          \
+        const char* name = kW > 1 ? "kge_points_kernel<wide>" : "kge_points_kernel";                             \
+        if (keys_out) {                                                                                          \
+            PS_LAUNCH_PDL(ps, name, (kge_points_kernel<kMaxNeg, kDim, kExact, kW, kAcc>), dim3(grid), dim3(256), 0, s, A); \
+        } else {                                                                                                 \
+            if (ps->prof) prof_before(ps, name, s);                                                              \
+            kge_points_kernel<kMaxNeg, kDim, kExact, kW, kAcc><<<grid, 256, 0, s>>>(A);                          \
+            if (ps->prof) prof_after(ps, s);                                                                     \
+            ps->launches++;                                                                                      \
+        }                                                                                                        \
     } while (0)
     if (wide) KGE_LAUNCH(29, 0, false, 8, true);
     else if (finished) {

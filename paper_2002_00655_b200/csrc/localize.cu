@@ -496,6 +496,9 @@ loc_small_kernel(const uint64_t* __restrict__ keys, uint32_t n, uint2* table, ui
     __shared__ uint32_t s_src[kLocSmallKeys / kLocSmallBlocks][2], s_dst[kLocSmallKeys / kLocSmallBlocks];
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const uint32_t b = blockIdx.x;
+    for (uint32_t i = tid; i < kSlots; i += kLocSmallThreads) t_key[i] = t_first[i] = kSentinelPad;
+    pdl_trigger();
+    pdl_wait();
     const unsigned long long top_w = tops[worker];
     uint32_t key[kPer], slot_of[kPer];
     int bad = 0;
@@ -506,7 +509,6 @@ loc_small_kernel(const uint64_t* __restrict__ keys, uint32_t n, uint2* table, ui
         bad |= i < n && k >= K;
         key[q] = i < n ? (uint32_t)k : kSentinelPad;
     }
-    for (uint32_t i = tid; i < kSlots; i += kLocSmallThreads) t_key[i] = t_first[i] = kSentinelPad;
     if (__syncthreads_or(bad)) {                            // the same decision in every block: nothing has been written
         if (b == 0 && tid == 0) latch_error(st, 0u, PS_ERR_KEY_RANGE);
         return;
@@ -612,9 +614,9 @@ bool localize_is_small(const ps_store* ps, uint64_t n) {
 void run_localize_small(ps_store* ps, uint32_t worker, const uint64_t* d_keys, uint32_t n, cudaStream_t s) {
     static std::atomic<unsigned long long> smem_set{0};
     opt_in_smem((const void*)loc_small_kernel, kLocSmallSmem, &smem_set);
-    PS_LAUNCH_SMEM(ps, loc_small_kernel, kLocSmallBlocks, kLocSmallThreads, kLocSmallSmem, s, d_keys, n, ps->table, worker,
-                   ps->cfg.slots_per_part, (uint32_t)ps->cfg.num_keys, ps->tops, ps->stacks, (float4*)ps->store,
-                   ps->cfg.row_len / 4, div_up_u32(ps->cfg.num_keys, ps->cfg.num_workers), ps->status);
+    PS_LAUNCH_PDL(ps, "loc_small_kernel", loc_small_kernel, dim3(kLocSmallBlocks), dim3(kLocSmallThreads), kLocSmallSmem, s,
+                  d_keys, n, ps->table, worker, ps->cfg.slots_per_part, (uint32_t)ps->cfg.num_keys, ps->tops, ps->stacks,
+                  (float4*)ps->store, ps->cfg.row_len / 4, div_up_u32(ps->cfg.num_keys, ps->cfg.num_workers), ps->status);
 }
 
 // Second half of a relocation that ran beside another call: the moving keys that call touched (flag[m] = 1) get

@@ -181,6 +181,32 @@ void prof_after(ps_store* ps, cudaStream_t s);
         (ps)->launches++;                                                    \
     } while (0)
 
+// Programmatic dependent launch, for the kernels of small calls: the kernel may be set up while the one before it on the
+// stream still runs, as soon as all blocks of that one have passed pdl_trigger(); it touches no memory before pdl_wait(),
+// which returns when everything before has completed.  Takes a launch's latency (a microsecond or two) off each of a
+// chain of kernels that run a few microseconds.  Without a trigger in the kernel before it is an ordinary launch.
+template <class... P, class... A>
+inline void launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, const A&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+#define PS_LAUNCH_PDL(ps, name, kernel, grid, block, smem, stream, ...)        \
+    do {                                                                     \
+        if ((ps)->prof) psb::prof_before((ps), name, (stream));              \
+        psb::launch_pdl(kernel, (grid), (block), (smem), (stream), __VA_ARGS__); \
+        if ((ps)->prof) psb::prof_after((ps), (stream));                     \
+        (ps)->launches++;                                                    \
+    } while (0)
+
 // ---- sort.cu ----
 // Stable LSD radix sort of (key, value) pairs on the low `bits` bits of the key, one cooperative launch.
 // Values are the positions 0..n-1 of the input.  Input in the A buffers (start = 0) or the B buffers
@@ -325,6 +351,8 @@ uint32_t launch_step_sgns(ps_store* ps, const uint32_t* d_tokens, uint64_t tok_f
 
 // ---- device helpers ----
 #ifdef __CUDACC__
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 // epoch 0: a call without later kernels to cancel (pull, set rows, get location); only the sticky code is latched
 __device__ __forceinline__ void latch_error(DevStatus* st, unsigned int epoch, unsigned int code) {
     atomicCAS(&st->sticky, 0u, code);

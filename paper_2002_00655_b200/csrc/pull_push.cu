@@ -84,6 +84,8 @@ pull_bulk_kernel(const uint64_t* __restrict__ keys, uint64_t n, char* __restrict
     if (lane < 2) mbar_init(&bars[w][lane], 1);
     mbar_init_fence();
     __syncwarp();
+    pdl_trigger();
+    pdl_wait();
     uint32_t uses = 0;
     int stage = 0;
     // the round whose loads are in flight: its first key, how many rows were asked for, whether this lane has one
@@ -187,8 +189,9 @@ void launch_pull(ps_store* ps, const uint64_t* d_keys, uint64_t n, float* d_out,
         const uint32_t per_round = tmin<uint32_t>(32u, kPullStageBytes / row_bytes);
         const uint64_t rounds = (n + per_round - 1) / per_round;
         const uint32_t grid = (uint32_t)tmin<uint64_t>((rounds + 7) / 8, (uint64_t)ps->sm_count * 3);
-        PS_LAUNCH_SMEM(ps, pull_bulk_kernel, grid, 256, kPullSmem, s, d_keys, n, (char*)d_out, (const char*)ps->store,
-                       ps->table, ps->cfg.slots_per_part, ps->cfg.num_keys, row_bytes, per_round, ps->status, 0u);
+        PS_LAUNCH_PDL(ps, "pull_bulk_kernel", pull_bulk_kernel, dim3(grid), dim3(256), kPullSmem, s, d_keys, n, (char*)d_out,
+                      (const char*)ps->store, ps->table, ps->cfg.slots_per_part, ps->cfg.num_keys, row_bytes, per_round,
+                      ps->status, 0u);
         return;
     }
     const uint32_t grid = (uint32_t)tmin<uint64_t>((n + 31) / 32, (uint64_t)ps->sm_count * 8);

@@ -100,9 +100,11 @@ __global__ void __launch_bounds__(kPointThreads, 2) rescal_points_kernel(const R
     double* const W = U + kPoints * ld;                         // R^T x_s
     float* const R = reinterpret_cast<float*>(W + kPoints * ld);        // [d][ld]
     float* const E = R + d * ld;                                // [points][n_ent][d]: the entities' rows
-    if (kSorted && call_failed(A.st, A.epoch)) return;
     if (tid == 0) mbar_init(&bar, 1);
     mbar_init_fence();
+    pdl_trigger();
+    pdl_wait();
+    if (kSorted && call_failed(A.st, A.epoch)) return;
     const uint64_t L = 2 * (uint64_t)d;
     const uint32_t row_bytes = d * 4;
     const uint32_t n_items = kSorted ? A.L.counts[2] : A.n;
@@ -589,8 +591,9 @@ const double* run_rescal_small(ps_store* ps, const RescalBatch& B, uint32_t* key
     A.loss_of = ps->loss_partial;               // (kSmallOcc key occurrences are fewer data points than it has room for)
     static std::atomic<unsigned long long> smem_set{0};
     opt_in_smem((const void*)rescal_points_kernel<false>, kMaxSmem, &smem_set);
-    PS_LAUNCH_SMEM(ps, rescal_points_kernel<false>, (uint32_t)tmin<uint64_t>(B.n, (uint64_t)ps->sm_count * 2), kPointThreads,
-                   points_smem(B.dim, B.n_neg, 1), s, A);
+    PS_LAUNCH_PDL(ps, "rescal_points_kernel<false>", rescal_points_kernel<false>,
+                  dim3((uint32_t)tmin<uint64_t>(B.n, (uint64_t)ps->sm_count * 2)), dim3(kPointThreads),
+                  points_smem(B.dim, B.n_neg, 1), s, A);
     return A.loss_of;
 }
 

@@ -78,12 +78,19 @@ __global__ void __launch_bounds__(kThreads, kCh == 1 ? 2 : 1) small_push_kernel(
         }
         return A.keys32[i];
     };
+    pdl_trigger();
+    for (int i = tid; i < kTable; i += kThreads) {
+        t_key[i] = t_first[i] = kSentinelPad;
+        t_count[i] = 0;
+    }
+    if (tid == 0) s_n_firsts = s_over = 0;
+    pdl_wait();
     // ---- the occurrences whose keys fall into this block's bucket; warp w looks at its 16th of the call ----
     const uint32_t rounds = (n + kThreads - 1) / kThreads;  // at most 32: lane r keeps the bucket's lanes of round r
     const uint32_t w0 = w * rounds * 32;
     uint32_t mask_of = 0, cnt_w = 0;
     int bad = 0;
-#pragma unroll 4
+#pragma unroll 8
     for (uint32_t r = 0; r < rounds; ++r) {
         const uint32_t i = w0 + r * 32 + lane;
         const uint32_t k = i < n ? key_at(i) : K;
@@ -93,11 +100,6 @@ __global__ void __launch_bounds__(kThreads, kCh == 1 ? 2 : 1) small_push_kernel(
         cnt_w += __popc(m);
     }
     if (lane == 0) s_cnt[w] = cnt_w;
-    for (int i = tid; i < kTable; i += kThreads) {
-        t_key[i] = t_first[i] = kSentinelPad;
-        t_count[i] = 0;
-    }
-    if (tid == 0) s_n_firsts = s_over = 0;
     if (__syncthreads_or(bad)) {                // the same decision in every block: nothing has been written yet
         if (A.keys64 && bucket == 0 && blockIdx.y == 0 && tid == 0) latch_error(A.st, 0u, PS_ERR_KEY_RANGE);
         return;
@@ -183,8 +185,7 @@ __global__ void __launch_bounds__(kThreads, kCh == 1 ? 2 : 1) small_push_kernel(
     };
     auto ada = [&](const float4& g, const float4& G, float4& step, float4& q) {
         q = make_float4(g.x * g.x, g.y * g.y, g.z * g.z, g.w * g.w);
-        step = make_float4(adagrad_step(g.x, G.x + q.x, A.lr, A.eps), adagrad_step(g.y, G.y + q.y, A.lr, A.eps),
-                           adagrad_step(g.z, G.z + q.z, A.lr, A.eps), adagrad_step(g.w, G.w + q.w, A.lr, A.eps));
+        adagrad_steps4(g, make_float4(G.x + q.x, G.y + q.y, G.z + q.z, G.w + q.w), A.lr, A.eps, step);
     };
     auto finish = [&](float4 r, const acc4& a) {
         r.x = (float)((double)r.x + a.x); r.y = (float)((double)r.y + a.y);
@@ -346,10 +347,8 @@ void launch_as(ps_store* ps, const SmallArgs& a, uint32_t strips, cudaStream_t s
     const size_t smem = ((size_t)a.n * 6 + 15) & ~(size_t)15;
     static std::atomic<unsigned long long> smem_set{0};
     opt_in_smem((const void*)small_push_kernel<kMode, kCh>, (size_t)kSmallOcc * 6, &smem_set);
-    if (ps->prof) prof_before(ps, kMode == kAdaGrad ? "small_push_kernel<adagrad>" : kMode == kScaled ? "small_push_kernel<scaled>" : "small_push_kernel", s);
-    small_push_kernel<kMode, kCh><<<dim3(buckets + 1, div_up_u32(strips, kCh)), kThreads, smem, s>>>(a);
-    if (ps->prof) prof_after(ps, s);
-    ps->launches++;
+    const char* name = kMode == kAdaGrad ? "small_push_kernel<adagrad>" : kMode == kScaled ? "small_push_kernel<scaled>" : "small_push_kernel";
+    PS_LAUNCH_PDL(ps, name, (small_push_kernel<kMode, kCh>), dim3(buckets + 1, div_up_u32(strips, kCh)), dim3(kThreads), smem, s, a);
 }
 template <int kMode>
 void launch(ps_store* ps, const SmallArgs& a, cudaStream_t s) {

@@ -56,6 +56,8 @@ mf_step_kernel(const uint32_t* __restrict__ ci, const uint32_t* __restrict__ cj,
     const uint64_t n_warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
     constexpr int kRegs = kCh > 0 ? kCh : 1;
     double loss = 0;
+    pdl_trigger();
+    pdl_wait();
     for (uint64_t t = warp; t < n; t += n_warps) {
         const uint32_t i = ci[t], j = cj[t];
         const float v = cv[t];
@@ -135,6 +137,8 @@ mf_step_small_kernel(const uint32_t* __restrict__ ci, const uint32_t* __restrict
     const uint64_t n_warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
     const bool act = (uint32_t)lane < L4;
     double loss = 0;
+    pdl_trigger();
+    pdl_wait();
     for (uint64_t t0 = warp * kCells; t0 < n; t0 += n_warps * kCells) {
         uint64_t kw[kCells], kh[kCells];
         float v[kCells];
@@ -201,11 +205,17 @@ uint32_t launch_step_mf(ps_store* ps, const uint32_t* d_i, const uint32_t* d_j, 
                 ps->cfg.slots_per_part, ps->cfg.num_keys, L4, (float4*)ps->upd, keys_out, ps->loss_partial,    \
                 ps->status, epoch
     // (a warp per cell for the calls without a sort: they do not fill the chip with four cells a warp)
-    if (L4 <= 32 && keys_out) PS_LAUNCH(ps, mf_step_small_kernel<1>, grid, 256, s, MF_ARGS);
-    else if (L4 <= 32) PS_LAUNCH(ps, mf_step_small_kernel<4>, grid, 256, s, MF_ARGS);
-    else if (L4 <= 64) PS_LAUNCH(ps, mf_step_kernel<2>, grid, 256, s, MF_ARGS);
-    else if (L4 <= 128) PS_LAUNCH(ps, mf_step_kernel<4>, grid, 256, s, MF_ARGS);
-    else PS_LAUNCH(ps, mf_step_kernel<0>, grid, 256, s, MF_ARGS);
+#define MF_LAUNCH(kernel)                                                                                          \
+    do {                                                                                                         \
+        if (keys_out) PS_LAUNCH_PDL(ps, #kernel, kernel, dim3(grid), dim3(256), 0, s, MF_ARGS);                    \
+        else PS_LAUNCH(ps, kernel, grid, 256, s, MF_ARGS);                                                         \
+    } while (0)
+    if (L4 <= 32 && keys_out) MF_LAUNCH(mf_step_small_kernel<1>);
+    else if (L4 <= 32) MF_LAUNCH(mf_step_small_kernel<4>);
+    else if (L4 <= 64) MF_LAUNCH(mf_step_kernel<2>);
+    else if (L4 <= 128) MF_LAUNCH(mf_step_kernel<4>);
+    else MF_LAUNCH(mf_step_kernel<0>);
+#undef MF_LAUNCH
 #undef MF_ARGS
     return grid;
 }
@@ -254,6 +264,8 @@ sgns_step_kernel(const uint32_t* __restrict__ tokens, uint64_t tok_first, uint64
     const uint64_t pairs0 = sgns_pairs_before(first_pos, T, window);
     constexpr int kQuad = 4;
     double loss = 0;
+    pdl_trigger();
+    pdl_wait();
     for (uint64_t cidx = warp; cidx < n_centers; cidx += n_warps) {
         const uint64_t p = first_pos + cidx;
         const uint64_t lo = p >= window ? p - window : 0;
@@ -420,10 +432,14 @@ uint32_t launch_step_sgns(ps_store* ps, const uint32_t* d_tokens, uint64_t tok_f
                 (float4*)ps->upd, sgns_scales(ps, n_centers), keys_out, ps->loss_partial, ps->status, epoch
 #define SG_LAUNCH(kCh, kL4, kW, kN)                                                                                  \
     do {                                                                                                             \
-        if (ps->prof) prof_before(ps, "sgns_step_kernel<" #kCh ">", s);                                              \
-        sgns_step_kernel<kCh, kL4, kW, kN><<<grid, 256, 0, s>>>(SG_ARGS);                                            \
-        if (ps->prof) prof_after(ps, s);                                                                             \
-        ps->launches++;                                                                                              \
+        if (keys_out) {                                                                                              \
+            PS_LAUNCH_PDL(ps, "sgns_step_kernel<" #kCh ">", (sgns_step_kernel<kCh, kL4, kW, kN>), dim3(grid), dim3(256), 0, s, SG_ARGS); \
+        } else {                                                                                                     \
+            if (ps->prof) prof_before(ps, "sgns_step_kernel<" #kCh ">", s);                                          \
+            sgns_step_kernel<kCh, kL4, kW, kN><<<grid, 256, 0, s>>>(SG_ARGS);                                        \
+            if (ps->prof) prof_after(ps, s);                                                                         \
+            ps->launches++;                                                                                          \
+        }                                                                                                            \
     } while (0)
     if (L4 == 75 && window == 5 && n_neg == 3) SG_LAUNCH(3, 75, 5, 3);     // 300 values, window 5, 3 negatives
     else if (L4 <= 32) SG_LAUNCH(1, 0, 0, -1);
