@@ -5,6 +5,10 @@ calls; tensors are passed as raw device (or host) pointers, the stream as the
 current torch CUDA stream.  Nothing is computed in Python.  There is no
 fallback: if the CUDA library has not been built, loading it raises.
 
+The functions called once per batch (pull, push, localize, the steps) do their
+marshalling in native code (csrc/native.cpp): through ctypes it takes 3 to 4 us
+of host time, as much as the calls of a few rows take altogether.
+
 `Store` is a small convenience wrapper that lets torch own the four device
 buffers a store needs (torch is used for device memory and streams only).
 """
@@ -90,6 +94,22 @@ SIGNATURES = {
 }
 
 _lib = None
+_native = None          # the module of csrc/native.cpp, once loaded
+
+
+def _load_native():
+    """The native part of the binding, bound to the loaded library; raises if it has not been built."""
+    global _native
+    if _native is None:
+        lib = load_library()
+        try:
+            from . import _native as mod
+        except ImportError as e:
+            raise RuntimeError(f"the native part of the binding cannot be loaded ({e}): build it with "
+                               "`python -m paper_2002_00655_b200.build`") from e
+        mod.setup({name: C.cast(getattr(lib, name), C.c_void_p).value for name in SIGNATURES}, PSError)
+        _native = mod
+    return _native
 
 
 def load_library() -> C.CDLL:
@@ -181,21 +201,19 @@ def ps_init_range_partition(ps):
 
 
 def ps_set_rows(ps, d_keys, d_vals):
-    _check(load_library().ps_set_rows(ps, _dptr(d_keys, _U64), d_keys.numel(), _dptr(d_vals, _F32), _stream()),
-           "ps_set_rows")
+    (_native or _load_native()).ps_set_rows(ps, d_keys, d_vals)
 
 
 def ps_pull(ps, d_keys, d_out):
-    _check(load_library().ps_pull(ps, _dptr(d_keys, _U64), d_keys.numel(), _dptr(d_out, _F32), _stream()), "ps_pull")
+    (_native or _load_native()).ps_pull(ps, d_keys, d_out)
 
 
 def ps_push(ps, d_keys, d_updates):
-    _check(load_library().ps_push(ps, _dptr(d_keys, _U64), d_keys.numel(), _dptr(d_updates, _F32), _stream()),
-           "ps_push")
+    (_native or _load_native()).ps_push(ps, d_keys, d_updates)
 
 
 def ps_localize(ps, worker, d_keys):
-    _check(load_library().ps_localize(ps, worker, _dptr(d_keys, _U64), d_keys.numel(), _stream()), "ps_localize")
+    (_native or _load_native()).ps_localize(ps, worker, d_keys)
 
 
 def ps_localize_beside(ps, worker, d_keys, loc_stream):
@@ -215,51 +233,39 @@ def ps_localize_stats(ps) -> dict:
 
 
 def ps_step_mf(ps, d_i, d_j, d_v, col_key_base, lr, lam, d_loss_accum=None):
-    _check(load_library().ps_step_mf(ps, _dptr(d_i, _U32), _dptr(d_j, _U32), _dptr(d_v, _F32), d_i.numel(),
-                                     col_key_base, lr, lam, _dptr(d_loss_accum, _F64), _stream()), "ps_step_mf")
+    (_native or _load_native()).ps_step_mf(ps, d_i, d_j, d_v, col_key_base, lr, lam, d_loss_accum)
 
 
 def ps_step_kge(ps, d_s, d_r, d_o, d_neg_ent, d_neg_side, n_neg, rel_key_base, dim_complex, lr, eps,
                 d_loss_accum=None):
-    _check(load_library().ps_step_kge(ps, _dptr(d_s, _U32), _dptr(d_r, _U32), _dptr(d_o, _U32),
-                                      _dptr(d_neg_ent, _U32), _dptr(d_neg_side, _U8), d_s.numel(), n_neg,
-                                      rel_key_base, dim_complex, lr, eps, _dptr(d_loss_accum, _F64), _stream()),
-           "ps_step_kge")
+    (_native or _load_native()).ps_step_kge(ps, d_s, d_r, d_o, d_neg_ent, d_neg_side, n_neg, rel_key_base, dim_complex, lr,
+                                            eps, d_loss_accum)
 
 
 def ps_step_rescal(ps, d_s, d_r, d_o, d_neg_ent, d_neg_side, n_neg, rel_key_base, dim, lr, eps, d_loss_accum=None):
-    _check(load_library().ps_step_rescal(ps, _dptr(d_s, _U32), _dptr(d_r, _U32), _dptr(d_o, _U32),
-                                         _dptr(d_neg_ent, _U32), _dptr(d_neg_side, _U8), d_s.numel(), n_neg,
-                                         rel_key_base, dim, lr, eps, _dptr(d_loss_accum, _F64), _stream()),
-           "ps_step_rescal")
+    (_native or _load_native()).ps_step_rescal(ps, d_s, d_r, d_o, d_neg_ent, d_neg_side, n_neg, rel_key_base, dim, lr, eps,
+                                               d_loss_accum)
 
 
 def ps_step_sgns(ps, d_tokens, first_pos, n_centers, window, d_negs, n_neg, out_key_base, lr, d_loss_accum=None):
-    _check(load_library().ps_step_sgns(ps, _dptr(d_tokens, _U32), first_pos, n_centers, d_tokens.numel(), window,
-                                       _dptr(d_negs, _U32), n_neg, out_key_base, lr, _dptr(d_loss_accum, _F64),
-                                       _stream()), "ps_step_sgns")
+    (_native or _load_native()).ps_step_sgns(ps, d_tokens, first_pos, n_centers, window, d_negs, n_neg, out_key_base, lr,
+                                             d_loss_accum)
 
 
 def ps_step_mf_host(ps, h_i, h_j, h_v, col_key_base, lr, lam, d_loss_accum, h_loss):
-    _check(load_library().ps_step_mf_host(ps, _hptr(h_i, _U32), _hptr(h_j, _U32), _hptr(h_v, _F32), h_i.numel(),
-                                          col_key_base, lr, lam, _dptr(d_loss_accum, _F64), _hptr(h_loss, _F64),
-                                          _stream()), "ps_step_mf_host")
+    (_native or _load_native()).ps_step_mf_host(ps, h_i, h_j, h_v, col_key_base, lr, lam, d_loss_accum, h_loss)
 
 
 def ps_step_kge_host(ps, h_s, h_r, h_o, h_neg_ent, h_neg_side, n_neg, rel_key_base, dim_complex, lr, eps,
                      d_loss_accum, h_loss):
-    _check(load_library().ps_step_kge_host(ps, _hptr(h_s, _U32), _hptr(h_r, _U32), _hptr(h_o, _U32),
-                                           _hptr(h_neg_ent, _U32), _hptr(h_neg_side, _U8), h_s.numel(), n_neg,
-                                           rel_key_base, dim_complex, lr, eps, _dptr(d_loss_accum, _F64),
-                                           _hptr(h_loss, _F64), _stream()), "ps_step_kge_host")
+    (_native or _load_native()).ps_step_kge_host(ps, h_s, h_r, h_o, h_neg_ent, h_neg_side, n_neg, rel_key_base, dim_complex,
+                                                 lr, eps, d_loss_accum, h_loss)
 
 
 def ps_step_sgns_host(ps, h_tokens, tok_first, first_pos, n_centers, corpus_len, window, h_negs, n_neg,
                       out_key_base, lr, d_loss_accum, h_loss):
-    _check(load_library().ps_step_sgns_host(ps, _hptr(h_tokens, _U32), tok_first, h_tokens.numel(), first_pos,
-                                            n_centers, corpus_len, window, _hptr(h_negs, _U32), h_negs.numel(),
-                                            n_neg, out_key_base, lr, _dptr(d_loss_accum, _F64),
-                                            _hptr(h_loss, _F64), _stream()), "ps_step_sgns_host")
+    (_native or _load_native()).ps_step_sgns_host(ps, h_tokens, tok_first, first_pos, n_centers, corpus_len, window, h_negs,
+                                                  n_neg, out_key_base, lr, d_loss_accum, h_loss)
 
 
 def ps_push_static(d_store, d_table, num_keys, row_len, slots_per_part, d_keys, d_updates) -> int:
@@ -362,13 +368,11 @@ def ps_keymap_destroy(m):
 
 
 def ps_keymap_insert(m, d_sparse, d_dense):
-    _check(load_library().ps_keymap_insert(m, _dptr(d_sparse, _U64), d_sparse.numel(), _dptr(d_dense, _U64), _stream()),
-           "ps_keymap_insert")
+    (_native or _load_native()).ps_keymap_insert(m, d_sparse, d_dense)
 
 
 def ps_keymap_lookup(m, d_sparse, d_dense):
-    _check(load_library().ps_keymap_lookup(m, _dptr(d_sparse, _U64), d_sparse.numel(), _dptr(d_dense, _U64), _stream()),
-           "ps_keymap_lookup")
+    (_native or _load_native()).ps_keymap_lookup(m, d_sparse, d_dense)
 
 
 def ps_keymap_sync(m):
@@ -387,20 +391,17 @@ class KeyMap:
 
     def __init__(self, capacity: int, max_batch_keys: int = 1 << 20, device: int = 0):
         self.device = torch.device("cuda", device)
+        self._ordinal = device
         n = ps_keymap_query_bytes(capacity, max_batch_keys)
         with torch.cuda.device(self.device):
             self.mem = torch.empty((n + 7) // 8, dtype=torch.int64, device=self.device)
             self.h = ps_keymap_create(capacity, max_batch_keys, self.mem, device)
 
     def insert(self, sparse):
-        out = torch.empty(sparse.numel(), dtype=torch.int64, device=self.device)
-        ps_keymap_insert(self.h, sparse, out)
-        return out
+        return (_native or _load_native()).map_insert(self.h, sparse, self._ordinal)
 
     def lookup(self, sparse):
-        out = torch.empty(sparse.numel(), dtype=torch.int64, device=self.device)
-        ps_keymap_lookup(self.h, sparse, out)
-        return out
+        return (_native or _load_native()).map_lookup(self.h, sparse, self._ordinal)
 
     def sync(self):
         return ps_keymap_sync(self.h)
@@ -435,6 +436,7 @@ class Store:
         self.sizes = sz
         dev = torch.device("cuda", device)
         self.device = dev
+        self._ordinal = device
         with torch.cuda.device(dev):
             self.store = torch.zeros(sz.store_bytes // 4, dtype=torch.float32, device=dev)
             self.table = torch.empty(sz.table_bytes // 8, dtype=torch.int64, device=dev)
@@ -473,15 +475,13 @@ class Store:
         torch.cuda.synchronize(self.device)
 
     def pull(self, keys):
-        out = torch.empty((keys.numel(), self.L), dtype=torch.float32, device=self.device)
-        ps_pull(self.h, keys, out)
-        return out
+        return (_native or _load_native()).pull_rows(self.h, keys, self._ordinal, self.L)
 
     def push(self, keys, updates):
-        ps_push(self.h, keys, updates)
+        (_native or _load_native()).ps_push(self.h, keys, updates)
 
     def localize(self, worker, keys):
-        ps_localize(self.h, worker, keys)
+        (_native or _load_native()).ps_localize(self.h, worker, keys)
 
     def export(self, rows=True, table=True):
         """(rows_by_key [K, L] | None, owner [K] | None, slot [K] | None) as CPU tensors."""

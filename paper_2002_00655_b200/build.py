@@ -2,7 +2,9 @@
 
 `python -m paper_2002_00655_b200.build` compiles every `csrc/*.cu` into
 `libps_b200.so` next to this file.  The library is plain C-ABI (include/ps.h);
-it links the CUDA runtime statically and depends on nothing else.
+it links the CUDA runtime statically and depends on nothing else.  Beside it,
+`csrc/native.cpp` becomes `_native`, the part of the Python binding that is
+called per batch (it links torch, whose tensors it takes).
 """
 from __future__ import annotations
 
@@ -11,6 +13,7 @@ import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 PKG = os.path.dirname(os.path.abspath(__file__))
@@ -18,6 +21,8 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 OBJ = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libps_b200.so")
+
+NATIVE = os.path.join(PKG, "_native" + sysconfig.get_config_var("EXT_SUFFIX"))
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include"), "-I", CSRC]
@@ -54,13 +59,36 @@ def build(force: bool = False, verbose: bool = False) -> str:
                 sys.stderr.write(out.stderr)
         return obj
 
-    with ThreadPoolExecutor(max_workers=4) as pool:
+    with ThreadPoolExecutor(max_workers=5) as pool:
+        native = pool.submit(build_native, force)
         objs = list(pool.map(compile_one, sources))
+        native.result()
     if force or _stale(LIB, objs):
         tmp = LIB + f".tmp{os.getpid()}"
         subprocess.check_call([nvcc, "-shared", "-o", tmp, *objs, "-gencode", "arch=compute_100a,code=sm_100a"])
         os.replace(tmp, LIB)
     return LIB
+
+
+def build_native(force: bool = False) -> str:
+    src = os.path.join(CSRC, "native.cpp")
+    if not force and not _stale(NATIVE, [src, os.path.join(ROOT, "include", "ps.h")]):
+        return NATIVE
+    import torch
+    troot = os.path.dirname(torch.__file__)
+    cuda = os.path.dirname(os.path.dirname(os.path.realpath(_nvcc())))
+    inc = [os.path.join(ROOT, "include"), os.path.join(troot, "include"),
+           os.path.join(troot, "include", "torch", "csrc", "api", "include"), sysconfig.get_paths()["include"],
+           os.path.join(cuda, "include")]
+    tmp = NATIVE + f".tmp{os.getpid()}"
+    cmd = ["g++", "-shared", "-fPIC", "-O2", "-std=c++17", "-w", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           *(x for i in inc for x in ("-isystem", i)), src, "-o", tmp, "-L", os.path.join(troot, "lib"),
+           "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"]
+    out = subprocess.run(cmd, capture_output=True, text=True)
+    if out.returncode != 0:
+        raise RuntimeError(f"g++ failed on {src}:\n{out.stdout}\n{out.stderr}")
+    os.replace(tmp, NATIVE)
+    return NATIVE
 
 
 if __name__ == "__main__":
