@@ -12,9 +12,7 @@
 namespace psb {
 
 constexpr uint32_t kSentinelPad = 0xFFFFFFFFu;   // never a key: num_keys < 2^32 - 1
-constexpr int kSortThreads = 256;
-constexpr int kSortItems = 8;
-constexpr int kSortTile = kSortThreads * kSortItems;   // keys per sort block
+constexpr int kSortTile = 2048;                  // the sort's counters have room for a block per half of this
 constexpr int kRadixBits = 8;
 constexpr int kRadix = 1 << kRadixBits;
 constexpr int kMaxSortPasses = 4;                // 32-bit keys

@@ -12,7 +12,7 @@
 // counts are gathered while the PREVIOUS pass scatters: a key that goes to
 // position pos adds one to counter [next pass][chunk of pos][next digit].  So
 // a pass is: grid barrier, read one column of counters per digit, rank the
-// chunk's keys tile by tile (warp match + per-warp counters: stable), scatter.
+// chunk's keys tile by tile (warp_rank: stable), scatter.
 // The key source of the first pass and the sink of the last pass are functors:
 // a step extracts its keys from the batch arrays inside the sort, and the
 // matrix-factorization step has the last pass emit, per sorted position, the
@@ -93,6 +93,66 @@ struct SinkMF {
     uint32_t* cellpos;                  // sorted position of each cell's row-factor occurrence
 };
 
+// the records of `len` sorted (key, value) pairs in shared memory, positions c0 on: a thread has kAtOnce of them under way
+// (all index loads, then all table loads, then the records)
+__device__ __forceinline__ void sink_records(const SinkMF& sink, const uint2* buf, uint32_t len, uint32_t c0, uint32_t* kout) {
+    constexpr int kAtOnce = 4;
+    for (uint32_t l0 = threadIdx.x; l0 < len; l0 += kAtOnce * blockDim.x) {
+        uint2 x[kAtOnce];
+        uint32_t pk[kAtOnce];
+        float cval[kAtOnce];
+        uint2 e_own[kAtOnce], e_par[kAtOnce];
+#pragma unroll
+        for (int i = 0; i < kAtOnce; ++i) {
+            const uint32_t l = l0 + i * blockDim.x;
+            x[i] = l < len ? buf[l] : make_uint2(sink.K, 0u);
+            pk[i] = sink.K;                             // cells with an index out of range carry the mark K
+            cval[i] = 0.f;
+            if (x[i].x < sink.K) {
+                const uint32_t cell = x[i].y >> 1;
+                pk[i] = (x[i].y & 1u) ? sink.ci[cell] : sink.col_base + sink.cj[cell];
+                cval[i] = sink.cv[cell];
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < kAtOnce; ++i) {
+            e_own[i] = x[i].x < sink.K ? sink.table[x[i].x] : make_uint2(0u, 0u);
+            e_par[i] = x[i].x < sink.K ? sink.table[pk[i]] : make_uint2(0u, 0u);
+        }
+#pragma unroll
+        for (int i = 0; i < kAtOnce; ++i) {
+            const uint32_t l = l0 + i * blockDim.x;
+            if (l >= len) break;
+            const uint32_t pos = c0 + l;
+            kout[pos] = x[i].x;
+            if (!(x[i].y & 1u)) sink.cellpos[x[i].y >> 1] = pos;
+            sink.rec[pos] = make_uint4(x[i].y >> 1, __float_as_uint(cval[i]), (uint32_t)phys_row(e_own[i], sink.S),
+                                       (uint32_t)phys_row(e_par[i], sink.S));
+        }
+    }
+}
+
+// Rank of a lane's digit among the warp's keys so far (stable: item by item, lane by lane), and the warp's counter of the
+// digit moved on.  Lanes with equal digits find one another through a word per digit in shared memory (every lane ORs its
+// bit in); __match_any_sync takes 61 cycles of an SM per instruction, the OR and the read 6.  `mask` is all zero before
+// and after.
+__device__ __forceinline__ uint32_t warp_rank(volatile uint32_t* mask, volatile uint32_t* hist, uint32_t digit, bool valid,
+                                              int lane) {
+    if (valid) atomicOr(const_cast<uint32_t*>(mask) + digit, 1u << lane);
+    __syncwarp();
+    const uint32_t peers = valid ? mask[digit] : 1u << lane;
+    const int leader = 31 - __clz(peers);
+    uint32_t old = 0;
+    if (valid && lane == leader) {
+        old = hist[digit];
+        hist[digit] = old + __popc(peers);
+    }
+    old = __shfl_sync(0xffffffffu, old, leader);
+    if (valid && lane == leader) mask[digit] = 0u;
+    __syncwarp();
+    return old + __popc(peers & ((1u << lane) - 1u));
+}
+
 // Exclusive scan of one value per digit held by threads 0..255 of a block of kThreads; every thread calls.
 template <int kThreads>
 __device__ __forceinline__ uint32_t scan_digits(uint32_t v, uint32_t* sm8, uint32_t* total) {
@@ -120,7 +180,7 @@ __device__ __forceinline__ uint32_t scan_digits(uint32_t v, uint32_t* sm8, uint3
 // A tile is kThreads x kItems keys.  Small sorts use many threads with few keys each (every phase of a pass is a
 // short chain of dependent steps, and all SMs get a tile); large sorts use 256 threads with 8 keys each.
 template <class Src, class Sink, int kThreads, int kItems>
-__global__ void __launch_bounds__(kThreads, kThreads == 256 ? 3 : 2)
+__global__ void __launch_bounds__(kThreads, kThreads == 256 ? 3 : kThreads == 512 ? 2 : 1)
 sort_all_kernel(Src src, Sink sink, SortParams P) {
     constexpr int kTile = kThreads * kItems;
     constexpr int kWarps = kThreads / 32;
@@ -128,10 +188,11 @@ sort_all_kernel(Src src, Sink sink, SortParams P) {
     constexpr int kRowsAtOnce = kThreads >= 512 ? 16 : 8;
     __shared__ uint32_t digit_base[kRadix];          // global position of the tile's first key with each digit
     __shared__ uint32_t local_base[kRadix];          // the same inside the tile
-    __shared__ uint32_t warp_hist[kWarps][kRadix];
-    extern __shared__ uint32_t s_dyn[];               // the tile in digit order, on its way out: keys, then values
+    extern __shared__ __align__(16) uint32_t s_dyn[];  // the tile in digit order, on its way out: keys, then values
     uint32_t* const s_key = s_dyn;
     uint32_t* const s_val = s_dyn + kTile;
+    uint32_t (*const warp_hist)[kRadix] = reinterpret_cast<uint32_t (*)[kRadix]>(s_dyn + 2 * kTile);
+    uint32_t (*const warp_mask)[kRadix] = warp_hist + kWarps;
     __shared__ uint32_t sm[8];
     __shared__ int s_ok;
     const uint32_t n = P.n_dev ? tmin<uint32_t>(*((const volatile unsigned int*)P.n_dev), P.n_host) : P.n_host;
@@ -144,7 +205,7 @@ sort_all_kernel(Src src, Sink sink, SortParams P) {
     const uint32_t c0 = c0_64 < n ? (uint32_t)c0_64 : n;
     const uint32_t c1 = (uint64_t)c0 + chunk < n ? c0 + chunk : n;
     const uint32_t my_tiles = (c1 - c0 + kTile - 1) / kTile;
-    const unsigned lt = (1u << lane) - 1u;
+    const uint32_t magic = (uint32_t)tmin<uint64_t>(((1ull << 32) + chunk - 1) / chunk, 0xFFFFFFFFull);
     unsigned int barriers = 0;
 
     // ---- before the first barrier: clear what must start at zero, count the digits of pass 0 ----
@@ -152,6 +213,7 @@ sort_all_kernel(Src src, Sink sink, SortParams P) {
         for (int p = 1; p < P.n_passes; ++p) P.counts[((size_t)p * G + b) * kRadix + tid] = 0u;
         digit_base[tid] = 0u;
     }
+    for (int i = tid; i < kWarps * kRadix; i += kThreads) (&warp_mask[0][0])[i] = 0u;
     if (b == 0) {
         for (uint32_t i = tid; i < P.n_zero_a; i += kThreads) P.zero_a[i] = 0u;
         if (tid == 0 && P.zero_b) P.zero_b[0] = P.zero_b[1] = 0u;     // (the list counter of the coming reduction and its neighbour)
@@ -257,28 +319,9 @@ sort_all_kernel(Src src, Sink sink, SortParams P) {
             const uint32_t tb = t0 + w * (32 * kItems);
             const uint32_t in_tile = tmin<uint32_t>((uint32_t)kTile, c1 - t0);
             uint32_t rank[kItems];
-            unsigned peers[kItems];
-            // lanes of the warp that hold the same digit (lanes past the end get a pseudo-digit of their own)
 #pragma unroll
-            for (int it = 0; it < kItems; ++it) {
-                const bool valid = tb + it * 32 + lane < c1;
-                const uint32_t digit = (key[it] >> shift) & (kRadix - 1);
-                peers[it] = __match_any_sync(0xffffffffu, valid ? digit : (kRadix + lane));
-            }
-#pragma unroll
-            for (int it = 0; it < kItems; ++it) {
-                const bool valid = tb + it * 32 + lane < c1;
-                const uint32_t digit = (key[it] >> shift) & (kRadix - 1);
-                const int leader = __ffs(peers[it]) - 1;
-                uint32_t old = 0;
-                if (valid && lane == leader) {
-                    old = warp_hist[w][digit];
-                    warp_hist[w][digit] = old + __popc(peers[it]);
-                }
-                old = __shfl_sync(0xffffffffu, old, leader);
-                rank[it] = old + __popc(peers[it] & lt);
-                __syncwarp();
-            }
+            for (int it = 0; it < kItems; ++it)
+                rank[it] = warp_rank(warp_mask[w], warp_hist[w], (key[it] >> shift) & (kRadix - 1), tb + it * 32 + lane < c1, lane);
             __syncthreads();
             // thread d: this tile's count of digit d; the per-warp counters become offsets inside the digit
             uint32_t run = 0;
@@ -322,13 +365,16 @@ sort_all_kernel(Src src, Sink sink, SortParams P) {
                         kout[pos[it]] = key[it];
                         vout[pos[it]] = val[it];
                     }
-                    // one more key with this digit of the next pass in the chunk the key lands in; lanes that
-                    // agree on both send one addition
+                    // one more key with this digit of the next pass in the chunk the key lands in; neighbouring lanes that
+                    // agree on both (a frequent key's occurrences stand together) send one addition
                     const uint32_t nd = (key[it] >> (shift + kRadixBits)) & (kRadix - 1);
-                    const uint32_t cell = valid ? (pos[it] / chunk) * kRadix + nd : 0xFFFFFFFFu - lane;
-                    const unsigned same = __match_any_sync(0xffffffffu, cell);
-                    if (valid && lane == __ffs(same) - 1)
-                        atomicAdd(P.counts + (size_t)(p + 1) * G * kRadix + cell, (uint32_t)__popc(same));
+                    uint32_t to = __umulhi(pos[it], magic);         // pos / chunk, or one more
+                    if (to * chunk > pos[it]) --to;
+                    const uint32_t cell = valid ? to * kRadix + nd : 0xFFFFFFFFu;
+                    const uint32_t left = __shfl_up_sync(0xffffffffu, cell, 1);
+                    const bool head = lane == 0 || left != cell;
+                    const unsigned later = __ballot_sync(0xffffffffu, head) & ~((2u << lane) - 1u);
+                    if (valid && head) atomicAdd(P.counts + (size_t)(p + 1) * G * kRadix + cell, (uint32_t)((later ? __ffs(later) - 1 : 32) - lane));
                 }
             } else if constexpr (Sink::kPairs) {
 #pragma unroll
@@ -388,13 +434,184 @@ sort_all_kernel(Src src, Sink sink, SortParams P) {
     grid_leave(P.bar, G);
 }
 
+// ------------------------------------------------------------------------------------------------
+// Sorts of at most kClusterSort keys as one cluster of sixteen blocks.  The keys stay in the blocks' shared memory from
+// the first pass to the last; a pass ranks a block's chunk (warp_rank: stable), tells every
+// other block its digit counts (a 16 x 256 matrix in each block's shared memory) and scatters each key to its place in
+// another block's shared memory.  The blocks meet at the cluster's hardware barrier, twice per pass.
+// 20,000 24-bit keys: 18.5 us against 24.7 of the cooperative form, whose passes go through global memory and a grid barrier.
+// With 16 keys a thread it would take 131,072, but sixteen SMs are too few for that many (48 us against 26), and the
+// records of the matrix-factorization step's sink want the whole chip's loads in flight (74 us against 34).
+constexpr int kClThreads = 512, kClItems = 4, kClBlocks = 16, kClWarps = kClThreads / 32;
+constexpr uint32_t kClChunk = kClThreads * kClItems;
+constexpr uint32_t kClusterSort = kClBlocks * kClChunk;         // 32,768
+static_assert(kClusterSort <= (1u << 17) && kClItems * 32 <= (1 << 15), "value and rank share a register");
+
+struct ClusterSmem {
+    uint2 buf[kClChunk];                    // the chunk's (key, value) pairs
+    uint32_t warp_hist[kClWarps][kRadix], warp_mask[kClWarps][kRadix];
+    uint32_t counts[kClBlocks][kRadix];     // digit counts of all blocks, written by them
+    uint32_t base[kRadix];
+    uint32_t sm[8];
+};
+
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory"); }
+__device__ __forceinline__ uint32_t peer_smem(const void* p, uint32_t rank) {
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(r) : "r"(smem_addr(p)), "r"(rank));
+    return r;
+}
+
+template <class Src, class Sink>
+__global__ void __launch_bounds__(kClThreads, 2)
+sort_cluster_kernel(Src src, Sink sink, SortParams P) {
+    extern __shared__ __align__(16) unsigned char cl_dyn[];
+    ClusterSmem& M = *reinterpret_cast<ClusterSmem*>(cl_dyn);
+    const uint32_t n = P.n_dev ? tmin<uint32_t>(*((const volatile unsigned int*)P.n_dev), P.n_host) : P.n_host;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const uint32_t b = blockIdx.x;
+    cluster_arrive();                       // (every block has started: before the first write to another's memory)
+    if (b == 0) {
+        for (uint32_t i = tid; i < P.n_zero_a; i += kClThreads) P.zero_a[i] = 0u;
+        if (tid == 0 && P.zero_b) P.zero_b[0] = P.zero_b[1] = 0u;
+    }
+    const uint32_t chunk = tmax<uint32_t>((n + kClBlocks - 1) / kClBlocks, 32u);    // (at least two: `magic` has 32 bits)
+    const uint32_t magic = (uint32_t)(((1ull << 32) + chunk - 1) / chunk);      // pos / chunk, exact for 17-bit positions
+    const uint32_t c0 = tmin<uint32_t>(b * chunk, n), len = tmin<uint32_t>(chunk, n - c0);
+    const uint32_t share = ((chunk + kClWarps - 1) / kClWarps + 31) & ~31u;     // consecutive positions per warp
+    const uint32_t l0 = w * share + lane;
+    for (int i = lane; i < kRadix; i += 32) M.warp_mask[w][i] = 0u;
+    uint32_t key[kClItems], vr[kClItems];
+    {
+        const uint32_t* kin = (P.start & 1) ? P.kB : P.kA;
+#pragma unroll
+        for (int it = 0; it < kClItems; ++it) {
+            const uint32_t l = l0 + it * 32;
+            key[it] = 0u;
+            vr[it] = c0 + l;
+            if (it * 32 < share && l < len) key[it] = Src::kFromBuffer ? __ldcg(kin + c0 + l) : src(c0 + l, P);
+        }
+    }
+    cluster_wait();
+    for (int p = 0; p < P.n_passes; ++p) {
+        const int shift = p * kRadixBits;
+        if (p > 0) {
+#pragma unroll
+            for (int it = 0; it < kClItems; ++it) {
+                const uint32_t l = l0 + it * 32;
+                if (it * 32 < share && l < len) {
+                    const uint2 x = M.buf[l];
+                    key[it] = x.x;
+                    vr[it] = x.y;
+                }
+            }
+        }
+        for (int i = lane; i < kRadix; i += 32) M.warp_hist[w][i] = 0u;
+        __syncwarp();
+#pragma unroll
+        for (int it = 0; it < kClItems; ++it) {
+            if (it * 32 >= share) break;
+            vr[it] |= warp_rank(M.warp_mask[w], M.warp_hist[w], (key[it] >> shift) & (kRadix - 1), l0 + it * 32 < len, lane) << 17;
+        }
+        __syncthreads();
+        if (tid < kRadix) {
+            uint32_t run = 0;
+#pragma unroll
+            for (int i = 0; i < kClWarps; ++i) {
+                const uint32_t c = M.warp_hist[i][tid];
+                M.warp_hist[i][tid] = run;
+                run += c;
+            }
+#pragma unroll
+            for (uint32_t r = 0; r < kClBlocks; ++r)
+                asm volatile("st.shared::cluster.u32 [%0], %1;\n" ::"r"(peer_smem(&M.counts[b][tid], r)), "r"(run) : "memory");
+        }
+        cluster_arrive();
+        cluster_wait();
+        uint32_t before = 0, total = 0;
+        if (tid < kRadix) {
+#pragma unroll
+            for (uint32_t r = 0; r < kClBlocks; ++r) {
+                const uint32_t c = M.counts[r][tid];
+                if (r < b) before += c;
+                total += c;
+            }
+        }
+        uint32_t all;
+        const uint32_t gbase = scan_digits<kClThreads>(total, M.sm, &all);      // has barriers
+        if (tid < kRadix) M.base[tid] = gbase + before;
+        __syncthreads();
+#pragma unroll
+        for (int it = 0; it < kClItems; ++it) {
+            if (it * 32 >= share) break;
+            if (l0 + it * 32 < len) {
+                const uint32_t digit = (key[it] >> shift) & (kRadix - 1);
+                const uint32_t pos = M.base[digit] + M.warp_hist[w][digit] + (vr[it] >> 17);
+                const uint32_t to = __umulhi(pos, magic);
+                asm volatile("st.shared::cluster.v2.u32 [%0], {%1, %2};\n" ::"r"(peer_smem(&M.buf[pos - to * chunk], to)),
+                             "r"(key[it]), "r"(vr[it] & 0x1ffffu)
+                             : "memory");
+            }
+        }
+        cluster_arrive();
+        cluster_wait();
+    }
+    uint32_t* kout = ((P.start + P.n_passes) & 1) ? P.kB : P.kA;
+    uint32_t* vout = ((P.start + P.n_passes) & 1) ? P.vB : P.vA;
+    if constexpr (Sink::kPairs) {
+        for (uint32_t l = tid; l < len; l += kClThreads) {
+            const uint2 x = M.buf[l];
+            kout[c0 + l] = x.x;
+            vout[c0 + l] = x.y;
+        }
+    } else {
+        sink_records(sink, M.buf, len, c0, kout);
+    }
+}
+
 // Small sorts: few blocks of many threads.  The sort of the next step runs beside the current step's kernels;
 // its blocks spend most of their life waiting at grid barriers, so it should hold few SMs' registers while it
 // does, and the cost of a pass grows with the number of blocks (barrier, counter read) more than with the keys
 // per block.
 constexpr int kSmallThreads = 512, kSmallItems = 4;      // tiles of 2048 keys
 constexpr int kSmallTile = kSmallThreads * kSmallItems;
+// Large sorts (more than a short tile per block): tiles of 4,096 keys.  1M keys in 88 us with 256 threads x 8, 71 us with 512 x 4,
+// 69 with 512 x 8, 65 with 1024 x 8, which holds whole SMs while kernels of other streams run beside it (skip-gram step
+// 788 us against 783).
+constexpr int kBigThreads = 512, kBigItems = 8;
+constexpr size_t sort_smem(int threads, int items) { return ((size_t)2 * threads * items + 2 * (threads / 32) * kRadix) * sizeof(uint32_t); }
 static_assert(kSmallTile >= kSortTile / 2, "the digit counters are sized for tiles of at least kSortTile / 2 keys");
+
+// Once per device: the opt-ins (shared memory, a cluster of more than eight blocks), and whether such a cluster can be
+// resident at all (a GPU's clusters are as large as its smallest partition of multiprocessors allows).
+template <class Src, class Sink>
+static bool cluster_sort_fits() {
+    static std::atomic<unsigned long long> asked{0}, fits{0};
+    int d = -1;
+    if (cudaGetDevice(&d) != cudaSuccess || d < 0 || d >= 64) return false;
+    if (!((asked.load(std::memory_order_acquire) >> d) & 1ull)) {
+        const void* fn = (const void*)sort_cluster_kernel<Src, Sink>;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(kClBlocks);
+        cfg.blockDim = dim3(kClThreads);
+        cfg.dynamicSmemBytes = sizeof(ClusterSmem);
+        cudaLaunchAttribute attr;
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = kClBlocks;
+        attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        int clusters = 0;
+        if (cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+            cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(ClusterSmem)) == cudaSuccess &&
+            cudaOccupancyMaxActiveClusters(&clusters, sort_cluster_kernel<Src, Sink>, &cfg) == cudaSuccess && clusters > 0)
+            fits.fetch_or(1ull << d, std::memory_order_relaxed);
+        cudaGetLastError();
+        asked.fetch_or(1ull << d, std::memory_order_release);
+    }
+    return (fits.load(std::memory_order_relaxed) >> d) & 1ull;
+}
 
 template <class Src, class Sink>
 static int sort_launch(ps_store* ps, const Src& src, const Sink& sink, uint32_t n, const unsigned int* n_dev, int bits,
@@ -409,7 +626,7 @@ static int sort_launch(ps_store* ps, const Src& src, const Sink& sink, uint32_t 
     const uint32_t max_grid = (uint32_t)tmax(ps->sm_count, 1);
     // short tiles while they still give every block at most one (and the counters have room for that many blocks)
     const bool small = n <= max_grid * (uint32_t)kSmallTile && div_up_u32(n, kSmallTile) <= ps->sort_blocks_cap;
-    const uint32_t tile = small ? kSmallTile : kSortTile;
+    const uint32_t tile = small ? kSmallTile : kBigThreads * kBigItems;
     const uint32_t n_tiles = div_up_u32(n, tile);
     P.tiles_per_block = div_up_u32(n_tiles, max_grid);
     const uint32_t grid = div_up_u32(n_tiles, P.tiles_per_block);
@@ -420,21 +637,39 @@ static int sort_launch(ps_store* ps, const Src& src, const Sink& sink, uint32_t 
     P.zero_b = zero_me;
     P.st = ps->status;
     P.epoch = ps->epoch;
+    if (n <= kClusterSort && Sink::kPairs && cluster_sort_fits<Src, Sink>()) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(kClBlocks);
+        cfg.blockDim = dim3(kClThreads);
+        cfg.dynamicSmemBytes = sizeof(ClusterSmem);
+        cfg.stream = stream;
+        cudaLaunchAttribute attr;
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = kClBlocks;
+        attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        if (ps->prof) prof_before(ps, "sort_cluster_kernel", stream);
+        cudaLaunchKernelEx(&cfg, sort_cluster_kernel<Src, Sink>, src, sink, P);
+        if (ps->prof) prof_after(ps, stream);
+        ps->launches++;
+        return (start + P.n_passes) & 1;
+    }
     if (ps->prof) prof_before(ps, "sort_all_kernel", stream);
     void* args[] = {(void*)&src, (void*)&sink, (void*)&P};
     // cooperative: the blocks wait for one another at the grid barrier, so all of them must be resident
     if (small) {
         static std::atomic<unsigned long long> attr_set{0};
         const void* fn = (const void*)sort_all_kernel<Src, Sink, kSmallThreads, kSmallItems>;
-        const size_t smem = (size_t)2 * kSmallTile * sizeof(uint32_t);
+        const size_t smem = sort_smem(kSmallThreads, kSmallItems);
         opt_in_smem(fn, smem, &attr_set);
         cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(kSmallThreads), args, smem, stream);
     } else {
         static std::atomic<unsigned long long> attr_set{0};
-        const void* fn = (const void*)sort_all_kernel<Src, Sink, kSortThreads, kSortItems>;
-        const size_t smem = (size_t)2 * kSortTile * sizeof(uint32_t);
+        const void* fn = (const void*)sort_all_kernel<Src, Sink, kBigThreads, kBigItems>;
+        const size_t smem = sort_smem(kBigThreads, kBigItems);
         opt_in_smem(fn, smem, &attr_set);
-        cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(kSortThreads), args, smem, stream);
+        cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(kBigThreads), args, smem, stream);
     }
     if (ps->prof) prof_after(ps, stream);
     ps->launches++;

@@ -94,3 +94,27 @@ def test_localize_around_the_limit_of_the_single_launch(N, L, counts):
     g.localize(0, dev(np.array([3, K])))
     assert g.sync(check=False) == ps.PS_ERR_KEY_RANGE
     compare_state(g, o, exact_rows=True, what="bad key")
+
+
+@pytest.mark.parametrize("n", [8_193, 16_384, 32_767, 32_768, 32_769, 303_104, 303_105, 606_300])
+@pytest.mark.parametrize("K", [200, 70_000])
+def test_sorted_pushes_around_the_limits_of_the_sorts(n, K):
+    """The sort in one cluster, the cooperative one with a short tile per block and with longer ones: sizes around the
+    changes, keys of one and of three digits, a key that is a third of the batch and runs of equal keys."""
+    L = 4
+    g, o = make_pair(K, L, 3, max_batch_keys=n)
+    rng = np.random.default_rng(n + K)
+    keys = rng.integers(0, K, size=n)
+    keys[rng.random(n) < 0.33] = K // 3
+    keys[n // 2:n // 2 + 3000] = K - 1
+    upd = rng.normal(size=(n, L)).astype(np.float32)
+    rows = torch.from_numpy(o.rows.copy())
+    out = []
+    for _ in range(2):                                              # the order of a key's terms is that of the call: same bits again
+        g.set_all_rows(rows)
+        g.push(dev(keys), dev(upd))
+        g.sync()
+        out.append(g.export(table=False)[0])
+    assert torch.equal(out[0], out[1])
+    o.push(keys, upd)
+    compare_state(g, o, what=f"push of {n}")
