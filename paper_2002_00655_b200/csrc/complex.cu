@@ -41,24 +41,342 @@ struct KgeArgs {
     unsigned int epoch;
 };
 
-// kMaxNeg bounds n_neg at compile time so that a data point's values live in registers: for every block of 32
-// dimensions the Re and Im of all its rows are requested together, before any is used.  kDim / kExact: the complex
-// dimension and "n_neg equals kMaxNeg" known at compile time (0 / false: taken from the arguments).
-// kAcc: some slots need their accumulators here (rows updated in place, finished rows).
-// kW: warps per data point.  One for rows of up to 128 complex dimensions (eight data points per block); eight for
-// longer ones: a data point's rows are then read by one block within a short time, so that the second pass over them
-// finds them in L2 (13 rows of 32 KB per block, one or two blocks per SM, fit; a data point per warp does not).
-template <int kMaxNeg, int kDim, bool kExact, int kW, bool kAcc>
-__global__ void __launch_bounds__(256, kMaxNeg <= 10 ? 2 : 1) kge_points_kernel(const KgeArgs A) {
-    constexpr int kGroups = 8 / kW;                             // data points per block at a time
+// Sums over the 32 lanes of NP values each, NP a power of two: halves are exchanged, so that each step leaves half as many
+// values per lane to add (NP + 5 - log2 NP exchanges in place of 5 NP).  Lane l is left with value l / (32 / NP).
+template <int NP>
+__device__ __forceinline__ double lane_sums(double (&v)[NP], int lane) {
+    int o = 16;
+#pragma unroll
+    for (int w = NP / 2; w >= 1; w >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int i = 0; i < w; ++i) {
+            const double send = up ? v[i] : v[i + w], keep = up ? v[i + w] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+        o >>= 1;
+    }
+    for (; o; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+    return v[0];
+}
+
+// Rows of at most 128 complex dimensions: a warp per data point.  The embeddings of its rows arrive in the warp's shared
+// memory as bulk copies asked for all at once, the next data point's keys and table entries are looked up meanwhile, and
+// both passes over the dimensions read from there: no load inside a pass.  (With loads into registers before each block of
+// dimensions the passes were chains of memory latencies at 16 warps per SM: 66 us for 8,192 data points of dimension 100,
+// 113 us where it also updated the rows whose key occurs once, with 84 and 45 us for the reduction; this one takes 89 with
+// those updates, 43 instead of 78 at 3,000 data points of dimension 60 with 20 negatives.  Four dimensions per lane at a time
+// spill: 100 us.)
+// A lane has two dimensions at a time.  kV2: consecutive ones, as pairs (d even); otherwise 32 apart.
+constexpr int kShortWarps = 4;
+
+template <bool kV2> struct Dims {                               // dimensions at and at + kStep
+    static constexpr uint32_t kStep = kV2 ? 1 : 32;
+    __device__ static __forceinline__ void load(const float* row, uint32_t at, uint32_t d, float (&v)[2]) {
+        if constexpr (kV2) {
+            const float2 x = *reinterpret_cast<const float2*>(row + at);
+            v[0] = x.x; v[1] = x.y;
+        } else {
+            v[0] = row[at];
+            v[1] = at + kStep < d ? row[at + kStep] : 0.f;
+        }
+    }
+    __device__ static __forceinline__ void store(float* row, uint32_t at, uint32_t d, const float (&v)[2]) {
+        if constexpr (kV2) {
+            *reinterpret_cast<float2*>(row + at) = make_float2(v[0], v[1]);
+        } else {
+            row[at] = v[0];
+            if (at + kStep < d) row[at + kStep] = v[1];
+        }
+    }
+};
+
+// kAcc: some slots need their accumulators here (rows updated in place, finished rows); otherwise gradients are all it writes.
+template <int kMaxNeg, bool kV2, bool kAcc>
+__global__ void __launch_bounds__(32 * kShortWarps, kMaxNeg <= 10 ? 4 : 2) kge_short_kernel(const KgeArgs A) {
+    constexpr int NP = kMaxNeg < 8 ? 8 : kMaxNeg < 16 ? 16 : 32;
+    using D = Dims<kV2>;
+    extern __shared__ __align__(128) float row_mem[];           // [warp][slot][row_len]
+    __shared__ __align__(8) uint64_t bars[kShortWarps];
+    __shared__ double s_w[kShortWarps][3][32];                  // coefficient of negative q; weights of a slot's two directions
+    __shared__ uint64_t s_off[kShortWarps][32];
+    __shared__ double s_loss[kShortWarps];
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const uint32_t d = A.d, n_neg = A.n_neg;
+    const int n_slots = 3 + (int)n_neg;
+    const bool slot = lane < n_slots;
+    const uint64_t L = 4 * (uint64_t)d, K = A.K;
+    const uint32_t rl = (2 * d + 3) & ~3u;                      // floats copied per row: the embedding, to a multiple of 16 bytes
+    float* const rows = row_mem + (size_t)w * n_slots * rl;
+    if (lane == 0) mbar_init(&bars[w], 1);
+    mbar_init_fence();
+    pdl_trigger();
+    pdl_wait();
+    if (A.single && call_failed(A.st, A.epoch)) return;
+    const uint64_t n_warps = (uint64_t)gridDim.x * kShortWarps;
+    uint64_t t = (uint64_t)blockIdx.x * kShortWarps + w;
+    // a data point's slots, lane u slot u: key (K: no slot; all ones: out of range) and side
+    auto key_of = [&](uint64_t t2, int& side) -> uint64_t {
+        side = 0;
+        if (!slot || t2 >= A.n) return K;
+        if (lane == 1) {
+            const uint64_t k = A.rel_base + A.tr[t2];
+            return k < K ? k : ~0ull;
+        }
+        const uint32_t e = lane == 0 ? A.ts[t2] : (lane == 2 ? A.to[t2] : A.neg_ent[t2 * n_neg + (lane - 3)]);
+        if (lane >= 3) side = A.neg_side[t2 * n_neg + (lane - 3)] != 0;
+        return e < A.rel_base ? e : ~0ull;
+    };
+    auto entry_of = [&](uint64_t k) { return k < K ? A.table[k] : make_uint2(0u, 0u); };
+    auto once_of = [&](uint64_t t2) { return slot && A.single && t2 < A.n && A.single[t2 * n_slots + lane]; };
+    int side, next_side = 0;
+    uint64_t key = key_of(t, side);
+    uint2 entry = entry_of(key);
+    bool alone = once_of(t);
+    unsigned parity = 0;
+    double loss = 0;
+    for (; t < A.n; t += n_warps) {
+        const bool bad = __any_sync(full, key == ~0ull);
+        const unsigned same = __match_any_sync(full, slot ? (uint32_t)key : kSentinelPad);
+        const int rep = slot ? __ffs(same) - 1 : lane;
+        const bool once = alone && rep == lane;
+        const uint64_t off = phys_row(entry, A.S) * L;
+        const int my_side = side;
+        if (!bad && lane == 0) mbar_expect_tx(&bars[w], (uint32_t)n_slots * rl * 4);
+        __syncwarp();
+        if (!bad && slot) {
+            bulk_g2s(rows + lane * rl, A.store + off, rl * 4, &bars[w]);
+            if (once)                                           // its accumulators are wanted at the end
+                for (uint32_t o = 0; o < 2 * d; o += 32) asm volatile("prefetch.global.L2 [%0];" ::"l"(A.store + off + 2 * d + o));
+        }
+        s_off[w][lane] = off;
+        if (A.keys_out && slot) A.keys_out[t * n_slots + lane] = bad ? kSentinelPad : rep == lane ? (uint32_t)key : (uint32_t)K;
+        // the next data point's look-ups travel beside this one's rows
+        const uint64_t next_key = key_of(t + n_warps, next_side);
+        const bool next_alone = once_of(t + n_warps);
+        const unsigned subj_mask = __ballot_sync(full, lane >= 3 && slot && my_side == 0) >> 3;
+        const unsigned rep_mask = __ballot_sync(full, slot && rep == lane), once_mask = __ballot_sync(full, once);
+        const unsigned acc_mask = !kAcc ? 0u : A.finished ? rep_mask : once_mask;   // slots whose accumulators are needed here
+        const int rep_o = __shfl_sync(full, rep, 2);            // 0 if object == subject
+        const uint2 next_entry = entry_of(next_key);
+        if (bad) {                                              // (the same decision in every lane)
+            if (lane == 0) latch_error(A.st, A.keys_out ? 0u : A.epoch, PS_ERR_KEY_RANGE);
+            key = next_key; entry = next_entry; alone = next_alone; side = next_side;
+            continue;
+        }
+        if (!mbar_wait(&bars[w], parity) && !mbar_wait(&bars[w], parity)) {
+            if (lane == 0) latch_error(A.st, A.epoch, PS_ERR_CUDA);
+            break;                                              // a copy that does not arrive: give the call up
+        }
+        parity ^= 1;
+        auto emb = [&](int u, int part, uint32_t at, float (&v)[2]) { D::load(rows + u * rl + part * d, at, d, v); };
+        // ---- pass A: partial scores of the 1 + n_neg triples over this lane's dimensions ----
+        double part[NP];
+#pragma unroll
+        for (int q = 0; q < NP; ++q) part[q] = 0.0;
+        for (uint32_t c0 = 0; c0 < d; c0 += 64) {
+            const uint32_t at = c0 + (kV2 ? 2 * lane : lane);
+            if (at >= d) continue;
+            float av[2], bv[2], crv[2], civ[2], ev[2], fv[2];
+            emb(0, 0, at, av); emb(0, 1, at, bv); emb(1, 0, at, crv); emb(1, 1, at, civ); emb(2, 0, at, ev); emb(2, 1, at, fv);
+            double re_o[2], im_o[2], re_s[2], im_s[2];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const double a = av[i], b = bv[i], cr = crv[i], ci = civ[i], e = ev[i], f = fv[i];
+                part[0] += cr * (a * e + b * f) + ci * (a * f - b * e);
+                // (n, r, o): cr (na e + nb f) + ci (na f - nb e);   (s, r, n): cr (a na + b nb) + ci (a nb - b na)
+                re_o[i] = cr * e + ci * f; im_o[i] = cr * f - ci * e;       // multiplies (na, nb) in the subject's place
+                re_s[i] = cr * a - ci * b; im_s[i] = cr * b + ci * a;       // ... in the object's place
+            }
+#pragma unroll
+            for (int q = 0; q < kMaxNeg; ++q) {
+                if (q >= (int)n_neg) break;
+                float na[2], nb[2];
+                emb(3 + q, 0, at, na); emb(3 + q, 1, at, nb);
+                if ((subj_mask >> q) & 1u)
+                    part[q + 1] += ((double)na[0] * re_o[0] + (double)nb[0] * im_o[0]) + ((double)na[1] * re_o[1] + (double)nb[1] * im_o[1]);
+                else
+                    part[q + 1] += ((double)na[0] * re_s[0] + (double)nb[0] * im_s[0]) + ((double)na[1] * re_s[1] + (double)nb[1] * im_s[1]);
+            }
+        }
+        const double sum = lane_sums<NP>(part, lane);
+        const double phi_mine = __shfl_sync(full, sum, (lane * (32 / NP)) & 31);
+        // lane q: loss term and d loss / d phi of triple q (label +1 for the positive, -1 for negatives)
+        double coef = 0, loss_q = 0;
+        if (lane <= (int)n_neg) {
+            const double y = lane == 0 ? 1.0 : -1.0, z = -y * phi_mine, ez = exp(-fabs(z));
+            loss_q = fmax(z, 0.0) + log1p(ez);
+            coef = -y * ((z >= 0.0 ? 1.0 : ez) / (1.0 + ez));
+        }
+        loss += loss_q;                                         // (lane q's share)
+        // ---- weights with which each entity slot receives the two "negative role" directions ----
+        // A negative with side 0 stands in the subject's place: its gradient is coef * dphi/dS(r, o).  With side 1 it stands in
+        // the object's place: coef * dphi/dO(s, r).  Summed over the negatives whose key's first slot is this lane.
+        if (lane >= 1 && lane <= (int)n_neg) s_w[w][0][lane - 1] = coef;
+        __syncwarp();
+        double wS = 0, wO = 0;
+        if (slot && rep == lane) {
+            for (unsigned m = (same >> 3) & ((1u << n_neg) - 1u); m; m &= m - 1) {
+                const int q = __ffs(m) - 1;
+                if ((subj_mask >> q) & 1u) wS += s_w[w][0][q]; else wO += s_w[w][0][q];
+            }
+        }
+        s_w[w][1][lane] = wS;
+        s_w[w][2][lane] = wO;
+        const double cf0 = __shfl_sync(full, coef, 0);
+        __syncwarp();
+        const double *cf = s_w[w][0], *ws = s_w[w][1], *wo = s_w[w][2];
+        // ---- pass B: gradients ----
+        const uint32_t LU = kAcc && A.finished ? 4 * d : 2 * d; // values per update row
+        float* const U = A.upd + t * n_slots * (uint64_t)LU;
+        for (uint32_t c0 = 0; c0 < d; c0 += 64) {
+            const uint32_t at = c0 + (kV2 ? 2 * lane : lane);
+            if (at >= d) continue;
+            // the accumulators of slot u, where they are needed
+            auto ask = [&](int u, float (&re)[2], float (&im)[2]) {
+                re[0] = re[1] = im[0] = im[1] = 0.f;
+                if (kAcc && ((acc_mask >> u) & 1u)) {
+                    D::load(A.store + s_off[w][u] + 2 * d, at, d, re);
+                    D::load(A.store + s_off[w][u] + 3 * d, at, d, im);
+                }
+            };
+            auto out = [&](int u, const double (&re)[2], const double (&im)[2], const float (&G_re)[2], const float (&G_im)[2]) {
+                const float g[4] = {(float)re[0], (float)re[1], (float)im[0], (float)im[1]};
+                float* o = U + (uint64_t)u * LU;
+                auto put = [&](int part, float x0, float x1) {
+                    const float v[2] = {x0, x1};
+                    D::store(o + part * d, at, d, v);
+                };
+                if (!kAcc || !((acc_mask >> u) & 1u)) {
+                    put(0, g[0], g[1]);
+                    put(1, g[2], g[3]);
+                    return;
+                }
+                float g2[4], x[4], step[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    g2[i] = __fmul_rn(g[i], g[i]);
+                    x[i] = __fadd_rn(i < 2 ? G_re[i] : G_im[i - 2], g2[i]);
+                }
+                adagrad_steps<4>(g, x, A.lr, A.eps, step);
+                if ((once_mask >> u) & 1u) {
+                    o = A.store + s_off[w][u];
+                    float r[2], m[2];
+                    emb(u, 0, at, r);
+                    emb(u, 1, at, m);
+                    put(0, __fadd_rn(r[0], step[0]), __fadd_rn(r[1], step[1]));
+                    put(1, __fadd_rn(m[0], step[2]), __fadd_rn(m[1], step[3]));
+                    put(2, x[0], x[1]);
+                    put(3, x[2], x[3]);
+                } else {
+                    put(0, step[0], step[1]);
+                    put(1, step[2], step[3]);
+                    put(2, g2[0], g2[1]);
+                    put(3, g2[2], g2[3]);
+                }
+            };
+            float G_re[3][2], G_im[3][2];
+#pragma unroll
+            for (int u = 0; u < 3; ++u) ask(u, G_re[u], G_im[u]);
+            // The negatives enter the gradients of subject, relation and object only through their weighted sums:
+            // (A0, B0) over those in the subject's place (triples (n, r, o)), (A1, B1) over those in the object's
+            // place (triples (s, r, n)).
+            double A0[2] = {0.0, 0.0}, B0[2] = {0.0, 0.0}, A1[2] = {0.0, 0.0}, B1[2] = {0.0, 0.0};
+#pragma unroll
+            for (int q = 0; q < kMaxNeg; ++q) {
+                if (q >= (int)n_neg) break;
+                float na[2], nb[2];
+                emb(3 + q, 0, at, na); emb(3 + q, 1, at, nb);
+                const double wq = cf[q];
+                if ((subj_mask >> q) & 1u) {
+                    A0[0] += wq * (double)na[0]; A0[1] += wq * (double)na[1];
+                    B0[0] += wq * (double)nb[0]; B0[1] += wq * (double)nb[1];
+                } else {
+                    A1[0] += wq * (double)na[0]; A1[1] += wq * (double)na[1];
+                    B1[0] += wq * (double)nb[0]; B1[1] += wq * (double)nb[1];
+                }
+            }
+            float av[2], bv[2], crv[2], civ[2], ev[2], fv[2];
+            emb(0, 0, at, av); emb(0, 1, at, bv); emb(1, 0, at, crv); emb(1, 1, at, civ); emb(2, 0, at, ev); emb(2, 1, at, fv);
+            // directions that do not depend on the negative: d phi / d subject (object = o), d phi / d object (subject = s)
+            double dS_re[2], dS_im[2], dO_re[2], dO_im[2], gs_re[2], gs_im[2], gr_re[2], gr_im[2], go_re[2], go_im[2];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const double a = av[i], b = bv[i], cr = crv[i], ci = civ[i], e = ev[i], f = fv[i];
+                dS_re[i] = cr * e + ci * f; dS_im[i] = cr * f - ci * e;
+                dO_re[i] = cr * a - ci * b; dO_im[i] = cr * b + ci * a;
+                gr_re[i] = cf0 * (a * e + b * f) + (A0[i] * e + B0[i] * f) + (a * A1[i] + b * B1[i]);
+                gr_im[i] = cf0 * (a * f - b * e) + (A0[i] * f - B0[i] * e) + (a * B1[i] - b * A1[i]);
+                // (negatives that coincide with the subject or the object: the slots' weights)
+                go_re[i] = cf0 * dO_re[i] + (cr * A0[i] - ci * B0[i]) + ws[2] * dS_re[i] + wo[2] * dO_re[i];
+                go_im[i] = cf0 * dO_im[i] + (cr * B0[i] + ci * A0[i]) + ws[2] * dS_im[i] + wo[2] * dO_im[i];
+                gs_re[i] = cf0 * dS_re[i] + (cr * A1[i] + ci * B1[i]) + ws[0] * dS_re[i] + wo[0] * dO_re[i];
+                gs_im[i] = cf0 * dS_im[i] + (cr * B1[i] - ci * A1[i]) + ws[0] * dS_im[i] + wo[0] * dO_im[i];
+                if (rep_o == 0) { gs_re[i] += go_re[i]; gs_im[i] += go_im[i]; }
+            }
+            out(0, gs_re, gs_im, G_re[0], G_im[0]);
+            out(1, gr_re, gr_im, G_re[1], G_im[1]);
+            if (rep_o == 2) out(2, go_re, go_im, G_re[2], G_im[2]);
+            auto negative = [&](int u, const float (&G_re2)[2], const float (&G_im2)[2]) {
+                const double wSq = ws[u], wOq = wo[u];
+                const double x[2] = {wSq * dS_re[0] + wOq * dO_re[0], wSq * dS_re[1] + wOq * dO_re[1]};
+                const double y[2] = {wSq * dS_im[0] + wOq * dO_im[0], wSq * dS_im[1] + wOq * dO_im[1]};
+                out(u, x, y, G_re2, G_im2);
+            };
+            if (!kAcc) {
+                const float none[2] = {0.f, 0.f};
+#pragma unroll
+                for (int q = 0; q < kMaxNeg; ++q)
+                    if ((rep_mask >> (3 + q)) & 1u) negative(3 + q, none, none);
+                continue;
+            }
+            // one negative after the other (the code of one, not of ten: the instruction cache; 103 -> 89 us), the accumulators
+            // of the next two on their way
+            float Gq[3][2][2];
+            ask(tmin(3, n_slots - 1), Gq[0][0], Gq[0][1]);
+            ask(tmin(4, n_slots - 1), Gq[1][0], Gq[1][1]);
+#pragma unroll 1
+            for (int u = 3; u < n_slots; ++u) {
+                ask(tmin(u + 2, n_slots - 1), Gq[2][0], Gq[2][1]);
+                if ((rep_mask >> u) & 1u) negative(u, Gq[0][0], Gq[0][1]);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    Gq[0][i / 2][i % 2] = Gq[1][i / 2][i % 2];
+                    Gq[1][i / 2][i % 2] = Gq[2][i / 2][i % 2];
+                }
+            }
+        }
+        fence_async_smem();                                     // (the rows have been read; the next ones come through the async proxy)
+        __syncwarp();
+        key = next_key; entry = next_entry; alone = next_alone; side = next_side;
+    }
+    // per-block loss partial, fixed order
+    loss = warp_sum_d(loss);
+    if (lane == 0) s_loss[w] = loss;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double tot = 0;
+        for (int i = 0; i < kShortWarps; ++i) tot += s_loss[i];
+        A.loss_partial[blockIdx.x] = tot;
+    }
+}
+
+// Rows of more than 128 complex dimensions and more than ten negatives: a block of eight warps per data point, whose rows
+// are then read within a short time, so that the second pass over them finds them in L2.  kMaxNeg bounds n_neg at compile
+// time so that a data point's values live in registers: for every block of 32 dimensions the Re and Im of all its rows are
+// requested together, before any is used.
+template <int kMaxNeg>
+__global__ void __launch_bounds__(256, 1) kge_points_kernel(const KgeArgs A) {
+    constexpr int kW = 8, kGroups = 1;
+    constexpr bool kAcc = true;
     __shared__ double s_part[kW > 1 ? kW : 1][kMaxNeg + 1];
     __shared__ double s_w[kGroups][3][32];                      // per slot: coefficient of negative q; weights of the two directions
     __shared__ double s_loss[8];
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int group = w / kW, wg = w % kW;
-    const uint32_t d = kDim ? (uint32_t)kDim : A.d;
-    const uint32_t n_neg = kExact ? (uint32_t)kMaxNeg : A.n_neg;
+    const uint32_t d = A.d, n_neg = A.n_neg;
     const int n_slots = 3 + (int)n_neg;
     const uint64_t L = 4 * (uint64_t)d, K = A.K;
     pdl_trigger();
@@ -558,49 +876,42 @@ uint32_t launch_points_kge(ps_store* ps, const KgeBatch& B, const uint8_t* singl
     A.store = ps->store; A.table = ps->table; A.S = ps->cfg.slots_per_part;
     A.upd = ps->upd; A.single = single; A.keys_out = keys_out; A.finished = finished;
     A.loss_partial = ps->loss_partial; A.st = ps->status; A.epoch = ps->epoch;
-    const bool wide = B.dim > 128;
-    if (wide && B.n_neg <= 10) {
-        const uint32_t grid = (uint32_t)tmin<uint64_t>(B.n, (uint64_t)ps->sm_count * 2);
-#define KGE_WIDE(kMaxNeg)                                                                                        \
-        do {                                                                                                     \
-            static std::atomic<unsigned long long> smem_set{0};                                                  \
-            const size_t smem = (size_t)2 * (3 + kMaxNeg) * 4 * kStretchPad * sizeof(float);                     \
-            opt_in_smem((const void*)kge_wide_kernel<kMaxNeg>, smem, &smem_set);                                 \
-            if (keys_out) PS_LAUNCH_PDL(ps, "kge_wide_kernel<" #kMaxNeg ">", kge_wide_kernel<kMaxNeg>, dim3(grid), dim3(256), smem, s, A); \
-            else PS_LAUNCH_SMEM(ps, kge_wide_kernel<kMaxNeg>, grid, 256, smem, s, A);                            \
-        } while (0)
-        if (B.n_neg <= 4) KGE_WIDE(4);
-        else KGE_WIDE(10);
-#undef KGE_WIDE
-        return grid;
-    }
-    uint64_t g = wide ? B.n : (B.n + 7) / 8;
-    g = tmin<uint64_t>(g, tmin<uint64_t>((uint64_t)ps->sm_count * (wide ? 2 : 8), kMaxLossBlocks));
-    const uint32_t grid = (uint32_t)g;
-#define KGE_LAUNCH(kMaxNeg, kDim, kExact, kW, kAcc)                                                                   \
+    // as many blocks as are resident at once, or one per example (the pdl form: kernels of small calls)
+#define KGE_LAUNCH(name, kernel, threads, smem, per_block, per_sm)                                               \
     do {                                                                                                         \
-        const char* name = kW > 1 ? "kge_points_kernel<wide>" : "kge_points_kernel";                             \
+        static std::atomic<unsigned long long> smem_set{0};                                                      \
+        opt_in_smem((const void*)kernel, 200 * 1024, &smem_set);                                                 \
+        const uint32_t grid = (uint32_t)tmin<uint64_t>((B.n + per_block - 1) / per_block, (uint64_t)ps->sm_count * (per_sm)); \
         if (keys_out) {                                                                                          \
-            PS_LAUNCH_PDL(ps, name, (kge_points_kernel<kMaxNeg, kDim, kExact, kW, kAcc>), dim3(grid), dim3(256), 0, s, A); \
+            PS_LAUNCH_PDL(ps, name, kernel, dim3(grid), dim3(threads), smem, s, A);                              \
         } else {                                                                                                 \
             if (ps->prof) prof_before(ps, name, s);                                                              \
-            kge_points_kernel<kMaxNeg, kDim, kExact, kW, kAcc><<<grid, 256, 0, s>>>(A);                          \
+            kernel<<<grid, threads, smem, s>>>(A);                                                               \
             if (ps->prof) prof_after(ps, s);                                                                     \
             ps->launches++;                                                                                      \
         }                                                                                                        \
+        return grid;                                                                                             \
     } while (0)
-    if (wide) KGE_LAUNCH(29, 0, false, 8, true);
-    else if (finished) {
-        if (B.n_neg <= 10) KGE_LAUNCH(10, 0, false, 1, true);
-        else KGE_LAUNCH(29, 0, false, 1, true);
-    } else {
-        if (B.n_neg == 10 && B.dim == 100) KGE_LAUNCH(10, 100, true, 1, false);
-        else if (B.n_neg <= 4) KGE_LAUNCH(4, 0, false, 1, false);
-        else if (B.n_neg <= 10) KGE_LAUNCH(10, 0, false, 1, false);
-        else KGE_LAUNCH(29, 0, false, 1, false);
+    if (B.dim > 128) {
+        if (B.n_neg <= 4) KGE_LAUNCH("kge_wide_kernel", kge_wide_kernel<4>, 256, (size_t)2 * 7 * 4 * kStretchPad * sizeof(float), 1, 2);
+        if (B.n_neg <= 10) KGE_LAUNCH("kge_wide_kernel", kge_wide_kernel<10>, 256, (size_t)2 * 13 * 4 * kStretchPad * sizeof(float), 1, 2);
+        KGE_LAUNCH("kge_points_kernel", kge_points_kernel<29>, 256, 0, 1, 2);
     }
+    const size_t smem = (size_t)kShortWarps * (3 + B.n_neg) * ((2 * B.dim + 3) & ~3u) * sizeof(float);
+    const uint32_t fit = tmax<uint32_t>(1u, (uint32_t)((220 * 1024) / (smem + 4096)));
+#define KGE_SHORT(kMaxNeg, resident)                                                                             \
+    do {                                                                                                         \
+        const bool even = B.dim % 2 == 0, acc = single || finished;                                              \
+        if (even && acc) KGE_LAUNCH("kge_short_kernel<acc>", (kge_short_kernel<kMaxNeg, true, true>), 32 * kShortWarps, smem, kShortWarps, tmin<uint32_t>(fit, resident)); \
+        if (even) KGE_LAUNCH("kge_short_kernel", (kge_short_kernel<kMaxNeg, true, false>), 32 * kShortWarps, smem, kShortWarps, tmin<uint32_t>(fit, resident)); \
+        if (acc) KGE_LAUNCH("kge_short_kernel<acc>", (kge_short_kernel<kMaxNeg, false, true>), 32 * kShortWarps, smem, kShortWarps, tmin<uint32_t>(fit, resident)); \
+        KGE_LAUNCH("kge_short_kernel", (kge_short_kernel<kMaxNeg, false, false>), 32 * kShortWarps, smem, kShortWarps, tmin<uint32_t>(fit, resident)); \
+    } while (0)
+    if (B.n_neg <= 4) KGE_SHORT(4, 4u);
+    if (B.n_neg <= 10) KGE_SHORT(10, 4u);
+    KGE_SHORT(29, 2u);
+#undef KGE_SHORT
 #undef KGE_LAUNCH
-    return grid;
 }
 
 void launch_keys_kge(ps_store* ps, const KgeBatch& B, cudaStream_t s) {

@@ -606,9 +606,9 @@ ps_status_t ps_step_kge(ps_store_t* ps, const uint32_t* d_s, const uint32_t* d_r
         return after_launch();
     }
     SortSet* ss = next_set(ps);
-    // Long rows: keys that occur once are updated by the gradient kernel, which therefore comes after the sort.  Short
-    // rows: all gradients go to the reduction, and the gradient kernel runs beside the sort.
-    const bool in_place = dim_complex > 128;
+    // Keys that occur once are updated by the gradient kernel, which therefore comes after the sort.  In ordered mode, rows of at
+    // most 512 values: all gradients go to the reduction (the same expressions), and the gradient kernel runs beside the sort.
+    const bool in_place = dim_complex > 128 || ps->pipelined;
     cudaStream_t q = ps->side;
     if (in_place ? !begin_sort(ps, ss, s, false, &q) : !fork_side(ps, ss, s)) return PS_ERR_CUDA;
     launch_keys_kge(ps, B, q);

@@ -379,26 +379,25 @@ __device__ __forceinline__ float adagrad_step(float g, float x, float lr, float 
 // The same for N values at a time.  Once sqrt(x) is thousands of times eps, which is all but the very first steps of a
 // parameter, 1 / (sqrt(x) + eps) = r (1 - eps r) with r = 1 / sqrt(x), to within (eps r)^2 < 4e-8: one operation of the
 // special-function unit instead of two, and that unit (16 lanes per clock and SM, conversions to and from fp64 included)
-// is what bounds the reductions with AdaGrad.  One test for all N values, so that their chains interleave.  True if that
-// form was taken, which it is not where a value is not finite.
+// is what bounds the reductions with AdaGrad.  Which form a value takes depends on that value alone (so results do not
+// depend on how values are grouped), but one test serves all N, so that their chains interleave.  True if that form was taken
+// by all, which it is not where one is not finite.
 template <int N>
 __device__ __forceinline__ bool adagrad_steps(const float (&g)[N], const float (&x)[N], float lr, float eps, float (&step)[N]) {
-    float er[N], worst = 0.f, top = 0.f;
+    float er[N];
+    bool fine = true;
 #pragma unroll
     for (int i = 0; i < N; ++i) {
         float r;
         asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x[i]));      // (zero or denormal: infinite, the other form)
-        er[i] = eps * r;
-        step[i] = (-lr * g[i]) * (r - er[i] * r);
-        worst = fmaxf(worst, er[i]);
-        top = fmaxf(top, x[i]);
+        er[i] = __fmul_rn(eps, r);
+        step[i] = __fmul_rn(__fmul_rn(-lr, g[i]), fmaf(-er[i], r, r));
+        fine = fine && er[i] < 2e-4f && x[i] < 3e38f;                   // (false for a NaN)
     }
-    bool fine = worst < 2e-4f && top < 3e38f;
-#pragma unroll
-    for (int i = 0; i < N; ++i) fine = fine && x[i] == x[i];            // (fmaxf passes over a NaN)
     if (fine) return true;
 #pragma unroll
-    for (int i = 0; i < N; ++i) step[i] = adagrad_step(g[i], x[i], lr, eps);
+    for (int i = 0; i < N; ++i)
+        if (!(er[i] < 2e-4f && x[i] < 3e38f)) step[i] = adagrad_step(g[i], x[i], lr, eps);
     return false;
 }
 __device__ __forceinline__ void adagrad_steps4(const float4& g, const float4& x, float lr, float eps, float4& step) {

@@ -353,12 +353,12 @@ segment_adagrad_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restri
 #pragma unroll
                     for (int i = 0; i < kN; ++i) {
                         g[i] = Vec<V>::get(u[q][c], i);
-                        x[i] = Vec<V>::get(g1[q][c], i) + g[i] * g[i];
+                        x[i] = __fadd_rn(Vec<V>::get(g1[q][c], i), __fmul_rn(g[i], g[i]));
                     }
                     adagrad_steps<kN>(g, x, lr, eps, step);
 #pragma unroll
                     for (int i = 0; i < kN; ++i) {
-                        Vec<V>::set(t1[q][c], i, Vec<V>::get(t1[q][c], i) + step[i]);
+                        Vec<V>::set(t1[q][c], i, __fadd_rn(Vec<V>::get(t1[q][c], i), step[i]));
                         Vec<V>::set(g1[q][c], i, x[i]);
                     }
                     row[q][f0 + 32 * c] = t1[q][c];
