@@ -756,6 +756,27 @@ static void sgns_small(ps_store_t* ps, const uint32_t* d_tokens, uint64_t tok_fi
                      (uint32_t)(occ / n_centers));
 }
 
+// The sorted form, the side stream being forked already.  Pipelined, long rows: the keys are sorted beside the step before, and the gradient
+// kernel, which comes after the sort, updates the rows of keys that occur once.  Otherwise it runs beside the sort, and all
+// updates go to the reduction (the same expressions).
+static ps_status_t sgns_sorted(ps_store_t* ps, SortSet* ss, const uint32_t* d_tokens, uint64_t tok_first, uint64_t first_pos,
+                               uint64_t n_centers, uint64_t corpus_len, uint32_t window, const uint32_t* d_negs,
+                               uint32_t n_neg, uint64_t out_key_base, float lr, uint64_t occ, double* d_loss_accum,
+                               cudaStream_t s) {
+    launch_keys_sgns(ps, d_tokens, tok_first, first_pos, n_centers, corpus_len, window, d_negs, n_neg, out_key_base, ps->side);
+    const int which = run_push_sort(ps, (uint32_t)occ, ps->side);
+    if (!sorted_keys_at(ps, ss, which, (uint32_t)occ, ps->side)) return PS_ERR_CUDA;
+    // (rows of less than 1 KB: 159 us against 155 at 64 values, 10,000 centers; with 500 values 333 against 344)
+    const uint8_t* single = ps->pipelined && ps->cfg.row_len >= 256 ? launch_singles(ps, (uint32_t)occ, which, ps->side) : nullptr;
+    if (single && !join_side(ps, s)) return PS_ERR_CUDA;
+    const uint32_t lb = launch_step_sgns(ps, d_tokens, tok_first, first_pos, n_centers, corpus_len, window, d_negs, n_neg,
+                                         out_key_base, lr, nullptr, s, single);
+    if (!single && !join_side(ps, s)) return PS_ERR_CUDA;
+    run_push_reduce(ps, (uint32_t)occ, which, ps->upd, d_loss_accum, d_loss_accum ? lb : 0, s, sgns_scales(ps, n_centers),
+                    (uint32_t)(occ / n_centers), single != nullptr);
+    return PS_OK;
+}
+
 ps_status_t ps_step_sgns(ps_store_t* ps, const uint32_t* d_tokens, uint64_t first_pos, uint64_t n_centers,
                          uint64_t corpus_len, uint32_t window, const uint32_t* d_negs, uint32_t n_neg,
                          uint64_t out_key_base, float lr, double* d_loss_accum, void* stream) {
@@ -772,14 +793,9 @@ ps_status_t ps_step_sgns(ps_store_t* ps, const uint32_t* d_tokens, uint64_t firs
     }
     SortSet* ss = next_set(ps);
     if (!fork_side(ps, ss, s)) return PS_ERR_CUDA;
-    launch_keys_sgns(ps, d_tokens, 0, first_pos, n_centers, corpus_len, window, d_negs, n_neg, out_key_base, ps->side);
-    const int which = run_push_sort(ps, (uint32_t)occ, ps->side);
-    if (!sorted_keys_at(ps, ss, which, (uint32_t)occ, ps->side)) return PS_ERR_CUDA;
-    const uint32_t lb = launch_step_sgns(ps, d_tokens, 0, first_pos, n_centers, corpus_len, window, d_negs, n_neg,
-                                         out_key_base, lr, nullptr, s);
-    if (!join_side(ps, s)) return PS_ERR_CUDA;
-    run_push_reduce(ps, (uint32_t)occ, which, ps->upd, d_loss_accum, d_loss_accum ? lb : 0, s,
-                    sgns_scales(ps, n_centers), (uint32_t)(occ / n_centers));
+    const ps_status_t rc = sgns_sorted(ps, ss, d_tokens, 0, first_pos, n_centers, corpus_len, window, d_negs, n_neg, out_key_base,
+                                       lr, occ, d_loss_accum, s);
+    if (rc != PS_OK) return rc;
     return release_set(ss, s);
 }
 
@@ -925,14 +941,9 @@ ps_status_t ps_step_sgns_host(ps_store_t* ps, const uint32_t* h_tokens, uint64_t
     } else if (cudaEventRecord(ps->ev_fork, s) != cudaSuccess || cudaStreamWaitEvent(ps->side, ps->ev_fork, 0) != cudaSuccess) {
         return PS_ERR_CUDA;                                  // the batch was just copied on the caller's stream
     }
-    launch_keys_sgns(ps, d_tok, tok_first, first_pos, n_centers, corpus_len, window, d_negs, n_neg, out_key_base,
-                     ps->side);
-    const int which = run_push_sort(ps, (uint32_t)occ, ps->side);
-    const uint32_t lb = launch_step_sgns(ps, d_tok, tok_first, first_pos, n_centers, corpus_len, window, d_negs, n_neg,
-                                         out_key_base, lr, nullptr, s);
-    if (!join_side(ps, s)) return PS_ERR_CUDA;
-    run_push_reduce(ps, (uint32_t)occ, which, ps->upd, d_loss_accum, d_loss_accum ? lb : 0, s,
-                    sgns_scales(ps, n_centers), (uint32_t)(occ / n_centers));
+    c = sgns_sorted(ps, ss, d_tok, tok_first, first_pos, n_centers, corpus_len, window, d_negs, n_neg, out_key_base, lr, occ,
+                    d_loss_accum, s);
+    if (c != PS_OK) return c;
     c = release_set(ss, s);
     if (c != PS_OK) return c;
     return finish_host_step(ps, hb, d_loss_accum, h_loss, s);

@@ -242,7 +242,8 @@ void run_push_pipeline(ps_store* ps, uint32_t n, const float* d_upd, double* d_l
 int run_push_sort(ps_store* ps, uint32_t n, cudaStream_t s);
 int run_segment_sort(ps_store* ps, uint32_t n, cudaStream_t s);     // the same; also clears the counters of seg_lists
 void run_push_reduce(ps_store* ps, uint32_t n, int which, const float* d_upd, double* d_loss_accum,
-                     uint32_t loss_blocks, cudaStream_t s, const float* d_scales = nullptr, uint32_t slots = 0);
+                     uint32_t loss_blocks, cudaStream_t s, const float* d_scales = nullptr, uint32_t slots = 0,
+                     bool skip_singles = false);        // keys that occur once have been updated already
 
 // push by atomic adds, no sort (ps_set_push_mode)
 void run_push_atomic(ps_store* ps, const uint64_t* d_keys, uint64_t n, const float* d_upd, cudaStream_t s);
@@ -283,6 +284,7 @@ struct SegLists {
 };
 constexpr uint32_t kSegCounters = 8;             // (rows whose single keys are reduced have at most two stretches of columns)
 SegLists seg_lists(ps_store* ps);   // of the current buffer set
+const uint8_t* launch_singles(ps_store* ps, uint32_t n, int which, cudaStream_t s);     // per occurrence: its key occurs once
 // after the sort, on its stream; keys from rel_key_base on are RESCAL's relations (num_keys: none)
 void launch_segments(ps_store* ps, uint32_t n, int which, uint32_t half_row, uint64_t rel_key_base, cudaStream_t s);
 // gradient rows (half_row values per occurrence, in ps->upd) -> AdaGrad, of the keys that occur several times and, with
@@ -345,7 +347,8 @@ uint32_t launch_step_mf(ps_store* ps, const uint32_t* d_i, const uint32_t* d_j, 
 float* sgns_scales(ps_store* ps, uint64_t n_centers);     // where launch_step_sgns puts the per-slot factors
 uint32_t launch_step_sgns(ps_store* ps, const uint32_t* d_tokens, uint64_t tok_first, uint64_t first_pos,
                           uint64_t n_centers, uint64_t corpus_len, uint32_t window, const uint32_t* d_negs,
-                          uint32_t n_neg, uint64_t out_key_base, float lr, uint32_t* keys_out, cudaStream_t s);
+                          uint32_t n_neg, uint64_t out_key_base, float lr, uint32_t* keys_out, cudaStream_t s,
+                          const uint8_t* single = nullptr);     // per slot: such rows are updated in place
 
 // ---- device helpers ----
 #ifdef __CUDACC__

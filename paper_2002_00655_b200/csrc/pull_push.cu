@@ -343,10 +343,12 @@ __device__ __noinline__ void group_preadd(const uint32_t* __restrict__ sk, uint3
 //
 // kL4 / kSlots: the row length in float4 and the slots per example if known at compile time (0: taken from the
 // arguments); row offsets, the copy size and the division by the slots then fold.
+//
+// skip_singles: keys that occur once have been updated by the gradient kernel.
 template <int kCh, bool kScaled, int kL4, int kSlots>
 __global__ void __launch_bounds__(256)
 push_reduce_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restrict__ sv, uint32_t n,
-                   const float4* __restrict__ upd, const float* __restrict__ scales, uint32_t slots_arg,
+                   const float4* __restrict__ upd, const float* __restrict__ scales, uint32_t slots_arg, bool skip_singles,
                    float4* __restrict__ store, const uint2* __restrict__ table,
                    uint64_t S, uint32_t K, uint32_t L4_arg, double* __restrict__ carry,
                    uint4* __restrict__ starters, unsigned int* __restrict__ starter_count,
@@ -364,7 +366,13 @@ push_reduce_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restrict__
     const uint32_t n_valid = base < n ? (uint32_t)tmin<uint64_t>((uint64_t)kReduceTile, n - base) : 0u;
     const uint32_t key = lane < n_valid ? sk[base + lane] : kSentinelPad;
     uint32_t occ = lane < n_valid ? sv[base + lane] : 0u;
-    const bool usable = key < K;                    // "no key" marks and padding sort last
+    uint32_t prev = __shfl_up_sync(full, key, 1);
+    if (lane == 0) prev = (base > 0 && base - 1 < n) ? sk[base - 1] : kSentinelPad;
+    const uint32_t next_after = (base + kReduceTile < n) ? sk[base + kReduceTile] : kSentinelPad;
+    uint32_t next = __shfl_down_sync(full, key, 1);
+    if (lane == 31) next = next_after;
+    // "no key" marks and padding sort last
+    const bool usable = key < K && !(kScaled && skip_singles && key != prev && key != next);
     float scale = 1.f;
     if (kScaled && usable) {
         scale = scales[occ];
@@ -373,11 +381,6 @@ push_reduce_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restrict__
     }
     uint64_t row = 0;
     if (usable) row = phys_row(table[key], S);
-    uint32_t prev = __shfl_up_sync(full, key, 1);
-    if (lane == 0) prev = (base > 0 && base - 1 < n) ? sk[base - 1] : kSentinelPad;
-    const uint32_t next_after = (base + kReduceTile < n) ? sk[base + kReduceTile] : kSentinelPad;
-    uint32_t next = __shfl_down_sync(full, key, 1);
-    if (lane == 31) next = next_after;
     const unsigned head_mask = __ballot_sync(full, key != prev);
     const unsigned usable_mask = __ballot_sync(full, usable);
     // positions at which a segment's part in this tile ends: its true end, or the tile's last position
@@ -1200,13 +1203,13 @@ void run_mf_fused(ps_store* ps, uint32_t n_cells, int which, uint64_t col_key_ba
 }
 
 void run_push_reduce(ps_store* ps, uint32_t n, int which, const float* d_upd, double* d_loss_accum,
-                     uint32_t loss_blocks, cudaStream_t s, const float* d_scales, uint32_t slots) {
+                     uint32_t loss_blocks, cudaStream_t s, const float* d_scales, uint32_t slots, bool skip_singles) {
     const uint32_t* sk = which ? ps->keysB : ps->keysA;
     const uint32_t* sv = which ? ps->valsB : ps->valsA;
     const uint32_t tiles = div_up_u32(n, kReduceTile);
     const uint32_t blocks = div_up_u32(tiles, 8);
     const uint32_t L4 = ps->cfg.row_len / 4;
-#define REDUCE_ARGS sk, sv, n, (const float4*)d_upd, d_scales, slots, (float4*)ps->store, ps->table,                 \
+#define REDUCE_ARGS sk, sv, n, (const float4*)d_upd, d_scales, slots, skip_singles, (float4*)ps->store, ps->table,   \
                     ps->cfg.slots_per_part, (uint32_t)ps->cfg.num_keys, L4, ps->carry, ps->starters,                \
                     ps->starter_count, ps->group_done, ps->group_sum, ps->status, ps->epoch
 #define REDUCE_LAUNCH(kCh, kScaled, kL4, kSlots)                                                                     \

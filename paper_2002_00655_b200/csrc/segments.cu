@@ -80,6 +80,24 @@ segment_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restrict__ sv,
     }
 }
 
+// The flags alone, for the skip-gram step (its other keys go through push_reduce_kernel).
+__global__ void __launch_bounds__(256)
+single_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restrict__ sv, uint32_t n, uint32_t K, uint8_t* __restrict__ single,
+              const DevStatus* st, unsigned int epoch) {
+    if (call_failed(st, epoch)) return;
+    const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= n) return;
+    const uint32_t key = sk[p];
+    if (key < K) single[sv[p]] = (p == 0 || sk[p - 1] != key) && (p + 1 == n || sk[p + 1] != key);
+}
+
+const uint8_t* launch_singles(ps_store* ps, uint32_t n, int which, cudaStream_t s) {
+    uint8_t* single = (uint8_t*)ps->cellpos;
+    PS_LAUNCH(ps, single_kernel, div_up_u32(n, 256), 256, s, which ? ps->keysB : ps->keysA, which ? ps->valsB : ps->valsA, n,
+              (uint32_t)ps->cfg.num_keys, single, ps->status, ps->epoch);
+    return single;
+}
+
 SegLists seg_lists(ps_store* ps) {
     SegLists L;
     L.counts = ps->group_done;                  // (zeroed by the sort)

@@ -13,10 +13,10 @@ namespace psb {
 
 __device__ __forceinline__ float softplusf(float z) { return fmaxf(z, 0.f) + log1pf(expf(-fabsf(z))); }
 __device__ __forceinline__ float sigmoidf(float z) {
-    if (z >= 0.f) return 1.f / (1.f + expf(-z));
-    const float e = expf(z);
-    return e / (1.f + e);
+    const float e = expf(-fabsf(z));
+    return (z >= 0.f ? 1.f : e) / (1.f + e);
 }
+
 // Sum of the warps' loss terms -> loss_partial[blockIdx.x]; fixed order.
 __device__ __forceinline__ void block_loss_out(double loss, double* __restrict__ loss_partial) {
     __shared__ double wl[8];
@@ -245,11 +245,13 @@ __device__ __forceinline__ uint64_t sgns_pairs_before(uint64_t p, uint64_t T, ui
 // the rows are then read four slots at a time, all loads of the four before the first dot product.
 // kL4, kWindow, kNeg: row length (float4), window and negatives per context if known at compile time (0: taken
 // from the arguments; kNeg < 0: from the argument); divisions by the slots per context and row offsets then fold.
-template <int kCh, int kL4, int kWindow, int kNeg>
+// kOnce: rows whose key occurs once in the batch (`single`, per slot) are updated here, in place, with the values in hand; a
+// third of the skip-gram batch's occurrences, each of which cost the reduction three rows of traffic.
+template <int kCh, int kL4, int kWindow, int kNeg, bool kOnce>
 __global__ void __launch_bounds__(256, 2)
 sgns_step_kernel(const uint32_t* __restrict__ tokens, uint64_t tok_first, uint64_t first_pos, uint64_t n_centers,
                  uint64_t T, uint32_t window_arg, const uint32_t* __restrict__ negs, uint32_t n_neg_arg, uint64_t out_base,
-                 float lr, const float4* __restrict__ store, const uint2* __restrict__ table, uint64_t S, uint64_t K,
+                 float lr, float4* store, const uint2* __restrict__ table, uint64_t S, uint64_t K, const uint8_t* __restrict__ single,
                  uint32_t L4_arg, float4* __restrict__ upd, float* __restrict__ scales, uint32_t* __restrict__ keys_out,
                  double* __restrict__ loss_partial, DevStatus* st, unsigned int epoch) {
     const unsigned full = 0xffffffffu;
@@ -263,9 +265,15 @@ sgns_step_kernel(const uint32_t* __restrict__ tokens, uint64_t tok_first, uint64
     const uint64_t slots = 1 + (uint64_t)2 * window * per_ctx;
     const uint64_t pairs0 = sgns_pairs_before(first_pos, T, window);
     constexpr int kQuad = 4;
+    float4 u[kQuad][kCh];                                       // (elements past the row are never loaded: zero throughout)
+#pragma unroll
+    for (int a = 0; a < kQuad; ++a)
+#pragma unroll
+        for (int c = 0; c < kCh; ++c) u[a][c] = make_float4(0.f, 0.f, 0.f, 0.f);
     double loss = 0;
     pdl_trigger();
     pdl_wait();
+    if (kOnce && call_failed(st, epoch)) return;        // (the key kernel found an index out of range: nothing may be written)
     for (uint64_t cidx = warp; cidx < n_centers; cidx += n_warps) {
         const uint64_t p = first_pos + cidx;
         const uint64_t lo = p >= window ? p - window : 0;
@@ -284,7 +292,8 @@ sgns_step_kernel(const uint32_t* __restrict__ tokens, uint64_t tok_first, uint64
             if (lane == 0) latch_error(st, epoch, PS_ERR_KEY_RANGE);
             continue;
         }
-        const float4* V = store + phys_row(table[wtok], S) * L4;
+        float4* V = store + phys_row(table[wtok], S) * L4;
+        const bool center_once = kOnce && single[cidx * slots];
         float4 v[kCh], dv[kCh];
 #pragma unroll
         for (int c = 0; c < kCh; ++c) {
@@ -292,7 +301,6 @@ sgns_step_kernel(const uint32_t* __restrict__ tokens, uint64_t tok_first, uint64
             v[c] = f < L4 ? V[f] : make_float4(0.f, 0.f, 0.f, 0.f);
             dv[c] = make_float4(0.f, 0.f, 0.f, 0.f);
         }
-        float loss_c = 0.f;
         bool bad = false;
         for (uint32_t t0 = 0; t0 < n_out; t0 += 32) {
             // this lane's slot of the round
@@ -313,22 +321,20 @@ sgns_step_kernel(const uint32_t* __restrict__ tokens, uint64_t tok_first, uint64
                 if (keys_out) keys_out[cidx * slots + 1 + t] = my_ok ? (uint32_t)ku : kSentinelPad;
             }
             const unsigned ok_mask = __ballot_sync(full, my_ok);
+            const unsigned once_mask = kOnce ? __ballot_sync(full, my_ok && single[cidx * slots + 1 + t]) : 0u;
             const uint32_t in_round = tmin<uint32_t>(32u, n_out - t0);
-            float my_scale = 0.f;                                               // factor of this lane's slot
+            float my_scale = 0.f, my_x = 0.f;                                   // factor and score of this lane's slot
             for (uint32_t b = 0; b < in_round; b += kQuad) {
-                float4 u[kQuad][kCh];
-                float x[kQuad];
 #pragma unroll
-                for (int a = 0; a < kQuad; ++a) {
-                    const uint64_t r = __shfl_sync(full, my_row, (b + a) & 31);
-                    const bool ok = (ok_mask >> (b + a)) & 1u;                  // b + a <= 31; bits past the round are 0
-                    const float4* Urow = store + r * L4;
+                for (int a = 0; a < kQuad; ++a) {                               // (a slot without a row reads row 0, and is skipped below)
+                    const float4* Urow = store + __shfl_sync(full, my_row, (b + a) & 31) * L4;
 #pragma unroll
                     for (int c = 0; c < kCh; ++c) {
                         const uint32_t f = lane + 32 * c;
-                        u[a][c] = (ok && f < L4) ? Urow[f] : make_float4(0.f, 0.f, 0.f, 0.f);
+                        if (f < L4) u[a][c] = Urow[f];
                     }
                 }
+                float x[kQuad];
 #pragma unroll
                 for (int a = 0; a < kQuad; ++a) {
                     x[a] = 0.f;
@@ -336,46 +342,57 @@ sgns_step_kernel(const uint32_t* __restrict__ tokens, uint64_t tok_first, uint64
                     for (int c = 0; c < kCh; ++c)
                         x[a] += v[c].x * u[a][c].x + v[c].y * u[a][c].y + v[c].z * u[a][c].z + v[c].w * u[a][c].w;
                 }
+                // The four sums over the lanes by exchanging halves (6 exchanges, not 20): lanes 8 a .. 8 a + 7 are left with
+                // the a-th score, and turn it into the slot's factor.
+                const bool up = lane & 16, right = lane & 8;
+                float y0 = (up ? x[2] : x[0]) + __shfl_xor_sync(full, up ? x[0] : x[2], 16);
+                float y1 = (up ? x[3] : x[1]) + __shfl_xor_sync(full, up ? x[1] : x[3], 16);
+                float xa = (right ? y1 : y0) + __shfl_xor_sync(full, right ? y0 : y1, 8);
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-                    for (int a = 0; a < kQuad; ++a) x[a] += __shfl_xor_sync(full, x[a], o);
-                }
-                // lane a < 4 turns the a-th score of the four into the slot's factor and loss term
-                float xa = x[0];
-#pragma unroll
-                for (int a = 1; a < kQuad; ++a) xa = lane == a ? x[a] : xa;
-                float sc_mine = 0.f;
-                if (lane < kQuad && ((ok_mask >> (b + lane)) & 1u)) {
-                    const bool positive = (t0 + b + lane) % per_ctx == 0;
-                    sc_mine = -lr * (sigmoidf(xa) - (positive ? 1.f : 0.f));
-                    loss_c += positive ? softplusf(-xa) : softplusf(xa);
-                }
+                for (int o = 4; o > 0; o >>= 1) xa += __shfl_xor_sync(full, xa, o);
+                const bool positive = (t0 + b + (lane >> 3)) % per_ctx == 0;
+                const float sc_mine = -lr * (sigmoidf(xa) - (positive ? 1.f : 0.f));
 #pragma unroll
                 for (int a = 0; a < kQuad; ++a) {
-                    const float sc = __shfl_sync(full, sc_mine, a);
+                    const float sc = __shfl_sync(full, sc_mine, 8 * a), xs = __shfl_sync(full, xa, 8 * a);
                     if (!((ok_mask >> (b + a)) & 1u)) continue;
-                    if (lane == (int)(b + a)) my_scale = sc;
+                    if (lane == (int)(b + a)) {
+                        my_scale = sc;
+                        my_x = xs;
+                    }
 #pragma unroll
                     for (int c = 0; c < kCh; ++c) {
                         dv[c].x += sc * u[a][c].x; dv[c].y += sc * u[a][c].y;
                         dv[c].z += sc * u[a][c].z; dv[c].w += sc * u[a][c].w;
                     }
+                    if (kOnce && ((once_mask >> (b + a)) & 1u)) {           // nobody else reads this row: its update, in place
+                        float4* Urow = store + __shfl_sync(full, my_row, (b + a) & 31) * L4;
+#pragma unroll
+                        for (int c = 0; c < kCh; ++c) {
+                            const uint32_t f = lane + 32 * c;
+                            const float4 x = make_float4(fmaf(sc, v[c].x, u[a][c].x), fmaf(sc, v[c].y, u[a][c].y),
+                                                         fmaf(sc, v[c].z, u[a][c].z), fmaf(sc, v[c].w, u[a][c].w));
+                            if (f < L4) Urow[f] = x;
+                        }
+                    }
                 }
             }
-            if (my_ok) F[1 + t] = my_scale;
+            if (my_ok) {
+                F[1 + t] = my_scale;
+                loss += (double)softplusf(t % per_ctx == 0 ? -my_x : my_x);
+            }
         }
         if (__any_sync(full, bad) && lane == 0) latch_error(st, epoch, PS_ERR_KEY_RANGE);
 #pragma unroll
         for (int c = 0; c < kCh; ++c) {
             const uint32_t f = lane + 32 * c;
             if (f < L4) {
-                U[f] = dv[c];
+                if (center_once) V[f] = make_float4(dv[c].x + v[c].x, dv[c].y + v[c].y, dv[c].z + v[c].z, dv[c].w + v[c].w);
+                else U[f] = dv[c];
                 U[L4 + f] = v[c];
             }
         }
         if (lane == 0) F[0] = 1.f;
-        loss += (double)loss_c;                             // this lane's share (lanes 0..3 hold the terms)
     }
     block_loss_out(warp_sum_d(loss), loss_partial);
 }
@@ -423,20 +440,21 @@ float* sgns_scales(ps_store* ps, uint64_t n_centers) { return ps->upd + n_center
 
 uint32_t launch_step_sgns(ps_store* ps, const uint32_t* d_tokens, uint64_t tok_first, uint64_t first_pos,
                           uint64_t n_centers, uint64_t corpus_len, uint32_t window, const uint32_t* d_negs,
-                          uint32_t n_neg, uint64_t out_key_base, float lr, uint32_t* keys_out, cudaStream_t s) {
+                          uint32_t n_neg, uint64_t out_key_base, float lr, uint32_t* keys_out, cudaStream_t s, const uint8_t* single) {
     const uint32_t L4 = ps->cfg.row_len / 4;
     const uint32_t epoch = keys_out ? 0u : ps->epoch;
     const uint32_t grid = step_grid(ps, n_centers, 2);      // the kernels are bounded to two blocks per SM
 #define SG_ARGS d_tokens, tok_first, first_pos, n_centers, corpus_len, window, d_negs, n_neg, out_key_base, lr,   \
-                (const float4*)ps->store, ps->table, ps->cfg.slots_per_part, ps->cfg.num_keys, L4,              \
+                (float4*)ps->store, ps->table, ps->cfg.slots_per_part, ps->cfg.num_keys, single, L4,            \
                 (float4*)ps->upd, sgns_scales(ps, n_centers), keys_out, ps->loss_partial, ps->status, epoch
 #define SG_LAUNCH(kCh, kL4, kW, kN)                                                                                  \
     do {                                                                                                             \
         if (keys_out) {                                                                                              \
-            PS_LAUNCH_PDL(ps, "sgns_step_kernel<" #kCh ">", (sgns_step_kernel<kCh, kL4, kW, kN>), dim3(grid), dim3(256), 0, s, SG_ARGS); \
+            PS_LAUNCH_PDL(ps, "sgns_step_kernel<" #kCh ">", (sgns_step_kernel<kCh, kL4, kW, kN, false>), dim3(grid), dim3(256), 0, s, SG_ARGS); \
         } else {                                                                                                     \
             if (ps->prof) prof_before(ps, "sgns_step_kernel<" #kCh ">", s);                                          \
-            sgns_step_kernel<kCh, kL4, kW, kN><<<grid, 256, 0, s>>>(SG_ARGS);                                        \
+            if (single) sgns_step_kernel<kCh, kL4, kW, kN, true><<<grid, 256, 0, s>>>(SG_ARGS);                      \
+            else sgns_step_kernel<kCh, kL4, kW, kN, false><<<grid, 256, 0, s>>>(SG_ARGS);                            \
             if (ps->prof) prof_after(ps, s);                                                                         \
             ps->launches++;                                                                                          \
         }                                                                                                            \
