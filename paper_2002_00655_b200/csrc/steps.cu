@@ -242,7 +242,7 @@ __device__ __forceinline__ uint64_t sgns_pairs_before(uint64_t p, uint64_t T, ui
 // batch) and one factor per slot (1 for slot 0); the reduction multiplies as it adds.
 // A warp takes one center at a time.  The output-vector slots are handled 32 at a time: every lane first
 // resolves one slot (word -> key -> table entry -> row address), so those lookups are in flight together;
-// the rows are then read four slots at a time, all loads of the four before the first dot product.
+// the rows are then read kQuad slots at a time, all their loads before the first dot product.
 // kL4, kWindow, kNeg: row length (float4), window and negatives per context if known at compile time (0: taken
 // from the arguments; kNeg < 0: from the argument); divisions by the slots per context and row offsets then fold.
 // kOnce: rows whose key occurs once in the batch (`single`, per slot) are updated here, in place, with the values in hand; a
@@ -264,7 +264,8 @@ sgns_step_kernel(const uint32_t* __restrict__ tokens, uint64_t tok_first, uint64
     const uint32_t per_ctx = 1 + n_neg;
     const uint64_t slots = 1 + (uint64_t)2 * window * per_ctx;
     const uint64_t pairs0 = sgns_pairs_before(first_pos, T, window);
-    constexpr int kQuad = 4;
+    constexpr int kQuad = kCh == 4 ? 2 : kCh == 1 ? 8 : 4;     // rows in flight: as many as leave 128 registers without spills
+    constexpr int kLanes = 32 / kQuad;
     float4 u[kQuad][kCh];                                       // (elements past the row are never loaded: zero throughout)
 #pragma unroll
     for (int a = 0; a < kQuad; ++a)
@@ -342,19 +343,28 @@ sgns_step_kernel(const uint32_t* __restrict__ tokens, uint64_t tok_first, uint64
                     for (int c = 0; c < kCh; ++c)
                         x[a] += v[c].x * u[a][c].x + v[c].y * u[a][c].y + v[c].z * u[a][c].z + v[c].w * u[a][c].w;
                 }
-                // The four sums over the lanes by exchanging halves (6 exchanges, not 20): lanes 8 a .. 8 a + 7 are left with
-                // the a-th score, and turn it into the slot's factor.
-                const bool up = lane & 16, right = lane & 8;
-                float y0 = (up ? x[2] : x[0]) + __shfl_xor_sync(full, up ? x[0] : x[2], 16);
-                float y1 = (up ? x[3] : x[1]) + __shfl_xor_sync(full, up ? x[1] : x[3], 16);
-                float xa = (right ? y1 : y0) + __shfl_xor_sync(full, right ? y0 : y1, 8);
+                // The sums over the lanes by exchanging halves: each step leaves half as many values per lane (6 exchanges for
+                // four scores, not 20).  Lanes kLanes a .. kLanes (a + 1) are left with the a-th score, and turn it into the
+                // slot's factor.
+                int o = 16;
 #pragma unroll
-                for (int o = 4; o > 0; o >>= 1) xa += __shfl_xor_sync(full, xa, o);
-                const bool positive = (t0 + b + (lane >> 3)) % per_ctx == 0;
+                for (int half = kQuad / 2; half >= 1; half >>= 1) {
+                    const bool up = lane & o;
+#pragma unroll
+                    for (int a = 0; a < half; ++a) {
+                        const float send = up ? x[a] : x[a + half], keep = up ? x[a + half] : x[a];
+                        x[a] = keep + __shfl_xor_sync(full, send, o);
+                    }
+                    o >>= 1;
+                }
+                float xa = x[0];
+#pragma unroll
+                for (int o2 = kLanes / 2; o2 > 0; o2 >>= 1) xa += __shfl_xor_sync(full, xa, o2);
+                const bool positive = (t0 + b + lane / kLanes) % per_ctx == 0;
                 const float sc_mine = -lr * (sigmoidf(xa) - (positive ? 1.f : 0.f));
 #pragma unroll
                 for (int a = 0; a < kQuad; ++a) {
-                    const float sc = __shfl_sync(full, sc_mine, 8 * a), xs = __shfl_sync(full, xa, 8 * a);
+                    const float sc = __shfl_sync(full, sc_mine, kLanes * a), xs = __shfl_sync(full, xa, kLanes * a);
                     if (!((ok_mask >> (b + a)) & 1u)) continue;
                     if (lane == (int)(b + a)) {
                         my_scale = sc;
