@@ -469,6 +469,13 @@ __device__ __forceinline__ void grid_leave(unsigned int* bar, unsigned int n_blo
     }
 }
 
+// Asks for a row to be in L2 (lane by lane, so that a warp's rows are on their way from memory together).
+__device__ __forceinline__ void prefetch_row(const void* row, uint32_t bytes) {
+    const char* p = (const char*)row;
+    for (uint32_t o = 0; o < bytes; o += 128) asm volatile("prefetch.global.L2 [%0];" ::"l"(p + o));
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(p + bytes - 16));         // (rows need not start on a line)
+}
+
 // ---- bulk asynchronous copies global -> shared, reporting to a barrier word in shared memory ----
 __device__ __forceinline__ unsigned smem_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void mbar_init(uint64_t* bar, unsigned count) {

@@ -337,18 +337,12 @@ __device__ __noinline__ void group_preadd(const uint32_t* __restrict__ sk, uint3
 // go out together; then the positions are walked in groups whose update rows
 // and target rows are all requested before the first is used.
 //
-// kScaled: occurrence o does not have an update row of its own.  Its update is scales[o] times a source
-// row shared with other occurrences: the occurrences come in runs of `slots` per example, example e owning
-// source rows 2e (used, by its slot 0) and 2e + 1 (used by all its other slots) of `upd`.
-//
-// kL4 / kSlots: the row length in float4 and the slots per example if known at compile time (0: taken from the
-// arguments); row offsets, the copy size and the division by the slots then fold.
-//
-// skip_singles: keys that occur once have been updated by the gradient kernel.
-template <int kCh, bool kScaled, int kL4, int kSlots>
+// kL4: the row length in float4 if known at compile time (0: taken from the argument); row offsets and the copy size then
+// fold.
+template <int kCh, int kL4>
 __global__ void __launch_bounds__(256)
 push_reduce_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restrict__ sv, uint32_t n,
-                   const float4* __restrict__ upd, const float* __restrict__ scales, uint32_t slots_arg, bool skip_singles,
+                   const float4* __restrict__ upd,
                    float4* __restrict__ store, const uint2* __restrict__ table,
                    uint64_t S, uint32_t K, uint32_t L4_arg, double* __restrict__ carry,
                    uint4* __restrict__ starters, unsigned int* __restrict__ starter_count,
@@ -357,7 +351,6 @@ push_reduce_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restrict__
     __shared__ unsigned int s_ticket;
     __shared__ __align__(8) uint64_t bars[8][3];    // per warp and stage: the barrier word its copies report to
     const uint32_t L4 = kL4 ? (uint32_t)kL4 : L4_arg;
-    const uint32_t slots = kSlots ? (uint32_t)kSlots : slots_arg;
     if (call_failed(st, epoch)) return;
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
@@ -365,20 +358,13 @@ push_reduce_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restrict__
     const uint64_t base = (uint64_t)tile * kReduceTile;
     const uint32_t n_valid = base < n ? (uint32_t)tmin<uint64_t>((uint64_t)kReduceTile, n - base) : 0u;
     const uint32_t key = lane < n_valid ? sk[base + lane] : kSentinelPad;
-    uint32_t occ = lane < n_valid ? sv[base + lane] : 0u;
+    const uint32_t occ = lane < n_valid ? sv[base + lane] : 0u;
     uint32_t prev = __shfl_up_sync(full, key, 1);
     if (lane == 0) prev = (base > 0 && base - 1 < n) ? sk[base - 1] : kSentinelPad;
     const uint32_t next_after = (base + kReduceTile < n) ? sk[base + kReduceTile] : kSentinelPad;
     uint32_t next = __shfl_down_sync(full, key, 1);
     if (lane == 31) next = next_after;
-    // "no key" marks and padding sort last
-    const bool usable = key < K && !(kScaled && skip_singles && key != prev && key != next);
-    float scale = 1.f;
-    if (kScaled && usable) {
-        scale = scales[occ];
-        const uint32_t e = occ / slots;
-        occ = 2u * e + (occ != e * slots ? 1u : 0u);
-    }
+    const bool usable = key < K;                    // "no key" marks and padding sort last
     uint64_t row = 0;
     if (usable) row = phys_row(table[key], S);
     const unsigned head_mask = __ballot_sync(full, key != prev);
@@ -467,11 +453,9 @@ push_reduce_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restrict__
 #pragma unroll
             for (int k = 0; k < G; ++k) {
                 const int p = g * G + k;
-                const float sc = kScaled ? __shfl_sync(full, scale, p) : 1.f;
                 if (!((usable_mask >> p) & 1u)) continue;
-                // A segment of exactly one occurrence needs no fp64 sum: row + update (one fused multiply-add if
-                // the update is a factor times a source row) rounds the exact sum once, and the conversions to
-                // and from fp64, which share a pipe with little throughput, are not issued.
+                // A segment of exactly one occurrence needs no fp64 sum: row + update rounds the exact sum once, and the
+                // conversions to and from fp64, which share a pipe with little throughput, are not issued.
                 if ((((head_mask & fetch_mask) >> p) & 1u)) {
                     const uint64_t rw1 = __shfl_sync(full, row, p);
 #pragma unroll
@@ -479,28 +463,17 @@ push_reduce_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restrict__
                         if (fl + 32 * c >= L4) continue;
                         const float4 u = slot[(k * 2 * kCh + c) * 32];
                         float4 v = slot[(k * 2 * kCh + kCh + c) * 32];
-                        if (kScaled) {
-                            v.x = fmaf(sc, u.x, v.x); v.y = fmaf(sc, u.y, v.y);
-                            v.z = fmaf(sc, u.z, v.z); v.w = fmaf(sc, u.w, v.w);
-                        } else {
-                            v.x += u.x; v.y += u.y; v.z += u.z; v.w += u.w;
-                        }
+                        v.x += u.x; v.y += u.y; v.z += u.z; v.w += u.w;
                         store[rw1 * L4 + fl + 32 * c] = v;
                     }
                     continue;
                 }
-                const double d = (double)sc;
 #pragma unroll
                 for (int c = 0; c < kCh; ++c) {
                     if (fl + 32 * c >= L4) continue;
                     const float4 u = slot[(k * 2 * kCh + c) * 32];
-                    if (kScaled) {
-                        acc[c].x += d * (double)u.x; acc[c].y += d * (double)u.y;
-                        acc[c].z += d * (double)u.z; acc[c].w += d * (double)u.w;
-                    } else {
-                        acc[c].x += (double)u.x; acc[c].y += (double)u.y;
-                        acc[c].z += (double)u.z; acc[c].w += (double)u.w;
-                    }
+                    acc[c].x += (double)u.x; acc[c].y += (double)u.y;
+                    acc[c].z += (double)u.z; acc[c].w += (double)u.w;
                 }
                 if (!((end_mask >> p) & 1u)) continue;
                 const uint64_t rw = __shfl_sync(full, row, p);
@@ -531,6 +504,149 @@ push_reduce_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restrict__
     // the staging memory is free by now (every warp has waited for all its copies) and serves as scratch
     group_preadd(sk, n, L4, carry, group_done, group_sum, group, gpos, kg, reinterpret_cast<d4 (*)[32]>(stage_mem),
                  &s_ticket, kReduceTile, tmin<uint32_t>(kGroupTiles / 8, gridDim.x - group * (kGroupTiles / 8)));
+}
+
+// The reduction of occurrences that are a factor times a shared source row (skip-gram: rows of at most 512 values), with
+// the tiles, masks, parked partials and pre-added groups of push_reduce_kernel.  Occurrence o's update is scales[o] times a
+// row that it shares with others: the occurrences come in runs of `slots` per example, example e owning source rows 2e
+// (used, by its slot 0) and 2e + 1 (used by all its other slots) of `upd`.  Source rows (in L2, mostly: the gradient kernel
+// has just written them) go from there to registers, kG positions at a time; the rows of segments that end in the tile are
+// asked for at its start (prefetch_row) and read where they end.  Staged by bulk copies, a position at a time, the walk was
+// bound by its instructions (215 per position, issue slots 74 % used; now 85): 276 us for 1.04M positions of rows of 300
+// values, now 242 with two positions in flight at three blocks per SM (four at two blocks 287, three 297), bound by the
+// latency of its loads and the unit that widens values to fp64 (60 %).
+// skip_singles: keys that occur once have been updated by the gradient kernel.
+// kL4 / kSlots: the row length in float4 and the slots per example if known at compile time (0: taken from the
+// arguments); row offsets and the division by the slots then fold.
+template <int kCh, int kL4, int kSlots>
+__global__ void __launch_bounds__(256, kCh == 3 || kCh == 1 ? 3 : 2)
+scaled_reduce_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restrict__ sv, uint32_t n,
+                     const float4* __restrict__ upd, const float* __restrict__ scales, uint32_t slots_arg, bool skip_singles,
+                     float4* __restrict__ store, const uint2* __restrict__ table, uint64_t S, uint32_t K, uint32_t L4_arg,
+                     double* __restrict__ carry, uint4* __restrict__ starters, unsigned int* __restrict__ starter_count,
+                     unsigned int* __restrict__ group_done, double* __restrict__ group_sum, DevStatus* st, unsigned int epoch) {
+    __shared__ unsigned int s_ticket;
+    __shared__ d4 s_pre[8][32];
+    const uint32_t L4 = kL4 ? (uint32_t)kL4 : L4_arg;
+    const uint32_t slots = kSlots ? (uint32_t)kSlots : slots_arg;
+    if (call_failed(st, epoch)) return;
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const uint32_t tile = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const uint64_t base = (uint64_t)tile * kReduceTile;
+    const uint32_t n_valid = base < n ? (uint32_t)tmin<uint64_t>((uint64_t)kReduceTile, n - base) : 0u;
+    const uint32_t key = lane < n_valid ? sk[base + lane] : kSentinelPad;
+    uint32_t occ = lane < n_valid ? sv[base + lane] : 0u;
+    uint32_t prev = __shfl_up_sync(full, key, 1);
+    if (lane == 0) prev = (base > 0 && base - 1 < n) ? sk[base - 1] : kSentinelPad;
+    const uint32_t next_after = (base + kReduceTile < n) ? sk[base + kReduceTile] : kSentinelPad;
+    uint32_t next = __shfl_down_sync(full, key, 1);
+    if (lane == 31) next = next_after;
+    // "no key" marks and padding sort last
+    const bool usable = key < K && !(skip_singles && key != prev && key != next);
+    float scale = 0.f;
+    if (usable) {
+        scale = scales[occ];
+        const uint32_t e = occ / slots;
+        occ = 2u * e + (occ != e * slots ? 1u : 0u);
+    } else {
+        occ = 0;
+    }
+    uint64_t row = 0;
+    if (usable) row = phys_row(table[key], S);
+    const unsigned head_mask = __ballot_sync(full, key != prev);
+    const unsigned usable_mask = __ballot_sync(full, usable);
+    // positions at which a segment's part in this tile ends: its true end, or the tile's last position
+    const unsigned end_mask = __ballot_sync(full, usable && (key != next || lane == 31));
+    const int first_head = head_mask ? (__ffs(head_mask) - 1) : 32;
+    const uint32_t key31 = __shfl_sync(full, key, 31);
+    const bool runs_on = key31 < K && next_after == key31;
+    if (runs_on && head_mask != 0u && lane == 31)
+        starters[atomicAdd(starter_count, 1u)] = make_uint4(tile, key, (uint32_t)row, (uint32_t)(row >> 32));
+    // positions whose target row is updated: a segment ends there and is neither parked on the way in nor out
+    const bool fetch_me = usable && (key != next || lane == 31) && !(lane < first_head || (lane == 31 && runs_on));
+    const unsigned fetch_mask = __ballot_sync(full, fetch_me);
+    if (fetch_me) prefetch_row(store + row * L4, L4 * 16);
+    const uint32_t group = blockIdx.x / (kGroupTiles / 8);
+    const uint64_t gpos = (uint64_t)group * kGroupTiles * kReduceTile;
+    uint32_t kg = kSentinelPad, kg_prev = kSentinelPad - 1, kg_far = kSentinelPad - 2;
+    if (gpos > 0 && gpos + kGroupMinSpan - 1 < n) {
+        kg = sk[gpos];
+        kg_prev = sk[gpos - 1];
+        kg_far = sk[gpos + kGroupMinSpan - 1];
+    }
+    const uint32_t L = L4 * 4;
+    constexpr int kG = kCh >= 3 ? 2 : 4;
+    d4 acc[kCh];
+#pragma unroll
+    for (int c = 0; c < kCh; ++c) acc[c] = d4{0.0, 0.0, 0.0, 0.0};
+    float4 u[kG][kCh];                                          // (elements past the row are never loaded: zero throughout)
+#pragma unroll
+    for (int k = 0; k < kG; ++k)
+#pragma unroll
+        for (int c = 0; c < kCh; ++c) u[k][c] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (unsigned todo = usable_mask; todo;) {
+        int at[kG];
+#pragma unroll
+        for (int k = 0; k < kG; ++k) {
+            at[k] = todo ? __ffs(todo) - 1 : -1;
+            todo &= todo - 1;                                   // 0 stays 0
+            const float4* src = upd + (uint64_t)__shfl_sync(full, occ, at[k] & 31) * L4 + lane;
+#pragma unroll
+            for (int c = 0; c < kCh; ++c)
+                if (lane + 32 * c < L4) u[k][c] = __ldg(src + 32 * c);      // (past the last: some other row, not used)
+        }
+#pragma unroll
+        for (int k = 0; k < kG; ++k) {
+            const int p = at[k];
+            if (p < 0) break;
+            const float sc = __shfl_sync(full, scale, p);
+            const bool ends = (end_mask >> p) & 1u, whole = (fetch_mask >> p) & 1u;
+            if (whole && ((head_mask >> p) & 1u)) {             // one occurrence: a multiply-add rounds the exact sum once
+                float4* to = store + __shfl_sync(full, row, p) * L4 + lane;
+#pragma unroll
+                for (int c = 0; c < kCh; ++c) {
+                    if (lane + 32 * c >= L4) continue;
+                    float4 v = to[32 * c];
+                    v.x = fmaf(sc, u[k][c].x, v.x); v.y = fmaf(sc, u[k][c].y, v.y);
+                    v.z = fmaf(sc, u[k][c].z, v.z); v.w = fmaf(sc, u[k][c].w, v.w);
+                    to[32 * c] = v;
+                }
+                continue;
+            }
+            const double d = (double)sc;
+#pragma unroll
+            for (int c = 0; c < kCh; ++c) {
+                acc[c].x += d * (double)u[k][c].x; acc[c].y += d * (double)u[k][c].y;
+                acc[c].z += d * (double)u[k][c].z; acc[c].w += d * (double)u[k][c].w;
+            }
+            if (!ends) continue;
+            if (whole) {
+                float4* to = store + __shfl_sync(full, row, p) * L4 + lane;
+#pragma unroll
+                for (int c = 0; c < kCh; ++c) {
+                    if (lane + 32 * c >= L4) continue;
+                    float4 v = to[32 * c];
+                    v.x = (float)((double)v.x + acc[c].x); v.y = (float)((double)v.y + acc[c].y);
+                    v.z = (float)((double)v.z + acc[c].z); v.w = (float)((double)v.w + acc[c].w);
+                    to[32 * c] = v;
+                }
+            } else {
+                double* cs = carry + ((uint64_t)tile * 2 + (p < first_head ? 0 : 1)) * L + (uint64_t)lane * 4;
+#pragma unroll
+                for (int c = 0; c < kCh; ++c) {
+                    if (lane + 32 * c >= L4) continue;
+                    *(double2*)(cs + 128 * c) = make_double2(acc[c].x, acc[c].y);
+                    *(double2*)(cs + 128 * c + 2) = make_double2(acc[c].z, acc[c].w);
+                }
+            }
+#pragma unroll
+            for (int c = 0; c < kCh; ++c) acc[c] = d4{0.0, 0.0, 0.0, 0.0};
+        }
+    }
+    if (!(kg < K && kg_prev == kg && kg_far == kg)) return;     // nothing to pre-add for this group
+    group_preadd(sk, n, L4, carry, group_done, group_sum, group, gpos, kg, s_pre, &s_ticket, kReduceTile,
+                 tmin<uint32_t>(kGroupTiles / 8, gridDim.x - group * (kGroupTiles / 8)));
 }
 
 // ------------------------------------------------- MF: gradient inside the reduction ----
@@ -1209,32 +1325,42 @@ void run_push_reduce(ps_store* ps, uint32_t n, int which, const float* d_upd, do
     const uint32_t tiles = div_up_u32(n, kReduceTile);
     const uint32_t blocks = div_up_u32(tiles, 8);
     const uint32_t L4 = ps->cfg.row_len / 4;
-#define REDUCE_ARGS sk, sv, n, (const float4*)d_upd, d_scales, slots, skip_singles, (float4*)ps->store, ps->table,   \
+#define REDUCE_ARGS sk, sv, n, (const float4*)d_upd, (float4*)ps->store, ps->table,                                  \
                     ps->cfg.slots_per_part, (uint32_t)ps->cfg.num_keys, L4, ps->carry, ps->starters,                \
                     ps->starter_count, ps->group_done, ps->group_sum, ps->status, ps->epoch
-#define REDUCE_LAUNCH(kCh, kScaled, kL4, kSlots)                                                                     \
+#define REDUCE_LAUNCH(kCh, kL4)                                                                                      \
     do {                                                                                                             \
         static std::atomic<unsigned long long> smem_set{0};                                                          \
-        opt_in_smem((const void*)push_reduce_kernel<kCh, kScaled, kL4, kSlots>, reduce_smem(kCh), &smem_set);        \
-        if (ps->prof) prof_before(ps, "push_reduce_kernel<" #kCh "," #kScaled ">", s);                               \
-        push_reduce_kernel<kCh, kScaled, kL4, kSlots><<<blocks, 256, reduce_smem(kCh), s>>>(REDUCE_ARGS);            \
+        opt_in_smem((const void*)push_reduce_kernel<kCh, kL4>, reduce_smem(kCh), &smem_set);                         \
+        if (ps->prof) prof_before(ps, "push_reduce_kernel<" #kCh ">", s);                                            \
+        push_reduce_kernel<kCh, kL4><<<blocks, 256, reduce_smem(kCh), s>>>(REDUCE_ARGS);                             \
         if (ps->prof) prof_after(ps, s);                                                                             \
         ps->launches++;                                                                                              \
     } while (0)
     // the row lengths of the paper's workloads get kernels of their own: 128, 300 (41 slots per center) and 400 values
     if (d_scales) {
-        if (L4 == 75 && slots == 41) REDUCE_LAUNCH(3, true, 75, 41);
-        else if (L4 <= 32) REDUCE_LAUNCH(1, true, 0, 0);
-        else if (L4 <= 64) REDUCE_LAUNCH(2, true, 0, 0);
-        else if (L4 <= 96) REDUCE_LAUNCH(3, true, 0, 0);
-        else REDUCE_LAUNCH(4, true, 0, 0);
+#define SCALED_LAUNCH(kCh, kL4, kSlots)                                                                              \
+    do {                                                                                                             \
+        if (ps->prof) prof_before(ps, "scaled_reduce_kernel<" #kCh ">", s);                                          \
+        scaled_reduce_kernel<kCh, kL4, kSlots><<<blocks, 256, 0, s>>>(sk, sv, n, (const float4*)d_upd, d_scales, slots, \
+            skip_singles, (float4*)ps->store, ps->table, ps->cfg.slots_per_part, (uint32_t)ps->cfg.num_keys, L4, ps->carry, \
+            ps->starters, ps->starter_count, ps->group_done, ps->group_sum, ps->status, ps->epoch);                  \
+        if (ps->prof) prof_after(ps, s);                                                                             \
+        ps->launches++;                                                                                              \
+    } while (0)
+        if (L4 == 75 && slots == 41) SCALED_LAUNCH(3, 75, 41);
+        else if (L4 <= 32) SCALED_LAUNCH(1, 0, 0);
+        else if (L4 <= 64) SCALED_LAUNCH(2, 0, 0);
+        else if (L4 <= 96) SCALED_LAUNCH(3, 0, 0);
+        else SCALED_LAUNCH(4, 0, 0);
+#undef SCALED_LAUNCH
     } else {
-        if (L4 == 32) REDUCE_LAUNCH(1, false, 32, 0);
-        else if (L4 == 100) REDUCE_LAUNCH(4, false, 100, 0);
-        else if (L4 <= 32) REDUCE_LAUNCH(1, false, 0, 0);
-        else if (L4 <= 64) REDUCE_LAUNCH(2, false, 0, 0);
-        else if (L4 <= 96) REDUCE_LAUNCH(3, false, 0, 0);
-        else REDUCE_LAUNCH(4, false, 0, 0);
+        if (L4 == 32) REDUCE_LAUNCH(1, 32);
+        else if (L4 == 100) REDUCE_LAUNCH(4, 100);
+        else if (L4 <= 32) REDUCE_LAUNCH(1, 0);
+        else if (L4 <= 64) REDUCE_LAUNCH(2, 0);
+        else if (L4 <= 96) REDUCE_LAUNCH(3, 0);
+        else REDUCE_LAUNCH(4, 0);
     }
 #undef REDUCE_LAUNCH
 #undef REDUCE_ARGS
