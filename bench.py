@@ -117,14 +117,17 @@ def smi_clocks():
 # keyed by (workload, kernel).  An entry is removed when its kernel changes after the capture.
 TRAFFIC = {
     ("mf_large", "mf_sub_kernel<4,gather4>"): 46.1e6,                 # profiles/mf_step_kernels_ncu_full.md (same-batch twin)
-    ("kge", "kge_reduce_kernel<2>"): 321.6e6,                   # profiles/kge_step_kernels_ncu_full.md
-    ("rescal", "rescal_grad_kernel<4>"): 501.4e6,               # profiles/rescal_step_kernels_ncu_full.md
-    ("sgns", "push_reduce_kernel<3,true>"): 1561.1e6,           # profiles/sgns_step_kernels_ncu_full.md
 }
 
 
 def n_unique(*tensors) -> int:
     return int(torch.unique(torch.cat([t.reshape(-1).to(torch.int64) for t in tensors])).numel())
+
+
+def key_counts(keys):
+    """(distinct keys, keys that occur once) of a batch's occurrence keys."""
+    c = torch.unique(keys.reshape(-1).to(torch.int64), return_counts=True)[1]
+    return int(c.numel()), int((c == 1).sum())
 
 
 def sort_bytes(occ, key_bits, extra=0):
@@ -157,6 +160,8 @@ def kernel_bytes_of_step(batch_bytes, occ, u, rb, keys_prefix, step_prefix, key_
         "push_fixup_kernel": fixup_bytes(keys, 32, rb) if keys is not None else None,
         keys_prefix: batch_bytes + occ * 4,                      # batch arrays in, one 32-bit key per occurrence out
         "sort_all_kernel": sort_bytes(occ, key_bits),
+        "sort_cluster_kernel": sort_bytes(occ, key_bits),
+        "segment_kernel": occ * (8 + 1),                         # sorted pairs in, a mark per occurrence out (and short lists)
         step_prefix: batch_bytes + occ * (8 + rb) + occ * rb,    # table entry + row per occurrence in, update row out
         "push_reduce_kernel": occ * (8 + rb) + u * (8 + 2 * rb), # sorted pair + update row in; row read-modify-write
     }
@@ -492,7 +497,7 @@ class KGEWorkload:
         return self.cfg.batch
 
     def side_stream_kernels(self):
-        return ("sort_all_kernel", "kge_keys")
+        return ("sort_all_kernel", "sort_cluster_kernel", "segment_kernel", "kge_keys")
 
     def _sl(self, k):
         b = self.cfg.batch
@@ -529,15 +534,17 @@ class KGEWorkload:
         u = n_unique(self.s[sl], self.o[sl], self.neg[sl]) + n_unique(self.r[sl])
         keys = torch.cat([t.reshape(-1).to(torch.int64) for t in (self.s[sl], self.o[sl], self.neg[sl])] +
                          [c.rel_key_base + self.r[sl].to(torch.int64)])
-        kb = kernel_bytes_of_step(b * (12 + c.n_neg * 5), (3 + c.n_neg) * b, u, self.row_bytes, "kge_keys", "kge_step",
+        kb = kernel_bytes_of_step(b * (12 + c.n_neg * 5), (3 + c.n_neg) * b, u, self.row_bytes, "kge_keys", "kge_short_kernel",
                                   int(c.num_keys).bit_length(), keys)
         occ, rb = (3 + c.n_neg) * b, self.row_bytes
-        # the step kernel reads the embedding half of every row and writes a gradient row of the same size; the
-        # reduction reads those and read-modify-writes every distinct row
-        if c.dim % 2 == 0 and c.dim <= 128:
-            kb["kge_step"] = b * (12 + c.n_neg * 5) + occ * (8 + rb // 2) + occ * (rb // 2)
-            kb["kge_reduce_kernel"] = occ * (8 + rb // 2) + u * (8 + 2 * rb)
-        # (wider rows: the step kernel reads whole rows and writes finished update rows, reduced like a push's)
+        _, once = key_counts(keys)
+        # The gradient kernel reads the embedding half of every occurrence's row.  Keys that occur once in the batch it
+        # updates in place (the accumulator half in, the row out); for the others it writes a gradient row of dim x 2
+        # values, which the reduction reads before it read-modify-writes the keys' rows.
+        grad = b * (12 + c.n_neg * 5) + occ * (8 + rb // 2) + once * (rb // 2 + rb) + (occ - once) * (rb // 2)
+        for name in ("kge_short_kernel", "kge_points_kernel", "kge_wide_kernel"):
+            kb[name] = grad
+        kb["segment_adagrad_kernel"] = (occ - once) * (8 + rb // 2) + (u - once) * (8 + 2 * rb)
         return kb
 
     def oracle_setup(self, device):
@@ -611,7 +618,7 @@ class RescalWorkload(KGEWorkload):
         torch.cuda.synchronize(device)
 
     def side_stream_kernels(self):
-        return ("sort_all_kernel", "rescal_keys")
+        return ("sort_all_kernel", "sort_cluster_kernel", "segment_kernel", "rescal_keys")
 
     def step(self, k):
         c, sl = self.cfg, self._sl(k)
@@ -630,16 +637,23 @@ class RescalWorkload(KGEWorkload):
 
     def kernel_bytes(self, k, moved=0.0):
         c, sl, b = self.cfg, self._sl(k), self.cfg.batch
-        u, occ, rb = self._distinct(sl), self._occ(), self.row_bytes
-        rows_of = (c.rel_key_base + self.r[sl].to(torch.int64)[:, None] * c.dim +
-                   torch.arange(c.dim, device=self.r.device, dtype=torch.int64)[None, :])
-        keys = torch.cat([t.reshape(-1).to(torch.int64) for t in (self.s[sl], self.o[sl], self.neg[sl])] + [rows_of.reshape(-1)])
-        kb = kernel_bytes_of_step(b * (12 + c.n_neg * 5), occ, u, rb, "rescal_keys", "rescal_grad",
-                                  int(c.num_keys).bit_length(), keys)
-        # the gradient kernel reads the value half of every row (the matrix once per data point) and writes a gradient
-        # row of the same size per occurrence; the reduction reads those and read-modify-writes every distinct row
-        kb["rescal_grad"] = b * (12 + c.n_neg * 5) + occ * (8 + rb // 2) + occ * (rb // 2)
-        kb["kge_reduce_kernel"] = occ * (8 + rb // 2) + u * (8 + 2 * rb)
+        rb = self.row_bytes
+        # one slot per data point for its relation: its d matrix rows are worked on as one
+        occ = (3 + c.n_neg) * b
+        keys = torch.cat([t.reshape(-1).to(torch.int64) for t in (self.s[sl], self.o[sl], self.neg[sl])])
+        u_ent, once = key_counts(keys)
+        n_rel = n_unique(self.r[sl])
+        groups = (torch.unique(self.r[sl], return_counts=True)[1] + 7) // 8
+        kb = kernel_bytes_of_step(b * (12 + c.n_neg * 5), occ, u_ent + n_rel, rb, "rescal_keys", "rescal_points_kernel",
+                                  int(c.num_keys).bit_length())
+        # The points kernel reads the value half of every entity occurrence's row and, per up to eight data points of one
+        # relation, its matrix; entities that occur once are updated in place, the others get a gradient row; four vectors
+        # of fp64 per data point go to the matrix kernel, which read-modify-writes each relation's rows once.
+        kb["rescal_points_kernel"] = (b * (12 + c.n_neg * 5) + (2 + c.n_neg) * b * (8 + rb // 2) +
+                                      int(groups.sum()) * c.dim * (8 + rb // 2) + once * (rb // 2 + rb) +
+                                      ((2 + c.n_neg) * b - once) * (rb // 2) + b * 32 * c.dim)
+        kb["rescal_matrix_kernel"] = b * 32 * c.dim + n_rel * c.dim * (8 + 2 * rb)
+        kb["segment_adagrad_kernel"] = ((2 + c.n_neg) * b - once) * (8 + rb // 2) + (u_ent - once) * (8 + 2 * rb)
         return kb
 
     def oracle_setup(self, device):
@@ -699,7 +713,7 @@ class SGNSWorkload:
         return self.cfg.batch
 
     def side_stream_kernels(self):
-        return ("sort_all_kernel", "sgns_keys")
+        return ("sort_all_kernel", "sort_cluster_kernel", "single_kernel", "sgns_keys")
 
     def step(self, k):
         c = self.cfg
@@ -752,10 +766,14 @@ class SGNSWorkload:
                           (c.out_key_base + span).repeat(2 * c.window), c.out_key_base + self.negs[k].to(torch.int64)])
         kb = kernel_bytes_of_step(c.batch * 4 + pairs * (1 + c.n_neg) * 4, occ, u, self.row_bytes,
                                   "sgns_keys", "sgns_step", int(c.num_keys).bit_length(), keys)
-        # the step kernel writes two source rows per center and one factor per occurrence, not a row per occurrence
-        kb["sgns_step"] += c.batch * 2 * self.row_bytes + occ * 4 - occ * self.row_bytes
-        # ... and the reduction reads a factor per occurrence and those 2 x centers source rows (from L2 after the first touch)
-        kb["push_reduce_kernel"] += occ * 4 + c.batch * 2 * self.row_bytes - occ * self.row_bytes
+        # The gradient kernel writes two source rows per center and, for keys that occur several times, one factor per
+        # occurrence; rows of keys that occur once it updates in place.  The reduction reads factors and source rows (those
+        # from L2 after the first touch) and read-modify-writes the other keys' rows.
+        rb = self.row_bytes
+        _, once = key_counts(keys)
+        kb["single_kernel"] = occ * 9
+        kb["sgns_step"] += c.batch * 2 * rb + occ * 4 - occ * rb + once * rb
+        kb["scaled_reduce_kernel"] = occ * 12 + (occ - once) * 8 + c.batch * 2 * rb + (u - once) * 2 * rb
         return kb
 
     def oracle_setup(self, device):
