@@ -602,20 +602,27 @@ __global__ void __launch_bounds__(256, 1) kge_points_kernel(const KgeArgs A) {
     }
 }
 
-// Rows of more than 128 complex dimensions and up to ten negatives: a block per data point, the rows streamed through
-// shared memory 256 dimensions at a time as bulk copies, the next stretch on its way while one is worked on, across the two
-// passes and across data points.  (With loads into registers, one stretch after the other, the memory system was idle
-// three quarters of the time: 1,199 us for 2,048 data points of 4,000 dimensions whose rows take 440 us.)  A stretch of a part
-// (Re, Im, G_Re or G_Im) of a row starts at a multiple of 16 bytes only if d is a multiple of four: the copy starts at the
-// boundary before it, and `shift` floats are skipped.
+// Rows of more than 128 complex dimensions and up to ten negatives: a block per data point (batches of few data points: a
+// cluster of up to four, which meets to add up the scores), the rows streamed through shared memory in stretches of 256
+// dimensions as bulk copies, what the next job needs on its way while one is worked on, across the two passes and across
+// data points.  (With loads into registers, one stretch after the other, the memory system was idle three quarters of the
+// time: 1,199 us for 2,048 data points of 4,000 dimensions whose rows take 440 us; streamed 808 us; with two stretches per job
+// in the first pass, which has little to do on them and waits for their arrival, and the two kinds of update row compiled
+// apart, 747.)  It is bound by the second pass's instructions (1,300 per warp and stretch, half of them AdaGrad's, issued at
+// 16 warps per SM in chains) and by those arrivals.  Filling a stage when its last reader leaves, without a barrier per
+// job, gained nothing; asking L2 for the rows two jobs earlier cost 200 us.  A stretch of a part (Re, Im, G_Re or G_Im) of a
+// row starts at a multiple of 16 bytes only if d is a multiple of four: the copy starts at the boundary before it, and
+// `shift` floats are skipped.
 constexpr uint32_t kStretch = 256, kStretchPad = kStretch + 4;
 
-template <int kMaxNeg>
+template <int kMaxNeg, bool kFinished>
 __global__ void __launch_bounds__(256, 2) kge_wide_kernel(const KgeArgs A) {
     constexpr int kSlots = 3 + kMaxNeg, kWarps = 8;
     extern __shared__ __align__(128) float stage_mem[];         // [2 stages][slot][part][kStretchPad]
     __shared__ __align__(8) uint64_t bars[2];
     __shared__ double s_part[kWarps][kMaxNeg + 1];
+    __shared__ double s_tot[2][kMaxNeg + 1];                    // the block's share of the scores, by the data point's parity
+    __shared__ int s_failed;
     __shared__ double s_w[3][32];
     __shared__ uint64_t s_off[32];
     const unsigned full = 0xffffffffu;
@@ -628,9 +635,24 @@ __global__ void __launch_bounds__(256, 2) kge_wide_kernel(const KgeArgs A) {
     mbar_init_fence();
     pdl_trigger();
     pdl_wait();
-    if (A.single && call_failed(A.st, A.epoch)) return;
+    uint32_t rank, C;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    asm("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(C));
+    if (A.single) {
+        bool failed = call_failed(A.st, A.epoch);
+        if (C > 1) {                                            // a block that started later may see more: one decision
+            if (tid == 0) s_failed = failed;
+            cluster_arrive();
+            cluster_wait();
+            for (uint32_t r = 0; r < C; ++r) failed |= peer_i32(&s_failed, r) != 0;
+            cluster_arrive();
+            cluster_wait();
+        }
+        if (failed) return;
+    }
     __syncthreads();
-    const uint32_t n_str = (d + kStretch - 1) / kStretch;
+    const uint32_t n_str = ((d + kStretch - 1) / kStretch - rank + C - 1) / C;         // stretches rank, rank + C, ... are the block's
+    const uint64_t stride = gridDim.x / C;
     double loss = 0;
     // what a warp knows of a data point: lane u its slot u
     struct Point {
@@ -667,31 +689,38 @@ __global__ void __launch_bounds__(256, 2) kge_wide_kernel(const KgeArgs A) {
         P.once = __ballot_sync(full, once);
         return P;
     };
-    // warp 0 asks for stretch number `str` of a data point's rows; with_acc: of their accumulators too where they are needed
-    auto issue = [&](const Point& P, uint32_t str, bool with_acc, int stage) {
-        const uint32_t c0 = str * kStretch, len = d - c0 < kStretch ? d - c0 : kStretch;
-        const unsigned acc = with_acc ? (A.finished ? P.reps : P.once) : 0u;
+    // Warp 0 asks for what a job of a data point reads.  First pass: the next two stretches of its rows' Re and Im (as many
+    // bytes as a job of the second pass: there is little to do on them, so it is their arrival that counts).  Second pass: one
+    // stretch, and of the accumulators too where they are needed.
+    const uint32_t n_first = (n_str + 1) / 2, n_jobs = n_first + n_str;
+    auto issue = [&](const Point& P, uint32_t job, int stage) {
+        const bool second = job >= n_first;
+        const uint32_t str = second ? job - n_first : 2 * job;
+        const uint32_t c0 = (str * C + rank) * kStretch, c1 = c0 + C * kStretch;        // c1: the stretch after it
+        const uint32_t len0 = tmin(d - c0, kStretch), len1 = second || str + 1 == n_str ? 0u : tmin(d - c1, kStretch);
+        const unsigned acc = !second ? 0u : kFinished ? P.reps : P.once;
         uint32_t bytes[4], total = 0;
 #pragma unroll
         for (int p = 0; p < 4; ++p) {
-            bytes[p] = ((len + ((p * d) & 3) + 3) & ~3u) * 4;
-            total += bytes[p] * (p < 2 ? (uint32_t)n_slots : (uint32_t)__popc(acc));
+            const uint32_t q = second ? p : p & 1, len = second || p < 2 ? len0 : len1;
+            bytes[p] = len ? ((len + ((q * d) & 3) + 3) & ~3u) * 4 : 0u;
+            total += bytes[p] * (second && p >= 2 ? (uint32_t)__popc(acc) : (uint32_t)n_slots);
         }
         if (lane == 0) mbar_expect_tx(&bars[stage], total);
         __syncwarp();
         if (!slot) return;
-        const int parts = ((acc >> lane) & 1u) ? 4 : 2;
+        const int parts = (second ? (acc >> lane) & 1u : len1 != 0) ? 4 : 2;
         for (int p = 0; p < parts; ++p)
-            bulk_g2s(stage_mem + (((size_t)stage * kSlots + lane) * 4 + p) * kStretchPad, A.store + P.off + ((p * d + c0) & ~3u),
-                     bytes[p], &bars[stage]);
+            bulk_g2s(stage_mem + (((size_t)stage * kSlots + lane) * 4 + p) * kStretchPad,
+                     A.store + P.off + (second ? (p * d + c0) & ~3u : ((p & 1) * d + (p < 2 ? c0 : c1)) & ~3u), bytes[p], &bars[stage]);
     };
-    uint64_t t = blockIdx.x;
+    uint64_t t = blockIdx.x / C;
     Point P = {}, N = {};
     // the first data point (from `from` on) whose indexes are all valid; marks the others (the same in every warp)
     auto next_valid = [&](uint64_t from, Point& Q) {
-        for (; from < A.n; from += gridDim.x) {
+        for (; from < A.n; from += stride) {
             Q = look_up(from);
-            if (A.keys_out && slot && w == 0)
+            if (A.keys_out && slot && w == 0 && rank == 0)
                 A.keys_out[from * n_slots + lane] = Q.bad ? kSentinelPad : Q.rep == lane ? Q.key : (uint32_t)K;
             if (!Q.bad) break;
             if (tid == 0) latch_error(A.st, A.keys_out ? 0u : A.epoch, PS_ERR_KEY_RANGE);
@@ -702,35 +731,36 @@ __global__ void __launch_bounds__(256, 2) kge_wide_kernel(const KgeArgs A) {
     unsigned uses = 0;
     int stage = 0;
     bool dead = false;
-    if (t < A.n && w == 0) issue(P, 0, false, 0);
+    int parity = 0;
+    if (t < A.n && w == 0) issue(P, 0, 0);
     while (t < A.n) {
-        const uint64_t tn = next_valid(t + gridDim.x, N);
-        const unsigned subj_mask = P.subj, rep_mask = P.reps, once_mask = P.once, acc_mask = A.finished ? P.reps : P.once;
+        const uint64_t tn = next_valid(t + stride, N);
+        const unsigned subj_mask = P.subj, rep_mask = P.reps, acc_mask = kFinished ? P.reps : P.once;
         double part[kMaxNeg + 1];
 #pragma unroll
         for (int q = 0; q <= kMaxNeg; ++q) part[q] = 0.0;
         double cf0 = 0;
         int rep_o = 2;
-        const uint32_t LU = A.finished ? 4 * d : 2 * d;         // values per update row
+        const uint32_t LU = kFinished ? 4 * d : 2 * d;         // values per update row
         float* const U = A.upd + t * n_slots * (uint64_t)LU;
-        for (uint32_t job = 0; job < 2 * n_str; ++job) {
-            const bool pass_b = job >= n_str;
-            const uint32_t str = pass_b ? job - n_str : job;
+        for (uint32_t job = 0; job < n_jobs; ++job) {
+            const bool pass_b = job >= n_first;
+            const uint32_t str = pass_b ? job - n_first : 2 * job;
             // the job after this one; its stage was read two jobs ago (and the warps have met since)
             if (w == 0) {
-                if (job + 1 < 2 * n_str) issue(P, job + 1 >= n_str ? job + 1 - n_str : job + 1, job + 1 >= n_str, stage ^ 1);
-                else if (tn < A.n) issue(N, 0, false, stage ^ 1);
+                if (job + 1 < n_jobs) issue(P, job + 1, stage ^ 1);
+                else if (tn < A.n) issue(N, 0, stage ^ 1);
             }
             if (!mbar_wait(&bars[stage], (uses >> stage) & 1u) && !mbar_wait(&bars[stage], (uses >> stage) & 1u)) dead = true;
             uses ^= 1u << stage;
-            const float* const base = stage_mem + (size_t)stage * kSlots * 4 * kStretchPad + tid;
+            const float* base = stage_mem + (size_t)stage * kSlots * 4 * kStretchPad + tid;
             const uint32_t sh1 = d & 3, sh2 = (2 * d) & 3, sh3 = (3 * d) & 3;
             auto re = [&](int u) { return base[u * 4 * kStretchPad]; };
             auto im = [&](int u) { return base[(u * 4 + 1) * kStretchPad + sh1]; };
             auto gre = [&](int u) { return base[(u * 4 + 2) * kStretchPad + sh2]; };
             auto gim = [&](int u) { return base[(u * 4 + 3) * kStretchPad + sh3]; };
-            const uint32_t c = str * kStretch + tid;
-            if (c < d) {
+            uint32_t c = (str * C + rank) * kStretch + tid;
+            for (int half = 0; half < (pass_b ? 1 : 2) && c < d; ++half, c += C * kStretch, base += 2 * kStretchPad) {
                 const float a_f = re(0), b_f = im(0), cr_f = re(1), ci_f = im(1), e_f = re(2), f_f = im(2);
                 const double a = a_f, b = b_f, cr = cr_f, ci = ci_f, e = e_f, f = f_f;
                 // directions that do not depend on the negative: d phi / d subject (object = o), d phi / d object (subject = s)
@@ -775,12 +805,11 @@ __global__ void __launch_bounds__(256, 2) kge_wide_kernel(const KgeArgs A) {
                         const float g2[2] = {g[0] * g[0], g[1] * g[1]}, x[2] = {gre(u) + g2[0], gim(u) + g2[1]};
                         float step[2];
                         adagrad_steps<2>(g, x, A.lr, A.eps, step);
-                        const bool in_place = (once_mask >> u) & 1u;
-                        if (in_place) o = A.store + s_off[u] + c;
-                        o[0] = in_place ? re(u) + step[0] : step[0];
-                        o[d] = in_place ? im(u) + step[1] : step[1];
-                        o[2 * d] = in_place ? x[0] : g2[0];
-                        o[3 * d] = in_place ? x[1] : g2[1];
+                        if (!kFinished) o = A.store + s_off[u] + c;     // in place
+                        o[0] = kFinished ? step[0] : re(u) + step[0];
+                        o[d] = kFinished ? step[1] : im(u) + step[1];
+                        o[2 * d] = kFinished ? g2[0] : x[0];
+                        o[3 * d] = kFinished ? g2[1] : x[1];
                     };
                     out(0, gs_re, gs_im);
                     out(1, gr_re, gr_im);
@@ -795,7 +824,7 @@ __global__ void __launch_bounds__(256, 2) kge_wide_kernel(const KgeArgs A) {
                 }
             }
             stage ^= 1;
-            if (job + 1 == n_str) {             // the scores are complete: coefficients and weights, as in kge_points_kernel
+            if (job + 1 == n_first) {           // the scores are complete: coefficients and weights, as in kge_points_kernel
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
@@ -807,6 +836,15 @@ __global__ void __launch_bounds__(256, 2) kge_wide_kernel(const KgeArgs A) {
                 double phi = 0, coef = 0, loss_q = 0;
                 if (lane <= kMaxNeg)
                     for (int i = 0; i < kWarps; ++i) phi += s_part[i][lane];
+                if (C > 1) {                    // the blocks' shares, in rank order
+                    if (w == 0 && lane <= kMaxNeg) s_tot[parity][lane] = phi;
+                    cluster_arrive();
+                    cluster_wait();
+                    phi = 0;
+                    if (lane <= kMaxNeg)
+                        for (uint32_t r = 0; r < C; ++r) phi += peer_f64(&s_tot[parity][lane], r);
+                    parity ^= 1;                // (two data points on, all have met again: the reads above are done)
+                }
                 if (lane <= (int)n_neg) {
                     const double y = lane == 0 ? 1.0 : -1.0, z = -y * phi, ez = exp(-fabs(z));
                     loss_q = fmax(z, 0.0) + log1p(ez);
@@ -833,13 +871,29 @@ __global__ void __launch_bounds__(256, 2) kge_wide_kernel(const KgeArgs A) {
             }
             if (__syncthreads_or(dead)) {
                 if (tid == 0) latch_error(A.st, A.epoch, PS_ERR_CUDA);
+                if (C == 1) return;
+                // the cluster's other blocks go on: meet them as often as they will, with nothing done in between
+                if (job + 1 < n_first) {
+                    cluster_arrive();
+                    cluster_wait();
+                }
+                for (uint64_t r = tn; r < A.n; r = next_valid(r + stride, N)) {
+                    cluster_arrive();
+                    cluster_wait();
+                }
+                cluster_arrive();
+                cluster_wait();
                 return;
             }
         }
         P = N;
         t = tn;
     }
-    if (tid == 0) A.loss_partial[blockIdx.x] = loss;
+    if (tid == 0) A.loss_partial[blockIdx.x] = rank == 0 ? loss : 0.0;
+    if (C > 1) {                                // (nobody reads a block's shared memory after it has left)
+        cluster_arrive();
+        cluster_wait();
+    }
 }
 
 // Keys of the occurrence slots of each data point; a slot that repeats an earlier slot's key, and every
@@ -864,6 +918,48 @@ kge_keys_kernel(const uint32_t* __restrict__ ts, const uint32_t* __restrict__ tr
     if (any_bad && lane == 0) latch_error(st, epoch, PS_ERR_KEY_RANGE);
     const unsigned same = __match_any_sync(0xffffffffu, slot ? (uint32_t)key : kSentinelPad);
     if (slot) keys_out[t * n_slots + lane] = (!any_bad && __ffs(same) - 1 == lane) ? (uint32_t)key : (uint32_t)K;
+}
+
+// A cluster of several blocks per data point where the data points alone would leave blocks' places empty (60 data points of
+// 4,000 dimensions: 77 us with one block each, 46 with two, 32 with four, 36 with eight).  Not otherwise, although fewer data
+// points in flight would keep more of their rows in L2 between the passes: the meetings cost more than the 0.4 of 1.7 GB
+// fewer reads save (2,048 data points: 747 us with one block, 791 with two, 950 with four).
+template <int kMaxNeg, bool kFinished>
+uint32_t launch_wide(ps_store* ps, const KgeArgs& A, cudaStream_t s) {
+    const size_t smem = (size_t)2 * (3 + kMaxNeg) * 4 * kStretchPad * sizeof(float);
+    static std::atomic<unsigned long long> smem_set{0};
+    static std::atomic<int> fit[64][3];                         // clusters resident at once, by device and size (0: not asked yet)
+    opt_in_smem((const void*)kge_wide_kernel<kMaxNeg, kFinished>, smem, &smem_set);
+    const uint32_t stretches = (A.d + kStretch - 1) / kStretch;
+    int lg = 0;
+    while (lg < 2 && ((uint64_t)A.n << (lg + 1)) <= (uint64_t)ps->sm_count * 2 && (2u << lg) <= stretches) ++lg;
+    cudaLaunchConfig_t cfg = {};
+    cfg.blockDim = dim3(256);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 1u << lg;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    int clusters = ps->cfg.device < 64 ? fit[ps->cfg.device][lg].load(std::memory_order_relaxed) : 0;
+    if (clusters == 0) {
+        cfg.gridDim = dim3(1u << lg);
+        cfg.numAttrs = 1;
+        if (cudaOccupancyMaxActiveClusters(&clusters, kge_wide_kernel<kMaxNeg, kFinished>, &cfg) != cudaSuccess || clusters < 1)
+            clusters = tmax(1, ps->sm_count * 2 >> lg);
+        if (ps->cfg.device < 64) fit[ps->cfg.device][lg].store(clusters, std::memory_order_relaxed);
+    }
+    const uint32_t grid = (uint32_t)tmin<uint64_t>(A.n, (uint64_t)clusters) << lg;
+    cfg.gridDim = dim3(grid);
+    cfg.numAttrs = A.keys_out ? 2 : 1;                          // (the pdl form: kernels of small calls)
+    if (ps->prof) prof_before(ps, "kge_wide_kernel", s);
+    cudaLaunchKernelEx(&cfg, kge_wide_kernel<kMaxNeg, kFinished>, A);
+    if (ps->prof) prof_after(ps, s);
+    ps->launches++;
+    return grid;
 }
 
 }  // namespace
@@ -893,8 +989,8 @@ uint32_t launch_points_kge(ps_store* ps, const KgeBatch& B, const uint8_t* singl
         return grid;                                                                                             \
     } while (0)
     if (B.dim > 128) {
-        if (B.n_neg <= 4) KGE_LAUNCH("kge_wide_kernel", kge_wide_kernel<4>, 256, (size_t)2 * 7 * 4 * kStretchPad * sizeof(float), 1, 2);
-        if (B.n_neg <= 10) KGE_LAUNCH("kge_wide_kernel", kge_wide_kernel<10>, 256, (size_t)2 * 13 * 4 * kStretchPad * sizeof(float), 1, 2);
+        if (B.n_neg <= 4) return finished ? launch_wide<4, true>(ps, A, s) : launch_wide<4, false>(ps, A, s);
+        if (B.n_neg <= 10) return finished ? launch_wide<10, true>(ps, A, s) : launch_wide<10, false>(ps, A, s);
         KGE_LAUNCH("kge_points_kernel", kge_points_kernel<29>, 256, 0, 1, 2);
     }
     const size_t smem = (size_t)kShortWarps * (3 + B.n_neg) * ((2 * B.dim + 3) & ~3u) * sizeof(float);

@@ -476,8 +476,28 @@ __device__ __forceinline__ void prefetch_row(const void* row, uint32_t bytes) {
     asm volatile("prefetch.global.L2 [%0];" ::"l"(p + bytes - 16));         // (rows need not start on a line)
 }
 
-// ---- bulk asynchronous copies global -> shared, reporting to a barrier word in shared memory ----
 __device__ __forceinline__ unsigned smem_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+
+// ---- thread-block clusters: the hardware barrier (all threads of all blocks), addresses in another block's shared memory ----
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory"); }
+__device__ __forceinline__ uint32_t peer_smem(const void* p, uint32_t rank) {
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(r) : "r"(smem_addr(p)), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ int peer_i32(const int* p, uint32_t rank) {
+    int v;
+    asm volatile("ld.shared::cluster.s32 %0, [%1];\n" : "=r"(v) : "r"(peer_smem(p, rank)) : "memory");
+    return v;
+}
+__device__ __forceinline__ double peer_f64(const double* p, uint32_t rank) {
+    double v;
+    asm volatile("ld.shared::cluster.f64 %0, [%1];\n" : "=d"(v) : "r"(peer_smem(p, rank)) : "memory");
+    return v;
+}
+
+// ---- bulk asynchronous copies global -> shared, reporting to a barrier word in shared memory ----
 __device__ __forceinline__ void mbar_init(uint64_t* bar, unsigned count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_addr(bar)), "r"(count) : "memory");
 }

@@ -455,14 +455,6 @@ struct ClusterSmem {
     uint32_t sm[8];
 };
 
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory"); }
-__device__ __forceinline__ uint32_t peer_smem(const void* p, uint32_t rank) {
-    uint32_t r;
-    asm("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(r) : "r"(smem_addr(p)), "r"(rank));
-    return r;
-}
-
 template <class Src, class Sink>
 __global__ void __launch_bounds__(kClThreads, 2)
 sort_cluster_kernel(Src src, Sink sink, SortParams P) {

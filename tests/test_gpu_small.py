@@ -75,6 +75,14 @@ def test_small_complex_steps(n, dim, n_neg):
     assert float(g.loss.cpu()[0]) == before
 
 
+@pytest.mark.parametrize("n,dim,n_neg", [(1, 129, 2), (74, 256, 4), (75, 257, 10), (148, 515, 3), (149, 512, 10), (33, 1028, 9),
+                                         (700, 514, 10)])
+def test_wide_complex_steps(n, dim, n_neg):
+    """Clusters of four, two and one block per data point, stretches that do and do not divide among them and among the
+    jobs of a pass, rows whose parts start off a 16-byte boundary; the last one with a sort and rows updated in place."""
+    test_small_complex_steps(n, dim, n_neg)
+
+
 @pytest.mark.parametrize("N,L,counts", [(8, 128, (1, 7, 600, 2047, 2048, 2049)), (1500, 4, (5, 700, 2048, 2500, 4000)),
                                         (3, 256, (2048, 1, 2049, 1025))])
 def test_localize_around_the_limit_of_the_single_launch(N, L, counts):
