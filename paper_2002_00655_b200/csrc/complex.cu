@@ -362,247 +362,7 @@ __global__ void __launch_bounds__(32 * kShortWarps, kMaxNeg <= 10 ? 4 : 2) kge_s
     }
 }
 
-// Rows of more than 128 complex dimensions and more than ten negatives: a block of eight warps per data point, whose rows
-// are then read within a short time, so that the second pass over them finds them in L2.  kMaxNeg bounds n_neg at compile
-// time so that a data point's values live in registers: for every block of 32 dimensions the Re and Im of all its rows are
-// requested together, before any is used.
-template <int kMaxNeg>
-__global__ void __launch_bounds__(256, 1) kge_points_kernel(const KgeArgs A) {
-    constexpr int kW = 8, kGroups = 1;
-    constexpr bool kAcc = true;
-    __shared__ double s_part[kW > 1 ? kW : 1][kMaxNeg + 1];
-    __shared__ double s_w[kGroups][3][32];                      // per slot: coefficient of negative q; weights of the two directions
-    __shared__ double s_loss[8];
-    const unsigned full = 0xffffffffu;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int group = w / kW, wg = w % kW;
-    const uint32_t d = A.d, n_neg = A.n_neg;
-    const int n_slots = 3 + (int)n_neg;
-    const uint64_t L = 4 * (uint64_t)d, K = A.K;
-    pdl_trigger();
-    pdl_wait();
-    if (A.single && call_failed(A.st, A.epoch)) return;
-    double loss = 0;
-    for (uint64_t t = (uint64_t)blockIdx.x * kGroups + group; t < A.n; t += (uint64_t)gridDim.x * kGroups) {
-        // ---- keys, validity, rows, first slot with the same key (lane u holds slot u) ----
-        uint64_t key = K;
-        int side = 0;
-        bool bad = false;
-        const bool slot = lane < n_slots;
-        if (slot) {
-            if (lane == 1) {
-                key = A.rel_base + A.tr[t];
-                bad = key >= K;
-            } else {
-                const uint32_t e = lane == 0 ? A.ts[t] : (lane == 2 ? A.to[t] : A.neg_ent[t * n_neg + (lane - 3)]);
-                key = e;
-                bad = e >= A.rel_base;
-                if (lane >= 3) side = A.neg_side[t * n_neg + (lane - 3)] != 0;
-            }
-        }
-        if (__any_sync(full, bad)) {                            // (the same decision in every warp of the data point)
-            if (lane == 0 && wg == 0) latch_error(A.st, A.keys_out ? 0u : A.epoch, PS_ERR_KEY_RANGE);
-            if (A.keys_out && slot && wg == 0) A.keys_out[t * n_slots + lane] = kSentinelPad;
-            continue;
-        }
-        const unsigned same = __match_any_sync(full, slot ? (uint32_t)key : kSentinelPad);
-        const int rep = slot ? __ffs(same) - 1 : lane;
-        if (A.keys_out && slot && wg == 0) A.keys_out[t * n_slots + lane] = rep == lane ? (uint32_t)key : (uint32_t)K;
-        const bool once = slot && A.single && rep == lane && A.single[t * n_slots + lane];
-        uint64_t off = 0;
-        if (slot) off = phys_row(A.table[key], A.S) * L;
-        float* const Srow = A.store + __shfl_sync(full, off, 0);
-        float* const Rrow = A.store + __shfl_sync(full, off, 1);
-        float* const Orow = A.store + __shfl_sync(full, off, 2);
-        float* Nrow[kMaxNeg];
-#pragma unroll
-        for (int q = 0; q < kMaxNeg; ++q) Nrow[q] = A.store + __shfl_sync(full, off, (3 + q) & 31);
-        // bit q: negative q stands in the subject's place; bit u: slot u is the first with its key / its key occurs once
-        const unsigned subj_mask = __ballot_sync(full, lane >= 3 && slot && side == 0) >> 3;
-        const unsigned rep_mask = __ballot_sync(full, slot && rep == lane), once_mask = __ballot_sync(full, once);
-        const unsigned acc_mask = !kAcc ? 0u : A.finished ? rep_mask : once_mask;       // slots whose accumulators are needed here
-
-        // ---- pass A: partial scores of the 1 + n_neg triples over this lane's dimensions ----
-        double part[kMaxNeg + 1];
-#pragma unroll
-        for (int q = 0; q <= kMaxNeg; ++q) part[q] = 0.0;
-        for (uint32_t c = wg * 32 + lane; c < d; c += 32 * kW) {
-            const float a_f = Srow[c], b_f = Srow[d + c], cr_f = Rrow[c], ci_f = Rrow[d + c];
-            const float e_f = Orow[c], f_f = Orow[d + c];
-            float na_f[kMaxNeg], nb_f[kMaxNeg];
-#pragma unroll
-            for (int q = 0; q < kMaxNeg; ++q) {
-                na_f[q] = q < (int)n_neg ? Nrow[q][c] : 0.f;
-                nb_f[q] = q < (int)n_neg ? Nrow[q][d + c] : 0.f;
-            }
-            const double a = a_f, b = b_f, cr = cr_f, ci = ci_f, e = e_f, f = f_f;
-            part[0] += cr * (a * e + b * f) + ci * (a * f - b * e);
-            // (n, r, o): cr (na e + nb f) + ci (na f - nb e);   (s, r, n): cr (a na + b nb) + ci (a nb - b na)
-            const double re_o = cr * e + ci * f, im_o = cr * f - ci * e;        // multiplies (na, nb) for side 0
-            const double re_s = cr * a - ci * b, im_s = cr * b + ci * a;        // multiplies (na, nb) for side 1
-#pragma unroll
-            for (int q = 0; q < kMaxNeg; ++q) {
-                const double na = na_f[q], nb = nb_f[q];
-                part[q + 1] += ((subj_mask >> q) & 1u) ? (na * re_o + nb * im_o) : (na * re_s + nb * im_s);
-            }
-        }
-        // the sums over the lanes, all triples' chains interleaved; lane q keeps triple q's score
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-            for (int q = 0; q <= kMaxNeg; ++q) part[q] += __shfl_xor_sync(full, part[q], o);
-        double phi_mine = 0;
-        if (kW > 1) {
-            __syncthreads();                                    // (the data point before has been read)
-            if (lane == 0)
-#pragma unroll
-                for (int q = 0; q <= kMaxNeg; ++q) s_part[wg][q] = part[q];
-            __syncthreads();
-            if (lane <= kMaxNeg)
-                for (int i = 0; i < kW; ++i) phi_mine += s_part[i][lane];
-        } else {
-#pragma unroll
-            for (int q = 0; q <= kMaxNeg; ++q)
-                if (lane == q) phi_mine = part[q];
-        }
-        // lane q: loss term and d loss / d phi of triple q (label +1 for the positive, -1 for negatives)
-        double coef = 0, loss_q = 0;
-        if (lane <= (int)n_neg) {
-            const double y = lane == 0 ? 1.0 : -1.0, z = -y * phi_mine, ez = exp(-fabs(z));
-            loss_q = fmax(z, 0.0) + log1p(ez);
-            coef = -y * ((z >= 0.0 ? 1.0 : ez) / (1.0 + ez));
-        }
-        loss_q = warp_sum_d(loss_q);
-        if (wg == 0) loss += loss_q;
-
-        // ---- weights with which each entity slot receives the two "negative role" directions ----
-        // A negative with side 0 stands in the subject's place: its gradient is coef * dphi/dS(r, o).
-        // With side 1 it stands in the object's place: coef * dphi/dO(s, r).  Summed over the
-        // negatives whose key's first slot is this lane.
-        double wS = 0, wO = 0;
-#pragma unroll
-        for (int q = 0; q < kMaxNeg; ++q) {
-            const int rq = __shfl_sync(full, rep, (3 + q) & 31);
-            const double cfq = __shfl_sync(full, coef, (q + 1) & 31);
-            if (q < (int)n_neg && rq == lane) {
-                if ((subj_mask >> q) & 1u) wS += cfq; else wO += cfq;
-            }
-        }
-        const double cf0 = __shfl_sync(full, coef, 0);
-        const int rep_o = __shfl_sync(full, rep, 2);            // 0 if object == subject
-        // (read back as broadcasts; the warps of a data point write the same values)
-        if (lane >= 1 && lane <= (int)n_neg) s_w[group][0][lane - 1] = coef;
-        s_w[group][1][lane] = wS;
-        s_w[group][2][lane] = wO;
-        __syncwarp();
-        const double* const cf = s_w[group][0];
-        const double* const ws = s_w[group][1];
-        const double* const wo = s_w[group][2];
-
-        // ---- pass B: gradients per block of 32 complex dimensions ----
-        const uint32_t LU = kAcc && A.finished ? 4 * d : 2 * d; // values per update row
-        float* const U = A.upd + t * n_slots * (uint64_t)LU;
-        auto out = [&](int u, float* row, uint32_t c, double gd_re, double gd_im, float x_re, float x_im, float G_re, float G_im) {
-            const float g[2] = {(float)gd_re, (float)gd_im};
-            if (!kAcc || !((acc_mask >> u) & 1u)) {
-                U[(uint64_t)u * LU + c] = g[0];
-                U[(uint64_t)u * LU + d + c] = g[1];
-                return;
-            }
-            const float g2[2] = {g[0] * g[0], g[1] * g[1]}, x[2] = {G_re + g2[0], G_im + g2[1]};
-            float step[2];
-            adagrad_steps<2>(g, x, A.lr, A.eps, step);
-            if ((once_mask >> u) & 1u) {
-                row[c] = x_re + step[0];
-                row[d + c] = x_im + step[1];
-                row[2 * d + c] = x[0];
-                row[3 * d + c] = x[1];
-            } else {
-                float* o = U + (uint64_t)u * LU;
-                o[c] = step[0];
-                o[d + c] = step[1];
-                o[2 * d + c] = g2[0];
-                o[3 * d + c] = g2[1];
-            }
-        };
-        for (uint32_t c = wg * 32 + lane; c < d; c += 32 * kW) {
-            // every value this block of dimensions needs, requested before the first use
-            const float a_f = Srow[c], b_f = Srow[d + c], cr_f = Rrow[c], ci_f = Rrow[d + c];
-            const float e_f = Orow[c], f_f = Orow[d + c];
-            float na_f[kMaxNeg], nb_f[kMaxNeg];
-#pragma unroll
-            for (int q = 0; q < kMaxNeg; ++q) {
-                const bool live = q < (int)n_neg;
-                na_f[q] = live ? Nrow[q][c] : 0.f;
-                nb_f[q] = live ? Nrow[q][d + c] : 0.f;
-            }
-            float G_re[3] = {0.f, 0.f, 0.f}, G_im[3] = {0.f, 0.f, 0.f};
-            if (kAcc && (acc_mask & 1u)) { G_re[0] = Srow[2 * d + c]; G_im[0] = Srow[3 * d + c]; }
-            if (kAcc && (acc_mask & 2u)) { G_re[1] = Rrow[2 * d + c]; G_im[1] = Rrow[3 * d + c]; }
-            if (kAcc && (acc_mask & 4u)) { G_re[2] = Orow[2 * d + c]; G_im[2] = Orow[3 * d + c]; }
-            const double a = a_f, b = b_f, cr = cr_f, ci = ci_f, e = e_f, f = f_f;
-            // directions that do not depend on the negative
-            const double dS_re = cr * e + ci * f, dS_im = cr * f - ci * e;      // d phi / d subject, object = o
-            const double dO_re = cr * a - ci * b, dO_im = cr * b + ci * a;      // d phi / d object, subject = s
-            // The negatives enter the gradients of subject, relation and object only through their weighted sums:
-            // (A0, B0) over those in the subject's place (triples (n, r, o)), (A1, B1) over those in the object's
-            // place (triples (s, r, n)).
-            double A0 = 0.0, B0 = 0.0, A1 = 0.0, B1 = 0.0;
-#pragma unroll
-            for (int q = 0; q < kMaxNeg; ++q) {
-                if (q >= (int)n_neg) break;
-                const double na = na_f[q], nb = nb_f[q], wq = cf[q];
-                if ((subj_mask >> q) & 1u) { A0 += wq * na; B0 += wq * nb; }
-                else { A1 += wq * na; B1 += wq * nb; }
-            }
-            double gs_re = cf0 * dS_re, gs_im = cf0 * dS_im;
-            double go_re = cf0 * dO_re, go_im = cf0 * dO_im;
-            double gr_re = cf0 * (a * e + b * f), gr_im = cf0 * (a * f - b * e);
-            gr_re += (A0 * e + B0 * f) + (a * A1 + b * B1); gr_im += (A0 * f - B0 * e) + (a * B1 - b * A1);
-            go_re += cr * A0 - ci * B0; go_im += cr * B0 + ci * A0;
-            gs_re += cr * A1 + ci * B1; gs_im += cr * B1 - ci * A1;
-            // negatives that coincide with the subject or the object
-            gs_re += ws[0] * dS_re + wo[0] * dO_re; gs_im += ws[0] * dS_im + wo[0] * dO_im;
-            go_re += ws[2] * dS_re + wo[2] * dO_re; go_im += ws[2] * dS_im + wo[2] * dO_im;
-            if (rep_o == 0) { gs_re += go_re; gs_im += go_im; }
-            out(0, Srow, c, gs_re, gs_im, a_f, b_f, G_re[0], G_im[0]);
-            out(1, Rrow, c, gr_re, gr_im, cr_f, ci_f, G_re[1], G_im[1]);
-            if (rep_o == 2) out(2, Orow, c, go_re, go_im, e_f, f_f, G_re[2], G_im[2]);
-            constexpr int kB = kMaxNeg < 5 ? kMaxNeg : 5;       // accumulators of so many negatives asked for together
-#pragma unroll
-            for (int q0 = 0; q0 < kMaxNeg; q0 += kB) {
-                float Gq_re[kB], Gq_im[kB];
-#pragma unroll
-                for (int i = 0; i < kB; ++i) {
-                    const int q = q0 + i;
-                    Gq_re[i] = Gq_im[i] = 0.f;
-                    if (kAcc && q < kMaxNeg && ((acc_mask >> (3 + q)) & 1u)) {
-                        Gq_re[i] = Nrow[q][2 * d + c];
-                        Gq_im[i] = Nrow[q][3 * d + c];
-                    }
-                }
-#pragma unroll
-                for (int i = 0; i < kB; ++i) {
-                    const int q = q0 + i;
-                    if (q >= kMaxNeg || !((rep_mask >> (3 + q)) & 1u)) continue;
-                    const double wSq = ws[3 + q], wOq = wo[3 + q];
-                    out(3 + q, Nrow[q], c, wSq * dS_re + wOq * dO_re, wSq * dS_im + wOq * dO_im, na_f[q], nb_f[q], Gq_re[i], Gq_im[i]);
-                }
-            }
-        }
-        __syncwarp();
-    }
-    // per-block loss partial, fixed order
-    if (lane == 0) s_loss[w] = loss;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double tot = 0;
-        for (int i = 0; i < 8; ++i) tot += s_loss[i];
-        A.loss_partial[blockIdx.x] = tot;
-    }
-}
-
-// Rows of more than 128 complex dimensions and up to ten negatives: a block per data point (batches of few data points: a
+// Rows of more than 128 complex dimensions: a block per data point (batches of few data points: a
 // cluster of up to four, which meets to add up the scores), the rows streamed through shared memory in stretches of 256
 // dimensions as bulk copies, what the next job needs on its way while one is worked on, across the two passes and across
 // data points.  (With loads into registers, one stretch after the other, the memory system was idle three quarters of the
@@ -613,14 +373,30 @@ __global__ void __launch_bounds__(256, 1) kge_points_kernel(const KgeArgs A) {
 // job, gained nothing; asking L2 for the rows two jobs earlier cost 200 us.  A stretch of a part (Re, Im, G_Re or G_Im) of a
 // row starts at a multiple of 16 bytes only if d is a multiple of four: the copy starts at the boundary before it, and
 // `shift` floats are skipped.
-constexpr uint32_t kStretch = 256, kStretchPad = kStretch + 4;
+//
+// kGroups = 2 (more than ten negatives): a stretch is 128 dimensions, and the block's halves share the negatives, so that a
+// thread's score sums stay in registers and two blocks' stages fit an SM (up to 20 negatives).  The first half, which also
+// has the subject, the relation and the object, gets fewer of them; the second hands it its weighted sums.  1,000 data points
+// of 400 dimensions with 20 negatives: 287 us with a block per data point and loads into registers at 8 warps per SM, now 146.
+template <int kMaxNeg>
+struct Wide {
+    static constexpr int kGroups = kMaxNeg > 10 ? 2 : 1, kSlots = 3 + kMaxNeg;
+    static constexpr uint32_t kStretch = 256 / kGroups, kPad = kStretch + 4;
+    static constexpr int kFirst = kGroups == 1 ? kMaxNeg : (kMaxNeg - 2) / 2;          // negatives of the first half
+    static constexpr int kMine = kGroups == 1 ? kMaxNeg : kMaxNeg - kFirst;            // of either, at most
+    static constexpr size_t kSmem = (size_t)2 * kSlots * 4 * kPad * sizeof(float);     // [2 stages][slot][part][kPad]
+    static constexpr int kPerSm = kMaxNeg > 20 ? 1 : 2;
+};
 
 template <int kMaxNeg, bool kFinished>
-__global__ void __launch_bounds__(256, 2) kge_wide_kernel(const KgeArgs A) {
-    constexpr int kSlots = 3 + kMaxNeg, kWarps = 8;
-    extern __shared__ __align__(128) float stage_mem[];         // [2 stages][slot][part][kStretchPad]
+__global__ void __launch_bounds__(256, Wide<kMaxNeg>::kPerSm) kge_wide_kernel(const KgeArgs A) {
+    constexpr int kGroups = Wide<kMaxNeg>::kGroups, kSlots = Wide<kMaxNeg>::kSlots, kMine = Wide<kMaxNeg>::kMine;
+    constexpr uint32_t kStretch = Wide<kMaxNeg>::kStretch, kStretchPad = Wide<kMaxNeg>::kPad;
+    constexpr int kWarps = 8, kGroupWarps = kWarps / kGroups;
+    extern __shared__ __align__(128) float stage_mem[];
     __shared__ __align__(8) uint64_t bars[2];
-    __shared__ double s_part[kWarps][kMaxNeg + 1];
+    __shared__ double s_part[kWarps][kMine + 1];
+    __shared__ double s_sum[4][kGroups == 1 ? 1 : kStretch];        // the second half's weighted sums
     __shared__ double s_tot[2][kMaxNeg + 1];                    // the block's share of the scores, by the data point's parity
     __shared__ int s_failed;
     __shared__ double s_w[3][32];
@@ -628,6 +404,9 @@ __global__ void __launch_bounds__(256, 2) kge_wide_kernel(const KgeArgs A) {
     const unsigned full = 0xffffffffu;
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const uint32_t d = A.d, n_neg = A.n_neg;
+    const int group = kGroups == 1 ? 0 : w / kGroupWarps, q0 = group ? Wide<kMaxNeg>::kFirst : 0;
+    const int n_mine = group ? tmax(0, (int)n_neg - q0) : tmin((int)n_neg, Wide<kMaxNeg>::kFirst);
+    const uint32_t gtid = tid % kStretch;                       // the thread's dimension in a stretch
     const int n_slots = 3 + (int)n_neg;
     const bool slot = lane < n_slots;
     const uint64_t L = 4 * (uint64_t)d, K = A.K;
@@ -736,9 +515,9 @@ __global__ void __launch_bounds__(256, 2) kge_wide_kernel(const KgeArgs A) {
     while (t < A.n) {
         const uint64_t tn = next_valid(t + stride, N);
         const unsigned subj_mask = P.subj, rep_mask = P.reps, acc_mask = kFinished ? P.reps : P.once;
-        double part[kMaxNeg + 1];
+        double part[kMine + 1];                                 // scores of the triple (first half) and of the thread's negatives
 #pragma unroll
-        for (int q = 0; q <= kMaxNeg; ++q) part[q] = 0.0;
+        for (int q = 0; q <= kMine; ++q) part[q] = 0.0;
         double cf0 = 0;
         int rep_o = 2;
         const uint32_t LU = kFinished ? 4 * d : 2 * d;         // values per update row
@@ -753,89 +532,122 @@ __global__ void __launch_bounds__(256, 2) kge_wide_kernel(const KgeArgs A) {
             }
             if (!mbar_wait(&bars[stage], (uses >> stage) & 1u) && !mbar_wait(&bars[stage], (uses >> stage) & 1u)) dead = true;
             uses ^= 1u << stage;
-            const float* base = stage_mem + (size_t)stage * kSlots * 4 * kStretchPad + tid;
+            const float* base = stage_mem + (size_t)stage * kSlots * 4 * kStretchPad + gtid;
             const uint32_t sh1 = d & 3, sh2 = (2 * d) & 3, sh3 = (3 * d) & 3;
             auto re = [&](int u) { return base[u * 4 * kStretchPad]; };
             auto im = [&](int u) { return base[(u * 4 + 1) * kStretchPad + sh1]; };
             auto gre = [&](int u) { return base[(u * 4 + 2) * kStretchPad + sh2]; };
             auto gim = [&](int u) { return base[(u * 4 + 3) * kStretchPad + sh3]; };
-            uint32_t c = (str * C + rank) * kStretch + tid;
-            for (int half = 0; half < (pass_b ? 1 : 2) && c < d; ++half, c += C * kStretch, base += 2 * kStretchPad) {
+            uint32_t c = (str * C + rank) * kStretch + gtid;
+            // the values of the triple's rows in dimension c, and the directions that do not depend on the negative:
+            // d phi / d subject (object = o), d phi / d object (subject = s)
+            struct Triple {
+                double a, b, cr, ci, e, f, dS_re, dS_im, dO_re, dO_im;
+            };
+            auto triple = [&]() {
+                Triple T;
                 const float a_f = re(0), b_f = im(0), cr_f = re(1), ci_f = im(1), e_f = re(2), f_f = im(2);
-                const double a = a_f, b = b_f, cr = cr_f, ci = ci_f, e = e_f, f = f_f;
-                // directions that do not depend on the negative: d phi / d subject (object = o), d phi / d object (subject = s)
-                const double dS_re = cr * e + ci * f, dS_im = cr * f - ci * e;
-                const double dO_re = cr * a - ci * b, dO_im = cr * b + ci * a;
-                if (!pass_b) {
-                    part[0] += cr * (a * e + b * f) + ci * (a * f - b * e);
+                T.a = a_f; T.b = b_f; T.cr = cr_f; T.ci = ci_f; T.e = e_f; T.f = f_f;
+                T.dS_re = T.cr * T.e + T.ci * T.f; T.dS_im = T.cr * T.f - T.ci * T.e;
+                T.dO_re = T.cr * T.a - T.ci * T.b; T.dO_im = T.cr * T.b + T.ci * T.a;
+                return T;
+            };
+            if (!pass_b) {
+                for (int half = 0; half < 2 && c < d; ++half, c += C * kStretch, base += 2 * kStretchPad) {
+                    const Triple T = triple();
+                    if (group == 0) part[0] += T.cr * (T.a * T.e + T.b * T.f) + T.ci * (T.a * T.f - T.b * T.e);
 #pragma unroll
-                    for (int q = 0; q < kMaxNeg; ++q) {
-                        if (q >= (int)n_neg) break;
+                    for (int i = 0; i < kMine; ++i) {
+                        if (i >= n_mine) break;
+                        const int q = q0 + i;
                         const double na = re(3 + q), nb = im(3 + q);
-                        part[q + 1] += ((subj_mask >> q) & 1u) ? (na * dS_re + nb * dS_im) : (na * dO_re + nb * dO_im);
+                        part[i + 1] += ((subj_mask >> q) & 1u) ? (na * T.dS_re + nb * T.dS_im) : (na * T.dO_re + nb * T.dO_im);
                     }
-                } else {
-                    const double *cf = s_w[0], *ws = s_w[1], *wo = s_w[2];
-                    double A0 = 0.0, B0 = 0.0, A1 = 0.0, B1 = 0.0;      // weighted sums of the negatives in either place
+                }
+            } else {
+                const double *cf = s_w[0], *ws = s_w[1], *wo = s_w[2];
+                auto out = [&](int u, double gd_re, double gd_im) {
+                    const float g[2] = {(float)gd_re, (float)gd_im};
+                    float* o = U + (uint64_t)u * LU + c;
+                    if (!((acc_mask >> u) & 1u)) {
+                        o[0] = g[0];
+                        o[d] = g[1];
+                        return;
+                    }
+                    const float g2[2] = {g[0] * g[0], g[1] * g[1]}, x[2] = {gre(u) + g2[0], gim(u) + g2[1]};
+                    float step[2];
+                    adagrad_steps<2>(g, x, A.lr, A.eps, step);
+                    if (!kFinished) o = A.store + s_off[u] + c;     // in place
+                    o[0] = kFinished ? step[0] : re(u) + step[0];
+                    o[d] = kFinished ? step[1] : im(u) + step[1];
+                    o[2 * d] = kFinished ? g2[0] : x[0];
+                    o[3 * d] = kFinished ? g2[1] : x[1];
+                };
+                double A0 = 0.0, B0 = 0.0, A1 = 0.0, B1 = 0.0;      // weighted sums of the negatives in either place
+                // subject, relation and object
+                auto triple_out = [&](const Triple& T) {
+                    double gs_re = cf0 * T.dS_re, gs_im = cf0 * T.dS_im;
+                    double go_re = cf0 * T.dO_re, go_im = cf0 * T.dO_im;
+                    double gr_re = cf0 * (T.a * T.e + T.b * T.f), gr_im = cf0 * (T.a * T.f - T.b * T.e);
+                    gr_re += (A0 * T.e + B0 * T.f) + (T.a * A1 + T.b * B1); gr_im += (A0 * T.f - B0 * T.e) + (T.a * B1 - T.b * A1);
+                    go_re += T.cr * A0 - T.ci * B0; go_im += T.cr * B0 + T.ci * A0;
+                    gs_re += T.cr * A1 + T.ci * B1; gs_im += T.cr * B1 - T.ci * A1;
+                    // negatives that coincide with the subject or the object
+                    gs_re += ws[0] * T.dS_re + wo[0] * T.dO_re; gs_im += ws[0] * T.dS_im + wo[0] * T.dO_im;
+                    go_re += ws[2] * T.dS_re + wo[2] * T.dO_re; go_im += ws[2] * T.dS_im + wo[2] * T.dO_im;
+                    if (rep_o == 0) { gs_re += go_re; gs_im += go_im; }
+                    out(0, gs_re, gs_im);
+                    out(1, gr_re, gr_im);
+                    if (rep_o == 2) out(2, go_re, go_im);
+                };
+                if (c < d) {
+                    const Triple T = triple();
 #pragma unroll
-                    for (int q = 0; q < kMaxNeg; ++q) {
-                        if (q >= (int)n_neg) break;
+                    for (int i = 0; i < kMine; ++i) {
+                        if (i >= n_mine) break;
+                        const int q = q0 + i;
                         const double na = re(3 + q), nb = im(3 + q), wq = cf[q];
                         if ((subj_mask >> q) & 1u) { A0 += wq * na; B0 += wq * nb; }
                         else { A1 += wq * na; B1 += wq * nb; }
                     }
-                    double gs_re = cf0 * dS_re, gs_im = cf0 * dS_im;
-                    double go_re = cf0 * dO_re, go_im = cf0 * dO_im;
-                    double gr_re = cf0 * (a * e + b * f), gr_im = cf0 * (a * f - b * e);
-                    gr_re += (A0 * e + B0 * f) + (a * A1 + b * B1); gr_im += (A0 * f - B0 * e) + (a * B1 - b * A1);
-                    go_re += cr * A0 - ci * B0; go_im += cr * B0 + ci * A0;
-                    gs_re += cr * A1 + ci * B1; gs_im += cr * B1 - ci * A1;
-                    // negatives that coincide with the subject or the object
-                    gs_re += ws[0] * dS_re + wo[0] * dO_re; gs_im += ws[0] * dS_im + wo[0] * dO_im;
-                    go_re += ws[2] * dS_re + wo[2] * dO_re; go_im += ws[2] * dS_im + wo[2] * dO_im;
-                    if (rep_o == 0) { gs_re += go_re; gs_im += go_im; }
-                    auto out = [&](int u, double gd_re, double gd_im) {
-                        const float g[2] = {(float)gd_re, (float)gd_im};
-                        float* o = U + (uint64_t)u * LU + c;
-                        if (!((acc_mask >> u) & 1u)) {
-                            o[0] = g[0];
-                            o[d] = g[1];
-                            return;
-                        }
-                        const float g2[2] = {g[0] * g[0], g[1] * g[1]}, x[2] = {gre(u) + g2[0], gim(u) + g2[1]};
-                        float step[2];
-                        adagrad_steps<2>(g, x, A.lr, A.eps, step);
-                        if (!kFinished) o = A.store + s_off[u] + c;     // in place
-                        o[0] = kFinished ? step[0] : re(u) + step[0];
-                        o[d] = kFinished ? step[1] : im(u) + step[1];
-                        o[2 * d] = kFinished ? g2[0] : x[0];
-                        o[3 * d] = kFinished ? g2[1] : x[1];
-                    };
-                    out(0, gs_re, gs_im);
-                    out(1, gr_re, gr_im);
-                    if (rep_o == 2) out(2, go_re, go_im);
+                    if (kGroups == 1) {
+                        triple_out(T);
+                    } else if (group == 1) {
+                        s_sum[0][gtid] = A0; s_sum[1][gtid] = B0; s_sum[2][gtid] = A1; s_sum[3][gtid] = B1;
+                    }
 #pragma unroll
-                    for (int q = 0; q < kMaxNeg; ++q) {
-                        if (q >= (int)n_neg) break;
+                    for (int i = 0; i < kMine; ++i) {
+                        if (i >= n_mine) break;
+                        const int q = q0 + i;
                         if (!((rep_mask >> (3 + q)) & 1u)) continue;
                         const double wSq = ws[3 + q], wOq = wo[3 + q];
-                        out(3 + q, wSq * dS_re + wOq * dO_re, wSq * dS_im + wOq * dO_im);
+                        out(3 + q, wSq * T.dS_re + wOq * T.dO_re, wSq * T.dS_im + wOq * T.dO_im);
+                    }
+                }
+                if (kGroups > 1) {
+                    __syncthreads();
+                    if (group == 0 && c < d) {
+                        A0 += s_sum[0][gtid]; B0 += s_sum[1][gtid]; A1 += s_sum[2][gtid]; B1 += s_sum[3][gtid];
+                        triple_out(triple());
                     }
                 }
             }
             stage ^= 1;
-            if (job + 1 == n_first) {           // the scores are complete: coefficients and weights, as in kge_points_kernel
+            if (job + 1 == n_first) {           // the scores are complete: coefficients and weights
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
-                    for (int q = 0; q <= kMaxNeg; ++q) part[q] += __shfl_xor_sync(full, part[q], o);
+                    for (int q = 0; q <= kMine; ++q) part[q] += __shfl_xor_sync(full, part[q], o);
                 if (lane == 0)
 #pragma unroll
-                    for (int q = 0; q <= kMaxNeg; ++q) s_part[w][q] = part[q];
+                    for (int q = 0; q <= kMine; ++q) s_part[w][q] = part[q];
                 __syncthreads();
-                double phi = 0, coef = 0, loss_q = 0;
-                if (lane <= kMaxNeg)
-                    for (int i = 0; i < kWarps; ++i) phi += s_part[i][lane];
+                double phi = 0, coef = 0, loss_q = 0;           // lane q + 1: negative q; lane 0: the triple
+                if (lane <= kMaxNeg) {
+                    const bool later = lane > Wide<kMaxNeg>::kFirst;
+                    const int from = later ? kWarps - kGroupWarps : 0, at = later ? lane - Wide<kMaxNeg>::kFirst : lane;
+                    for (int i = 0; i < kGroupWarps; ++i) phi += s_part[from + i][at];
+                }
                 if (C > 1) {                    // the blocks' shares, in rank order
                     if (w == 0 && lane <= kMaxNeg) s_tot[parity][lane] = phi;
                     cluster_arrive();
@@ -926,13 +738,14 @@ kge_keys_kernel(const uint32_t* __restrict__ ts, const uint32_t* __restrict__ tr
 // fewer reads save (2,048 data points: 747 us with one block, 791 with two, 950 with four).
 template <int kMaxNeg, bool kFinished>
 uint32_t launch_wide(ps_store* ps, const KgeArgs& A, cudaStream_t s) {
-    const size_t smem = (size_t)2 * (3 + kMaxNeg) * 4 * kStretchPad * sizeof(float);
+    const size_t smem = Wide<kMaxNeg>::kSmem;
+    const uint32_t places = (uint32_t)ps->sm_count * Wide<kMaxNeg>::kPerSm;
     static std::atomic<unsigned long long> smem_set{0};
     static std::atomic<int> fit[64][3];                         // clusters resident at once, by device and size (0: not asked yet)
     opt_in_smem((const void*)kge_wide_kernel<kMaxNeg, kFinished>, smem, &smem_set);
-    const uint32_t stretches = (A.d + kStretch - 1) / kStretch;
+    const uint32_t stretches = (A.d + Wide<kMaxNeg>::kStretch - 1) / Wide<kMaxNeg>::kStretch;
     int lg = 0;
-    while (lg < 2 && ((uint64_t)A.n << (lg + 1)) <= (uint64_t)ps->sm_count * 2 && (2u << lg) <= stretches) ++lg;
+    while (lg < 2 && ((uint64_t)A.n << (lg + 1)) <= places && (2u << lg) <= stretches) ++lg;
     cudaLaunchConfig_t cfg = {};
     cfg.blockDim = dim3(256);
     cfg.dynamicSmemBytes = smem;
@@ -949,7 +762,7 @@ uint32_t launch_wide(ps_store* ps, const KgeArgs& A, cudaStream_t s) {
         cfg.gridDim = dim3(1u << lg);
         cfg.numAttrs = 1;
         if (cudaOccupancyMaxActiveClusters(&clusters, kge_wide_kernel<kMaxNeg, kFinished>, &cfg) != cudaSuccess || clusters < 1)
-            clusters = tmax(1, ps->sm_count * 2 >> lg);
+            clusters = tmax(1, (int)(places >> lg));
         if (ps->cfg.device < 64) fit[ps->cfg.device][lg].store(clusters, std::memory_order_relaxed);
     }
     const uint32_t grid = (uint32_t)tmin<uint64_t>(A.n, (uint64_t)clusters) << lg;
@@ -989,9 +802,12 @@ uint32_t launch_points_kge(ps_store* ps, const KgeBatch& B, const uint8_t* singl
         return grid;                                                                                             \
     } while (0)
     if (B.dim > 128) {
-        if (B.n_neg <= 4) return finished ? launch_wide<4, true>(ps, A, s) : launch_wide<4, false>(ps, A, s);
-        if (B.n_neg <= 10) return finished ? launch_wide<10, true>(ps, A, s) : launch_wide<10, false>(ps, A, s);
-        KGE_LAUNCH("kge_points_kernel", kge_points_kernel<29>, 256, 0, 1, 2);
+#define KGE_WIDE(kMaxNeg) return finished ? launch_wide<kMaxNeg, true>(ps, A, s) : launch_wide<kMaxNeg, false>(ps, A, s)
+        if (B.n_neg <= 4) KGE_WIDE(4);
+        if (B.n_neg <= 10) KGE_WIDE(10);
+        if (B.n_neg <= 20) KGE_WIDE(20);
+        KGE_WIDE(29);
+#undef KGE_WIDE
     }
     const size_t smem = (size_t)kShortWarps * (3 + B.n_neg) * ((2 * B.dim + 3) & ~3u) * sizeof(float);
     const uint32_t fit = tmax<uint32_t>(1u, (uint32_t)((220 * 1024) / (smem + 4096)));
