@@ -619,7 +619,8 @@ ps_status_t ps_step_kge(ps_store_t* ps, const uint32_t* d_s, const uint32_t* d_r
     if (!in_place) lb = launch_points_kge(ps, B, nullptr, false, nullptr, s);
     if (!end_sort(ps, s, q)) return PS_ERR_CUDA;
     if (in_place) lb = launch_points_kge(ps, B, seg_lists(ps).single, false, nullptr, s);
-    run_segment_adagrad(ps, occ, which, 2 * dim_complex, !in_place, lr, eps, ps->loss_partial, d_loss_accum ? lb : 0, d_loss_accum, s);
+    run_segment_adagrad(ps, occ, which, 2 * dim_complex, !in_place, lr, eps, ps->carry, ps->loss_partial, d_loss_accum ? lb : 0,
+                        d_loss_accum, s);
     return release_set(ss, s);
 }
 
@@ -652,8 +653,7 @@ ps_status_t ps_step_rescal(ps_store_t* ps, const uint32_t* d_s, const uint32_t* 
     const int which = run_segment_sort(ps, occ, q);
     launch_segments(ps, occ, which, dim, rel_key_base, q);
     if (!end_sort(ps, s, q)) return PS_ERR_CUDA;
-    const double* loss_terms = run_rescal_sorted(ps, B, which, s);
-    run_segment_adagrad(ps, occ, which, dim, false, lr, eps, loss_terms, n_loss, d_loss_accum, s);
+    run_rescal_sorted(ps, B, which, n_loss, d_loss_accum, s);
     return release_set(ss, s);
 }
 

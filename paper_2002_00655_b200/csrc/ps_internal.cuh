@@ -288,9 +288,10 @@ const uint8_t* launch_singles(ps_store* ps, uint32_t n, int which, cudaStream_t 
 // after the sort, on its stream; keys from rel_key_base on are RESCAL's relations (num_keys: none)
 void launch_segments(ps_store* ps, uint32_t n, int which, uint32_t half_row, uint64_t rel_key_base, cudaStream_t s);
 // gradient rows (half_row values per occurrence, in ps->upd) -> AdaGrad, of the keys that occur several times and, with
-// singles, of those that occur once; loss terms
+// singles, of those that occur once; loss terms.  parked: room for the long segments' partial sums.  beside: the kernel before
+// it on the stream has triggered it, is still running, and touches none of what this one does
 void run_segment_adagrad(ps_store* ps, uint32_t n, int which, uint32_t half_row, bool singles, float lr, float eps,
-                         const double* loss_terms, uint32_t n_loss, double* d_loss_accum, cudaStream_t s);
+                         double* parked, const double* loss_terms, uint32_t n_loss, double* d_loss_accum, cudaStream_t s, bool beside = false);
 
 // ---- complex.cu ----
 struct KgeBatch {
@@ -321,7 +322,7 @@ void launch_keys_rescal(ps_store* ps, const RescalBatch& B, cudaStream_t s);    
 // Return where the data points' loss terms are.  small: gradient rows and keys of all 2 + n_neg + dim slots; sorted:
 // matrices and keys that occur once are updated, gradient rows of the other entity slots written.
 const double* run_rescal_small(ps_store* ps, const RescalBatch& B, uint32_t* keys_out, cudaStream_t s);
-const double* run_rescal_sorted(ps_store* ps, const RescalBatch& B, int which, cudaStream_t s);
+void run_rescal_sorted(ps_store* ps, const RescalBatch& B, int which, uint32_t n_loss, double* d_loss_accum, cudaStream_t s);
 
 // ---- localize.cu ----
 // busy_keys: sorted keys of a call that may run beside this relocation (null: none); moving keys among them keep

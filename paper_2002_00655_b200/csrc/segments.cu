@@ -159,6 +159,11 @@ segment_adagrad_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restri
     constexpr int kN = Vec<V>::kN, kWarps = 8;
     constexpr int kFly = 4;                     // gradient rows a warp has in flight
     __shared__ double s_part[kWarps][32 * kN];
+    // Beside RESCAL's matrix kernel (launched while that one's last blocks run, on other rows): what follows on the stream has
+    // to come after both.  Elsewhere nothing is waited for.
+    struct AtExit {
+        __device__ ~AtExit() { pdl_wait(); }
+    } at_exit;
     if (call_failed(st, epoch)) return;
     const unsigned full = 0xffffffffu;
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
@@ -387,21 +392,21 @@ segment_adagrad_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restri
 }
 
 void run_segment_adagrad(ps_store* ps, uint32_t n, int which, uint32_t half_row, bool singles, float lr, float eps,
-                         const double* loss_terms, uint32_t n_loss, double* d_loss_accum, cudaStream_t s) {
+                         double* parked, const double* loss_terms, uint32_t n_loss, double* d_loss_accum, cudaStream_t s, bool beside) {
     const uint32_t* sk = which ? ps->keysB : ps->keysA;
     const uint32_t* sv = which ? ps->valsB : ps->valsA;
     const SegLists L = seg_lists(ps);
     if (!n_loss) d_loss_accum = nullptr;
+#define SEG_ARGS(V) sk, sv, (const V*)ps->upd, (V*)ps->store, (const uint2*)ps->table, ps->cfg.slots_per_part, (uint32_t)ps->cfg.num_keys, \
+                 singles ? n : 0u, GV, lr, eps, L, parked, loss_terms, n_loss, d_loss_accum, (const DevStatus*)ps->status, ps->epoch
 #define SEG_LAUNCH(V, kCh)                                                                                              \
     do {                                                                                                                \
         const uint32_t GV = half_row / Vec<V>::kN, strips = seg_strips(half_row);                                       \
         /* as many blocks as are resident over all stretches of columns; the warps loop over the lists */               \
         const uint32_t gx = tmax<uint32_t>(1u, tmin<uint32_t>(div_up_u32(n, 32), (uint32_t)ps->sm_count * 2 / strips)); \
         if (ps->prof) prof_before(ps, "segment_adagrad_kernel", s);                                                     \
-        segment_adagrad_kernel<V, kCh><<<dim3(gx + 1, strips), 256, 0, s>>>(                                            \
-            sk, sv, (const V*)ps->upd, (V*)ps->store, ps->table, ps->cfg.slots_per_part, (uint32_t)ps->cfg.num_keys,   \
-            singles ? n : 0u, GV, lr, eps, L, ps->carry,                                                                \
-            loss_terms, n_loss, d_loss_accum, ps->status, ps->epoch);                                                               \
+        if (beside) launch_pdl(segment_adagrad_kernel<V, kCh>, dim3(gx + 1, strips), dim3(256), 0, s, SEG_ARGS(V));     \
+        else segment_adagrad_kernel<V, kCh><<<dim3(gx + 1, strips), 256, 0, s>>>(SEG_ARGS(V));                           \
         if (ps->prof) prof_after(ps, s);                                                                                \
         ps->launches++;                                                                                                 \
     } while (0)
@@ -413,6 +418,7 @@ void run_segment_adagrad(ps_store* ps, uint32_t n, int which, uint32_t half_row,
         else SEG_LAUNCH(float2, 2);
     }
 #undef SEG_LAUNCH
+#undef SEG_ARGS
 }
 
 }  // namespace psb
