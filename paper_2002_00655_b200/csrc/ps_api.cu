@@ -26,8 +26,10 @@ WsLayout ws_layout(const ps_config_t& cfg, uint64_t max_keys) {
     const size_t sort_tiles = (mk + kSortTile / 2 - 1) / (kSortTile / 2);   // the sort's blocks, at its shortest tile
     // tiles of the reduction: 32 positions, or 8 for the matrix-factorization step on rows of at most 128 values
     const size_t tile_len = cfg.row_len <= 128 ? 8 : kReduceTile;
-    const size_t reduce_tiles = (mk + tile_len - 1) / tile_len;
-    const size_t groups = (mk + tile_len * 64 - 1) / (tile_len * 64);
+    size_t reduce_tiles = (mk + tile_len - 1) / tile_len;
+    if (cfg.row_len <= kTiledRow) reduce_tiles = tmax(reduce_tiles, tmin<size_t>((mk + 7) / 8, kMidTiles));
+    l.reduce_tiles = reduce_tiles;
+    const size_t groups = (reduce_tiles + 63) / 64;
     const size_t row_bytes = (size_t)cfg.row_len * 4;
     l.status = take(sizeof(DevStatus));
     for (int b = 0; b < kSortSets; ++b) {
@@ -301,6 +303,7 @@ ps_status_t ps_create(const ps_config_t* cfg, void* d_store, void* d_table, void
     ps->upd = (float*)(ps->ws + l.upd);
     ps->carry = (double*)(ps->ws + l.carry);
     ps->group_sum = (double*)(ps->ws + l.group_sum);
+    ps->tile_cap = (uint32_t)tmin<size_t>(l.reduce_tiles, 0xffffffffu);
     ps->loss_partial = (double*)(ps->ws + l.loss_partial);
     ps->apply_rows = (uint64_t*)(ps->ws + l.apply_rows);
     for (int b = 0; b < kHostStages; ++b) ps->stagings[b] = ps->ws + l.staging[b];
@@ -452,7 +455,7 @@ ps_status_t ps_push(ps_store_t* ps, const uint64_t* d_keys, uint64_t n, const fl
     SortSet* ss = next_set(ps);
     cudaStream_t q;
     if (!begin_sort(ps, ss, s, false, &q)) return PS_ERR_CUDA;  // pipelined: the keys are sorted beside earlier calls' kernels
-    const int which = radix_sort_keys64(ps, d_keys, (uint32_t)n, q, ps->starter_count, div_up_u32(n, kGroupSpan));
+    const int which = radix_sort_keys64(ps, d_keys, (uint32_t)n, q, ps->starter_count, reduce_groups(ps, (uint32_t)n));
     if (!sorted_keys_at(ps, ss, which, (uint32_t)n, q) || !end_sort(ps, s, q)) return PS_ERR_CUDA;
     run_push_reduce(ps, (uint32_t)n, which, d_updates, nullptr, 0, s);
     return release_set(ss, s);
@@ -563,7 +566,7 @@ ps_status_t ps_step_mf(ps_store_t* ps, const uint32_t* d_i, const uint32_t* d_j,
     cudaStream_t q = ps->side;                      // (rows of more than 128 values: the sort runs beside the gradient kernel)
     if (fused ? !begin_sort(ps, ss, s, true, &q) : !fork_side(ps, ss, s, true)) return PS_ERR_CUDA;
     const int which = radix_sort_mf(ps, d_i, d_j, d_v, (uint32_t)n, col_key_base, fused, q, ps->starter_count,
-                                    div_up_u32(2 * n, fused ? 64 * 8 : kGroupSpan));
+                                    fused ? div_up_u32(2 * n, 64 * 8) : reduce_groups(ps, (uint32_t)(2 * n)));
     if (!sorted_keys_at(ps, ss, which, (uint32_t)(2 * n), q)) return PS_ERR_CUDA;
     if (by_column) {
         launch_mf_plan(ps, (uint32_t)n, which, q);

@@ -17,8 +17,9 @@ constexpr int kRadixBits = 8;
 constexpr int kRadix = 1 << kRadixBits;
 constexpr int kMaxSortPasses = 4;                // 32-bit keys
 constexpr int kSortCtlWords = kMaxSortPasses * kRadix + kMaxSortPasses;   // digit histograms of every pass, then tickets
-constexpr int kReduceTile = 32;                  // sorted occurrences per warp in the segmented reduction
-constexpr int kGroupSpan = 64 * kReduceTile;      // sorted positions whose parked parts are pre-added together
+constexpr int kReduceTile = 32;                  // sorted occurrences per warp in the segmented reduction of long rows
+constexpr uint32_t kTiledRow = 512;              // ... rows up to this many values: 8 to 128 (reduce_tile)
+constexpr uint32_t kMidTiles = 4096;             // shorter tiles than 32 positions that a call has at most
 constexpr int kMaxLossBlocks = 4096;
 constexpr uint32_t kSmallOcc = 8192;             // calls of at most this many key occurrences are reduced without a sort (small.cu)
 constexpr int kHostStages = 3;                   // staging areas for batches that arrive from host memory
@@ -99,6 +100,7 @@ struct ps_store {
     double* carry;                  // nReduceTiles x 2 x row_len partial sums of segments that span tiles
     uint4* starters;                // {tile, key, row} of the tiles that start a border-crossing segment
     unsigned int* starter_count;
+    uint32_t tile_cap;              // tiles that carry and starters have room for
     double* loss_partial;           // max(kMaxLossBlocks, one per 256 key occurrences)
     uint64_t* apply_rows;           // per sorted position: address of the row staged there, or all ones
     char* staging;                  // host-batch staging, max_keys x 8 bytes (the first of `stagings`)
@@ -141,7 +143,7 @@ namespace psb {
 struct WsLayout {
     size_t status, keysA[kSortSets], keysB[kSortSets], valsA[kSortSets], valsB[kSortSets], tile_state[kSortSets],
         sort_ctl[kSortSets], rec[kSortSets], cellpos[kSortSets], mf_dup[kSortSets], mf_tickets[kSortSets], scan_sums, loc_counts, loc_scratch, upd, carry, group_sum, starters[kSortSets], starter_count[kSortSets],
-        loss_partial, apply_rows, staging[kHostStages], total;
+        loss_partial, apply_rows, staging[kHostStages], total, reduce_tiles;
 };
 WsLayout ws_layout(const ps_config_t& cfg, uint64_t max_keys);
 
@@ -224,6 +226,8 @@ int radix_sort_mf(ps_store* ps, const uint32_t* d_i, const uint32_t* d_j, const 
                   uint32_t zero_groups);
 
 // ---- pull_push.cu ----
+uint32_t reduce_tile(const ps_store* ps, uint32_t n, bool scaled);      // positions per tile of a push of n occurrences
+uint32_t reduce_groups(const ps_store* ps, uint32_t n);                 // groups of 64 tiles, at most
 void launch_init_range_partition(ps_store* ps, cudaStream_t s);
 void launch_set_rows(ps_store* ps, const uint64_t* d_keys, uint64_t n, const float* d_vals, cudaStream_t s);
 void launch_pull(ps_store* ps, const uint64_t* d_keys, uint64_t n, float* d_out, cudaStream_t s);

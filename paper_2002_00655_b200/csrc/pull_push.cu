@@ -274,7 +274,6 @@ __host__ __device__ constexpr size_t reduce_smem(int kCh) {
 }
 static_assert(reduce_smem(1) >= 8 * 32 * 32 && reduce_smem(4) <= 64 * 1024, "staging also serves as the pre-add scratch");
 constexpr int kFixupWarps = 8;
-constexpr int kGroupMinSpan = 8 * kReduceTile;   // a group's entering segment is pre-added only if at least this long
 constexpr int kGroupTiles = 64;     // tiles whose parked parts are pre-added per group (8 reduction blocks)
 
 // Tail of the reduction kernel, kept out of line so that it does not weigh on the main loop's registers.
@@ -327,7 +326,7 @@ __device__ __noinline__ void group_preadd(const uint32_t* __restrict__ sk, uint3
     }
 }
 
-// A warp owns sorted positions [tile*32, tile*32+32).  A segment (run of equal
+// A warp owns the tile_len sorted positions of one tile, 32 at most.  A segment (run of equal
 // keys) that starts and ends inside the tile is summed in fp64 and applied with
 // one read-modify-write of its row; a segment that continues from the previous
 // tile parks its partial sum in carry slot 0 of the tile, one that continues
@@ -347,49 +346,52 @@ push_reduce_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restrict__
                    uint64_t S, uint32_t K, uint32_t L4_arg, double* __restrict__ carry,
                    uint4* __restrict__ starters, unsigned int* __restrict__ starter_count,
                    unsigned int* __restrict__ group_done, double* __restrict__ group_sum,
-                   DevStatus* st, unsigned int epoch) {
+                   uint32_t tile_len, DevStatus* st, unsigned int epoch) {
     __shared__ unsigned int s_ticket;
     __shared__ __align__(8) uint64_t bars[8][3];    // per warp and stage: the barrier word its copies report to
     const uint32_t L4 = kL4 ? (uint32_t)kL4 : L4_arg;
     if (call_failed(st, epoch)) return;
     const unsigned full = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
+    const uint32_t lane = threadIdx.x & 31;
     const uint32_t tile = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const uint64_t base = (uint64_t)tile * kReduceTile;
-    const uint32_t n_valid = base < n ? (uint32_t)tmin<uint64_t>((uint64_t)kReduceTile, n - base) : 0u;
+    const uint64_t base = (uint64_t)tile * tile_len;
+    const bool at_end = lane == tile_len - 1;                   // the tile's last position
+    const uint32_t n_valid = base < n ? (uint32_t)tmin<uint64_t>(tile_len, n - base) : 0u;
     const uint32_t key = lane < n_valid ? sk[base + lane] : kSentinelPad;
     const uint32_t occ = lane < n_valid ? sv[base + lane] : 0u;
     uint32_t prev = __shfl_up_sync(full, key, 1);
     if (lane == 0) prev = (base > 0 && base - 1 < n) ? sk[base - 1] : kSentinelPad;
-    const uint32_t next_after = (base + kReduceTile < n) ? sk[base + kReduceTile] : kSentinelPad;
+    const uint32_t next_after = (base + tile_len < n) ? sk[base + tile_len] : kSentinelPad;
     uint32_t next = __shfl_down_sync(full, key, 1);
-    if (lane == 31) next = next_after;
+    if (lane == tile_len - 1) next = next_after;
     const bool usable = key < K;                    // "no key" marks and padding sort last
     uint64_t row = 0;
     if (usable) row = phys_row(table[key], S);
-    const unsigned head_mask = __ballot_sync(full, key != prev);
+    const unsigned head_mask = __ballot_sync(full, lane < n_valid && key != prev);
     const unsigned usable_mask = __ballot_sync(full, usable);
     // positions at which a segment's part in this tile ends: its true end, or the tile's last position
-    const unsigned end_mask = __ballot_sync(full, usable && (key != next || lane == 31));
+    const unsigned end_mask = __ballot_sync(full, usable && (key != next || at_end));
     // positions before the first head belong to a segment that came in from the previous tile
-    const int first_head = head_mask ? (__ffs(head_mask) - 1) : 32;
-    // the last segment runs on iff the position after the tile holds the same usable key
-    const uint32_t key31 = __shfl_sync(full, key, 31);
-    const bool runs_on = key31 < K && next_after == key31;
-    // a border-crossing segment starts in this tile iff it runs on and has its head here
-    if (runs_on && head_mask != 0u && lane == 31)
+    const uint32_t first_head = head_mask ? (uint32_t)(__ffs(head_mask) - 1) : 32u;
+    // the last segment runs on iff the position after the tile holds the same usable key; a border-crossing segment
+    // starts in this tile iff it runs on and has its head here
+    const bool runs_on = at_end && usable && next_after == key;
+    if (runs_on && head_mask)
         starters[atomicAdd(starter_count, 1u)] = make_uint4(tile, key, (uint32_t)row, (uint32_t)(row >> 32));
+    // positions whose target row is fetched: a segment ends there and is neither parked on the way in nor out
+    const bool fetch_me = ((end_mask >> lane) & 1u) && !(lane < first_head || runs_on);
+    const unsigned fetch_mask = __ballot_sync(full, fetch_me);
     // does a segment enter this block's group of 64 tiles from the group before?  (asked here, with the
     // walk's loads still to come, and needed only after the walk)
     const uint32_t group = blockIdx.x / (kGroupTiles / 8);
-    const uint64_t gpos = (uint64_t)group * kGroupTiles * kReduceTile;     // first sorted position of the group
-    // Only a segment that also covers the group's first kGroupMinSpan positions is worth it: shorter ones
+    const uint64_t gpos = (uint64_t)group * kGroupTiles * tile_len;     // first sorted position of the group
+    // Only a segment that also covers the group's first eight tiles is worth it: shorter ones
     // end within a few tiles and the fix-up kernel takes those tile by tile.
     uint32_t kg = kSentinelPad, kg_prev = kSentinelPad - 1, kg_far = kSentinelPad - 2;
-    if (gpos > 0 && gpos + kGroupMinSpan - 1 < n) {
+    if (gpos > 0 && gpos + 8 * tile_len - 1 < n) {
         kg = sk[gpos];
         kg_prev = sk[gpos - 1];
-        kg_far = sk[gpos + kGroupMinSpan - 1];
+        kg_far = sk[gpos + 8 * tile_len - 1];
     }
     const uint32_t L = L4 * 4;
     // Rows are staged through shared memory with bulk asynchronous copies: for a group of G positions the
@@ -404,13 +406,10 @@ push_reduce_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restrict__
     if (lane < ST) mbar_init(&bars[w][lane], 1);
     mbar_init_fence();
     __syncwarp();
-    const int n_groups = ((int)n_valid + G - 1) / G;
-    // positions whose target row is fetched: a segment ends there and is neither parked on the way in nor out
-    const bool fetch_me = usable && (key != next || lane == 31) && !(lane < first_head || (lane == 31 && runs_on));
-    const unsigned fetch_mask = __ballot_sync(full, fetch_me);
     const unsigned gmask0 = G == 32 ? full : ((1u << G) - 1u);
     uint32_t uses = 0;                                          // how often the warp has waited so far, per stage: parity
     bool dead = false;
+    const int n_groups = ((int)n_valid + G - 1) / G;
     for (uint32_t f0 = 0; f0 < L4 && !dead; f0 += 32 * kCh) {   // one round unless a row is longer than 128 kCh floats
         const uint32_t chunk4 = tmin<uint32_t>(L4 - f0, 32u * kCh);
         const uint32_t chunk_bytes = chunk4 * 16u;
@@ -420,10 +419,10 @@ push_reduce_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restrict__
             const unsigned gm = gmask0 << (g * G);
             const uint32_t n_rows = __popc(usable_mask & gm) + __popc(fetch_mask & gm);
             if (n_rows == 0) return;                            // nothing to wait for either: see the walk
-            if (lane == g * G) mbar_expect_tx(&bars[w][stage], n_rows * chunk_bytes);
+            if ((int)lane == g * G) mbar_expect_tx(&bars[w][stage], n_rows * chunk_bytes);
             __syncwarp();
             if ((gm >> lane) & 1u) {
-                float4* dst = my_stage + (size_t)stage * kSlotF4 + (size_t)(lane - g * G) * (2 * kCh * 32);
+                float4* dst = my_stage + (size_t)stage * kSlotF4 + (size_t)((int)lane - g * G) * (2 * kCh * 32);
                 if (usable) bulk_g2s(dst, upd + (uint64_t)occ * L4 + f0, chunk_bytes, &bars[w][stage]);
                 if (fetch_me) bulk_g2s(dst + kCh * 32, store + row * L4 + f0, chunk_bytes, &bars[w][stage]);
             }
@@ -477,8 +476,8 @@ push_reduce_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restrict__
                 }
                 if (!((end_mask >> p) & 1u)) continue;
                 const uint64_t rw = __shfl_sync(full, row, p);
-                const bool from_prev = p < first_head;
-                const bool parked = from_prev || (p == 31 && runs_on);
+                const bool from_prev = (uint32_t)p < first_head;
+                const bool parked = !((fetch_mask >> p) & 1u);
 #pragma unroll
                 for (int c = 0; c < kCh; ++c) {
                     const uint32_t f = fl + 32 * c;
@@ -503,7 +502,7 @@ push_reduce_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restrict__
     if (!(kg < K && kg_prev == kg && kg_far == kg)) return;     // nothing to pre-add for this group
     // the staging memory is free by now (every warp has waited for all its copies) and serves as scratch
     group_preadd(sk, n, L4, carry, group_done, group_sum, group, gpos, kg, reinterpret_cast<d4 (*)[32]>(stage_mem),
-                 &s_ticket, kReduceTile, tmin<uint32_t>(kGroupTiles / 8, gridDim.x - group * (kGroupTiles / 8)));
+                 &s_ticket, tile_len, tmin<uint32_t>(kGroupTiles / 8, gridDim.x - group * (kGroupTiles / 8)));
 }
 
 // The reduction of occurrences that are a factor times a shared source row (skip-gram: rows of at most 512 values), with
@@ -521,7 +520,7 @@ push_reduce_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restrict__
 template <int kCh, int kL4, int kSlots>
 __global__ void __launch_bounds__(256, kCh == 3 || kCh == 1 ? 3 : 2)
 scaled_reduce_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restrict__ sv, uint32_t n,
-                     const float4* __restrict__ upd, const float* __restrict__ scales, uint32_t slots_arg, bool skip_singles,
+                     const float4* __restrict__ upd, const float* __restrict__ scales, uint32_t slots_arg, uint32_t tile_len, bool skip_singles,
                      float4* __restrict__ store, const uint2* __restrict__ table, uint64_t S, uint32_t K, uint32_t L4_arg,
                      double* __restrict__ carry, uint4* __restrict__ starters, unsigned int* __restrict__ starter_count,
                      unsigned int* __restrict__ group_done, double* __restrict__ group_sum, DevStatus* st, unsigned int epoch) {
@@ -531,49 +530,16 @@ scaled_reduce_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restrict
     const uint32_t slots = kSlots ? (uint32_t)kSlots : slots_arg;
     if (call_failed(st, epoch)) return;
     const unsigned full = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
+    const uint32_t lane = threadIdx.x & 31;
     const uint32_t tile = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const uint64_t base = (uint64_t)tile * kReduceTile;
-    const uint32_t n_valid = base < n ? (uint32_t)tmin<uint64_t>((uint64_t)kReduceTile, n - base) : 0u;
-    const uint32_t key = lane < n_valid ? sk[base + lane] : kSentinelPad;
-    uint32_t occ = lane < n_valid ? sv[base + lane] : 0u;
-    uint32_t prev = __shfl_up_sync(full, key, 1);
-    if (lane == 0) prev = (base > 0 && base - 1 < n) ? sk[base - 1] : kSentinelPad;
-    const uint32_t next_after = (base + kReduceTile < n) ? sk[base + kReduceTile] : kSentinelPad;
-    uint32_t next = __shfl_down_sync(full, key, 1);
-    if (lane == 31) next = next_after;
-    // "no key" marks and padding sort last
-    const bool usable = key < K && !(skip_singles && key != prev && key != next);
-    float scale = 0.f;
-    if (usable) {
-        scale = scales[occ];
-        const uint32_t e = occ / slots;
-        occ = 2u * e + (occ != e * slots ? 1u : 0u);
-    } else {
-        occ = 0;
-    }
-    uint64_t row = 0;
-    if (usable) row = phys_row(table[key], S);
-    const unsigned head_mask = __ballot_sync(full, key != prev);
-    const unsigned usable_mask = __ballot_sync(full, usable);
-    // positions at which a segment's part in this tile ends: its true end, or the tile's last position
-    const unsigned end_mask = __ballot_sync(full, usable && (key != next || lane == 31));
-    const int first_head = head_mask ? (__ffs(head_mask) - 1) : 32;
-    const uint32_t key31 = __shfl_sync(full, key, 31);
-    const bool runs_on = key31 < K && next_after == key31;
-    if (runs_on && head_mask != 0u && lane == 31)
-        starters[atomicAdd(starter_count, 1u)] = make_uint4(tile, key, (uint32_t)row, (uint32_t)(row >> 32));
-    // positions whose target row is updated: a segment ends there and is neither parked on the way in nor out
-    const bool fetch_me = usable && (key != next || lane == 31) && !(lane < first_head || (lane == 31 && runs_on));
-    const unsigned fetch_mask = __ballot_sync(full, fetch_me);
-    if (fetch_me) prefetch_row(store + row * L4, L4 * 16);
+    const uint32_t span = tmin(tile_len, 32u);                  // positions at a time
     const uint32_t group = blockIdx.x / (kGroupTiles / 8);
-    const uint64_t gpos = (uint64_t)group * kGroupTiles * kReduceTile;
+    const uint64_t gpos = (uint64_t)group * kGroupTiles * tile_len;
     uint32_t kg = kSentinelPad, kg_prev = kSentinelPad - 1, kg_far = kSentinelPad - 2;
-    if (gpos > 0 && gpos + kGroupMinSpan - 1 < n) {
+    if (gpos > 0 && gpos + 8 * tile_len - 1 < n) {
         kg = sk[gpos];
         kg_prev = sk[gpos - 1];
-        kg_far = sk[gpos + kGroupMinSpan - 1];
+        kg_far = sk[gpos + 8 * tile_len - 1];
     }
     const uint32_t L = L4 * 4;
     constexpr int kG = kCh >= 3 ? 2 : 4;
@@ -585,67 +551,105 @@ scaled_reduce_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restrict
     for (int k = 0; k < kG; ++k)
 #pragma unroll
         for (int c = 0; c < kCh; ++c) u[k][c] = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (unsigned todo = usable_mask; todo;) {
-        int at[kG];
-#pragma unroll
-        for (int k = 0; k < kG; ++k) {
-            at[k] = todo ? __ffs(todo) - 1 : -1;
-            todo &= todo - 1;                                   // 0 stays 0
-            const float4* src = upd + (uint64_t)__shfl_sync(full, occ, at[k] & 31) * L4 + lane;
-#pragma unroll
-            for (int c = 0; c < kCh; ++c)
-                if (lane + 32 * c < L4) u[k][c] = __ldg(src + 32 * c);      // (past the last: some other row, not used)
+    bool entered = true;                                        // no segment has begun in this tile so far
+    for (uint32_t done = 0; done < tile_len; done += span) {
+        const uint64_t base = (uint64_t)tile * tile_len + done;
+        const bool at_end = done + span == tile_len && lane == span - 1;       // the tile's last position
+        const uint32_t n_valid = base < n ? (uint32_t)tmin<uint64_t>(span, n - base) : 0u;
+        const uint32_t key = lane < n_valid ? sk[base + lane] : kSentinelPad;
+        uint32_t occ = lane < n_valid ? sv[base + lane] : 0u;
+        uint32_t prev = __shfl_up_sync(full, key, 1);
+        if (lane == 0) prev = (base > 0 && base - 1 < n) ? sk[base - 1] : kSentinelPad;
+        const uint32_t next_after = (base + span < n) ? sk[base + span] : kSentinelPad;
+        uint32_t next = __shfl_down_sync(full, key, 1);
+        if (lane == span - 1) next = next_after;
+        // "no key" marks and padding sort last
+        const bool usable = key < K && !(skip_singles && key != prev && key != next);
+        float scale = 0.f;
+        if (usable) {
+            scale = scales[occ];
+            const uint32_t e = occ / slots;
+            occ = 2u * e + (occ != e * slots ? 1u : 0u);
+        } else {
+            occ = 0;
         }
+        uint64_t row = 0;
+        if (usable) row = phys_row(table[key], S);
+        const unsigned head_mask = __ballot_sync(full, lane < n_valid && key != prev);
+        const unsigned usable_mask = __ballot_sync(full, usable);
+        // positions at which a segment's part in this tile ends: its true end, or the tile's last position
+        const unsigned end_mask = __ballot_sync(full, usable && (key != next || at_end));
+        const uint32_t first_head = !entered ? 0 : head_mask ? (uint32_t)(__ffs(head_mask) - 1) : 32u;     // before it: parts of a segment that entered
+        if (head_mask) entered = false;
+        const bool runs_on = at_end && usable && next_after == key;
+        if (runs_on && !entered)
+            starters[atomicAdd(starter_count, 1u)] = make_uint4(tile, key, (uint32_t)row, (uint32_t)(row >> 32));
+        // positions whose target row is updated: a segment ends there and is neither parked on the way in nor out
+        const bool fetch_me = ((end_mask >> lane) & 1u) && !(lane < first_head || runs_on);
+        const unsigned fetch_mask = __ballot_sync(full, fetch_me);
+        if (fetch_me) prefetch_row(store + row * L4, L4 * 16);
+        for (unsigned todo = usable_mask; todo;) {
+            int at[kG];
 #pragma unroll
-        for (int k = 0; k < kG; ++k) {
-            const int p = at[k];
-            if (p < 0) break;
-            const float sc = __shfl_sync(full, scale, p);
-            const bool ends = (end_mask >> p) & 1u, whole = (fetch_mask >> p) & 1u;
-            if (whole && ((head_mask >> p) & 1u)) {             // one occurrence: a multiply-add rounds the exact sum once
-                float4* to = store + __shfl_sync(full, row, p) * L4 + lane;
+            for (int k = 0; k < kG; ++k) {
+                at[k] = todo ? __ffs(todo) - 1 : -1;
+                todo &= todo - 1;                                   // 0 stays 0
+                const float4* src = upd + (uint64_t)__shfl_sync(full, occ, at[k] & 31) * L4 + lane;
 #pragma unroll
-                for (int c = 0; c < kCh; ++c) {
-                    if (lane + 32 * c >= L4) continue;
-                    float4 v = to[32 * c];
-                    v.x = fmaf(sc, u[k][c].x, v.x); v.y = fmaf(sc, u[k][c].y, v.y);
-                    v.z = fmaf(sc, u[k][c].z, v.z); v.w = fmaf(sc, u[k][c].w, v.w);
-                    to[32 * c] = v;
-                }
-                continue;
-            }
-            const double d = (double)sc;
-#pragma unroll
-            for (int c = 0; c < kCh; ++c) {
-                acc[c].x += d * (double)u[k][c].x; acc[c].y += d * (double)u[k][c].y;
-                acc[c].z += d * (double)u[k][c].z; acc[c].w += d * (double)u[k][c].w;
-            }
-            if (!ends) continue;
-            if (whole) {
-                float4* to = store + __shfl_sync(full, row, p) * L4 + lane;
-#pragma unroll
-                for (int c = 0; c < kCh; ++c) {
-                    if (lane + 32 * c >= L4) continue;
-                    float4 v = to[32 * c];
-                    v.x = (float)((double)v.x + acc[c].x); v.y = (float)((double)v.y + acc[c].y);
-                    v.z = (float)((double)v.z + acc[c].z); v.w = (float)((double)v.w + acc[c].w);
-                    to[32 * c] = v;
-                }
-            } else {
-                double* cs = carry + ((uint64_t)tile * 2 + (p < first_head ? 0 : 1)) * L + (uint64_t)lane * 4;
-#pragma unroll
-                for (int c = 0; c < kCh; ++c) {
-                    if (lane + 32 * c >= L4) continue;
-                    *(double2*)(cs + 128 * c) = make_double2(acc[c].x, acc[c].y);
-                    *(double2*)(cs + 128 * c + 2) = make_double2(acc[c].z, acc[c].w);
-                }
+                for (int c = 0; c < kCh; ++c)
+                    if (lane + 32 * c < L4) u[k][c] = __ldg(src + 32 * c);      // (past the last: some other row, not used)
             }
 #pragma unroll
-            for (int c = 0; c < kCh; ++c) acc[c] = d4{0.0, 0.0, 0.0, 0.0};
+            for (int k = 0; k < kG; ++k) {
+                const int p = at[k];
+                if (p < 0) break;
+                const float sc = __shfl_sync(full, scale, p);
+                const bool ends = (end_mask >> p) & 1u, whole = (fetch_mask >> p) & 1u;
+                if (whole && ((head_mask >> p) & 1u)) {             // one occurrence: a multiply-add rounds the exact sum once
+                    float4* to = store + __shfl_sync(full, row, p) * L4 + lane;
+#pragma unroll
+                    for (int c = 0; c < kCh; ++c) {
+                        if (lane + 32 * c >= L4) continue;
+                        float4 v = to[32 * c];
+                        v.x = fmaf(sc, u[k][c].x, v.x); v.y = fmaf(sc, u[k][c].y, v.y);
+                        v.z = fmaf(sc, u[k][c].z, v.z); v.w = fmaf(sc, u[k][c].w, v.w);
+                        to[32 * c] = v;
+                    }
+                    continue;
+                }
+                const double d = (double)sc;
+#pragma unroll
+                for (int c = 0; c < kCh; ++c) {
+                    acc[c].x += d * (double)u[k][c].x; acc[c].y += d * (double)u[k][c].y;
+                    acc[c].z += d * (double)u[k][c].z; acc[c].w += d * (double)u[k][c].w;
+                }
+                if (!ends) continue;
+                if (whole) {
+                    float4* to = store + __shfl_sync(full, row, p) * L4 + lane;
+#pragma unroll
+                    for (int c = 0; c < kCh; ++c) {
+                        if (lane + 32 * c >= L4) continue;
+                        float4 v = to[32 * c];
+                        v.x = (float)((double)v.x + acc[c].x); v.y = (float)((double)v.y + acc[c].y);
+                        v.z = (float)((double)v.z + acc[c].z); v.w = (float)((double)v.w + acc[c].w);
+                        to[32 * c] = v;
+                    }
+                } else {
+                    double* cs = carry + ((uint64_t)tile * 2 + ((uint32_t)p < first_head ? 0 : 1)) * L + (uint64_t)lane * 4;
+#pragma unroll
+                    for (int c = 0; c < kCh; ++c) {
+                        if (lane + 32 * c >= L4) continue;
+                        *(double2*)(cs + 128 * c) = make_double2(acc[c].x, acc[c].y);
+                        *(double2*)(cs + 128 * c + 2) = make_double2(acc[c].z, acc[c].w);
+                    }
+                }
+#pragma unroll
+                for (int c = 0; c < kCh; ++c) acc[c] = d4{0.0, 0.0, 0.0, 0.0};
+            }
         }
     }
     if (!(kg < K && kg_prev == kg && kg_far == kg)) return;     // nothing to pre-add for this group
-    group_preadd(sk, n, L4, carry, group_done, group_sum, group, gpos, kg, s_pre, &s_ticket, kReduceTile,
+    group_preadd(sk, n, L4, carry, group_done, group_sum, group, gpos, kg, s_pre, &s_ticket, tile_len,
                  tmin<uint32_t>(kGroupTiles / 8, gridDim.x - group * (kGroupTiles / 8)));
 }
 
@@ -1248,8 +1252,26 @@ void run_push_atomic(ps_store* ps, const uint64_t* d_keys, uint64_t n, const flo
               ps->cfg.slots_per_part, ps->cfg.row_len / 4, ps->status, ps->epoch);
 }
 
+// Positions per warp (tile) of the segmented reductions of rows that one round of a warp holds.  Calls of fewer tiles of 32
+// than warps are resident at once (24 per SM): shorter tiles, as their time is that of one tile's chain (20,000 occurrences of 300
+// values, skip-gram: 29.4 us with 32, 18.4 with 8; 30,000 of 128 values, plain push: 19.3 and 14.7; at 100,000 of 64 values 8 would
+// be a loss, 26.5 against 24.7).  Skip-gram, calls of several rounds of warps: longer ones, as fewer segments then cross a border, each a
+// parked partial sum and an entry for the fix-up launch (1.34M occurrences of 300 values: reduction and fix-up 245 + 51 us
+// with 32, 235 + 37 with 64, 232 + 26 with 128; a plain push of 1M gains nothing, 187 + 22 against 190 + 18).
+uint32_t reduce_tile(const ps_store* ps, uint32_t n, bool scaled) {
+    if (ps->cfg.row_len > kTiledRow) return kReduceTile;
+    const uint32_t warps = (uint32_t)ps->sm_count * 24;
+    uint32_t tile = 8;
+    while (tile < kReduceTile && (n / tile > warps || div_up_u32(n, tile) > ps->tile_cap)) tile *= 2;
+    if (scaled)
+        while (tile < 128 && n / (tile * 2) >= warps * 5 / 2) tile *= 2;
+    return tile;
+}
+// (the longer tiles of skip-gram need fewer)
+uint32_t reduce_groups(const ps_store* ps, uint32_t n) { return div_up_u32(n, (uint32_t)kGroupTiles * reduce_tile(ps, n, false)); }
+
 int run_push_sort(ps_store* ps, uint32_t n, cudaStream_t s) {
-    return radix_sort_pairs(ps, n, nullptr, ps->key_bits, s, 0, ps->starter_count, div_up_u32(n, kGroupSpan));
+    return radix_sort_pairs(ps, n, nullptr, ps->key_bits, s, 0, ps->starter_count, reduce_groups(ps, n));
 }
 
 int run_segment_sort(ps_store* ps, uint32_t n, cudaStream_t s) {
@@ -1322,12 +1344,12 @@ void run_push_reduce(ps_store* ps, uint32_t n, int which, const float* d_upd, do
                      uint32_t loss_blocks, cudaStream_t s, const float* d_scales, uint32_t slots, bool skip_singles) {
     const uint32_t* sk = which ? ps->keysB : ps->keysA;
     const uint32_t* sv = which ? ps->valsB : ps->valsA;
-    const uint32_t tiles = div_up_u32(n, kReduceTile);
-    const uint32_t blocks = div_up_u32(tiles, 8);
+    const uint32_t tile_len = reduce_tile(ps, n, d_scales != nullptr);
+    const uint32_t blocks = div_up_u32(div_up_u32(n, tile_len), 8);
     const uint32_t L4 = ps->cfg.row_len / 4;
 #define REDUCE_ARGS sk, sv, n, (const float4*)d_upd, (float4*)ps->store, ps->table,                                  \
                     ps->cfg.slots_per_part, (uint32_t)ps->cfg.num_keys, L4, ps->carry, ps->starters,                \
-                    ps->starter_count, ps->group_done, ps->group_sum, ps->status, ps->epoch
+                    ps->starter_count, ps->group_done, ps->group_sum, tile_len, ps->status, ps->epoch
 #define REDUCE_LAUNCH(kCh, kL4)                                                                                      \
     do {                                                                                                             \
         static std::atomic<unsigned long long> smem_set{0};                                                          \
@@ -1342,8 +1364,8 @@ void run_push_reduce(ps_store* ps, uint32_t n, int which, const float* d_upd, do
 #define SCALED_LAUNCH(kCh, kL4, kSlots)                                                                              \
     do {                                                                                                             \
         if (ps->prof) prof_before(ps, "scaled_reduce_kernel<" #kCh ">", s);                                          \
-        scaled_reduce_kernel<kCh, kL4, kSlots><<<blocks, 256, 0, s>>>(sk, sv, n, (const float4*)d_upd, d_scales, slots, \
-            skip_singles, (float4*)ps->store, ps->table, ps->cfg.slots_per_part, (uint32_t)ps->cfg.num_keys, L4, ps->carry, \
+        scaled_reduce_kernel<kCh, kL4, kSlots><<<blocks, 256, 0, s>>>(sk, sv, n, (const float4*)d_upd, d_scales, slots,  \
+            tile_len, skip_singles, (float4*)ps->store, ps->table, ps->cfg.slots_per_part, (uint32_t)ps->cfg.num_keys, L4, ps->carry, \
             ps->starters, ps->starter_count, ps->group_done, ps->group_sum, ps->status, ps->epoch);                  \
         if (ps->prof) prof_after(ps, s);                                                                             \
         ps->launches++;                                                                                              \
@@ -1364,7 +1386,7 @@ void run_push_reduce(ps_store* ps, uint32_t n, int which, const float* d_upd, do
     }
 #undef REDUCE_LAUNCH
 #undef REDUCE_ARGS
-    launch_fixup(ps, sk, n, d_loss_accum, loss_blocks, false, kReduceTile, 0, s);
+    launch_fixup(ps, sk, n, d_loss_accum, loss_blocks, false, tile_len, 0, s);
 }
 
 void run_push_pipeline(ps_store* ps, uint32_t n, const float* d_upd, double* d_loss_accum, uint32_t loss_blocks,

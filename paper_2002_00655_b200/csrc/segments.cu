@@ -2,10 +2,9 @@
 //
 // Most keys of a batch occur once.  Such a key's row is read by one data point only, so that data point's gradient
 // kernel, which has the gradient in registers, can update the row in place; its gradient then never goes through memory.
-// RESCAL and ComplEx on rows of more than 512 values do that (the gradients of long rows do not stay in L2 between two
-// kernels); for shorter ComplEx rows it was no gain (gradient kernel 64 -> 113 us for 85 MB of gradients less, reduction
-// 73 -> 45), and single keys are a case of the reduction here.  The keys that occur several times are runs (segments) of
-// the sorted occurrences.
+// They do so but for ComplEx on rows of at most 512 values in ordered mode, where the gradient kernel runs beside the sort
+// and does not know yet which keys occur once: there single keys are a case of the reduction here.  The keys that occur
+// several times are runs (segments) of the sorted occurrences.
 //
 // segment_kernel (on the stream of the sort, right after it) looks at every sorted position and writes
 //   single[occurrence]     1 iff the occurrence's key occurs once
@@ -18,7 +17,9 @@
 namespace psb {
 
 namespace {
-constexpr uint32_t kLongRun = 24;               // occurrences from which on a block, not a warp, adds a segment
+// occurrences from which on a block, not a warp, adds a segment (106,496 key occurrences of ComplEx on Zipf(1) triples, 400
+// values: 47.4 us with 24, 44.8 with 12, 54.5 with 8)
+constexpr uint32_t kLongRun = 12;
 constexpr uint32_t kLongPiece = 96;             // ... and about as many as one block adds of it
 constexpr uint32_t kMaxStrips = 64;             // (wider rows, of 16,384 values and more, are not cut: the tickets' room)
 }  // namespace

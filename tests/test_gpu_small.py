@@ -127,3 +127,20 @@ def test_sorted_pushes_around_the_limits_of_the_sorts(n, K):
     assert torch.equal(out[0], out[1])
     o.push(keys, upd)
     compare_state(g, o, what=f"push of {n}")
+
+
+@pytest.mark.parametrize("n", [300, 1_000, 2_500, 14_500, 29_000])
+@pytest.mark.parametrize("pipelined", [False, True])
+def test_skip_gram_reduction_at_every_tile_length(n, pipelined):
+    """12,300 to 1.2M key occurrences: tiles of 8, 16, 32, 64 and 128 sorted positions, words that fill thousands of them and
+    words that occur once; a batch that ends inside a tile and, clipped windows, with "no key" marks."""
+    cfg = W.scaled(W.SGNS_TINY, vocab=20_000, n_tokens=n, dim=8, batch=n)
+    rows = torch.from_numpy(np.random.default_rng(n).normal(0, 0.1, size=(cfg.num_keys, cfg.dim)).astype(np.float32))
+    tokens, negs = W.sgns_tokens(cfg, 0, n, "cpu"), W.sgns_negatives(cfg, 0, n, "cpu")
+    g, o = make_pair(cfg.num_keys, cfg.dim, rows=rows, max_batch_keys=n * (1 + 2 * cfg.window * (1 + cfg.n_neg)))
+    ps.ps_set_pipelining(g.h, pipelined)
+    ps.ps_step_sgns(g.h, tokens.cuda(), 0, n, cfg.window, negs.cuda(), cfg.n_neg, cfg.out_key_base, cfg.lr, g.loss)
+    o.step_sgns(tokens, 0, n, cfg.window, negs, cfg.n_neg, cfg.out_key_base, cfg.lr)
+    g.sync()
+    compare_state(g, o, what=f"skip-gram, {n} centers")
+    assert close(float(g.loss.cpu()[0]), o.loss[0])
