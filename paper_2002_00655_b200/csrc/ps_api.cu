@@ -617,7 +617,7 @@ ps_status_t ps_step_kge(ps_store_t* ps, const uint32_t* d_s, const uint32_t* d_r
     launch_keys_kge(ps, B, q);
     const int which = run_segment_sort(ps, occ, q);
     if (!sorted_keys_at(ps, ss, which, occ, q)) return PS_ERR_CUDA;
-    launch_segments(ps, occ, which, 2 * dim_complex, ps->cfg.num_keys, q);
+    launch_segments(ps, occ, which, 2 * dim_complex, ps->cfg.num_keys, 0, q);
     uint32_t lb = 0;
     if (!in_place) lb = launch_points_kge(ps, B, nullptr, false, nullptr, s);
     if (!end_sort(ps, s, q)) return PS_ERR_CUDA;
@@ -654,7 +654,7 @@ ps_status_t ps_step_rescal(ps_store_t* ps, const uint32_t* d_s, const uint32_t* 
     if (!begin_sort(ps, ss, s, false, &q)) return PS_ERR_CUDA;
     launch_keys_rescal(ps, B, q);
     const int which = run_segment_sort(ps, occ, q);
-    launch_segments(ps, occ, which, dim, rel_key_base, q);
+    launch_segments(ps, occ, which, dim, rel_key_base, (uint32_t)n, q);
     if (!end_sort(ps, s, q)) return PS_ERR_CUDA;
     run_rescal_sorted(ps, B, which, n_loss, d_loss_accum, s);
     return release_set(ss, s);

@@ -275,7 +275,7 @@ void run_small_adagrad(ps_store* ps, uint32_t n, float lr, float eps, double* d_
                        cudaStream_t s, const double* loss_terms = nullptr);     // null: ps->loss_partial
 
 // ---- segments.cu ----
-constexpr uint32_t kRelPiece = 8;                // data points of one relation that a block of rescal_points_kernel takes
+constexpr uint32_t kRelPiece = 8;                // data points of one relation that a block of rescal_points_kernel takes, at most
 constexpr uint32_t kRelChunk = 64;               // ... that a block of rescal_matrix_kernel sums before parking
 constexpr uint32_t kRelTickets = 16;             // ticket words per chunk of a relation of several chunks
 struct SegLists {
@@ -289,8 +289,9 @@ struct SegLists {
 constexpr uint32_t kSegCounters = 8 + 64;        // lengths and single keys drawn (rows whose single keys are reduced have at most two stretches of columns); short segments drawn, by stretch
 SegLists seg_lists(ps_store* ps);   // of the current buffer set
 const uint8_t* launch_singles(ps_store* ps, uint32_t n, int which, cudaStream_t s);     // per occurrence: its key occurs once
-// after the sort, on its stream; keys from rel_key_base on are RESCAL's relations (num_keys: none)
-void launch_segments(ps_store* ps, uint32_t n, int which, uint32_t half_row, uint64_t rel_key_base, cudaStream_t s);
+// after the sort, on its stream; keys from rel_key_base on are RESCAL's relations (num_keys: none), of n_points data points
+void launch_segments(ps_store* ps, uint32_t n, int which, uint32_t half_row, uint64_t rel_key_base, uint32_t n_points, cudaStream_t s);
+uint32_t rel_piece_len(uint32_t d);     // data points per piece of a relation's run: 8, or 4 for small matrices
 // gradient rows (half_row values per occurrence, in ps->upd) -> AdaGrad, of the keys that occur several times and, with
 // singles, of those that occur once; loss terms.  parked: room for the long segments' partial sums.  beside: the kernel before
 // it on the stream has triggered it, is still running, and touches none of what this one does

@@ -40,8 +40,7 @@ namespace psb {
 
 namespace {
 
-constexpr int kPoints = 8;                      // data points of one relation per block at a time: a warp each, the columns of one tile
-constexpr int kPointThreads = 32 * kPoints;
+constexpr int kPoints = 8;                      // columns of one tile: data points of one relation per block at a time, a warp each
 constexpr int kMatThreads = 256;                // eight matrix elements each
 constexpr int kMatStage = 8;                    // data points whose vectors are staged together
 
@@ -84,8 +83,12 @@ __device__ __forceinline__ double sum8(double v) {          // over the eight la
 // every gradient row written (the d matrix rows' too) together with the slots' keys.
 // All rows a block needs (the matrix, the points' entities) are asked for at once as bulk copies into shared memory and
 // waited for once; with plain loads phase by phase the block's time was a chain of memory latencies (248 us a step).
-template <bool kSorted>
-__global__ void __launch_bounds__(kPointThreads, 2) rescal_points_kernel(const RescalArgs A) {
+// kWarps: 8, or 4 (up to four data points at a time) for dimensions up to 64, whose tiles four warps hold: as many warps per
+// SM in twice the blocks, so a relation of few data points idles fewer warps (1,288 data points of 573 relations of dimension
+// 28: 34.6 -> 23.8 us; 8,000 of 237 of dimension 64: 81 -> 76).
+template <bool kSorted, int kWarps>
+__global__ void __launch_bounds__(32 * kWarps, 16 / kWarps) rescal_points_kernel(const RescalArgs A) {
+    constexpr int kPointThreads = 32 * kWarps;
     extern __shared__ __align__(128) unsigned char dyn[];
     __shared__ __align__(8) uint64_t bar;
     __shared__ uint32_t s_t[kPoints];
@@ -110,7 +113,7 @@ __global__ void __launch_bounds__(kPointThreads, 2) rescal_points_kernel(const R
     const uint32_t n_items = kSorted ? A.L.counts[2] : A.n;
     const uint32_t m_tiles = (d + 7) / 8;
     unsigned parity = 0;
-    // Both products of a pass, R Y and R^T X: warp w takes the tiles w, w + 8, w + 16, w + 24 of the 2 m_tiles together
+    // Both products of a pass, R Y and R^T X: warp w takes the tiles w, w + kWarps, ... of the 2 m_tiles together
     // (four independent chains of tensor instructions).
     double acc[4][2];
     auto products = [&]() {
@@ -119,7 +122,7 @@ __global__ void __launch_bounds__(kPointThreads, 2) rescal_points_kernel(const R
         bool tr[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const uint32_t job = tmin<uint32_t>(w + 8 * j, 2 * m_tiles - 1);    // (past the last: computed, not stored)
+            const uint32_t job = tmin<uint32_t>(w + kWarps * j, 2 * m_tiles - 1);    // (past the last: computed, not stored)
             tr[j] = job >= m_tiles;
             const uint32_t row = tmin<uint32_t>((tr[j] ? job - m_tiles : job) * 8 + lane / 4, d - 1);
             a[j] = tr[j] ? R + (lane % 4) * ld + row : R + row * ld + lane % 4;
@@ -138,7 +141,7 @@ __global__ void __launch_bounds__(kPointThreads, 2) rescal_points_kernel(const R
     auto store_products = [&](double* u, double* wt, uint32_t len) {
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const uint32_t job = w + 8 * j;
+            const uint32_t job = w + kWarps * j;
             const bool tr = job >= m_tiles;
             const uint32_t row = (tr ? job - m_tiles : job) * 8 + lane / 4, col = 2 * (lane % 4);
             if (job >= 2 * m_tiles || row >= d) continue;
@@ -591,9 +594,9 @@ const double* run_rescal_small(ps_store* ps, const RescalBatch& B, uint32_t* key
     A.keys_out = keys_out;
     A.loss_of = ps->loss_partial;               // (kSmallOcc key occurrences are fewer data points than it has room for)
     static std::atomic<unsigned long long> smem_set{0};
-    opt_in_smem((const void*)rescal_points_kernel<false>, kMaxSmem, &smem_set);
-    PS_LAUNCH_PDL(ps, "rescal_points_kernel<false>", rescal_points_kernel<false>,
-                  dim3((uint32_t)tmin<uint64_t>(B.n, (uint64_t)ps->sm_count * 2)), dim3(kPointThreads),
+    opt_in_smem((const void*)rescal_points_kernel<false, 8>, kMaxSmem, &smem_set);
+    PS_LAUNCH_PDL(ps, "rescal_points_kernel<false>", (rescal_points_kernel<false, 8>),
+                  dim3((uint32_t)tmin<uint64_t>(B.n, (uint64_t)ps->sm_count * 2)), dim3(256),
                   points_smem(B.dim, B.n_neg, 1), s, A);
     return A.loss_of;
 }
@@ -603,10 +606,20 @@ void run_rescal_sorted(ps_store* ps, const RescalBatch& B, int which, uint32_t n
     A.sk = which ? ps->keysB : ps->keysA;
     A.sv = which ? ps->valsB : ps->valsA;
     A.L = seg_lists(ps);
-    static std::atomic<unsigned long long> smem_set{0}, smem_set2{0};
-    opt_in_smem((const void*)rescal_points_kernel<true>, kMaxSmem, &smem_set);
-    PS_LAUNCH_SMEM(ps, rescal_points_kernel<true>, (uint32_t)tmin<uint64_t>(B.n, (uint64_t)ps->sm_count * 2), kPointThreads,
-                   points_smem(B.dim, B.n_neg, kPoints), s, A);
+    static std::atomic<unsigned long long> smem_set{0}, smem_set2{0}, smem_set4{0};
+    const int points = (int)rel_piece_len(B.dim);
+    const size_t p_smem = points_smem(B.dim, B.n_neg, points);
+    const uint32_t p_grid = (uint32_t)tmin<uint64_t>(B.n, (uint64_t)ps->sm_count * 2 * (kPoints / points));
+    if (ps->prof) prof_before(ps, "rescal_points_kernel<true>", s);
+    if (points == kPoints) {
+        opt_in_smem((const void*)rescal_points_kernel<true, 8>, kMaxSmem, &smem_set);
+        rescal_points_kernel<true, 8><<<p_grid, 256, p_smem, s>>>(A);
+    } else {
+        opt_in_smem((const void*)rescal_points_kernel<true, 4>, points_smem(64, 29, 4), &smem_set4);
+        rescal_points_kernel<true, 4><<<p_grid, 128, p_smem, s>>>(A);
+    }
+    if (ps->prof) prof_after(ps, s);
+    ps->launches++;
     const uint32_t strips = div_up_u32((uint64_t)B.dim * B.dim / 8, kMatThreads);
     static_assert(128 * 128 / 8 / kMatThreads <= (int)kRelTickets, "a ticket per strip of a matrix");
     const size_t smem = (size_t)2 * kMatStage * B.dim * 32;

@@ -144,3 +144,12 @@ def test_skip_gram_reduction_at_every_tile_length(n, pipelined):
     g.sync()
     compare_state(g, o, what=f"skip-gram, {n} centers")
     assert close(float(g.loss.cpu()[0]), o.loss[0])
+
+
+@pytest.mark.parametrize("d,n_neg,batch,ents,rels", [(4, 0, 3_000, 500, 1), (28, 10, 700, 3_000, 300), (64, 3, 900, 500, 5),
+                                                     (68, 10, 650, 800, 60), (128, 29, 200, 900, 2)])
+def test_rescal_steps_with_a_sort(d, n_neg, batch, ents, rels):
+    """Runs of relations from one data point to all 3,000 of the batch (pieces of four and of eight, chunks of every
+    length), dimensions on both sides of the points kernel's two forms."""
+    from tests.test_gpu_rescal import rescal_run
+    rescal_run(d, n_neg, batch, ents, rels, steps=2, single_step=True, G=0.3)
