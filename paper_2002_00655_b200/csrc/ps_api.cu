@@ -833,11 +833,26 @@ static bool host_batch_copied(ps_store* ps, cudaStream_t s, const HostBatch& hb)
     ps->batch_ready = ps->ev_copied[hb.slot];       // picked up by the step's fork of the side stream
     return true;
 }
+// The loss word, to pinned host memory.  A copy of eight bytes by the copy engine stood between two steps on the caller's
+// stream for 4 to 6 us (matrix factorization: 65,536 cells 53.9 -> 49.5 us per step, 10,984 of rank 4 27.6 -> 22.4).
+__global__ void read_loss_kernel(double* __restrict__ h, const double* __restrict__ d) {
+    pdl_wait();
+    if (threadIdx.x == 0) *(volatile double*)h = *d;
+}
+
 static ps_status_t finish_host_step(ps_store* ps, const HostBatch& hb, double* d_loss_accum, double* h_loss,
                                     cudaStream_t s) {
-    if (d_loss_accum && h_loss &&
-        cudaMemcpyAsync(h_loss, d_loss_accum, sizeof(double), cudaMemcpyDeviceToHost, s) != cudaSuccess)
-        return PS_ERR_CUDA;
+    if (d_loss_accum && h_loss) {
+        cudaPointerAttributes at;
+        const bool known = hb.slot >= 0 && ((uintptr_t)h_loss & 7) == 0 && cudaPointerGetAttributes(&at, h_loss) == cudaSuccess;
+        if (known && at.type == cudaMemoryTypeHost && at.devicePointer) {
+            PS_LAUNCH_PDL(ps, "read_loss_kernel", read_loss_kernel, dim3(1), dim3(32), 0, s, (double*)at.devicePointer,
+                          (const double*)d_loss_accum);
+            if (cudaGetLastError() != cudaSuccess) return PS_ERR_CUDA;
+        } else if (cudaMemcpyAsync(h_loss, d_loss_accum, sizeof(double), cudaMemcpyDeviceToHost, s) != cudaSuccess) {
+            return PS_ERR_CUDA;
+        }
+    }
     if (hb.slot >= 0) {                              // overlapped mode: nothing waits; the area is free once s gets here
         if (cudaEventRecord(ps->ev_consumed[hb.slot], s) != cudaSuccess) return PS_ERR_CUDA;
         ps->consumed_valid[hb.slot] = true;

@@ -970,6 +970,7 @@ push_fixup_kernel(const uint32_t* __restrict__ sk, uint32_t n, float4* __restric
                   uint32_t loss_blocks, double* __restrict__ loss_accum, uint32_t fix_blocks,
                   const float4* __restrict__ staged, const uint64_t* __restrict__ apply_row, uint32_t tile_len,
                   uint32_t apply_lo, const DevStatus* st, unsigned int epoch) {
+    pdl_trigger();                                  // (for read_loss_kernel)
     if (call_failed(st, epoch)) return;
     if (blockIdx.x > fix_blocks) {
         // Blocks past the loss block move staged rows into the store (calls that stage rows only): the reduction

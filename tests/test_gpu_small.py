@@ -153,3 +153,28 @@ def test_rescal_steps_with_a_sort(d, n_neg, batch, ents, rels):
     length), dimensions on both sides of the points kernel's two forms."""
     from tests.test_gpu_rescal import rescal_run
     rescal_run(d, n_neg, batch, ents, rels, steps=2, single_step=True, G=0.3)
+
+
+@pytest.mark.parametrize("batch", [512, 8192])
+def test_losses_of_overlapped_host_steps_reach_pinned_and_pageable_words(batch):
+    """Steps without and with a sort, each with a loss word of its own, every other one in pageable memory (a copy there, a
+    kernel's store to pinned memory): all equal to what the device-batch calls accumulate."""
+    cfg = W.scaled(W.MF_TINY, rows=3000, cols=400, rank=12, n_cells=6 * batch, batch=batch, lr=0.0005)
+    rows = W.mf_init_rows(cfg, 0, cfg.num_keys, "cpu")
+    i, j, v = W.mf_cells(cfg, W.mf_planted(cfg, "cpu"), 0, cfg.n_cells, "cpu")
+    pinned = [t.pin_memory() for t in (i, j, v)]
+    a, _ = make_pair(cfg.num_keys, cfg.rank, rows=rows, max_batch_keys=2 * batch)
+    g, _ = make_pair(cfg.num_keys, cfg.rank, rows=rows, max_batch_keys=2 * batch)
+    ps.ps_set_pipelining(g.h, True)
+    ps.ps_set_host_overlap(g.h, True)
+    words = [torch.zeros(1, dtype=torch.float64) for _ in range(cfg.n_batches)]
+    words = [w.pin_memory() if b % 2 else w for b, w in enumerate(words)]
+    want = []
+    for b in range(cfg.n_batches):
+        sl = slice(b * batch, (b + 1) * batch)
+        ps.ps_step_mf(a.h, i[sl].cuda(), j[sl].cuda(), v[sl].cuda(), cfg.col_key_base, cfg.lr, cfg.lam, a.loss)
+        a.sync()
+        want.append(float(a.loss.cpu()[0]))
+        ps.ps_step_mf_host(g.h, *(t[sl] for t in pinned), cfg.col_key_base, cfg.lr, cfg.lam, g.loss, words[b])
+    g.sync()
+    assert [float(w[0]) for w in words] == want
