@@ -766,11 +766,13 @@ static ps_status_t sgns_sorted(ps_store_t* ps, SortSet* ss, const uint32_t* d_to
                                uint64_t n_centers, uint64_t corpus_len, uint32_t window, const uint32_t* d_negs,
                                uint32_t n_neg, uint64_t out_key_base, float lr, uint64_t occ, double* d_loss_accum,
                                cudaStream_t s) {
-    launch_keys_sgns(ps, d_tokens, tok_first, first_pos, n_centers, corpus_len, window, d_negs, n_neg, out_key_base, ps->side);
+    // (rows of less than 1 KB: 159 us against 155 at 64 values, 10,000 centers; with 500 values 333 against 344)
+    const bool in_place = ps->pipelined && ps->cfg.row_len >= 256;
+    launch_keys_sgns(ps, d_tokens, tok_first, first_pos, n_centers, corpus_len, window, d_negs, n_neg, out_key_base,
+                     in_place ? seg_lists(ps).single : nullptr, ps->side);
     const int which = run_push_sort(ps, (uint32_t)occ, ps->side);
     if (!sorted_keys_at(ps, ss, which, (uint32_t)occ, ps->side)) return PS_ERR_CUDA;
-    // (rows of less than 1 KB: 159 us against 155 at 64 values, 10,000 centers; with 500 values 333 against 344)
-    const uint8_t* single = ps->pipelined && ps->cfg.row_len >= 256 ? launch_singles(ps, (uint32_t)occ, which, ps->side) : nullptr;
+    const uint8_t* single = in_place ? launch_singles(ps, (uint32_t)occ, which, ps->side) : nullptr;
     if (single && !join_side(ps, s)) return PS_ERR_CUDA;
     const uint32_t lb = launch_step_sgns(ps, d_tokens, tok_first, first_pos, n_centers, corpus_len, window, d_negs, n_neg,
                                          out_key_base, lr, nullptr, s, single);

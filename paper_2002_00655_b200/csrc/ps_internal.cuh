@@ -347,7 +347,7 @@ void run_localize_deferred(ps_store* ps, uint32_t worker, uint32_t n, cudaStream
 // (calls without a sort, small.cu) they write the slots' keys there themselves and latch errors for no call number.
 void launch_keys_sgns(ps_store* ps, const uint32_t* d_tokens, uint64_t tok_first, uint64_t first_pos,
                       uint64_t n_centers, uint64_t corpus_len, uint32_t window, const uint32_t* d_negs, uint32_t n_neg,
-                      uint64_t out_key_base, cudaStream_t s);
+                      uint64_t out_key_base, uint8_t* single, cudaStream_t s);
 uint32_t launch_step_mf(ps_store* ps, const uint32_t* d_i, const uint32_t* d_j, const float* d_v, uint64_t n,
                         uint64_t col_key_base, float lr, float lambda, uint32_t* keys_out, cudaStream_t s);
 float* sgns_scales(ps_store* ps, uint64_t n_centers);     // where launch_step_sgns puts the per-slot factors
