@@ -234,6 +234,9 @@ __host__ __device__ __forceinline__ uint64_t sgns_pairs_before(uint64_t p, uint6
     return left + right;
 }
 
+// rows worked on together: as many as leave 128 registers without spills
+__host__ __device__ constexpr int sgns_quad(int kCh) { return kCh == 4 ? 2 : kCh == 1 ? 8 : 4; }
+
 // Occurrence slots of center number c of the batch: slot_base = c * (1 + 2W(1 + n_neg));
 // slot_base = the center's input vector; then per context j (ascending position) 1 + n_neg output vectors.
 // The update of an output vector is a multiple of the center's input vector, the same vector for all of
@@ -264,8 +267,23 @@ sgns_step_kernel(const uint32_t* __restrict__ tokens, uint64_t tok_first, uint64
     const uint32_t per_ctx = 1 + n_neg;
     const uint64_t slots = 1 + (uint64_t)2 * window * per_ctx;
     const uint64_t pairs0 = sgns_pairs_before(first_pos, T, window);
-    constexpr int kQuad = kCh == 4 ? 2 : kCh == 1 ? 8 : 4;     // rows in flight: as many as leave 128 registers without spills
+    constexpr int kQuad = sgns_quad(kCh);
     constexpr int kLanes = 32 / kQuad;
+    // Rows of more than 512 bytes arrive in shared memory as bulk copies, two groups of kQuad of them on their way while one
+    // is worked on from registers: [warp][2][kQuad][L4].  (With loads straight into the registers one group was on its way, and
+    // that only between two groups' arithmetic: 295 us for 32,768 centers of 300 values at 4.6 TB/s of DRAM, now 265.)
+    constexpr bool kStage = kCh >= 2;
+    extern __shared__ __align__(128) float4 sgns_stage[];
+    __shared__ __align__(8) uint64_t bars[8][2];
+    const int w = threadIdx.x >> 5;
+    float4* const ring = sgns_stage + (size_t)w * (2 * kQuad) * L4;
+    if (kStage) {
+        if (lane < 2) mbar_init(&bars[w][lane], 1);
+        mbar_init_fence();
+        __syncwarp();
+    }
+    unsigned uses = 0;                                          // parity of each stage's barrier
+    bool dead = false;
     float4 u[kQuad][kCh];                                       // (elements past the row are never loaded: zero throughout)
 #pragma unroll
     for (int a = 0; a < kQuad; ++a)
@@ -275,7 +293,7 @@ sgns_step_kernel(const uint32_t* __restrict__ tokens, uint64_t tok_first, uint64
     pdl_trigger();
     pdl_wait();
     if (kOnce && call_failed(st, epoch)) return;        // (the key kernel found an index out of range: nothing may be written)
-    for (uint64_t cidx = warp; cidx < n_centers; cidx += n_warps) {
+    for (uint64_t cidx = warp; cidx < n_centers && !dead; cidx += n_warps) {
         const uint64_t p = first_pos + cidx;
         const uint64_t lo = p >= window ? p - window : 0;
         const uint64_t hi = p + window < T ? p + window : T - 1;
@@ -303,7 +321,7 @@ sgns_step_kernel(const uint32_t* __restrict__ tokens, uint64_t tok_first, uint64
             dv[c] = make_float4(0.f, 0.f, 0.f, 0.f);
         }
         bool bad = false;
-        for (uint32_t t0 = 0; t0 < n_out; t0 += 32) {
+        for (uint32_t t0 = 0; t0 < n_out && !dead; t0 += 32) {
             // this lane's slot of the round
             const uint32_t t = t0 + lane;
             uint64_t my_row = 0;
@@ -325,9 +343,37 @@ sgns_step_kernel(const uint32_t* __restrict__ tokens, uint64_t tok_first, uint64
             const unsigned once_mask = kOnce ? __ballot_sync(full, my_ok && single[cidx * slots + 1 + t]) : 0u;
             const uint32_t in_round = tmin<uint32_t>(32u, n_out - t0);
             float my_scale = 0.f, my_x = 0.f;                                   // factor and score of this lane's slot
+            auto ask = [&](uint32_t b) {                                        // the rows of slots b .. b + kQuad
+                const unsigned group = (ok_mask >> b) & ((1u << kQuad) - 1u);
+                if (b >= in_round || group == 0) return;
+                const uint32_t stage = (b / kQuad) & 1;
+                if (lane == (int)b) mbar_expect_tx(&bars[w][stage], __popc(group) * L4 * 16);
+                __syncwarp();
+                if (my_ok && lane - b < kQuad) bulk_g2s(ring + (stage * kQuad + (lane - b)) * L4, store + my_row * L4, L4 * 16, &bars[w][stage]);
+            };
+            if (kStage) {
+                ask(0);
+                ask(kQuad);
+            }
             for (uint32_t b = 0; b < in_round; b += kQuad) {
+                if (kStage && ((ok_mask >> b) & ((1u << kQuad) - 1u))) {
+                    const uint32_t stage = (b / kQuad) & 1;
+                    if (!mbar_wait(&bars[w][stage], (uses >> stage) & 1u) && !mbar_wait(&bars[w][stage], (uses >> stage) & 1u)) {
+                        if (lane == 0) latch_error(st, epoch, PS_ERR_CUDA);
+                        dead = true;                                            // a copy that does not arrive: give the call up
+                        break;
+                    }
+                    uses ^= 1u << stage;
 #pragma unroll
-                for (int a = 0; a < kQuad; ++a) {                               // (a slot without a row reads row 0, and is skipped below)
+                    for (int a = 0; a < kQuad; ++a)                             // (a slot without a row: what was there, skipped below)
+#pragma unroll
+                        for (int c = 0; c < kCh; ++c)
+                            if (lane + 32 * c < L4) u[a][c] = ring[(stage * kQuad + a) * L4 + lane + 32 * c];
+                    __syncwarp();
+                }
+                if (kStage) ask(b + 2 * kQuad);
+#pragma unroll
+                for (int a = 0; a < kQuad && !kStage; ++a) {                    // (a slot without a row reads row 0, and is skipped below)
                     const float4* Urow = store + __shfl_sync(full, my_row, (b + a) & 31) * L4;
 #pragma unroll
                     for (int c = 0; c < kCh; ++c) {
@@ -462,12 +508,16 @@ uint32_t launch_step_sgns(ps_store* ps, const uint32_t* d_tokens, uint64_t tok_f
                 (float4*)ps->upd, sgns_scales(ps, n_centers), keys_out, ps->loss_partial, ps->status, epoch
 #define SG_LAUNCH(kCh, kL4, kW, kN)                                                                                  \
     do {                                                                                                             \
+        const size_t smem = (kCh) >= 2 ? (size_t)8 * 2 * sgns_quad(kCh) * L4 * 16 : 0;                               \
+        static std::atomic<unsigned long long> smem_set[2];                                                          \
+        const void* fn = single ? (const void*)sgns_step_kernel<kCh, kL4, kW, kN, true> : (const void*)sgns_step_kernel<kCh, kL4, kW, kN, false>; \
+        if ((kCh) >= 2) opt_in_smem(fn, (size_t)8 * 2 * sgns_quad(kCh) * (kCh) * 512, &smem_set[single ? 1 : 0]);    \
         if (keys_out) {                                                                                              \
-            PS_LAUNCH_PDL(ps, "sgns_step_kernel<" #kCh ">", (sgns_step_kernel<kCh, kL4, kW, kN, false>), dim3(grid), dim3(256), 0, s, SG_ARGS); \
+            PS_LAUNCH_PDL(ps, "sgns_step_kernel<" #kCh ">", (sgns_step_kernel<kCh, kL4, kW, kN, false>), dim3(grid), dim3(256), smem, s, SG_ARGS); \
         } else {                                                                                                     \
             if (ps->prof) prof_before(ps, "sgns_step_kernel<" #kCh ">", s);                                          \
-            if (single) sgns_step_kernel<kCh, kL4, kW, kN, true><<<grid, 256, 0, s>>>(SG_ARGS);                      \
-            else sgns_step_kernel<kCh, kL4, kW, kN, false><<<grid, 256, 0, s>>>(SG_ARGS);                            \
+            if (single) sgns_step_kernel<kCh, kL4, kW, kN, true><<<grid, 256, smem, s>>>(SG_ARGS);                   \
+            else sgns_step_kernel<kCh, kL4, kW, kN, false><<<grid, 256, smem, s>>>(SG_ARGS);                         \
             if (ps->prof) prof_after(ps, s);                                                                         \
             ps->launches++;                                                                                          \
         }                                                                                                            \
