@@ -228,6 +228,7 @@ map_insert_kernel(ps_keymap m, const uint64_t* __restrict__ in, uint32_t n, uint
         }
         const uint32_t s = new_slot(t, q);
         if (s < kSettled) out[t] = (uint64_t)__ldcg(&m.vals[s]);
+        else if (s != kSettled) out[t] = ~0ull;                 // the reserved key, behind an error latched earlier (bad_key is then false)
     }
     if (b == 0 && tid == 0) {
         if (!full && !bad_key) *m.size = size0 + total;

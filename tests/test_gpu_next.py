@@ -60,6 +60,24 @@ def test_keymap_full_and_reserved_key_add_nothing():
     assert g.sync() == (ps.PS_OK, 100)
 
 
+@pytest.mark.parametrize("n", [3, 700, 60_000])
+def test_keymap_reserved_key_behind_a_latched_error_reads_as_absent(n):
+    """With an earlier call's error still latched, the call takes the keys it can and says "absent" for the reserved one."""
+    g = ps.KeyMap(100_000, max_batch_keys=200_000)
+    known = np.arange(1, 2_000, dtype=np.uint64) * np.uint64(2654435761)
+    g.insert(u64(known))
+    assert g.sync() == (ps.PS_OK, 1_999)
+    g.insert(u64(np.arange(10_000_000, 10_150_000, dtype=np.uint64)))           # more than there is room for; no sync
+    keys = known[np.arange(n) % 1_999]
+    keys[n // 2] = np.uint64(2**64 - 1)
+    out = torch.full((n,), 12345, dtype=torch.int64, device="cuda")
+    ps.ps_keymap_insert(g.h, u64(keys), out)
+    want = (np.arange(n) % 1_999).astype(np.uint64)
+    want[n // 2] = ABSENT
+    assert (as_u64(out) == want).all()
+    assert g.sync() == (ps.PS_ERR_CAPACITY, 1_999)
+
+
 def test_store_behind_a_keymap_serves_sparse_keys():
     """push, localize and pull through the map against the oracle's map in front of the oracle's store."""
     rng = np.random.default_rng(4)
