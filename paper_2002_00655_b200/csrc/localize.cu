@@ -485,7 +485,7 @@ constexpr int kLocTableBits = 12;
 constexpr size_t kLocSmallSmem = ((size_t)kLocSmallKeys * 2 + ((size_t)2 << kLocTableBits)) * 4;
 
 __global__ void __cluster_dims__(kLocSmallBlocks, 1, 1) __launch_bounds__(kLocSmallThreads)
-loc_small_kernel(const uint64_t* __restrict__ keys, uint32_t n, uint2* table, uint32_t worker, uint64_t S, uint32_t K,
+loc_small_kernel(const uint64_t* keys, uint32_t n, uint2* table, uint32_t worker, uint64_t S, uint32_t K,
                  unsigned long long* tops, uint32_t* stacks, float4* store, uint32_t L4, uint32_t part_size, DevStatus* st) {
     constexpr uint32_t kSlots = 1u << kLocTableBits, kPer = kLocSmallKeys / kLocSmallThreads;
     extern __shared__ __align__(16) uint32_t loc_dyn[];

@@ -837,7 +837,7 @@ static bool host_batch_copied(ps_store* ps, cudaStream_t s, const HostBatch& hb)
 }
 // The loss word, to pinned host memory.  A copy of eight bytes by the copy engine stood between two steps on the caller's
 // stream for 4 to 6 us (matrix factorization: 65,536 cells 53.9 -> 49.5 us per step, 10,984 of rank 4 27.6 -> 22.4).
-__global__ void read_loss_kernel(double* __restrict__ h, const double* __restrict__ d) {
+__global__ void read_loss_kernel(double* h, const double* d) {
     pdl_wait();
     if (threadIdx.x == 0) *(volatile double*)h = *d;
 }

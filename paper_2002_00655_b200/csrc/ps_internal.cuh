@@ -185,6 +185,8 @@ void prof_after(ps_store* ps, cudaStream_t s);
 // stream still runs, as soon as all blocks of that one have passed pdl_trigger(); it touches no memory before pdl_wait(),
 // which returns when everything before has completed.  Takes a launch's latency (a microsecond or two) off each of a
 // chain of kernels that run a few microseconds.  Without a trigger in the kernel before it is an ordinary launch.
+// What such a kernel reads may be written while it is already on the chip: none of it is passed as `const __restrict__`, which
+// would let the compiler read it through the read-only path and before the wait.
 template <class... P, class... A>
 inline void launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, const A&... args) {
     cudaLaunchConfig_t cfg = {};

@@ -72,8 +72,8 @@ constexpr uint32_t kPullStageBytes = 4096;          // per warp and stage
 constexpr size_t kPullSmem = (size_t)8 * 2 * kPullStageBytes;
 
 __global__ void __launch_bounds__(256)
-pull_bulk_kernel(const uint64_t* __restrict__ keys, uint64_t n, char* __restrict__ out, const char* __restrict__ store,
-                 const uint2* __restrict__ table, uint64_t S, uint64_t K, uint32_t row_bytes, uint32_t per_round,
+pull_bulk_kernel(const uint64_t* keys, uint64_t n, char* __restrict__ out, const char* store,
+                 const uint2* table, uint64_t S, uint64_t K, uint32_t row_bytes, uint32_t per_round,
                  DevStatus* st, unsigned int epoch) {
     __shared__ __align__(8) uint64_t bars[8][2];
     extern __shared__ __align__(128) char pull_stage[];

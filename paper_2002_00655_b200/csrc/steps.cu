@@ -46,10 +46,10 @@ static uint32_t step_grid(ps_store* ps, uint64_t n_examples, uint32_t blocks_per
 // row length, rows re-read from cache for the second pass.
 template <int kCh>
 __global__ void __launch_bounds__(256)
-mf_step_kernel(const uint32_t* __restrict__ ci, const uint32_t* __restrict__ cj, const float* __restrict__ cv,
-               uint64_t n, uint64_t col_base, float lr, float lam, const float4* __restrict__ store,
-               const uint2* __restrict__ table, uint64_t S, uint64_t K, uint32_t L4,
-               float4* __restrict__ upd, uint32_t* __restrict__ keys_out, double* __restrict__ loss_partial,
+mf_step_kernel(const uint32_t* ci, const uint32_t* cj, const float* cv,
+               uint64_t n, uint64_t col_base, float lr, float lam, const float4* store,
+               const uint2* table, uint64_t S, uint64_t K, uint32_t L4,
+               float4* __restrict__ upd, uint32_t* keys_out, double* __restrict__ loss_partial,
                DevStatus* st, unsigned int epoch) {
     const int lane = threadIdx.x & 31;
     const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -127,10 +127,10 @@ mf_step_kernel(const uint32_t* __restrict__ ci, const uint32_t* __restrict__ cj,
 // dependent loads; one cell per warp leaves the memory system idle most of the time).
 template <int kCells>
 __global__ void __launch_bounds__(256)
-mf_step_small_kernel(const uint32_t* __restrict__ ci, const uint32_t* __restrict__ cj, const float* __restrict__ cv,
-                     uint64_t n, uint64_t col_base, float lr, float lam, const float4* __restrict__ store,
-                     const uint2* __restrict__ table, uint64_t S, uint64_t K, uint32_t L4,
-                     float4* __restrict__ upd, uint32_t* __restrict__ keys_out, double* __restrict__ loss_partial,
+mf_step_small_kernel(const uint32_t* ci, const uint32_t* cj, const float* cv,
+                     uint64_t n, uint64_t col_base, float lr, float lam, const float4* store,
+                     const uint2* table, uint64_t S, uint64_t K, uint32_t L4,
+                     float4* __restrict__ upd, uint32_t* keys_out, double* __restrict__ loss_partial,
                      DevStatus* st, unsigned int epoch) {
     const int lane = threadIdx.x & 31;
     const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -252,10 +252,10 @@ __host__ __device__ constexpr int sgns_quad(int kCh) { return kCh == 4 ? 2 : kCh
 // third of the skip-gram batch's occurrences, each of which cost the reduction three rows of traffic.
 template <int kCh, int kL4, int kWindow, int kNeg, bool kOnce>
 __global__ void __launch_bounds__(256, 2)
-sgns_step_kernel(const uint32_t* __restrict__ tokens, uint64_t tok_first, uint64_t first_pos, uint64_t n_centers,
-                 uint64_t T, uint32_t window_arg, const uint32_t* __restrict__ negs, uint32_t n_neg_arg, uint64_t out_base,
-                 float lr, float4* store, const uint2* __restrict__ table, uint64_t S, uint64_t K, const uint8_t* __restrict__ single,
-                 uint32_t L4_arg, float4* __restrict__ upd, float* __restrict__ scales, uint32_t* __restrict__ keys_out,
+sgns_step_kernel(const uint32_t* tokens, uint64_t tok_first, uint64_t first_pos, uint64_t n_centers,
+                 uint64_t T, uint32_t window_arg, const uint32_t* negs, uint32_t n_neg_arg, uint64_t out_base,
+                 float lr, float4* store, const uint2* table, uint64_t S, uint64_t K, const uint8_t* single,
+                 uint32_t L4_arg, float4* __restrict__ upd, float* __restrict__ scales, uint32_t* keys_out,
                  double* __restrict__ loss_partial, DevStatus* st, unsigned int epoch) {
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;

@@ -178,3 +178,63 @@ def test_losses_of_overlapped_host_steps_reach_pinned_and_pageable_words(batch):
         ps.ps_step_mf_host(g.h, *(t[sl] for t in pinned), cfg.col_key_base, cfg.lr, cfg.lam, g.loss, words[b])
     g.sync()
     assert [float(w[0]) for w in words] == want
+
+
+def small_step(mode, E, R, L, n, rng):
+    """(number of keys, step(store) on the GPU, the same on the oracle) of a small step with random indexes."""
+    d, q = {"kge": L // 4, "rescal": L // 2}.get(mode, L), 2
+    u32 = lambda a: a.astype(np.uint32)
+    if mode == "sgns":
+        tok, neg = u32(rng.integers(0, E, size=n + 4)), u32(rng.integers(0, E, size=(n * 4, q)))
+        a = [dev(tok, torch.int32), dev(neg, torch.int32)]
+        return (2 * E, lambda g: ps.ps_step_sgns(g.h, a[0], 2, n, 2, a[1], q, E, 0.01, g.loss),
+                lambda o: o.step_sgns(tok, 2, n, 2, neg, q, E, 0.01))
+    i, j = u32(rng.integers(0, E, size=n)), u32(rng.integers(0, R, size=n))
+    if mode == "mf":
+        v = rng.normal(size=n).astype(np.float32)
+        a = [dev(i, torch.int32), dev(j, torch.int32), dev(v)]
+        return (E + R, lambda g: ps.ps_step_mf(g.h, *a, E, 0.01, 0.05, g.loss), lambda o: o.step_mf(i, j, v, E, 0.01, 0.05))
+    t, ne = u32(rng.integers(0, E, size=n)), u32(rng.integers(0, E, size=(n, q)))
+    ns = rng.integers(0, 2, size=(n, q)).astype(np.uint8)
+    a = [dev(x, torch.int32) for x in (i, j, t, ne)] + [dev(ns)]
+    step = ps.ps_step_kge if mode == "kge" else ps.ps_step_rescal
+    return (E + R * (d if mode == "rescal" else 1), lambda g: step(g.h, *a, q, E, d, 0.1, 1e-8, g.loss),
+            lambda o: getattr(o, "step_" + mode)(i, j, t, ne, ns, E, d, 0.1, 1e-8))
+
+
+@pytest.mark.parametrize("L,mode", [(12, "mf"), (260, "mf"), (16, "kge"), (24, "sgns"), (300, "sgns"), (16, "rescal")])
+def test_small_calls_back_to_back(L, mode):
+    """Kernels of small calls are set up while the ones before them still run and write: relocation, step, push and pull over
+    the same few keys, with nothing waited for, against the same calls waited for one by one (bit for bit) and the oracle."""
+    rng = np.random.default_rng(L)
+    steps = [small_step(mode, 60, 10, L, 40, rng) for _ in range(60)]
+    K = steps[0][0]
+    rows = np.abs(rng.normal(0.2, 0.1, size=(K, L))).astype(np.float32)
+    calls = []
+    for _, on_gpu, on_cpu in steps:
+        keys, upd = rng.integers(0, K, size=50), np.abs(rng.normal(0, 0.01, size=(50, L))).astype(np.float32)
+        calls.append((int(rng.integers(0, 3)), on_gpu, on_cpu, keys, upd, dev(keys), dev(upd)))
+    (g, o), (h, _) = (make_pair(K, L, 3, K, rows=rows, max_batch_keys=4096) for _ in range(2))
+    torch.cuda.synchronize()
+    pulled = []
+    for w, on_gpu, _, _, _, keys, upd in calls:
+        g.localize(w, keys)
+        on_gpu(g)
+        g.push(keys, upd)
+        pulled.append(g.pull(keys))
+    g.sync()
+    for (w, on_gpu, on_cpu, keys, upd, dk, du), got in zip(calls, pulled):
+        for call in (lambda: h.localize(w, dk), lambda: on_gpu(h), lambda: h.push(dk, du)):
+            call()
+            h.sync()
+        assert torch.equal(h.pull(dk), got)
+        o.localize(w, keys)
+        if got is pulled[0]:                # (the oracle's rows drift from the GPU's roundings over the later steps)
+            on_cpu(o)
+            o.push(keys, upd)
+            assert close(got.cpu().numpy(), o.pull(keys)).all()
+    for x, y in zip(g.export(), h.export()):
+        assert torch.equal(x, y)
+    assert torch.equal(g.loss, h.loss)
+    o.set_rows(np.arange(K), g.export()[0].numpy())
+    compare_state(g, o, exact_rows=True, what="tables and free lists")
