@@ -41,6 +41,14 @@ struct KgeArgs {
     unsigned int epoch;
 };
 
+// A bulk copy that does not arrive: the call is given up.  What follows it on the stream sees that by the call's number or, in calls
+// without a sort, by a key out of range among the slots' keys (lane 0 wrote slot 0's).
+__device__ __forceinline__ void give_up(const KgeArgs& A, uint64_t t, int lane) {
+    if (lane != 0) return;
+    latch_error(A.st, A.keys_out ? 0u : A.epoch, PS_ERR_CUDA);
+    if (A.keys_out) A.keys_out[t * (3 + A.n_neg)] = kSentinelPad;
+}
+
 // Sums over the 32 lanes of NP values each, NP a power of two: halves are exchanged, so that each step leaves half as many
 // values per lane to add (NP + 5 - log2 NP exchanges in place of 5 NP).  Lane l is left with value l / (32 / NP).
 template <int NP>
@@ -166,7 +174,7 @@ __global__ void __launch_bounds__(32 * kShortWarps, kMaxNeg <= 10 ? 4 : 2) kge_s
             continue;
         }
         if (!mbar_wait(&bars[w], parity) && !mbar_wait(&bars[w], parity)) {
-            if (lane == 0) latch_error(A.st, A.epoch, PS_ERR_CUDA);
+            give_up(A, t, lane);
             break;                                              // a copy that does not arrive: give the call up
         }
         parity ^= 1;
@@ -682,8 +690,11 @@ __global__ void __launch_bounds__(256, Wide<kMaxNeg>::kPerSm) kge_wide_kernel(co
                 }
             }
             if (__syncthreads_or(dead)) {
-                if (tid == 0) latch_error(A.st, A.epoch, PS_ERR_CUDA);
-                if (C == 1) return;
+                if (C == 1) {
+                    give_up(A, t, tid);
+                    return;
+                }
+                if (tid == 0) latch_error(A.st, A.keys_out ? 0u : A.epoch, PS_ERR_CUDA);
                 // the cluster's other blocks go on: meet them as often as they will, with nothing done in between
                 if (job + 1 < n_first) {
                     cluster_arrive();
@@ -695,6 +706,7 @@ __global__ void __launch_bounds__(256, Wide<kMaxNeg>::kPerSm) kge_wide_kernel(co
                 }
                 cluster_arrive();
                 cluster_wait();
+                give_up(A, t, tid);                             // (after the block that writes the keys has written them all)
                 return;
             }
         }

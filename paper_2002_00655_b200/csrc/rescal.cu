@@ -209,7 +209,10 @@ __global__ void __launch_bounds__(32 * kWarps, 16 / kWarps) rescal_points_kernel
         if (tid < (int)d) bulk_g2s(R + tid * ld, A.store + phys_row(A.table[rk + tid], A.S) * L, row_bytes, &bar);
         const bool ok = mbar_wait(&bar, parity) || mbar_wait(&bar, parity);
         if (__syncthreads_or(!ok)) {
-            if (tid == 0) latch_error(A.st, A.epoch, PS_ERR_CUDA);
+            if (tid == 0) {
+                latch_error(A.st, kSorted ? A.epoch : 0u, PS_ERR_CUDA);
+                if (!kSorted) A.keys_out[(uint64_t)item * n_slots] = kSentinelPad;      // (the reduction then does nothing)
+            }
             return;                             // a copy that does not arrive: give the call up
         }
         parity ^= 1;

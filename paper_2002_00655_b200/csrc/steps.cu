@@ -458,6 +458,10 @@ sgns_step_kernel(const uint32_t* tokens, uint64_t tok_first, uint64_t first_pos,
             }
         }
         if (__any_sync(full, bad) && lane == 0) latch_error(st, epoch, PS_ERR_KEY_RANGE);
+        if (dead) {                                             // (dv is a partial sum: the center's row stays as it is)
+            if (keys_out && lane == 0) keys_out[cidx * slots] = kSentinelPad;   // without a sort: the reduction then does nothing
+            break;
+        }
 #pragma unroll
         for (int c = 0; c < kCh; ++c) {
             const uint32_t f = lane + 32 * c;
