@@ -237,7 +237,7 @@ ps_status_t ps_step_sgns_host(ps_store_t* ps, const uint32_t* h_tokens, uint64_t
  * that cannot afford the device-wide synchronisation an allocation implies.
  * Such a caller cannot provide the workspace of ps_create, so this call needs
  * no handle: all scratch memory (sort buffers, partial sums) lives in a static
- * device array inside the library, about 2.3 MB, present on every GPU that
+ * device array inside the library, about 9 MB, present on every GPU that
  * loads the library until the process exits.  The call itself calls neither
  * cudaMalloc nor cudaFree nor anything else that allocates.
  *   d_store, d_table: a store and its location table as laid out by ps_create /

@@ -236,15 +236,10 @@ void launch_pull(ps_store* ps, const uint64_t* d_keys, uint64_t n, float* d_out,
 void launch_get_location(ps_store* ps, const uint64_t* d_keys, uint64_t n, uint32_t* d_owner, uint32_t* d_slot,
                          cudaStream_t s);
 void launch_gather_rows_by_key(ps_store* ps, uint64_t first_key, uint64_t n, float* d_out, cudaStream_t s);
-// keys64 -> keysA (range-checked)
-void launch_prepare_keys(ps_store* ps, const uint64_t* d_keys, uint64_t n, cudaStream_t s);
-// sort keysA (values = occurrence index), reduce `upd` rows per key, apply to the store, and add the
-// first `loss_blocks` loss partials to *d_loss_accum (if not null)
-void run_push_pipeline(ps_store* ps, uint32_t n, const float* d_upd, double* d_loss_accum, uint32_t loss_blocks,
-                       cudaStream_t s);
-// the two halves of the above: sort keysA (returns which buffer holds the result), then reduce and apply.
-// With d_scales, occurrence o contributes d_scales[o] times a shared source row of d_upd: row 2e for slot 0
-// of example e = o / slots, row 2e + 1 for its other slots.
+// sort keysA (values = occurrence index; returns which buffer holds the result), then reduce `upd` rows per key, apply them
+// to the store, and add the first `loss_blocks` loss partials to *d_loss_accum (if not null).  With d_scales, occurrence
+// o contributes d_scales[o] times a shared source row of d_upd: row 2e for slot 0 of example e = o / slots, row 2e + 1
+// for its other slots.
 int run_push_sort(ps_store* ps, uint32_t n, cudaStream_t s);
 int run_segment_sort(ps_store* ps, uint32_t n, cudaStream_t s);     // the same; also clears the counters of seg_lists
 void run_push_reduce(ps_store* ps, uint32_t n, int which, const float* d_upd, double* d_loss_accum,

@@ -242,24 +242,6 @@ void launch_get_location(ps_store* ps, const uint64_t* d_keys, uint64_t n, uint3
 }
 
 // ---------------------------------------------------------------- push ----
-__global__ void prepare_keys_kernel(const uint64_t* __restrict__ keys, uint64_t n, uint32_t* __restrict__ out,
-                                    uint64_t K, DevStatus* st, unsigned int epoch) {
-    const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= n) return;
-    const uint64_t key = keys[t];
-    if (key >= K) {
-        latch_error(st, epoch, PS_ERR_KEY_RANGE);
-        out[t] = (uint32_t)K;
-    } else {
-        out[t] = (uint32_t)key;
-    }
-}
-
-void launch_prepare_keys(ps_store* ps, const uint64_t* d_keys, uint64_t n, cudaStream_t s) {
-    PS_LAUNCH(ps, prepare_keys_kernel, div_up_u32(n, 256), 256, s, d_keys, n, ps->keysA, ps->cfg.num_keys,
-              ps->status, ps->epoch);
-}
-
 struct d4 {
     double x, y, z, w;
 };
@@ -1388,12 +1370,6 @@ void run_push_reduce(ps_store* ps, uint32_t n, int which, const float* d_upd, do
 #undef REDUCE_LAUNCH
 #undef REDUCE_ARGS
     launch_fixup(ps, sk, n, d_loss_accum, loss_blocks, false, tile_len, 0, s);
-}
-
-void run_push_pipeline(ps_store* ps, uint32_t n, const float* d_upd, double* d_loss_accum, uint32_t loss_blocks,
-                       cudaStream_t s) {
-    const int which = run_push_sort(ps, n, s);
-    run_push_reduce(ps, n, which, d_upd, d_loss_accum, loss_blocks, s);
 }
 
 }  // namespace psb

@@ -29,7 +29,7 @@ constexpr size_t kOffValsB = kOffValsA + pad256(kStaticMaxKeys * 4);
 constexpr size_t kOffHist = kOffValsB + pad256(kStaticMaxKeys * 4);
 constexpr size_t kOffSortCtl =
     kOffHist + pad256((size_t)kMaxSortPasses * ((kStaticMaxKeys + kSortTile - 1) / kSortTile) * kRadix * 4);
-constexpr size_t kStaticTiles = (kStaticMaxKeys + kReduceTile - 1) / kReduceTile;
+constexpr size_t kStaticTiles = (kStaticMaxKeys + 7) / 8;       // ps_push's tiles at these sizes: eight positions (reduce_tile)
 constexpr size_t kStaticGroups = (kStaticTiles + 63) / 64;
 constexpr size_t kOffCarry = kOffSortCtl + pad256(((size_t)kSortCtlWords + kStaticGroups) * 4);
 constexpr size_t kOffStarters =
@@ -38,7 +38,7 @@ constexpr size_t kOffStarterCount = kOffStarters + pad256(kStaticTiles * 16);
 constexpr size_t kOffGroupSum = kOffStarterCount + 256;
 constexpr size_t kStaticBytes = kOffGroupSum + pad256(kStaticGroups * (size_t)kStaticMaxRowLen * 8);
 
-// About 2.3 MB per GPU.  In host code this name is only a handle for the
+// About 9 MB per GPU.  In host code this name is only a handle for the
 // runtime; the address a kernel can use comes from cudaGetSymbolAddress.
 static __device__ __align__(256) unsigned char g_push_scratch[kStaticBytes];
 
@@ -124,8 +124,13 @@ extern "C" ps_status_t ps_push_static(void* d_store, const void* d_table, uint64
     if (cudaMemsetAsync(tmp.status, 0, sizeof(DevStatus), s) != cudaSuccess) return PS_ERR_CUDA;
     // ... and so must the two words of the sort's grid barrier, should an earlier call have given up inside it
     if (cudaMemsetAsync(tmp.sort_ctl, 0, 2 * sizeof(uint32_t), s) != cudaSuccess) return PS_ERR_CUDA;
-    launch_prepare_keys(&tmp, d_keys, n, s);
-    run_push_pipeline(&tmp, (uint32_t)n, d_updates, nullptr, 0, s);
+    // the kernels, and so the order of every sum, of ps_push
+    if (small_call(n)) {
+        run_small_push_keys(&tmp, d_keys, (uint32_t)n, d_updates, s);
+    } else {
+        const int which = radix_sort_keys64(&tmp, d_keys, (uint32_t)n, s, tmp.starter_count, reduce_groups(&tmp, (uint32_t)n));
+        run_push_reduce(&tmp, (uint32_t)n, which, d_updates, nullptr, 0, s);
+    }
     if (cudaGetLastError() != cudaSuccess) return PS_ERR_CUDA;
     unsigned int code = 0;
     if (cudaMemcpyAsync(&code, &tmp.status->sticky, sizeof code, cudaMemcpyDeviceToHost, s) != cudaSuccess)

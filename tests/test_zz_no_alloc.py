@@ -76,6 +76,23 @@ def test_push_static_after_a_failed_call_of_the_maximum_size():
     assert (a.export(table=False)[0].numpy() == b.export(table=False)[0].numpy()).all()
 
 
+@pytest.mark.parametrize("L", [4, 128, 256])
+@pytest.mark.parametrize("n", [9, 700, 4097, 8192, 8193, 12_345, ps.PS_PUSH_STATIC_MAX_KEYS])
+def test_push_static_adds_in_the_order_of_ps_push(n, L):
+    """Terms of 1e20 and of 1, of either sign, on a few keys: another order of the fp64 sums gives another row."""
+    K = 40
+    a, _ = make_pair(K, L, 2, 30, max_batch_keys=n, seed=n)
+    b, _ = make_pair(K, L, 2, 30, max_batch_keys=n, seed=n)
+    rng = np.random.default_rng(n + L)
+    keys = (rng.zipf(1.3, size=n) - 1) % K
+    upd = (rng.normal(size=(n, L)) * 10.0 ** rng.choice([0, 5, 20], size=(n, 1))).astype(np.float32)
+    a.push(dev(keys), dev(upd))
+    a.sync()
+    assert ps.ps_push_static(b.store, b.table, K, L, b.S, dev(keys), dev(upd)) == ps.PS_OK
+    ra, rb = a.export(table=False)[0], b.export(table=False)[0]
+    assert torch.equal(ra, rb), (ra != rb).sum()
+
+
 def test_push_static_enforces_its_limits_and_reports_bad_keys():
     K, L = 500, 8
     g, o = make_pair(K, L)
