@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(256, 2)
 loc_fused_kernel(const uint32_t* __restrict__ sk, uint32_t n, uint32_t span, uint2* table, uint32_t worker,
                  uint32_t N, uint64_t S, uint32_t K, unsigned long long* tops, uint32_t* stacks, char* store,
                  uint32_t row_bytes, uint32_t* block_counts, uint32_t* owner_counts, LocScratch sc,
-                 const uint32_t* __restrict__ busy_keys, uint32_t n_busy, uint32_t part_size, unsigned int* bar,
+                 const BusyKeys busy, uint32_t part_size, unsigned int* bar,
                  DevStatus* st, unsigned int epoch) {
     __shared__ uint32_t s_hist[kLocFastWorkers];    // phase 2a: keys leaving each owner from this block; phase 3: next stack position
     __shared__ uint32_t s_top[kLocFastWorkers];     // stack heights before the call (S < 2^32)
@@ -281,13 +281,10 @@ loc_fused_kernel(const uint32_t* __restrict__ sk, uint32_t n, uint32_t span, uin
             // A key that the call running beside this one also touches keeps its table entry and its row until
             // that call is through (loc_deferred_kernel); its slot and its old owner's stack are settled now.
             bool wait_for_it = false;
-            if (busy_keys) {
-                uint32_t lo2 = 0, hi2 = n_busy;
-                while (lo2 < hi2) {
-                    const uint32_t mid = (lo2 + hi2) >> 1;
-                    if (busy_keys[mid] < key) lo2 = mid + 1; else hi2 = mid;
-                }
-                wait_for_it = lo2 < n_busy && busy_keys[lo2] == key;
+            if (busy.keys) {
+                const uint32_t look = key < busy.run_base ? key : key - (key - busy.run_base) % busy.run_len;
+                const uint32_t at = lower_bound_u32(busy.keys, busy.n, look);
+                wait_for_it = at < busy.n && busy.keys[at] == look;
             }
             sc.mkey[m] = key;
             sc.flag[m] = wait_for_it ? 1u : 0u;
@@ -666,8 +663,7 @@ void run_localize_deferred(ps_store* ps, uint32_t worker, uint32_t n, cudaStream
 }
 
 // The call's keys (range-checked) have been sorted already; `which` says into which buffers.
-void run_localize(ps_store* ps, uint32_t worker, uint32_t n, int which, cudaStream_t s, const uint32_t* busy_keys,
-                  uint32_t n_busy) {
+void run_localize(ps_store* ps, uint32_t worker, uint32_t n, int which, cudaStream_t s, BusyKeys busy) {
     LocScratch sc = loc_scratch(ps);
     const uint32_t* sk = which ? ps->keysB : ps->keysA;
     uint32_t* owner_keys = which ? ps->keysA : ps->keysB;    // the buffer the sorted keys are not in
@@ -695,7 +691,7 @@ void run_localize(ps_store* ps, uint32_t worker, uint32_t n, int which, cudaStre
         uint32_t part_size = div_up_u32(ps->cfg.num_keys, ps->cfg.num_workers);
         void* args[] = {(void*)&sk, (void*)&n, (void*)&span, (void*)&table, (void*)&worker, (void*)&N, (void*)&S, (void*)&K,
                         (void*)&tops, (void*)&stacks, (void*)&store, (void*)&row_bytes, (void*)&block_counts,
-                        (void*)&owner_counts, (void*)&sc, (void*)&busy_keys, (void*)&n_busy, (void*)&part_size,
+                        (void*)&owner_counts, (void*)&sc, (void*)&busy, (void*)&part_size,
                         (void*)&bar, (void*)&st, (void*)&epoch};
         if (ps->prof) prof_before(ps, "loc_fused_kernel", s);
         cudaLaunchCooperativeKernel((const void*)loc_fused_kernel, dim3(grid_f), dim3(256), args, kLocSmem, s);

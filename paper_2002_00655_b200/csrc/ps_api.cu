@@ -208,9 +208,12 @@ static bool begin_sort(ps_store* ps, SortSet* ss, cudaStream_t s, bool reads_tab
 }
 static bool end_sort(ps_store* ps, cudaStream_t s, cudaStream_t where) { return where == s || join_side(ps, s); }
 // after the call's sort has been enqueued: where its sorted keys are, for ps_localize_beside
-static bool sorted_keys_at(ps_store* ps, SortSet* ss, int which, uint32_t n, cudaStream_t where) {
+static bool sorted_keys_at(ps_store* ps, SortSet* ss, int which, uint32_t n, cudaStream_t where, uint64_t run_base = kSentinelPad,
+                           uint32_t run_len = 1) {
     ss->sorted_which = which;
     ss->sorted_n = n;
+    ss->run_base = (uint32_t)run_base;
+    ss->run_len = run_len;
     ps->last_set = ss;
     return cudaEventRecord(ps->ev_sorted, where) == cudaSuccess;
 }
@@ -512,13 +515,12 @@ ps_status_t ps_localize_beside(ps_store_t* ps, uint32_t worker, const uint64_t* 
     if (ps->loc_pending && cudaStreamWaitEvent(ls, ps->ev_loc, 0) != cudaSuccess) return PS_ERR_CUDA;
     if (cudaStreamWaitEvent(ls, ps->ev_before, 0) != cudaSuccess || cudaStreamWaitEvent(ls, ps->ev_sorted, 0) != cudaSuccess)
         return PS_ERR_CUDA;
-    const uint32_t* busy_keys = busy->sorted_which ? busy->keysB : busy->keysA;
-    const uint32_t n_busy = busy->sorted_n;
+    const BusyKeys busy_keys = {busy->sorted_which ? busy->keysB : busy->keysA, busy->sorted_n, busy->run_base, busy->run_len};
     const cudaEvent_t busy_done = busy->ev_free;
     SortSet* ss = next_set(ps);
     ss->sorted_which = -1;
     const int which = radix_sort_keys64(ps, d_keys, (uint32_t)n, ls, nullptr, 0);
-    run_localize(ps, worker, (uint32_t)n, which, ls, busy_keys, n_busy);
+    run_localize(ps, worker, (uint32_t)n, which, ls, busy_keys);
     if (cudaStreamWaitEvent(ls, busy_done, 0) != cudaSuccess) return PS_ERR_CUDA;
     run_localize_deferred(ps, worker, (uint32_t)n, ls);
     // (a later sort that reads the table forks after the caller's stream, which waits for ev_loc: table_dirty)
@@ -647,13 +649,13 @@ ps_status_t ps_step_rescal(ps_store_t* ps, const uint32_t* d_s, const uint32_t* 
         return after_launch();
     }
     // entity slots and one slot per data point for its relation are sorted; the matrices' rows follow from the latter
-    // (so the sorted keys do not list them, and a relocation is not run beside this call)
     const uint32_t occ = (uint32_t)((3 + (uint64_t)n_neg) * n);
     SortSet* ss = next_set(ps);
     cudaStream_t q;
     if (!begin_sort(ps, ss, s, false, &q)) return PS_ERR_CUDA;
     launch_keys_rescal(ps, B, q);
     const int which = run_segment_sort(ps, occ, q);
+    if (!sorted_keys_at(ps, ss, which, occ, q, rel_key_base, dim)) return PS_ERR_CUDA;
     launch_segments(ps, occ, which, dim, rel_key_base, (uint32_t)n, q);
     if (!end_sort(ps, s, q)) return PS_ERR_CUDA;
     run_rescal_sorted(ps, B, which, n_loss, d_loss_accum, s);

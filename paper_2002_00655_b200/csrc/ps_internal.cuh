@@ -65,6 +65,7 @@ struct SortSet {
     bool loc_reader;                // a relocation on another stream reads this set's sorted keys (ps_localize_beside)
     int sorted_which;               // which key buffer holds the call's sorted keys (-1: the call sorted none)
     uint32_t sorted_n;
+    uint32_t run_base, run_len;     // sorted keys from run_base on stand for run_len consecutive keys (RESCAL: a matrix's rows)
 };
 
 }  // namespace psb
@@ -329,8 +330,11 @@ void run_rescal_sorted(ps_store* ps, const RescalBatch& B, int which, uint32_t n
 // ---- localize.cu ----
 // busy_keys: sorted keys of a call that may run beside this relocation (null: none); moving keys among them keep
 // table entry and row until run_localize_deferred, which the caller enqueues once that call is through.
-void run_localize(ps_store* ps, uint32_t worker, uint32_t n, int which, cudaStream_t s,
-                  const uint32_t* busy_keys = nullptr, uint32_t n_busy = 0);
+struct BusyKeys {
+    const uint32_t* keys;
+    uint32_t n, run_base, run_len;      // as in SortSet
+};
+void run_localize(ps_store* ps, uint32_t worker, uint32_t n, int which, cudaStream_t s, BusyKeys busy = {nullptr, 0u, 0u, 1u});
 // Few keys: the whole call, without a sort, in one launch on the caller's stream.
 bool localize_is_small(const ps_store* ps, uint64_t n);
 void run_localize_small(ps_store* ps, uint32_t worker, const uint64_t* d_keys, uint32_t n, cudaStream_t s);

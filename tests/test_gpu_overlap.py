@@ -91,3 +91,36 @@ def test_mf_steps_with_the_next_batch_localized_beside_the_step(path):
     assert close(float(g.loss.cpu()[0]), o.loss[0])
     st = ps.ps_localize_stats(g.h)
     assert st["deferred"] > 0 and st["moved"] > st["deferred"]
+
+
+@pytest.mark.parametrize("pipelined", [False, True])
+@pytest.mark.parametrize("d,n,rels", [(16, 900, 40), (100, 700, 9)])
+def test_rescal_steps_with_the_next_batch_localized_beside_the_step(d, n, rels, pipelined):
+    """The step's sorted keys hold one key per relation for all rows of its matrix: each of those rows waits for the step, the
+    others (relations the batch does not have, single rows of one) are relocated beside it."""
+    E, n_neg, N = 4_000, 10, 8
+    K = E + rels * d
+    rng = np.random.default_rng(d)
+    rows = np.abs(rng.normal(0.2, 0.1, size=(K, 2 * d))).astype(np.float32)
+    pair = [make_pair(K, 2 * d, N, K, rows=rows, max_batch_keys=(2 + n_neg + d) * n) for _ in range(2)]
+    (ref, _), (g, _) = pair
+    for s in (ref, g):
+        ps.ps_set_pipelining(s.h, pipelined)
+    side = torch.cuda.Stream()
+    steps = []
+    for b in range(6):
+        a = [dev(x, torch.int32) for x in (rng.integers(0, E, size=n), rng.integers(0, rels // 2 + b, size=n),
+                                           rng.integers(0, E, size=n), rng.integers(0, E, size=(n, n_neg)))]
+        nxt = np.concatenate([rng.integers(0, E, size=2_000), E + rng.integers(0, rels * d, size=600), E + np.arange(d)])
+        steps.append((a + [dev(rng.integers(0, 2, size=(n, n_neg)).astype(np.uint8))], dev(nxt)))
+    torch.cuda.synchronize()
+    for b, (a, nxt) in enumerate(steps):
+        ps.ps_step_rescal(ref.h, *a, n_neg, E, d, 0.1, 1e-8, ref.loss)
+        ref.localize(b % N, nxt)
+        ps.ps_step_rescal(g.h, *a, n_neg, E, d, 0.1, 1e-8, g.loss)
+        ps.ps_localize_beside(g.h, b % N, nxt, side)
+    ref.sync()
+    g.sync()
+    same_state(ref, g, "relocations beside RESCAL steps")
+    sr, sg = ps.ps_localize_stats(ref.h), ps.ps_localize_stats(g.h)
+    assert sg["deferred"] > 0 and {**sg, "deferred": 0} == {**sr, "deferred": 0} and sr["moved"] > sg["deferred"]
