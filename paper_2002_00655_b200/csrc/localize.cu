@@ -536,7 +536,10 @@ loc_small_kernel(const uint64_t* keys, uint32_t n, uint2* table, uint32_t worker
         local += (uint32_t)__syncthreads_count(first && !moves);
     }
     if ((unsigned long long)total > top_w) {                // the same decision in every block
-        if (b == 0 && tid == 0) latch_error(st, 0u, PS_ERR_CAPACITY);
+        if (b == 0 && tid == 0) {
+            latch_error(st, 0u, PS_ERR_CAPACITY);
+            st->loc_requested += n;
+        }
         return;
     }
     // ---- the block's eighth of the positions, T neighbouring lanes per position ----

@@ -105,6 +105,18 @@ def test_localize_around_the_limit_of_the_single_launch(N, L, counts):
     compare_state(g, o, exact_rows=True, what="bad key")
 
 
+@pytest.mark.parametrize("n", [600, 3_000])
+def test_requested_counts_a_localize_that_finds_no_room(n):
+    """On either side of the limit of the single launch."""
+    K = 8_000
+    g, _ = make_pair(K, 8, 2, K // 2 + 100, max_batch_keys=4096)
+    g.localize(0, dev(np.arange(K - n, K)))
+    assert g.sync(check=False) == ps.PS_ERR_CAPACITY
+    g.localize(0, dev(np.arange(K - 50, K + 50) % K))
+    g.sync()
+    assert ps.ps_localize_stats(g.h) == {"requested": n + 100, "moved": 50, "already_local": 50, "moved_again": 0, "deferred": 0}
+
+
 @pytest.mark.parametrize("n", [8_193, 16_384, 32_767, 32_768, 32_769, 303_104, 303_105, 606_300])
 @pytest.mark.parametrize("K", [200, 70_000])
 def test_sorted_pushes_around_the_limits_of_the_sorts(n, K):
