@@ -391,23 +391,23 @@ __device__ __forceinline__ float adagrad_step(float g, float x, float lr, float 
 // special-function unit instead of two, and that unit (16 lanes per clock and SM, conversions to and from fp64 included)
 // is what bounds the reductions with AdaGrad.  Which form a value takes depends on that value alone (so results do not
 // depend on how values are grouped), but one test serves all N, so that their chains interleave.  True if that form was taken
-// by all, which it is not where one is not finite.
+// by all and all steps are finite: x < 3e38 bounds g by 2e19, and lr is bounded too.
 template <int N>
 __device__ __forceinline__ bool adagrad_steps(const float (&g)[N], const float (&x)[N], float lr, float eps, float (&step)[N]) {
     float er[N];
-    bool fine = true;
+    bool fine = fabsf(lr) < 1e18f;                                      // (false for a NaN, here and below)
 #pragma unroll
     for (int i = 0; i < N; ++i) {
         float r;
         asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x[i]));      // (zero or denormal: infinite, the other form)
         er[i] = __fmul_rn(eps, r);
         step[i] = __fmul_rn(__fmul_rn(-lr, g[i]), fmaf(-er[i], r, r));
-        fine = fine && er[i] < 2e-4f && x[i] < 3e38f;                   // (false for a NaN)
+        fine = fine && fabsf(er[i]) < 2e-4f && x[i] < 3e38f;
     }
     if (fine) return true;
 #pragma unroll
     for (int i = 0; i < N; ++i)
-        if (!(er[i] < 2e-4f && x[i] < 3e38f)) step[i] = adagrad_step(g[i], x[i], lr, eps);
+        if (!(fabsf(er[i]) < 2e-4f && x[i] < 3e38f)) step[i] = adagrad_step(g[i], x[i], lr, eps);
     return false;
 }
 __device__ __forceinline__ void adagrad_steps4(const float4& g, const float4& x, float lr, float eps, float4& step) {

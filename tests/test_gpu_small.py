@@ -167,6 +167,29 @@ def test_rescal_steps_with_a_sort(d, n_neg, batch, ents, rels):
     rescal_run(d, n_neg, batch, ents, rels, steps=2, single_step=True, G=0.3)
 
 
+@pytest.mark.parametrize("lr,eps", [(float("nan"), 1e-8), (float("inf"), 1e-8), (0.1, -1e-3), (0.1, 0.05)])
+@pytest.mark.parametrize("mode,n", [("kge", 40), ("kge", 700), ("rescal", 40), ("rescal", 700)])
+def test_adagrad_with_unusual_rates(mode, n, lr, eps):
+    """Learning rates that are not finite, an eps that is negative or not small against the accumulators' roots:
+    without and with a sort, keys that occur once, a few times and hundreds of times."""
+    E, R, n_neg, L = 1_500, 3, 10, 48
+    d = L // 4 if mode == "kge" else L // 2
+    rng = np.random.default_rng(n)
+    rows = np.abs(rng.normal(0, 0.4, size=(E + R * (d if mode == "rescal" else 1), L))).astype(np.float32) + 0.05
+    g, o = make_pair(len(rows), L, rows=rows, max_batch_keys=(3 + n_neg + d) * n)
+    s, t, ne = (((rng.zipf(1.3, size=z) - 1) % E).astype(np.uint32) for z in (n, n, (n, n_neg)))
+    r, ns = rng.integers(0, R, size=n).astype(np.uint32), rng.integers(0, 2, size=(n, n_neg)).astype(np.uint8)
+    step = ps.ps_step_kge if mode == "kge" else ps.ps_step_rescal
+    step(g.h, *(dev(x, torch.int32) for x in (s, r, t, ne)), dev(ns), n_neg, E, d, lr, eps, g.loss)
+    getattr(o, "step_" + mode)(s, r, t, ne, ns, E, d, lr, eps)
+    g.sync()
+    got = g.export(table=False)[0].numpy()
+    assert (np.isfinite(got) == np.isfinite(o.rows)).all()
+    assert (np.isnan(got) == np.isnan(o.rows)).mean() > 0.999       # (inf - inf: which of the two a sum of either sign becomes)
+    ok = np.isfinite(got)
+    assert close(got[ok], o.rows[ok]).all()
+
+
 @pytest.mark.parametrize("batch", [512, 8192])
 def test_losses_of_overlapped_host_steps_reach_pinned_and_pageable_words(batch):
     """Steps without and with a sort, each with a loss word of its own, every other one in pageable memory (a copy there, a
