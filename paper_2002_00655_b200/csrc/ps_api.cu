@@ -56,6 +56,7 @@ WsLayout ws_layout(const ps_config_t& cfg, uint64_t max_keys) {
     l.group_sum = take(groups * (size_t)cfg.row_len * 8);
     l.loss_partial = take(tmax<size_t>(kMaxLossBlocks, mk / 256 + 1) * 8);
     l.apply_rows = take(mk * 8);
+    l.hot_tickets = take((size_t)kHotStretches * kMaxHot * 4);
     for (int b = 0; b < kHostStages; ++b) l.staging[b] = take(mk * 8 + 256);
     l.total = off;
     return l;
@@ -309,6 +310,7 @@ ps_status_t ps_create(const ps_config_t* cfg, void* d_store, void* d_table, void
     ps->tile_cap = (uint32_t)tmin<size_t>(l.reduce_tiles, 0xffffffffu);
     ps->loss_partial = (double*)(ps->ws + l.loss_partial);
     ps->apply_rows = (uint64_t*)(ps->ws + l.apply_rows);
+    ps->hot_tickets = (unsigned int*)(ps->ws + l.hot_tickets);
     for (int b = 0; b < kHostStages; ++b) ps->stagings[b] = ps->ws + l.staging[b];
     ps->staging = ps->stagings[0];
     int sms = 0;
@@ -317,7 +319,8 @@ ps_status_t ps_create(const ps_config_t* cfg, void* d_store, void* d_table, void
         return PS_ERR_CUDA;
     }
     ps->sm_count = sms;
-    if (cudaMemset(ps->status, 0, sizeof(DevStatus)) != cudaSuccess) {
+    if (cudaMemset(ps->status, 0, sizeof(DevStatus)) != cudaSuccess ||
+        cudaMemset(ps->hot_tickets, 0, (size_t)kHotStretches * kMaxHot * 4) != cudaSuccess) {
         delete ps;
         return PS_ERR_CUDA;
     }

@@ -22,6 +22,8 @@ constexpr uint32_t kTiledRow = 512;              // ... rows up to this many val
 constexpr uint32_t kMidTiles = 4096;             // shorter tiles than 32 positions that a call has at most
 constexpr int kMaxLossBlocks = 4096;
 constexpr uint32_t kSmallOcc = 8192;             // calls of at most this many key occurrences are reduced without a sort (small.cu)
+constexpr uint32_t kMaxHot = 8;                  // keys of such a call that all blocks share, at most
+constexpr uint32_t kHotStretches = 128;          // ... on rows of at most this many stretches of columns
 constexpr int kHostStages = 3;                   // staging areas for batches that arrive from host memory
 constexpr int kSortSets = 4;                     // calls whose key sort may be in flight at once (see SortSet)
 constexpr int kSideStreams = 3;                  // internal streams that calls with a long sort take in turn
@@ -101,6 +103,7 @@ struct ps_store {
     double* carry;                  // nReduceTiles x 2 x row_len partial sums of segments that span tiles
     uint4* starters;                // {tile, key, row} of the tiles that start a border-crossing segment
     unsigned int* starter_count;
+    unsigned int* hot_tickets;      // calls without a sort: per stretch of columns and hot key, zero between calls
     uint32_t tile_cap;              // tiles that carry and starters have room for
     double* loss_partial;           // max(kMaxLossBlocks, one per 256 key occurrences)
     uint64_t* apply_rows;           // per sorted position: address of the row staged there, or all ones
@@ -144,7 +147,7 @@ namespace psb {
 struct WsLayout {
     size_t status, keysA[kSortSets], keysB[kSortSets], valsA[kSortSets], valsB[kSortSets], tile_state[kSortSets],
         sort_ctl[kSortSets], rec[kSortSets], cellpos[kSortSets], mf_dup[kSortSets], mf_tickets[kSortSets], scan_sums, loc_counts, loc_scratch, upd, carry, group_sum, starters[kSortSets], starter_count[kSortSets],
-        loss_partial, apply_rows, staging[kHostStages], total, reduce_tiles;
+        loss_partial, apply_rows, hot_tickets, staging[kHostStages], total, reduce_tiles;
 };
 WsLayout ws_layout(const ps_config_t& cfg, uint64_t max_keys);
 

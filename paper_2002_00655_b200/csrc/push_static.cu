@@ -36,7 +36,8 @@ constexpr size_t kOffStarters =
     kOffCarry + pad256(kStaticTiles * 2 * (size_t)kStaticMaxRowLen * 8);
 constexpr size_t kOffStarterCount = kOffStarters + pad256(kStaticTiles * 16);
 constexpr size_t kOffGroupSum = kOffStarterCount + 256;
-constexpr size_t kStaticBytes = kOffGroupSum + pad256(kStaticGroups * (size_t)kStaticMaxRowLen * 8);
+constexpr size_t kOffTickets = kOffGroupSum + pad256(kStaticGroups * (size_t)kStaticMaxRowLen * 8);
+constexpr size_t kStaticBytes = kOffTickets + (size_t)kHotStretches * kMaxHot * 4;      // (zero to begin with, and after every call)
 
 // About 9 MB per GPU.  In host code this name is only a handle for the
 // runtime; the address a kernel can use comes from cudaGetSymbolAddress.
@@ -113,6 +114,7 @@ extern "C" ps_status_t ps_push_static(void* d_store, const void* d_table, uint64
     tmp.group_done = tmp.sort_ctl + kSortCtlWords;
     tmp.group_sum = (double*)(dev.scratch + kOffGroupSum);
     tmp.tile_cap = (uint32_t)kStaticTiles;
+    tmp.hot_tickets = (unsigned int*)(dev.scratch + kOffTickets);
     tmp.carry = (double*)(dev.scratch + kOffCarry);
     tmp.starters = (uint4*)(dev.scratch + kOffStarters);
     tmp.starter_count = (unsigned int*)(dev.scratch + kOffStarterCount);

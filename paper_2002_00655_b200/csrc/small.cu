@@ -7,6 +7,13 @@
 // number of occurrences of each in a table in shared memory, and a warp per distinct key adds its occurrences' rows in
 // the order of the call, in fp64, and rounds once, as the sorted reduction does.  A key with more than kShortRun
 // occurrences is shared by the block's warps (a range of the list each, partial sums added in range order).
+// Hot keys, which are a large part of the call, are shared by all blocks: 8,192 occurrences of one key took its block 118 us
+// at 128 values and 242 at 400, where a sort and the tiled reduction take 39 and 52.  Every block finds the same ones by itself
+// in a sample of kSample keys at jittered positions (hot_hits of one key make it hot: a key that is a quarter of the call is
+// missed once in some hundred calls, which costs time only; at four in a hundred the largest key of 6,000 Zipf(0.9) ones,
+// 300 occurrences, is shared as well: a pull, push and relocation of them take 39 us instead of 26).  The call is cut into
+// pieces, a block sums a hot key's occurrences of one piece and parks the sum; the last block to finish a key adds its pieces
+// in order.
 // What grows with the call is the reading of all keys by every block: kSmallOcc is where the sort takes over.
 // (A first form compared every occurrence with all others, 128 keys per instruction: 1,200 to 1,800 warp instructions
 // per occurrence, 11 us at 2,048 and 27 us at 3,328 occurrences of AdaGrad.)
@@ -25,6 +32,10 @@ constexpr int kThreads = 512;
 constexpr int kWarps = kThreads / 32;
 constexpr uint32_t kShortRun = 8;               // occurrences of one key that a warp adds alone
 constexpr int kTableBits = 10, kTable = 1 << kTableBits;
+constexpr uint32_t kSample = 64;
+__host__ __device__ constexpr uint32_t hot_hits(int kCh) { return kCh == 1 ? 7 : 10; }   // (a warp has half as many rows of several column blocks in flight)
+constexpr uint32_t kHotCall = 2049;             // smaller calls are not sampled: 2,048 occurrences of one key take 33 us, sorted 31
+constexpr uint32_t kHotPiece = 256;             // occurrences per piece, at least
 static_assert(kSmallOcc <= 32 * kThreads, "a lane per round of the bucket's selection");
 
 // which of the blocks takes a key: a multiplicative hash, so that neighbouring keys (the frequent ones) are spread
@@ -54,10 +65,139 @@ struct SmallArgs {
     uint32_t loss_blocks;
     double* loss_accum;
     DevStatus* st;
+    uint32_t pieces, piece_len;     // of the call, for hot keys; piece_len a multiple of kWarps
+    double* parked;                 // [stretch][hot key][piece][stretch_vals]
+    uint32_t stretch_vals;
+    unsigned int* tickets;          // [stretch][hot key], zero between calls
 };
 
-// kCh: float4 per lane; blockIdx.y counts stretches of 32 kCh float4 of the row
+// position s of the sample: one in each of kSample equal parts of the call, so that no period of the batch escapes it
+__device__ __forceinline__ uint32_t sample_pos(uint32_t s, uint32_t n) {
+    const uint32_t jitter = (s * 0x9e3779b1u) >> 16;
+    return (uint32_t)(((uint64_t)(s * 0x10000u + jitter) * n) >> 22);
+}
+static_assert(kSample * 8 == kThreads && kSample == 1u << 6, "sample_pos divides by 2^16 times this");
+
+__device__ __forceinline__ uint32_t key_at(const SmallArgs& A, uint32_t i) {     // kSentinelPad: out of range
+    if (A.keys64) {
+        const uint64_t k = A.keys64[i];
+        return k < A.K ? (uint32_t)k : kSentinelPad;
+    }
+    return A.keys32[i];
+}
+
+
+// Hot keys: a piece of the call at a time, a sixteenth of it per warp, kFly rows of a warp in flight.  (A function of its own, so
+// that the registers of calls without hot keys stay as they are.)
 template <int kMode, int kCh>
+__device__ __noinline__ void hot_keys(const SmallArgs A, const uint32_t* s_hot, uint32_t n_hot, acc4 (*s_part)[32], uint32_t* s_ticket) {
+    constexpr int kHalves = kMode == kAdaGrad ? 2 : 1, kFly = kCh == 4 ? 2 : 4;
+    const unsigned full = 0xffffffffu;
+    const uint32_t tid = threadIdx.x, lane = tid & 31, w = tid >> 5, n = A.n, f0 = blockIdx.y * (32 * kCh) + lane;
+    for (uint32_t task = blockIdx.x; task < n_hot * A.pieces; task += gridDim.x - 1) {
+        const uint32_t h = task / A.pieces, p = task - h * A.pieces, k = s_hot[h], slot = blockIdx.y * kMaxHot + h;
+        float4* target = A.store + phys_row(A.table[k], A.S) * A.L4;
+        float4 G[kCh];                          // kAdaGrad: the accumulators before the call
+        acc4 a[kHalves][kCh];
+#pragma unroll
+        for (int c = 0; c < kCh; ++c) {
+            G[c] = kMode == kAdaGrad && f0 + 32 * c < A.F4 ? target[A.F4 + f0 + 32 * c] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int half = 0; half < kHalves; ++half) a[half][c] = acc4{0.0, 0.0, 0.0, 0.0};
+        }
+        const uint32_t from = tmin(p * A.piece_len + w * (A.piece_len / kWarps), n), to = tmin(from + A.piece_len / kWarps, n);
+        for (uint32_t b = from; b < to; b += 32) {
+            for (unsigned todo = __ballot_sync(full, b + lane < to && key_at(A, b + lane) == k); todo;) {
+                float4 u[kFly][kCh];
+                float sc[kFly];
+                bool have[kFly];
+#pragma unroll
+                for (int q = 0; q < kFly; ++q) {
+                    have[q] = todo != 0;
+                    const uint32_t o = b + (todo ? __ffs(todo) - 1 : 0);
+                    todo &= todo - 1;           // 0 stays 0
+                    uint64_t row = o;
+                    sc[q] = 1.f;
+                    if (kMode == kScaled) {
+                        sc[q] = A.scales[o];
+                        const uint32_t e = o / A.slots;
+                        row = 2u * e + (o != e * A.slots ? 1u : 0u);
+                    }
+#pragma unroll
+                    for (int c = 0; c < kCh; ++c)
+                        u[q][c] = have[q] && f0 + 32 * c < A.F4 ? A.upd[row * A.F4 + f0 + 32 * c] : make_float4(0.f, 0.f, 0.f, 0.f);
+                }
+#pragma unroll
+                for (int q = 0; q < kFly; ++q) {
+                    if (!have[q]) break;
+#pragma unroll
+                    for (int c = 0; c < kCh; ++c) {
+                        float4 v = u[q][c];
+                        if (kMode == kAdaGrad) {
+                            const float4 sq = make_float4(v.x * v.x, v.y * v.y, v.z * v.z, v.w * v.w);
+                            adagrad_steps4(u[q][c], make_float4(G[c].x + sq.x, G[c].y + sq.y, G[c].z + sq.z, G[c].w + sq.w), A.lr, A.eps, v);
+                            acc4& g = a[kHalves - 1][c];
+                            g.x += (double)sq.x; g.y += (double)sq.y; g.z += (double)sq.z; g.w += (double)sq.w;
+                        }
+                        const double d = (double)sc[q];
+                        a[0][c].x += d * (double)v.x; a[0][c].y += d * (double)v.y;
+                        a[0][c].z += d * (double)v.z; a[0][c].w += d * (double)v.w;
+                    }
+                }
+            }
+        }
+        // the warps' sums in warp order, parked
+        double* const mine = A.parked + (uint64_t)slot * A.pieces * A.stretch_vals;
+        const uint32_t per_half = tmin<uint32_t>(32 * kCh, A.F4);                // float4 from one half's sums to the other's
+#pragma unroll
+        for (int half = 0; half < kHalves; ++half)
+#pragma unroll
+            for (int c = 0; c < kCh; ++c) {
+                s_part[w][lane] = a[half][c];
+                __syncthreads();
+                if (w == 0 && f0 + 32 * c < A.F4) {
+                    acc4 tot = s_part[0][lane];
+                    for (int i = 1; i < kWarps; ++i) {
+                        tot.x += s_part[i][lane].x; tot.y += s_part[i][lane].y;
+                        tot.z += s_part[i][lane].z; tot.w += s_part[i][lane].w;
+                    }
+                    double2* to2 = reinterpret_cast<double2*>(mine + (uint64_t)p * A.stretch_vals) + 2 * (half * per_half + 32 * c + lane);
+                    to2[0] = make_double2(tot.x, tot.y);
+                    to2[1] = make_double2(tot.z, tot.w);
+                }
+                __syncthreads();
+            }
+        if (w == 0) __threadfence();
+        __syncthreads();
+        if (tid == 0) {
+            *s_ticket = atomicAdd(A.tickets + slot, 1u);
+            if (*s_ticket == A.pieces - 1) A.tickets[slot] = 0u;                // (nobody draws it again in this call)
+        }
+        __syncthreads();
+        if (*s_ticket != A.pieces - 1) continue;
+        __threadfence();
+        if (w < kHalves * kCh) {                // a warp per half and column block adds the pieces
+            const uint32_t half = w / kCh, c = w % kCh, f = f0 + 32 * c;
+            if (f < A.F4) {
+                const double2* at2 = reinterpret_cast<const double2*>(mine) + 2 * (half * per_half + 32 * c + lane);
+                acc4 tot = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 8
+                for (uint32_t i = 0; i < A.pieces; ++i) {
+                    const double2 x = __ldcg(at2 + (uint64_t)i * (A.stretch_vals / 2)), y = __ldcg(at2 + (uint64_t)i * (A.stretch_vals / 2) + 1);
+                    tot.x += x.x; tot.y += x.y; tot.z += y.x; tot.w += y.y;
+                }
+                float4 r = target[half * A.F4 + f];
+                r.x = (float)((double)r.x + tot.x); r.y = (float)((double)r.y + tot.y);
+                r.z = (float)((double)r.z + tot.z); r.w = (float)((double)r.w + tot.w);
+                target[half * A.F4 + f] = r;
+            }
+        }
+    }
+}
+
+// kCh: float4 per lane; blockIdx.y counts stretches of 32 kCh float4 of the row.  kHot: hot keys are looked for (compiled apart:
+// that costs calls without any half a microsecond)
+template <int kMode, int kCh, bool kHot>
 __global__ void __launch_bounds__(kThreads, kCh == 1 ? 2 : 1) small_push_kernel(const SmallArgs A) {
     extern __shared__ __align__(16) uint32_t s_dyn[];
     uint32_t* const s_key = s_dyn;                          // the bucket: keys of its occurrences, in the order of the call
@@ -66,6 +206,8 @@ __global__ void __launch_bounds__(kThreads, kCh == 1 ? 2 : 1) small_push_kernel(
     __shared__ uint16_t s_firsts[kTable];
     __shared__ uint32_t s_cnt[kWarps], s_n_firsts, s_over;
     __shared__ acc4 s_part[kWarps][32];
+    __shared__ __align__(16) uint32_t s_sample[kHot ? kSample : 4];
+    __shared__ uint32_t s_hot[kMaxHot], s_hot_mask[kWarps], s_ticket;
     constexpr int kHalves = kMode == kAdaGrad ? 2 : 1;      // AdaGrad: sums for the parameters and for their accumulators
     constexpr int kFly = kCh == 1 ? 4 : (kCh == 2 && kMode != kAdaGrad ? 4 : 2) / (kCh == 4 ? 2 : 1);      // update rows a warp has in flight
     const unsigned full = 0xffffffffu;
@@ -85,6 +227,10 @@ __global__ void __launch_bounds__(kThreads, kCh == 1 ? 2 : 1) small_push_kernel(
     }
     if (tid == 0) s_n_firsts = s_over = 0;
     pdl_wait();
+    uint32_t sample = K;
+    if constexpr (kHot) {
+        if (tid < (int)kSample) sample = key_at(sample_pos(tid, n));
+    }
     // ---- the occurrences whose keys fall into this block's bucket; warp w looks at its 16th of the call ----
     const uint32_t rounds = (n + kThreads - 1) / kThreads;  // at most 32: lane r keeps the bucket's lanes of round r
     const uint32_t w0 = w * rounds * 32;
@@ -100,6 +246,9 @@ __global__ void __launch_bounds__(kThreads, kCh == 1 ? 2 : 1) small_push_kernel(
         cnt_w += __popc(m);
     }
     if (lane == 0) s_cnt[w] = cnt_w;
+    if constexpr (kHot) {
+        if (tid < (int)kSample) s_sample[tid] = sample;
+    }
     if (__syncthreads_or(bad)) {                // the same decision in every block: nothing has been written yet
         if (A.keys64 && bucket == 0 && blockIdx.y == 0 && tid == 0) latch_error(A.st, 0u, PS_ERR_KEY_RANGE);
         return;
@@ -118,6 +267,51 @@ __global__ void __launch_bounds__(kThreads, kCh == 1 ? 2 : 1) small_push_kernel(
             *A.loss_accum += tot;
         }
         return;
+    }
+    if constexpr (kHot) {                       // eight threads compare a key of the sample with all of it
+        const uint32_t sampled = s_sample[tid / 8];
+        uint32_t hits = 0;
+#pragma unroll
+        for (uint32_t i = 0; i < kSample / 32; ++i) {
+            const uint4 x = reinterpret_cast<const uint4*>(s_sample)[8 * i + tid % 8];
+            hits += (x.x == sampled) + (x.y == sampled) + (x.z == sampled) + (x.w == sampled);
+        }
+        hits += __shfl_xor_sync(full, hits, 1);
+        hits += __shfl_xor_sync(full, hits, 2);
+        hits += __shfl_xor_sync(full, hits, 4);
+        bool is_hot = hits >= hot_hits(kCh) && sampled < K && tid % 8 == 0;
+        if (__builtin_expect(__syncthreads_or(is_hot), 0)) {
+            if (is_hot)                         // (its first place in the sample)
+                for (int i = 0; i < tid / 8; ++i) is_hot = is_hot && s_sample[i] != sampled;
+            const unsigned mine = __ballot_sync(full, is_hot);
+            if (lane == 0) s_hot_mask[w] = mine;
+            __syncthreads();
+            uint32_t rank = __popc(mine & ((1u << lane) - 1u)), n_hot = 0;
+            for (int i = 0; i < kWarps; ++i) {
+                if (i < w) rank += __popc(s_hot_mask[i]);
+                n_hot += __popc(s_hot_mask[i]);
+            }
+            n_hot = tmin(n_hot, kMaxHot);       // the same list, in the order of the sample, in every block
+            if (is_hot && rank < kMaxHot) s_hot[rank] = sampled;
+            __syncthreads();
+            // they leave the block's list
+            cnt_w = 0;
+            for (unsigned some = __ballot_sync(full, mask_of != 0); some; some &= some - 1) {
+                const int r = __ffs(some) - 1;
+                const unsigned mk = __shfl_sync(full, mask_of, r);
+                bool keep = (mk >> lane) & 1u;
+                if (keep) {
+                    const uint32_t k = key_at(w0 + r * 32 + lane);
+                    for (uint32_t h = 0; h < n_hot; ++h) keep = keep && k != s_hot[h];
+                }
+                const unsigned kept = __ballot_sync(full, keep);
+                if (lane == r) mask_of = kept;
+                cnt_w += __popc(kept);
+            }
+            if (lane == 0) s_cnt[w] = cnt_w;
+            hot_keys<kMode, kCh>(A, s_hot, n_hot, s_part, &s_ticket);
+            __syncthreads();
+        }
     }
     uint32_t at = 0, m = 0;                     // where the warp's part of the list begins; the length of the list
 #pragma unroll
@@ -340,15 +534,26 @@ __global__ void __launch_bounds__(kThreads, kCh == 1 ? 2 : 1) small_push_kernel(
     }
 }
 
-template <int kMode, int kCh>
-void launch_as(ps_store* ps, const SmallArgs& a, uint32_t strips, cudaStream_t s) {
+template <int kMode, int kCh, bool kHot>
+void launch_kernel(ps_store* ps, const SmallArgs& a, uint32_t strips, cudaStream_t s) {
     // about a dozen occurrences per block of 16 warps, two blocks per SM at most (more would only read the keys again)
     const uint32_t buckets = tmax<uint32_t>(1u, tmin<uint32_t>(div_up_u32(a.n, 12), (uint32_t)ps->sm_count * 2 - 1));
     const size_t smem = ((size_t)a.n * 6 + 15) & ~(size_t)15;
     static std::atomic<unsigned long long> smem_set{0};
-    opt_in_smem((const void*)small_push_kernel<kMode, kCh>, (size_t)kSmallOcc * 6, &smem_set);
+    opt_in_smem((const void*)small_push_kernel<kMode, kCh, kHot>, (size_t)kSmallOcc * 6, &smem_set);
     const char* name = kMode == kAdaGrad ? "small_push_kernel<adagrad>" : kMode == kScaled ? "small_push_kernel<scaled>" : "small_push_kernel";
-    PS_LAUNCH_PDL(ps, name, (small_push_kernel<kMode, kCh>), dim3(buckets + 1, div_up_u32(strips, kCh)), dim3(kThreads), smem, s, a);
+    PS_LAUNCH_PDL(ps, name, (small_push_kernel<kMode, kCh, kHot>), dim3(buckets + 1, div_up_u32(strips, kCh)), dim3(kThreads), smem, s, a);
+}
+template <int kMode, int kCh>
+void launch_as(ps_store* ps, const SmallArgs& a, uint32_t strips, cudaStream_t s) {
+    SmallArgs b = a;
+    const uint32_t stretches = div_up_u32(strips, kCh);
+    b.stretch_vals = tmin<uint32_t>(32 * kCh, a.F4) * 4 * (kMode == kAdaGrad ? 2 : 1);
+    const uint64_t room = (uint64_t)ps->tile_cap * 2 * ps->cfg.row_len / ((uint64_t)stretches * kMaxHot * b.stretch_vals);
+    b.pieces = a.n < kHotCall || stretches > kHotStretches ? 0u : (uint32_t)tmin<uint64_t>(div_up_u32(a.n, kHotPiece), room);
+    if (b.pieces < 2) return launch_kernel<kMode, kCh, false>(ps, a, strips, s);
+    b.piece_len = div_up_u32(a.n, b.pieces * kWarps) * kWarps;
+    launch_kernel<kMode, kCh, true>(ps, b, strips, s);
 }
 template <int kMode>
 void launch(ps_store* ps, const SmallArgs& a, cudaStream_t s) {
@@ -376,6 +581,8 @@ SmallArgs common(ps_store* ps, uint32_t n, double* d_loss_accum, uint32_t loss_b
     a.loss_blocks = loss_blocks;
     a.loss_accum = loss_blocks ? d_loss_accum : nullptr;
     a.st = ps->status;
+    a.parked = ps->carry;           // (the sorted reductions' partial sums: on the caller's stream, as all of this is)
+    a.tickets = ps->hot_tickets;
     return a;
 }
 

@@ -35,6 +35,47 @@ def test_small_push_is_exact_on_integers(n, hot, L):
         compare_state(g, o, exact_rows=True, what="small push with a bad key")
 
 
+@pytest.mark.parametrize("L", [4, 128, 132, 520, 1028, 4100])
+@pytest.mark.parametrize("n,n_hot,share", [(2048, 1, 1.0), (2049, 1, 1.0), (2500, 3, 0.5), (5000, 12, 1.0), (8192, 1, 0.4), (8192, 8, 0.9)])
+def test_small_pushes_with_hot_keys(n, n_hot, share, L):
+    """Keys that are a large part of the call are shared by all blocks: integers exactly, and, with terms of very different
+    size, the same bits again on a second store (whichever block finishes a key)."""
+    K = 300
+    rng = np.random.default_rng(n + L)
+    keys = rng.integers(0, K, size=n)
+    keys = np.where(rng.random(n) < share, 17 + 3 * rng.integers(0, n_hot, size=n), keys)
+    upd = rng.integers(-4, 5, size=(n, L)).astype(np.float32)
+    rough = (rng.normal(size=(n, L)) * 10.0 ** rng.choice([0, 5, 20], size=(n, 1))).astype(np.float32)
+    (g, o), (h, _) = (make_pair(K, L, 3, max_batch_keys=n) for _ in range(2))
+    rows = rng.integers(-100, 100, size=(K, L)).astype(np.float32)
+    o.set_rows(np.arange(K), rows)
+    for s in (g, h):
+        s.set_all_rows(torch.from_numpy(rows))
+        s.push(dev(keys), dev(upd))
+    o.push(keys, upd)
+    compare_state(g, o, exact_rows=True, what="hot keys")
+    for s in (g, h):
+        s.push(dev(keys), dev(rough))
+        s.push(dev(keys[::-1].copy()), dev(upd))
+        s.sync()
+    assert torch.equal(g.export()[0], h.export()[0])
+
+
+@pytest.mark.parametrize("mode,L,n,words", [("mf", 8, 4000, 1), ("mf", 260, 1500, 2), ("kge", 24, 700, 1), ("kge", 600, 500, 2),
+                                            ("rescal", 16, 400, 1), ("sgns", 24, 500, 2), ("sgns", 300, 400, 1)])
+def test_small_steps_with_hot_keys(mode, L, n, words):
+    """Batches whose cells share a column, whose triples share a relation and few entities, of one or two words."""
+    rng = np.random.default_rng(n)
+    K, on_gpu, on_cpu = small_step(mode, 400 if mode == "mf" else words, words, L, n, rng)
+    rows = np.abs(rng.normal(0.2, 0.05, size=(K, L))).astype(np.float32) * (0.1 if mode in ("mf", "sgns") else 1)
+    g, o = make_pair(K, L, rows=rows, max_batch_keys=8192)
+    on_gpu(g)
+    on_cpu(o)
+    g.sync()
+    compare_state(g, o, what="hot keys in a small step")
+    assert close(float(g.loss.cpu()[0]), o.loss[0])
+
+
 def test_small_push_with_more_keys_in_one_bucket_than_its_table_holds():
     """Keys whose hash puts them all into the same block: the table overflows and warps compare for themselves."""
     K, L, n = 2_000_000, 4, 8000
