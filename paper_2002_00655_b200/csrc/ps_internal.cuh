@@ -279,15 +279,17 @@ void run_small_adagrad(ps_store* ps, uint32_t n, float lr, float eps, double* d_
 constexpr uint32_t kRelPiece = 8;                // data points of one relation that a block of rescal_points_kernel takes, at most
 constexpr uint32_t kRelChunk = 64;               // ... that a block of rescal_matrix_kernel sums before parking
 constexpr uint32_t kRelTickets = 16;             // ticket words per chunk of a relation of several chunks
+constexpr uint32_t kRelGroup = 8;                // ... chunks whose sums are added before they meet the others
 struct SegLists {
     unsigned int* counts;           // entries of shorts, longs, pieces, chunks; partial sums parked; what warps have drawn
     uint8_t* single;                // per occurrence
     uint2 *shorts, *pieces;         // {first position, length}
+    uint32_t short_room;            // entries `shorts` has room for
     uint4 *longs, *chunks;          // {first position, length, the segment's first parked sum, piece | pieces << 16}
     unsigned int *tickets, *long_tickets;
     uint32_t strips;                // long_tickets per parked sum
 };
-constexpr uint32_t kSegCounters = 8 + 64;        // lengths and single keys drawn (rows whose single keys are reduced have at most two stretches of columns); short segments drawn, by stretch
+constexpr uint32_t kSegMediums = 8 + 64, kSegCounters = kSegMediums + 1;        // lengths and single keys drawn (rows whose single keys are reduced have at most two stretches of columns); short segments drawn, by stretch; medium ones
 SegLists seg_lists(ps_store* ps);   // of the current buffer set
 const uint8_t* launch_singles(ps_store* ps, uint32_t n, int which, cudaStream_t s);     // per occurrence: its key occurs once
 // after the sort, on its stream; keys from rel_key_base on are RESCAL's relations (num_keys: none), of n_points data points

@@ -483,25 +483,32 @@ __global__ void __launch_bounds__(kMatThreads, 3) rescal_matrix_kernel(const Res
         bool finish = true;
         if (nc > 1) {
             // laid out [chunk][value of the thread's eight][thread]: coalesced either way
-            double2* mine = reinterpret_cast<double2*>(parked) + (uint64_t)(it.z + chunk) * quads * 4;
-            if (act)
+            auto park = [&](uint32_t slot) {
+                double2* mine = reinterpret_cast<double2*>(parked) + (uint64_t)(it.z + slot) * quads * 4;
+                if (act)
 #pragma unroll
-                for (int i = 0; i < 2; ++i)
+                    for (int i = 0; i < 2; ++i)
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) mine[(uint64_t)(4 * i + k) * (quads / 2) + x] = make_double2(at[i][k], ag[i][k]);
-            __threadfence();
-            __syncthreads();
-            if (tid == 0) s_ticket = atomicAdd(&A.L.tickets[it.z * kRelTickets + blockIdx.y], 1u);
-            __syncthreads();
-            finish = s_ticket == nc - 1;
-            if (finish) {
+                        for (int k = 0; k < 4; ++k) mine[(uint64_t)(4 * i + k) * (quads / 2) + x] = make_double2(at[i][k], ag[i][k]);
+            };
+            // the last chunk of a group to finish adds the group's sums, the last group the groups' (one after the other, 47 chunks
+            // of one relation took 33 us; each is a round trip to memory)
+            auto drawn_last = [&](uint32_t word, uint32_t of) {
                 __threadfence();
+                __syncthreads();
+                if (tid == 0) s_ticket = atomicAdd(&A.L.tickets[(uint64_t)(it.z + word) * kRelTickets + blockIdx.y], 1u);
+                __syncthreads();
+                const bool last = s_ticket == of - 1;
+                if (last) __threadfence();
+                return last;
+            };
+            auto add_up = [&](uint32_t first, uint32_t step, uint32_t count) {
 #pragma unroll
                 for (int i = 0; i < 2; ++i)
 #pragma unroll
                     for (int k = 0; k < 4; ++k) at[i][k] = ag[i][k] = 0.0;
-                for (uint32_t c = 0; c < nc && act; ++c) {
-                    const double2* from = reinterpret_cast<const double2*>(parked) + (uint64_t)(it.z + c) * quads * 4;
+                for (uint32_t c = 0; c < count && act; ++c) {
+                    const double2* from = reinterpret_cast<const double2*>(parked) + (uint64_t)(it.z + first + c * step) * quads * 4;
 #pragma unroll
                     for (int i = 0; i < 2; ++i)
 #pragma unroll
@@ -510,6 +517,18 @@ __global__ void __launch_bounds__(kMatThreads, 3) rescal_matrix_kernel(const Res
                             at[i][k] += v.x;
                             ag[i][k] += v.y;
                         }
+                }
+            };
+            const uint32_t g0 = chunk / kRelGroup * kRelGroup, groups = (nc + kRelGroup - 1) / kRelGroup;
+            const uint32_t in_group = tmin(kRelGroup, nc - g0);
+            park(chunk);
+            finish = in_group == 1 || drawn_last(g0, in_group);
+            if (finish) {
+                if (in_group > 1) add_up(g0, 1, in_group);
+                if (groups > 1) {
+                    if (in_group > 1) park(g0);
+                    finish = drawn_last(1, groups);             // (no group begins with chunk 1)
+                    if (finish) add_up(0, kRelGroup, groups);
                 }
             }
         }

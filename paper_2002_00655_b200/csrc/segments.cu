@@ -8,7 +8,8 @@
 //
 // segment_kernel (on the stream of the sort, right after it) looks at every sorted position and writes
 //   single[occurrence]     1 iff the occurrence's key occurs once
-//   shorts                 {first position, length} of the other segments of fewer than kLongRun occurrences
+//   shorts                 {first position, length} of the other segments of fewer than kMediumRun occurrences; from the end of
+//                          the array backwards, those of fewer than kWholeRun, which a warp adds alone too, but first
 //   longs                  the longer ones, cut into pieces of about kLongPiece
 //   pieces, chunks         RESCAL only: the relations' segments (any length), cut into pieces for its two kernels
 // The lists' order is the hardware's, the sums' is not: a segment is summed in position order whoever takes it.
@@ -17,11 +18,13 @@
 namespace psb {
 
 namespace {
-// occurrences from which on a block, not a warp, adds a segment (106,496 key occurrences of ComplEx on Zipf(1) triples, 400
-// values: 47.4 us with 24, 44.8 with 12, 54.5 with 8)
-constexpr uint32_t kLongRun = 12;
+// Occurrences from which on a block, not a warp, adds a segment.  Where many segments are that long their warps are busy anyway,
+// and a block's meetings per segment cost more than they save (8,000 data points of 5,000 uniform entities, 19 occurrences each:
+// 125 us for the reduction with all from 12 on added by blocks, 63 now); the warps take those from kMediumRun on first, so
+// that no long one is left for the end.
+constexpr uint32_t kMediumRun = 12, kWholeRun = 40;
 constexpr uint32_t kLongPiece = 96;             // ... and about as many as one block adds of it
-constexpr uint32_t kMaxStrips = kSegCounters - 8;             // (wider rows, of 16,384 values and more, are not cut: the tickets' room)
+constexpr uint32_t kMaxStrips = 64;             // (wider rows, of 16,384 values and more, are not cut: the tickets' room)
 }  // namespace
 
 // The first position from `from` on whose key is not k (which the position before it holds), by all lanes: 32 probes at a time,
@@ -68,11 +71,12 @@ segment_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restrict__ sv,
         if ((int)lane == src) end = e;
     }
     const uint32_t len = end - p;
-    if (run && !rel && len < kLongRun) L.shorts[atomicAdd(L.counts, 1u)] = make_uint2(p, len);
+    if (run && !rel && len < kMediumRun) L.shorts[atomicAdd(L.counts, 1u)] = make_uint2(p, len);
+    else if (run && !rel && len < kWholeRun) L.shorts[L.short_room - 1 - atomicAdd(L.counts + kSegMediums, 1u)] = make_uint2(p, len);
     // pieces of nearly equal length: of a long run, or of a relation's, which also has chunks
     uint32_t np = 0, at = 0, park = 0, nc = 0, at_c = 0, park_c = 0;
-    if (run && !rel && len >= kLongRun) {
-        np = tmin<uint32_t>((uint32_t)(((uint64_t)len + long_piece - 1) / long_piece), 0xffffu);
+    if (run && !rel && len >= kWholeRun) {
+        np = tmax<uint32_t>(tmin<uint32_t>((uint32_t)(((uint64_t)len + long_piece / 2) / long_piece), 0xffffu), 1u);
         at = atomicAdd(L.counts + 1, np);
         if (np > 1) {
             park = atomicAdd(L.counts + 5, np);         // where its pieces leave their partial sums
@@ -83,10 +87,7 @@ segment_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restrict__ sv,
         at = atomicAdd(L.counts + 2, np);
         nc = (len + rel_chunk - 1) / rel_chunk;
         at_c = atomicAdd(L.counts + 3, nc);
-        if (nc > 1) {
-            park_c = atomicAdd(L.counts + 4, nc);       // where its chunks leave their partial sums
-            for (uint32_t i = 0; i < kRelTickets; ++i) L.tickets[park_c * kRelTickets + i] = 0u;
-        }
+        if (nc > 1) park_c = atomicAdd(L.counts + 4, nc);       // where its chunks leave their partial sums
     }
     auto cut = [](uint32_t l, uint32_t i, uint32_t of) { return (uint32_t)((uint64_t)l * i / of); };
     auto write = [&](bool r, uint32_t p0, uint32_t l, uint32_t i, uint32_t of, uint32_t to, uint32_t pk) {
@@ -97,6 +98,8 @@ segment_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restrict__ sv,
     auto write_chunk = [&](uint32_t p0, uint32_t l, uint32_t i, uint32_t of, uint32_t to, uint32_t pk) {
         const uint32_t x = cut(l, i, of), y = cut(l, i + 1, of);
         L.chunks[to + i] = make_uint4(p0 + x, y - x, pk, i | of << 16);
+        for (uint32_t t = 0; of > 1 && t < kRelTickets / 4; ++t)
+            reinterpret_cast<uint4*>(L.tickets + (uint64_t)(pk + i) * kRelTickets)[t] = make_uint4(0u, 0u, 0u, 0u);
     };
     const bool many = np > 4 || nc > 4;
     if (!many) {
@@ -139,8 +142,9 @@ SegLists seg_lists(ps_store* ps) {
     L.single = (uint8_t*)ps->cellpos;
     // the records of the matrix-factorization step (16 bytes per key occurrence) are not in use
     L.longs = ps->rec;
-    L.shorts = (uint2*)(L.longs + ps->max_keys / kLongRun + 2);
-    L.pieces = L.shorts + ps->max_keys / 2 + 1;
+    L.shorts = (uint2*)(L.longs + ps->max_keys / kMediumRun + 2);
+    L.short_room = (uint32_t)(ps->max_keys / 2 + 1);
+    L.pieces = L.shorts + L.short_room;
     L.long_tickets = (unsigned int*)(L.pieces + ps->max_keys / 6 + 1);     // at least six slots per data point of RESCAL
     L.chunks = ps->mf_dup;
     L.tickets = ps->mf_tickets;
@@ -159,13 +163,13 @@ uint32_t rel_piece_len(uint32_t d) { return d <= 64 ? kRelPiece / 2 : kRelPiece;
 
 // Data points per chunk of rescal_matrix_kernel: 64, and fewer (16 at least) while the batch's chunks, a block for each of a
 // matrix's strips, would not fill the chip (1,288 data points of 11 relations of dimension 28: 34.7 -> 22.9 us); but the block
-// that finishes a relation adds up its chunks' sums one after the other, about as long per chunk as per data point, so not
-// below twice the square root of a relation's share of the batch.  A chunk parks two sums per element, 2 d d doubles, where a
+// that finishes a relation adds up its groups of kRelGroup chunks one after the other, about twice as long per group as a data
+// point takes, so not below half the square root of a relation's share of the batch.  A chunk parks two sums per element, 2 d d doubles, where a
 // tile of the push's reductions has room for 4 d, and a relation's chunks may be half empty: at least n d / tiles.
 static uint32_t rel_chunk_len(const ps_store* ps, uint32_t n_points, uint64_t n_rel, uint32_t d) {
     const uint64_t strips = div_up_u32((uint64_t)d * d / 8, 256), blocks = (uint64_t)ps->sm_count * 3;
     uint64_t len = tmax<uint64_t>(n_points * strips / blocks, div_up_u32((uint64_t)n_points * d, ps->tile_cap));
-    while (len < kRelChunk && len * len < 4 * (uint64_t)n_points / tmax<uint64_t>(n_rel, 1)) ++len;
+    while (len < kRelChunk && 4 * len * len < (uint64_t)n_points / tmax<uint64_t>(n_rel, 1)) ++len;
     len = (len + 7) / 8 * 8;
     return (uint32_t)tmin<uint64_t>(tmax<uint64_t>(len, 16), kRelChunk);
 }
@@ -209,6 +213,7 @@ segment_adagrad_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restri
     constexpr int kN = Vec<V>::kN, kWarps = 8;
     constexpr int kFly = 4;                     // gradient rows a warp has in flight
     __shared__ double s_part[kWarps][32 * kN];
+    __shared__ uint32_t s_ticket;
     // Beside RESCAL's matrix kernel (launched while that one's last blocks run, on other rows): what follows on the stream has
     // to come after both.  Elsewhere nothing is waited for.
     struct AtExit {
@@ -306,15 +311,8 @@ segment_adagrad_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restri
                 row[GV + f0 + 32 * c] = G[c];
             }
     };
-    const uint32_t n_work = gridDim.x - 1;
-    const uint32_t n_longs = L.counts[1], n_shorts = L.counts[0];
-    for (uint32_t j = blockIdx.x; j < n_longs; j += n_work) {
-        const uint4 seg = L.longs[j];
-        V* row = store + phys_row(table[sk[seg.x]], S) * (2 * GV);
-        load_row(row);
-        const uint32_t a = (uint32_t)((uint64_t)seg.y * w / kWarps), b = (uint32_t)((uint64_t)seg.y * (w + 1) / kWarps);
-        sum(seg.x + a, b - a);
-        unscale();
+    // the warps' sums, added in warp order: warp 0 has the total
+    auto over_warps = [&]() {
 #pragma unroll
         for (int c = 0; c < kCh; ++c)
 #pragma unroll
@@ -333,6 +331,17 @@ segment_adagrad_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restri
                     }
                 }
             }
+    };
+    const uint32_t n_work = gridDim.x - 1;
+    const uint32_t n_longs = L.counts[1], n_mediums = L.counts[kSegMediums], n_shorts = n_mediums + L.counts[0];
+    for (uint32_t j = blockIdx.x; j < n_longs; j += n_work) {
+        const uint4 seg = L.longs[j];
+        V* row = store + phys_row(table[sk[seg.x]], S) * (2 * GV);
+        load_row(row);
+        const uint32_t a = (uint32_t)((uint64_t)seg.y * w / kWarps), b = (uint32_t)((uint64_t)seg.y * (w + 1) / kWarps);
+        sum(seg.x + a, b - a);
+        unscale();
+        over_warps();
         const uint32_t np = seg.w >> 16, piece = seg.w & 0xffffu;
         if (np > 1) {
             if (w == 0) {
@@ -346,29 +355,31 @@ segment_adagrad_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restri
                             p[(GV + f0 + 32 * c) * kN + i] = a_g[c][i];
                         }
                 __threadfence();
-                __syncwarp();
-                uint32_t ticket = 0;
-                if (lane == 0) ticket = atomicAdd(&L.long_tickets[(uint64_t)seg.z * gridDim.y + blockIdx.y], 1u);
-                ticket = __shfl_sync(full, ticket, 0);
-                if (ticket != np - 1) continue;
-                __threadfence();
+            }
+            __syncthreads();
+            if (tid == 0) s_ticket = atomicAdd(&L.long_tickets[(uint64_t)seg.z * gridDim.y + blockIdx.y], 1u);
+            __syncthreads();
+            if (s_ticket != np - 1) continue;
+            // the last of the segment's blocks: a stretch of the pieces per warp (one warp took 0.7 us for each, 42 of them for a
+            // relation that half of 8,000 data points have)
+            __threadfence();
+#pragma unroll
+            for (int c = 0; c < kCh; ++c)
+#pragma unroll
+                for (int i = 0; i < kN; ++i) a_t[c][i] = a_g[c][i] = 0.0;
+            for (uint32_t k = np * w / kWarps; k < np * (w + 1) / kWarps; ++k) {
+                const double* q = parked + (uint64_t)(seg.z + k) * (2 * GV * kN);
 #pragma unroll
                 for (int c = 0; c < kCh; ++c)
+                    if (f0 + 32 * c < GV)
 #pragma unroll
-                    for (int i = 0; i < kN; ++i) a_t[c][i] = a_g[c][i] = 0.0;
-                for (uint32_t k = 0; k < np; ++k) {
-                    const double* q = parked + (uint64_t)(seg.z + k) * (2 * GV * kN);
-#pragma unroll
-                    for (int c = 0; c < kCh; ++c)
-                        if (f0 + 32 * c < GV)
-#pragma unroll
-                            for (int i = 0; i < kN; ++i) {
-                                a_t[c][i] += __ldcg(q + (f0 + 32 * c) * kN + i);
-                                a_g[c][i] += __ldcg(q + (GV + f0 + 32 * c) * kN + i);
-                            }
-                }
-                finish(row);
+                        for (int i = 0; i < kN; ++i) {
+                            a_t[c][i] += __ldcg(q + (f0 + 32 * c) * kN + i);
+                            a_g[c][i] += __ldcg(q + (GV + f0 + 32 * c) * kN + i);
+                        }
             }
+            over_warps();
+            if (w == 0) finish(row);
             continue;
         }
         if (w == 0) finish(row);
@@ -384,7 +395,7 @@ segment_adagrad_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restri
         if (j >= n_shorts) break;
         next = j + n_work * kWarps;
         if (drawn && lane == 0) next = atomicAdd(L.counts + 8 + blockIdx.y, 1u);
-        const uint2 seg = L.shorts[j];
+        const uint2 seg = L.shorts[j < n_mediums ? L.short_room - 1 - j : j - n_mediums];
         V* row = store + phys_row(table[sk[seg.x]], S) * (2 * GV);
         load_row(row);
         sum(seg.x, seg.y);
