@@ -465,18 +465,20 @@ loc_fused_kernel(const uint32_t* __restrict__ sk, uint32_t n, uint32_t span, uin
 }
 
 // ------------------------------------------------------------------------------------------------
-// Few keys (kLocSmallKeys at most, kLocSmallBytes of rows): the whole call, sort included, as ONE launch of one cluster
+// Few keys (kLocSmallLimit at most, kLocSmallBytes of rows): the whole call, sort included, as ONE launch of one cluster
 // of eight blocks.  With the cooperative sort and the launch above, 600 keys took 30 us of which nearly all was grid
 // barriers and launches; here the blocks meet once, at the cluster's own barrier.
 // Every block reads all keys, drops repeats with a hash table in shared memory and looks the others up; no order is needed
 // beyond what counting gives: a moving key's place among the moving keys (= its slot from the top of the requester's
 // stack) is the number of smaller moving keys, its place on its old owner's stack the number of smaller ones
 // with that owner.  A block counts for its eighth of the keys, kLocSmallThreads / (n / 8) threads per key; the n^2 / 8
-// comparisons per block are what kLocSmallKeys limits (a microsecond at 1,024 keys, six at 2,048).
+// comparisons per block are what kLocSmallLimit limits (1,024 keys of 256 values 15.8 us, 1,200 20.3, 1,400 26.1, 2,048 41.5; the
+// sort and the launch above take 21).
 // Nothing is written before every block has read what it needs (cluster barrier), and each block then moves its own keys.
 constexpr int kLocSmallThreads = 1024;
 constexpr uint32_t kLocSmallBlocks = 8;
-constexpr uint32_t kLocSmallKeys = 2048;
+constexpr uint32_t kLocSmallLimit = 1152;
+constexpr uint32_t kLocSmallKeys = 2048;            // places in shared memory: the limit, to a multiple of the threads
 constexpr uint64_t kLocSmallBytes = 2u << 20;       // eight SMs move this in about 4 us; more is better spread over the chip
 constexpr int kLocTableBits = 12;
 constexpr size_t kLocSmallSmem = ((size_t)kLocSmallKeys * 2 + ((size_t)2 << kLocTableBits)) * 4;
@@ -608,7 +610,7 @@ loc_small_kernel(const uint64_t* keys, uint32_t n, uint2* table, uint32_t worker
 }
 
 bool localize_is_small(const ps_store* ps, uint64_t n) {
-    return n <= kLocSmallKeys && n * ps->cfg.row_len * 4 <= kLocSmallBytes;
+    return n <= kLocSmallLimit && n * ps->cfg.row_len * 4 <= kLocSmallBytes;
 }
 
 void run_localize_small(ps_store* ps, uint32_t worker, const uint64_t* d_keys, uint32_t n, cudaStream_t s) {

@@ -126,7 +126,7 @@ def test_wide_complex_steps(n, dim, n_neg):
 
 
 @pytest.mark.parametrize("N,L,counts", [(8, 128, (1, 7, 600, 2047, 2048, 2049)), (1500, 4, (5, 700, 2048, 2500, 4000)),
-                                        (3, 256, (2048, 1, 2049, 1025))])
+                                        (3, 256, (2048, 1, 2049, 1025)), (8, 64, (1151, 1152, 1153))])
 def test_localize_around_the_limit_of_the_single_launch(N, L, counts):
     K = 30_000
     g, o = make_pair(K, L, N, 2 * -(-K // N) + 4200, max_batch_keys=4000)
