@@ -107,7 +107,10 @@ def _load_native():
         except ImportError as e:
             raise RuntimeError(f"the native part of the binding cannot be loaded ({e}): build it with "
                                "`python -m paper_2002_00655_b200.build`") from e
-        mod.setup({name: C.cast(getattr(lib, name), C.c_void_p).value for name in SIGNATURES}, PSError)
+        if mod.torch_version != torch.__version__:
+            raise RuntimeError(f"the native part of the binding was built for torch {mod.torch_version}, this is {torch.__version__}: "
+                               "build it again with `python -m paper_2002_00655_b200.build`")
+        mod.setup({name: C.cast(getattr(lib, name), C.c_void_p).value for name in SIGNATURES}, PSError, C.c_void_p, _convert)
         _native = mod
     return _native
 
@@ -156,6 +159,20 @@ def _hptr(t, dtype=None):
     if dtype is not None:
         assert t.dtype in dtype, f"expected dtype in {dtype}, got {t.dtype}"
     return t.data_ptr()
+
+
+def _convert(what, o):
+    """What the native part does not convert itself, as a ctypes call of the library would: raises what that raises."""
+    if what == "handle":
+        if not isinstance(o, _vp):
+            _vp.from_param(o)
+        return C.cast(o, _vp).value or 0
+    if what in ("u64", "u32", "f32"):
+        kind = {"u64": _u64, "u32": _u32, "f32": _f32}[what]
+        kind.from_param(o)
+        return o.value if isinstance(o, kind) else kind(o).value
+    ptr = (_dptr if what[0] == "d" else _hptr)(o, (_U32, _U64, _F32, _F64, _U8)[int(what[1])])
+    return ptr, o.numel()
 
 
 # The current stream's handle, as torch.cuda.current_stream().cuda_stream gives it, without building a Stream object for

@@ -70,18 +70,25 @@ def build(force: bool = False, verbose: bool = False) -> str:
     return LIB
 
 
+def _built_for(path: str, version: str) -> bool:
+    """Was the module built for this torch?  (It carries the version it was compiled against.)"""
+    with open(path, "rb") as f:
+        return b"\0" + version.encode() + b"\0" in f.read()
+
+
 def build_native(force: bool = False) -> str:
     src = os.path.join(CSRC, "native.cpp")
-    if not force and not _stale(NATIVE, [src, os.path.join(ROOT, "include", "ps.h")]):
-        return NATIVE
     import torch
+    if not force and not _stale(NATIVE, [src, os.path.join(ROOT, "include", "ps.h")]) and _built_for(NATIVE, torch.__version__):
+        return NATIVE
     troot = os.path.dirname(torch.__file__)
     cuda = os.path.dirname(os.path.dirname(os.path.realpath(_nvcc())))
     inc = [os.path.join(ROOT, "include"), os.path.join(troot, "include"),
            os.path.join(troot, "include", "torch", "csrc", "api", "include"), sysconfig.get_paths()["include"],
            os.path.join(cuda, "include")]
     tmp = NATIVE + f".tmp{os.getpid()}"
-    cmd = ["g++", "-shared", "-fPIC", "-O2", "-std=c++17", "-w", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+    cmd = ["g++", "-shared", "-fPIC", "-O2", "-std=c++17", "-Wall", "-Wextra", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           f'-DPS_TORCH_VERSION="{torch.__version__}"',
            *(x for i in inc for x in ("-isystem", i)), src, "-o", tmp, "-L", os.path.join(troot, "lib"),
            "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"]
     out = subprocess.run(cmd, capture_output=True, text=True)

@@ -3,8 +3,10 @@
 // A call through ctypes spends 3 to 4 us on the host around the 2 us of a kernel launch (attribute look-ups on tensors,
 // argument conversion, the current stream as a Python object, an output tensor through the Python front end), which
 // is most of what a call of a few rows costs.  Each function here has the name and arguments of its counterpart in
-// include/ps.h, takes the same tensors, makes the same checks and raises the same errors as the ctypes form.
-// The library is not linked: `setup` is given the addresses of its functions, and the exception to raise.
+// include/ps.h, takes the same arguments, makes the same checks and raises the same errors as the ctypes form; what is not a
+// tensor, a plain number or a c_void_p is handed to that form's own conversions (pointers, ctypes numbers, tensor-like
+// objects).
+// The library is not linked: `setup` is given the addresses of its functions, the exception to raise and the conversions.
 #include <Python.h>
 
 #include <ATen/ops/empty.h>
@@ -24,6 +26,8 @@ PS_FUNCTIONS(X)
 #undef X
 PyObject* ps_error = nullptr;           // PSError(code, where)
 PyObject* s_value = nullptr;            // "value"
+PyObject* c_void_p = nullptr;           // ctypes.c_void_p
+PyObject* convert = nullptr;            // convert(what, object) -> int, float or (pointer, number of elements), as ctypes and binding.py do
 
 enum Kind { kU32, kU64, kF32, kF64, kU8 };
 const char* const kKindNames[] = {"(torch.int32, torch.uint32)", "(torch.int64, torch.uint64)", "(torch.float32,)",
@@ -46,10 +50,11 @@ struct Args {
 
     PyObject* next() { return at < n ? a[at++] : nullptr; }
     void fail() { bad = true; }
+    PyObject* converted(const char* what, PyObject* o) { return PyObject_CallFunction(convert, "sO", what, o); }
     template <class T> T* handle() {                        // a ctypes c_void_p, an integer or None
         PyObject* o = next();
         if (bad || !o || o == Py_None) return nullptr;
-        PyObject* v = PyLong_Check(o) ? Py_NewRef(o) : PyObject_GetAttr(o, s_value);
+        PyObject* v = PyLong_Check(o) ? Py_NewRef(o) : (PyObject*)Py_TYPE(o) == c_void_p ? PyObject_GetAttr(o, s_value) : converted("handle", o);
         if (!v) return fail(), nullptr;
         void* p = v == Py_None ? nullptr : PyLong_AsVoidPtr(v);
         Py_DECREF(v);
@@ -68,8 +73,14 @@ struct Args {
             return nullptr;
         }
         if (!THPVariable_Check(o)) {
-            PyErr_SetString(PyExc_TypeError, "expected a tensor");
-            return fail(), nullptr;
+            char what[] = {cuda ? 'd' : 'h', (char)('0' + k), 0};
+            PyObject* pair = converted(what, o);
+            unsigned long long p = 0, n = 0;
+            const bool ok = pair && PyArg_ParseTuple(pair, "KK", &p, &n);
+            Py_XDECREF(pair);
+            if (!ok) return fail(), nullptr;
+            if (numel) *numel = n;
+            return (T*)(uintptr_t)p;
         }
         const at::Tensor& t = THPVariable_Unpack(o);
         if (t.is_cuda() != cuda || !t.is_contiguous()) {
@@ -86,10 +97,10 @@ struct Args {
         if (numel) *numel = (uint64_t)t.numel();
         return (T*)t.data_ptr();
     }
-    uint64_t u64() {
+    uint64_t u64(const char* what = "u64") {
         PyObject* o = next();
         if (bad) return 0;
-        PyObject* i = o ? PyNumber_Index(o) : nullptr;
+        PyObject* i = !o ? nullptr : PyIndex_Check(o) ? PyNumber_Index(o) : converted(what, o);
         if (!i) {
             if (!PyErr_Occurred()) PyErr_SetString(PyExc_TypeError, "an integer is missing");
             return fail(), 0;
@@ -98,12 +109,18 @@ struct Args {
         Py_DECREF(i);
         return v;
     }
-    uint32_t u32() { return (uint32_t)u64(); }
+    uint32_t u32() { return (uint32_t)u64("u32"); }
     float f32() {
         PyObject* o = next();
         if (bad) return 0.f;
-        const double v = o ? PyFloat_AsDouble(o) : -1.0;
+        double v = o ? PyFloat_AsDouble(o) : -1.0;
         if (!o) PyErr_SetString(PyExc_TypeError, "a number is missing");
+        if (o && v == -1.0 && PyErr_Occurred()) {               // (a c_float; anything else raises again)
+            PyErr_Clear();
+            PyObject* f = converted("f32", o);
+            v = f ? PyFloat_AsDouble(f) : -1.0;
+            Py_XDECREF(f);
+        }
         if (PyErr_Occurred()) fail();
         return (float)v;
     }
@@ -336,10 +353,10 @@ template <bool kInsert> PyObject* map_keys(PyObject*, PyObject* const* args, Py_
     END
 }
 
-// setup({name: address}, exception class)
+// setup({name: address}, exception class, ctypes.c_void_p, convert)
 PyObject* py_setup(PyObject*, PyObject* args) {
-    PyObject *addresses, *error;
-    if (!PyArg_ParseTuple(args, "O!O", &PyDict_Type, &addresses, &error)) return nullptr;
+    PyObject *addresses, *error, *void_p, *conv;
+    if (!PyArg_ParseTuple(args, "O!OOO", &PyDict_Type, &addresses, &error, &void_p, &conv)) return nullptr;
 #define X(f)                                                                          \
     {                                                                                 \
         PyObject* v = PyDict_GetItemString(addresses, #f);                            \
@@ -352,8 +369,9 @@ PyObject* py_setup(PyObject*, PyObject* args) {
     }
     PS_FUNCTIONS(X)
 #undef X
-    Py_INCREF(error);
-    Py_XSETREF(ps_error, error);
+    Py_XSETREF(ps_error, Py_NewRef(error));
+    Py_XSETREF(c_void_p, Py_NewRef(void_p));
+    Py_XSETREF(convert, Py_NewRef(conv));
     Py_RETURN_NONE;
 }
 
@@ -371,5 +389,7 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "_native", nullptr, -1, methods, nu
 
 PyMODINIT_FUNC PyInit__native() {
     s_value = PyUnicode_InternFromString("value");
-    return s_value ? PyModule_Create(&module) : nullptr;
+    PyObject* m = s_value ? PyModule_Create(&module) : nullptr;
+    if (m && PyModule_AddStringConstant(m, "torch_version", PS_TORCH_VERSION) < 0) Py_CLEAR(m);
+    return m;
 }
