@@ -317,21 +317,17 @@ __device__ __noinline__ void group_preadd(const uint32_t* __restrict__ sk, uint3
 // Every lane looks up the row of its own position's key, so the 32 table reads
 // go out together; then the positions are walked in groups whose update rows
 // and target rows are all requested before the first is used.
-//
-// kL4: the row length in float4 if known at compile time (0: taken from the argument); row offsets and the copy size then
-// fold.
-template <int kCh, int kL4>
+template <int kCh>
 __global__ void __launch_bounds__(256)
 push_reduce_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restrict__ sv, uint32_t n,
                    const float4* __restrict__ upd,
                    float4* __restrict__ store, const uint2* __restrict__ table,
-                   uint64_t S, uint32_t K, uint32_t L4_arg, double* __restrict__ carry,
+                   uint64_t S, uint32_t K, uint32_t L4, double* __restrict__ carry,
                    uint4* __restrict__ starters, unsigned int* __restrict__ starter_count,
                    unsigned int* __restrict__ group_done, double* __restrict__ group_sum,
                    uint32_t tile_len, DevStatus* st, unsigned int epoch) {
     __shared__ unsigned int s_ticket;
     __shared__ __align__(8) uint64_t bars[8][3];    // per warp and stage: the barrier word its copies report to
-    const uint32_t L4 = kL4 ? (uint32_t)kL4 : L4_arg;
     if (call_failed(st, epoch)) return;
     const unsigned full = 0xffffffffu;
     const uint32_t lane = threadIdx.x & 31;
@@ -497,19 +493,15 @@ push_reduce_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restrict__
 // values, now 242 with two positions in flight at three blocks per SM (four at two blocks 287, three 297), bound by the
 // latency of its loads and the unit that widens values to fp64 (60 %).
 // skip_singles: keys that occur once have been updated by the gradient kernel.
-// kL4 / kSlots: the row length in float4 and the slots per example if known at compile time (0: taken from the
-// arguments); row offsets and the division by the slots then fold.
-template <int kCh, int kL4, int kSlots>
+template <int kCh>
 __global__ void __launch_bounds__(256, kCh == 3 || kCh == 1 ? 3 : 2)
 scaled_reduce_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restrict__ sv, uint32_t n,
-                     const float4* __restrict__ upd, const float* __restrict__ scales, uint32_t slots_arg, uint32_t tile_len, bool skip_singles,
-                     float4* __restrict__ store, const uint2* __restrict__ table, uint64_t S, uint32_t K, uint32_t L4_arg,
+                     const float4* __restrict__ upd, const float* __restrict__ scales, uint32_t slots, uint32_t tile_len, bool skip_singles,
+                     float4* __restrict__ store, const uint2* __restrict__ table, uint64_t S, uint32_t K, uint32_t L4,
                      double* __restrict__ carry, uint4* __restrict__ starters, unsigned int* __restrict__ starter_count,
                      unsigned int* __restrict__ group_done, double* __restrict__ group_sum, DevStatus* st, unsigned int epoch) {
     __shared__ unsigned int s_ticket;
     __shared__ d4 s_pre[8][32];
-    const uint32_t L4 = kL4 ? (uint32_t)kL4 : L4_arg;
-    const uint32_t slots = kSlots ? (uint32_t)kSlots : slots_arg;
     if (call_failed(st, epoch)) return;
     const unsigned full = 0xffffffffu;
     const uint32_t lane = threadIdx.x & 31;
@@ -524,6 +516,8 @@ scaled_reduce_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restrict
         kg_far = sk[gpos + 8 * tile_len - 1];
     }
     const uint32_t L = L4 * 4;
+    // (rows of more than 128 (kCh - 1) values: the dispatch's rule; only the last column block needs the comparison)
+    auto in_row = [&](int c) { return c + 1 < kCh || lane + 32 * c < L4; };
     constexpr int kG = kCh >= 3 ? 2 : 4;
     d4 acc[kCh];
 #pragma unroll
@@ -579,7 +573,7 @@ scaled_reduce_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restrict
                 const float4* src = upd + (uint64_t)__shfl_sync(full, occ, at[k] & 31) * L4 + lane;
 #pragma unroll
                 for (int c = 0; c < kCh; ++c)
-                    if (lane + 32 * c < L4) u[k][c] = __ldg(src + 32 * c);      // (past the last: some other row, not used)
+                    if (in_row(c)) u[k][c] = __ldg(src + 32 * c);      // (past the last: some other row, not used)
             }
 #pragma unroll
             for (int k = 0; k < kG; ++k) {
@@ -591,7 +585,7 @@ scaled_reduce_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restrict
                     float4* to = store + __shfl_sync(full, row, p) * L4 + lane;
 #pragma unroll
                     for (int c = 0; c < kCh; ++c) {
-                        if (lane + 32 * c >= L4) continue;
+                        if (!in_row(c)) continue;
                         float4 v = to[32 * c];
                         v.x = fmaf(sc, u[k][c].x, v.x); v.y = fmaf(sc, u[k][c].y, v.y);
                         v.z = fmaf(sc, u[k][c].z, v.z); v.w = fmaf(sc, u[k][c].w, v.w);
@@ -610,7 +604,7 @@ scaled_reduce_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restrict
                     float4* to = store + __shfl_sync(full, row, p) * L4 + lane;
 #pragma unroll
                     for (int c = 0; c < kCh; ++c) {
-                        if (lane + 32 * c >= L4) continue;
+                        if (!in_row(c)) continue;
                         float4 v = to[32 * c];
                         v.x = (float)((double)v.x + acc[c].x); v.y = (float)((double)v.y + acc[c].y);
                         v.z = (float)((double)v.z + acc[c].z); v.w = (float)((double)v.w + acc[c].w);
@@ -620,7 +614,7 @@ scaled_reduce_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restrict
                     double* cs = carry + ((uint64_t)tile * 2 + ((uint32_t)p < first_head ? 0 : 1)) * L + (uint64_t)lane * 4;
 #pragma unroll
                     for (int c = 0; c < kCh; ++c) {
-                        if (lane + 32 * c >= L4) continue;
+                        if (!in_row(c)) continue;
                         *(double2*)(cs + 128 * c) = make_double2(acc[c].x, acc[c].y);
                         *(double2*)(cs + 128 * c + 2) = make_double2(acc[c].z, acc[c].w);
                     }
@@ -1333,39 +1327,35 @@ void run_push_reduce(ps_store* ps, uint32_t n, int which, const float* d_upd, do
 #define REDUCE_ARGS sk, sv, n, (const float4*)d_upd, (float4*)ps->store, ps->table,                                  \
                     ps->cfg.slots_per_part, (uint32_t)ps->cfg.num_keys, L4, ps->carry, ps->starters,                \
                     ps->starter_count, ps->group_done, ps->group_sum, tile_len, ps->status, ps->epoch
-#define REDUCE_LAUNCH(kCh, kL4)                                                                                      \
+#define REDUCE_LAUNCH(kCh)                                                                                           \
     do {                                                                                                             \
         static std::atomic<unsigned long long> smem_set{0};                                                          \
-        opt_in_smem((const void*)push_reduce_kernel<kCh, kL4>, reduce_smem(kCh), &smem_set);                         \
+        opt_in_smem((const void*)push_reduce_kernel<kCh>, reduce_smem(kCh), &smem_set);                         \
         if (ps->prof) prof_before(ps, "push_reduce_kernel<" #kCh ">", s);                                            \
-        push_reduce_kernel<kCh, kL4><<<blocks, 256, reduce_smem(kCh), s>>>(REDUCE_ARGS);                             \
+        push_reduce_kernel<kCh><<<blocks, 256, reduce_smem(kCh), s>>>(REDUCE_ARGS);                             \
         if (ps->prof) prof_after(ps, s);                                                                             \
         ps->launches++;                                                                                              \
     } while (0)
-    // the row lengths of the paper's workloads get kernels of their own: 128, 300 (41 slots per center) and 400 values
     if (d_scales) {
-#define SCALED_LAUNCH(kCh, kL4, kSlots)                                                                              \
+#define SCALED_LAUNCH(kCh)                                                                                           \
     do {                                                                                                             \
         if (ps->prof) prof_before(ps, "scaled_reduce_kernel<" #kCh ">", s);                                          \
-        scaled_reduce_kernel<kCh, kL4, kSlots><<<blocks, 256, 0, s>>>(sk, sv, n, (const float4*)d_upd, d_scales, slots,  \
+        scaled_reduce_kernel<kCh><<<blocks, 256, 0, s>>>(sk, sv, n, (const float4*)d_upd, d_scales, slots,  \
             tile_len, skip_singles, (float4*)ps->store, ps->table, ps->cfg.slots_per_part, (uint32_t)ps->cfg.num_keys, L4, ps->carry, \
             ps->starters, ps->starter_count, ps->group_done, ps->group_sum, ps->status, ps->epoch);                  \
         if (ps->prof) prof_after(ps, s);                                                                             \
         ps->launches++;                                                                                              \
     } while (0)
-        if (L4 == 75 && slots == 41) SCALED_LAUNCH(3, 75, 41);
-        else if (L4 <= 32) SCALED_LAUNCH(1, 0, 0);
-        else if (L4 <= 64) SCALED_LAUNCH(2, 0, 0);
-        else if (L4 <= 96) SCALED_LAUNCH(3, 0, 0);
-        else SCALED_LAUNCH(4, 0, 0);
+        if (L4 <= 32) SCALED_LAUNCH(1);
+        else if (L4 <= 64) SCALED_LAUNCH(2);
+        else if (L4 <= 96) SCALED_LAUNCH(3);
+        else SCALED_LAUNCH(4);
 #undef SCALED_LAUNCH
     } else {
-        if (L4 == 32) REDUCE_LAUNCH(1, 32);
-        else if (L4 == 100) REDUCE_LAUNCH(4, 100);
-        else if (L4 <= 32) REDUCE_LAUNCH(1, 0);
-        else if (L4 <= 64) REDUCE_LAUNCH(2, 0);
-        else if (L4 <= 96) REDUCE_LAUNCH(3, 0);
-        else REDUCE_LAUNCH(4, 0);
+        if (L4 <= 32) REDUCE_LAUNCH(1);
+        else if (L4 <= 64) REDUCE_LAUNCH(2);
+        else if (L4 <= 96) REDUCE_LAUNCH(3);
+        else REDUCE_LAUNCH(4);
     }
 #undef REDUCE_LAUNCH
 #undef REDUCE_ARGS

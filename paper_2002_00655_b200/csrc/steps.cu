@@ -246,29 +246,26 @@ __host__ __device__ constexpr int sgns_quad(int kCh) { return kCh == 4 ? 2 : kCh
 // A warp takes one center at a time.  The output-vector slots are handled 32 at a time: every lane first
 // resolves one slot (word -> key -> table entry -> row address), so those lookups are in flight together;
 // the rows are then read kQuad slots at a time, all their loads before the first dot product.
-// kL4, kWindow, kNeg: row length (float4), window and negatives per context if known at compile time (0: taken
-// from the arguments; kNeg < 0: from the argument); divisions by the slots per context and row offsets then fold.
 // kOnce: rows whose key occurs once in the batch (`single`, per slot) are updated here, in place, with the values in hand; a
 // third of the skip-gram batch's occurrences, each of which cost the reduction three rows of traffic.
-template <int kCh, int kL4, int kWindow, int kNeg, bool kOnce>
+template <int kCh, bool kOnce>
 __global__ void __launch_bounds__(256, 2)
 sgns_step_kernel(const uint32_t* tokens, uint64_t tok_first, uint64_t first_pos, uint64_t n_centers,
-                 uint64_t T, uint32_t window_arg, const uint32_t* negs, uint32_t n_neg_arg, uint64_t out_base,
+                 uint64_t T, uint32_t window, const uint32_t* negs, uint32_t n_neg, uint64_t out_base,
                  float lr, float4* store, const uint2* table, uint64_t S, uint64_t K, const uint8_t* single,
-                 uint32_t L4_arg, float4* __restrict__ upd, float* __restrict__ scales, uint32_t* keys_out,
+                 uint32_t L4, float4* __restrict__ upd, float* __restrict__ scales, uint32_t* keys_out,
                  double* __restrict__ loss_partial, DevStatus* st, unsigned int epoch) {
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint64_t n_warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-    const uint32_t L4 = kL4 ? (uint32_t)kL4 : L4_arg;
-    const uint32_t window = kWindow ? (uint32_t)kWindow : window_arg;
-    const uint32_t n_neg = kNeg >= 0 ? (uint32_t)kNeg : n_neg_arg;
     const uint32_t per_ctx = 1 + n_neg;
     const uint64_t slots = 1 + (uint64_t)2 * window * per_ctx;
     const uint64_t pairs0 = sgns_pairs_before(first_pos, T, window);
     constexpr int kQuad = sgns_quad(kCh);
     constexpr int kLanes = 32 / kQuad;
+    // (rows of more than 128 (kCh - 1) values: the dispatch's rule; only the last column block needs the comparison)
+    auto in_row = [&](int c) { return c + 1 < kCh || lane + 32 * c < L4; };
     // Rows of more than 512 bytes arrive in shared memory as bulk copies, two groups of kQuad of them on their way while one
     // is worked on from registers: [warp][2][kQuad][L4].  (With loads straight into the registers one group was on its way, and
     // that only between two groups' arithmetic: 295 us for 32,768 centers of 300 values at 4.6 TB/s of DRAM, now 265.)
@@ -329,7 +326,7 @@ sgns_step_kernel(const uint32_t* tokens, uint64_t tok_first, uint64_t first_pos,
 #pragma unroll
         for (int c = 0; c < kCh; ++c) {
             const uint32_t f = lane + 32 * c;
-            v[c] = f < L4 ? V[f] : make_float4(0.f, 0.f, 0.f, 0.f);
+            v[c] = in_row(c) ? V[f] : make_float4(0.f, 0.f, 0.f, 0.f);
             dv[c] = make_float4(0.f, 0.f, 0.f, 0.f);
         }
         bool bad = false;
@@ -387,7 +384,7 @@ sgns_step_kernel(const uint32_t* tokens, uint64_t tok_first, uint64_t first_pos,
                     for (int a = 0; a < kQuad; ++a)                             // (a slot without a row: what was there, skipped below)
 #pragma unroll
                         for (int c = 0; c < kCh; ++c)
-                            if (lane + 32 * c < L4) u[a][c] = ring[(stage * kQuad + a) * L4 + lane + 32 * c];
+                            if (in_row(c)) u[a][c] = ring[(stage * kQuad + a) * L4 + lane + 32 * c];
                     __syncwarp();
                 }
                 if (kStage) ask(b + 2 * kQuad);
@@ -397,7 +394,7 @@ sgns_step_kernel(const uint32_t* tokens, uint64_t tok_first, uint64_t first_pos,
 #pragma unroll
                     for (int c = 0; c < kCh; ++c) {
                         const uint32_t f = lane + 32 * c;
-                        if (f < L4) u[a][c] = Urow[f];
+                        if (in_row(c)) u[a][c] = Urow[f];
                     }
                 }
                 float x[kQuad];
@@ -447,7 +444,7 @@ sgns_step_kernel(const uint32_t* tokens, uint64_t tok_first, uint64_t first_pos,
                             const uint32_t f = lane + 32 * c;
                             const float4 x = make_float4(fmaf(sc, v[c].x, u[a][c].x), fmaf(sc, v[c].y, u[a][c].y),
                                                          fmaf(sc, v[c].z, u[a][c].z), fmaf(sc, v[c].w, u[a][c].w));
-                            if (f < L4) Urow[f] = x;
+                            if (in_row(c)) Urow[f] = x;
                         }
                     }
                 }
@@ -465,7 +462,7 @@ sgns_step_kernel(const uint32_t* tokens, uint64_t tok_first, uint64_t first_pos,
 #pragma unroll
         for (int c = 0; c < kCh; ++c) {
             const uint32_t f = lane + 32 * c;
-            if (f < L4) {
+            if (in_row(c)) {
                 if (center_once) V[f] = make_float4(dv[c].x + v[c].x, dv[c].y + v[c].y, dv[c].z + v[c].z, dv[c].w + v[c].w);
                 else U[f] = dv[c];
                 U[L4 + f] = v[c];
@@ -529,27 +526,26 @@ uint32_t launch_step_sgns(ps_store* ps, const uint32_t* d_tokens, uint64_t tok_f
 #define SG_ARGS d_tokens, tok_first, first_pos, n_centers, corpus_len, window, d_negs, n_neg, out_key_base, lr,   \
                 (float4*)ps->store, ps->table, ps->cfg.slots_per_part, ps->cfg.num_keys, single, L4,            \
                 (float4*)ps->upd, sgns_scales(ps, n_centers), keys_out, ps->loss_partial, ps->status, epoch
-#define SG_LAUNCH(kCh, kL4, kW, kN)                                                                                  \
+#define SG_LAUNCH(kCh)                                                                                  \
     do {                                                                                                             \
         const size_t smem = (kCh) >= 2 ? (size_t)8 * 2 * sgns_quad(kCh) * L4 * 16 : 0;                               \
         static std::atomic<unsigned long long> smem_set[2];                                                          \
-        const void* fn = single ? (const void*)sgns_step_kernel<kCh, kL4, kW, kN, true> : (const void*)sgns_step_kernel<kCh, kL4, kW, kN, false>; \
+        const void* fn = single ? (const void*)sgns_step_kernel<kCh, true> : (const void*)sgns_step_kernel<kCh, false>; \
         if ((kCh) >= 2) opt_in_smem(fn, (size_t)8 * 2 * sgns_quad(kCh) * (kCh) * 512, &smem_set[single ? 1 : 0]);    \
         if (keys_out) {                                                                                              \
-            PS_LAUNCH_PDL(ps, "sgns_step_kernel<" #kCh ">", (sgns_step_kernel<kCh, kL4, kW, kN, false>), dim3(grid), dim3(256), smem, s, SG_ARGS); \
+            PS_LAUNCH_PDL(ps, "sgns_step_kernel<" #kCh ">", (sgns_step_kernel<kCh, false>), dim3(grid), dim3(256), smem, s, SG_ARGS); \
         } else {                                                                                                     \
             if (ps->prof) prof_before(ps, "sgns_step_kernel<" #kCh ">", s);                                          \
-            if (single) sgns_step_kernel<kCh, kL4, kW, kN, true><<<grid, 256, smem, s>>>(SG_ARGS);                   \
-            else sgns_step_kernel<kCh, kL4, kW, kN, false><<<grid, 256, smem, s>>>(SG_ARGS);                         \
+            if (single) sgns_step_kernel<kCh, true><<<grid, 256, smem, s>>>(SG_ARGS);                   \
+            else sgns_step_kernel<kCh, false><<<grid, 256, smem, s>>>(SG_ARGS);                         \
             if (ps->prof) prof_after(ps, s);                                                                         \
             ps->launches++;                                                                                          \
         }                                                                                                            \
     } while (0)
-    if (L4 == 75 && window == 5 && n_neg == 3) SG_LAUNCH(3, 75, 5, 3);     // 300 values, window 5, 3 negatives
-    else if (L4 <= 32) SG_LAUNCH(1, 0, 0, -1);
-    else if (L4 <= 64) SG_LAUNCH(2, 0, 0, -1);
-    else if (L4 <= 96) SG_LAUNCH(3, 0, 0, -1);
-    else SG_LAUNCH(4, 0, 0, -1);
+    if (L4 <= 32) SG_LAUNCH(1);
+    else if (L4 <= 64) SG_LAUNCH(2);
+    else if (L4 <= 96) SG_LAUNCH(3);
+    else SG_LAUNCH(4);
 #undef SG_LAUNCH
 #undef SG_ARGS
     return grid;
