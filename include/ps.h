@@ -107,7 +107,8 @@ ps_status_t ps_set_rows(ps_store_t* ps, const uint64_t* d_keys, uint64_t n, cons
 ps_status_t ps_pull(ps_store_t* ps, const uint64_t* d_keys, uint64_t n, float* d_out, void* stream);
 
 /* push (Table 2; cumulative, Section 2.1): row(k) += sum over {t : d_keys[t] = k} of
- * d_updates[t, :].  Occurrences are sorted by key and reduced segment by segment. */
+ * d_updates[t, :].  Occurrences are sorted by key and reduced segment by segment; calls of at most 8,192 are
+ * reduced without a sort. */
 ps_status_t ps_push(ps_store_t* ps, const uint64_t* d_keys, uint64_t n, const float* d_updates,
                     void* stream);
 
@@ -307,8 +308,8 @@ ps_status_t ps_set_host_overlap(ps_store_t* ps, int on);
 
 /* How ps_push adds (Section 2.1: the push is cumulative; the paper's servers serialise the adds of a key with
  * latches, Section 3.7).
- *   PS_PUSH_SORTED (default): occurrences sorted by key, per-key sums in fp64, one rounding, one write per key;
- *     results are reproducible bit for bit.
+ *   PS_PUSH_SORTED (default): occurrences grouped by key (sorted, but for calls of at most 8,192), per-key sums in
+ *     fp64, one rounding, one write per key; results are reproducible bit for bit.
  *   PS_PUSH_ATOMIC: no sort; every occurrence adds its row with vector atomic adds.  Kept as a measured
  *     alternative: each term is rounded into the row as it arrives and the order is the hardware's, so keys
  *     with more than two terms in a call are not reproducible from run to run (and differ from the sorted

@@ -24,7 +24,7 @@ WsLayout ws_layout(const ps_config_t& cfg, uint64_t max_keys) {
     };
     const uint64_t mk = max_keys ? max_keys : 1;
     const size_t sort_tiles = (mk + kSortTile / 2 - 1) / (kSortTile / 2);   // the sort's blocks, at its shortest tile
-    // tiles of the reduction: 32 positions, or 8 for the matrix-factorization step on rows of at most 128 values
+    // room for the reductions' tiles (reduce_tile: 8 to 128 positions by the size of the call; the matrix-factorization step: 8)
     const size_t tile_len = cfg.row_len <= 128 ? 8 : kReduceTile;
     size_t reduce_tiles = (mk + tile_len - 1) / tile_len;
     if (cfg.row_len <= kTiledRow) reduce_tiles = tmax(reduce_tiles, tmin<size_t>((mk + 7) / 8, kMidTiles));

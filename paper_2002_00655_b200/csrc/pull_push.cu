@@ -3,8 +3,8 @@
 // pull  (Table 2 of the paper): key -> (owner, slot) lookup, then a 128-bit
 //       vectorised gather of the row.
 // push  (Table 2; cumulative, Section 2.1): the occurrences of a call are
-//       sorted by key; a warp reduces 32 consecutive sorted occurrences in
-//       fp64, applies every segment that lies wholly inside its tile with one
+//       sorted by key; a warp reduces 8 to 128 consecutive sorted occurrences
+//       (reduce_tile) in fp64, applies every segment that lies wholly inside its tile with one
 //       read-modify-write of the row, and parks partial sums of segments that
 //       cross tile borders; a second kernel adds those partials in tile order.
 //       The order of every sum is fixed by the sorted positions, so results

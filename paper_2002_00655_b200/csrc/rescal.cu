@@ -29,7 +29,7 @@
 // The d * d gradients of a data point never go through memory (335 MB per 8,192 data points of dimension 100 did, with
 // a sort of 112 keys per data point where 13 do now), and a relation's rows are read and written once per batch.
 // Before: a warp per data point with two passes over the matrix in L2, 292 us, and the matrix rows through the sorted
-// reduction, 278 us, of 577 us per step of 8,192 data points of dimension 100; now 125 + 108 + 33 us, 273 us per step.
+// reduction, 278 us, of 577 us per step of 8,192 data points of dimension 100; now 125 + 105 us with the entities' reduction beside the latter, 237 us per step.
 // rescal_points_kernel is bound by the latency of its phases (16 warps per SM, issue slots 40 % used, tensor pipe 27 %),
 // rescal_matrix_kernel by instruction issue and the special-function unit.
 #include <string.h>
@@ -386,7 +386,8 @@ __global__ void __launch_bounds__(32 * kWarps, 16 / kWarps) rescal_points_kernel
 // widenings and roots (16 lanes per clock and SM: each such operation per element is 18 us of a step of 8,192 data points
 // of dimension 100), so the vectors are staged in fp64 (widened once per data point, not once per element), the squares
 // are summed as fp64 products and the steps widened by integer operations.  A relation of several chunks
-// leaves fp64 partial sums of each; the last of its chunks to finish (a ticket) adds them in chunk order.
+// leaves fp64 partial sums of each; the last chunk of a group of kRelGroup to finish (a ticket) adds the group's in chunk order, the
+// last group the groups'.
 __global__ void __launch_bounds__(kMatThreads, 3) rescal_matrix_kernel(const RescalArgs A, double* __restrict__ parked) {
     extern __shared__ __align__(128) unsigned char dyn[];
     __shared__ __align__(8) uint64_t bars[2];

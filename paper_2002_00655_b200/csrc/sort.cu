@@ -93,49 +93,10 @@ struct SinkMF {
     uint32_t* cellpos;                  // sorted position of each cell's row-factor occurrence
 };
 
-// the records of `len` sorted (key, value) pairs in shared memory, positions c0 on: a thread has kAtOnce of them under way
-// (all index loads, then all table loads, then the records)
-__device__ __forceinline__ void sink_records(const SinkMF& sink, const uint2* buf, uint32_t len, uint32_t c0, uint32_t* kout) {
-    constexpr int kAtOnce = 4;
-    for (uint32_t l0 = threadIdx.x; l0 < len; l0 += kAtOnce * blockDim.x) {
-        uint2 x[kAtOnce];
-        uint32_t pk[kAtOnce];
-        float cval[kAtOnce];
-        uint2 e_own[kAtOnce], e_par[kAtOnce];
-#pragma unroll
-        for (int i = 0; i < kAtOnce; ++i) {
-            const uint32_t l = l0 + i * blockDim.x;
-            x[i] = l < len ? buf[l] : make_uint2(sink.K, 0u);
-            pk[i] = sink.K;                             // cells with an index out of range carry the mark K
-            cval[i] = 0.f;
-            if (x[i].x < sink.K) {
-                const uint32_t cell = x[i].y >> 1;
-                pk[i] = (x[i].y & 1u) ? sink.ci[cell] : sink.col_base + sink.cj[cell];
-                cval[i] = sink.cv[cell];
-            }
-        }
-#pragma unroll
-        for (int i = 0; i < kAtOnce; ++i) {
-            e_own[i] = x[i].x < sink.K ? sink.table[x[i].x] : make_uint2(0u, 0u);
-            e_par[i] = x[i].x < sink.K ? sink.table[pk[i]] : make_uint2(0u, 0u);
-        }
-#pragma unroll
-        for (int i = 0; i < kAtOnce; ++i) {
-            const uint32_t l = l0 + i * blockDim.x;
-            if (l >= len) break;
-            const uint32_t pos = c0 + l;
-            kout[pos] = x[i].x;
-            if (!(x[i].y & 1u)) sink.cellpos[x[i].y >> 1] = pos;
-            sink.rec[pos] = make_uint4(x[i].y >> 1, __float_as_uint(cval[i]), (uint32_t)phys_row(e_own[i], sink.S),
-                                       (uint32_t)phys_row(e_par[i], sink.S));
-        }
-    }
-}
-
 // Rank of a lane's digit among the warp's keys so far (stable: item by item, lane by lane), and the warp's counter of the
 // digit moved on.  Lanes with equal digits find one another through a word per digit in shared memory (every lane ORs its
-// bit in); __match_any_sync takes 61 cycles of an SM per instruction, the OR and the read 6.  `mask` is all zero before
-// and after.
+// bit in, as in the atomic-OR form of the warp match of CUB's BlockRadixRankMatch); __match_any_sync takes 61 cycles of an SM
+// per instruction, the OR and the read 6.  `mask` is all zero before and after.
 __device__ __forceinline__ uint32_t warp_rank(volatile uint32_t* mask, volatile uint32_t* hist, uint32_t digit, bool valid,
                                               int lane) {
     if (valid) atomicOr(const_cast<uint32_t*>(mask) + digit, 1u << lane);
@@ -177,15 +138,15 @@ __device__ __forceinline__ uint32_t scan_digits(uint32_t v, uint32_t* sm8, uint3
     return wbase + incl - v;
 }
 
-// A tile is kThreads x kItems keys.  Small sorts use many threads with few keys each (every phase of a pass is a
-// short chain of dependent steps, and all SMs get a tile); large sorts use 256 threads with 8 keys each.
+// A tile is kThreads x kItems keys: 512 x 4 in small sorts (every phase of a pass is a short chain of dependent steps, and all
+// SMs get a tile), 512 x 8 in large ones.
 template <class Src, class Sink, int kThreads, int kItems>
-__global__ void __launch_bounds__(kThreads, kThreads == 256 ? 3 : kThreads == 512 ? 2 : 1)
+__global__ void __launch_bounds__(kThreads, 2)
 sort_all_kernel(Src src, Sink sink, SortParams P) {
     constexpr int kTile = kThreads * kItems;
     constexpr int kWarps = kThreads / 32;
     constexpr int kQ = kThreads / 64;                // threads per group of four digits in the counter read
-    constexpr int kRowsAtOnce = kThreads >= 512 ? 16 : 8;
+    constexpr int kRowsAtOnce = 16;
     __shared__ uint32_t digit_base[kRadix];          // global position of the tile's first key with each digit
     __shared__ uint32_t local_base[kRadix];          // the same inside the tile
     extern __shared__ __align__(16) uint32_t s_dyn[];  // the tile in digit order, on its way out: keys, then values
@@ -198,7 +159,6 @@ sort_all_kernel(Src src, Sink sink, SortParams P) {
     const uint32_t n = P.n_dev ? tmin<uint32_t>(*((const volatile unsigned int*)P.n_dev), P.n_host) : P.n_host;
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const bool digit_thread = tid < kRadix;
-    const int dg = tid & (kRadix - 1);
     const uint32_t b = blockIdx.x, G = gridDim.x;
     const uint32_t chunk = P.tiles_per_block * kTile;
     const uint64_t c0_64 = (uint64_t)b * chunk;
@@ -455,9 +415,9 @@ struct ClusterSmem {
     uint32_t sm[8];
 };
 
-template <class Src, class Sink>
+template <class Src>
 __global__ void __launch_bounds__(kClThreads, 2)
-sort_cluster_kernel(Src src, Sink sink, SortParams P) {
+sort_cluster_kernel(Src src, SortParams P) {
     extern __shared__ __align__(16) unsigned char cl_dyn[];
     ClusterSmem& M = *reinterpret_cast<ClusterSmem*>(cl_dyn);
     const uint32_t n = P.n_dev ? tmin<uint32_t>(*((const volatile unsigned int*)P.n_dev), P.n_host) : P.n_host;
@@ -551,14 +511,10 @@ sort_cluster_kernel(Src src, Sink sink, SortParams P) {
     }
     uint32_t* kout = ((P.start + P.n_passes) & 1) ? P.kB : P.kA;
     uint32_t* vout = ((P.start + P.n_passes) & 1) ? P.vB : P.vA;
-    if constexpr (Sink::kPairs) {
-        for (uint32_t l = tid; l < len; l += kClThreads) {
-            const uint2 x = M.buf[l];
-            kout[c0 + l] = x.x;
-            vout[c0 + l] = x.y;
-        }
-    } else {
-        sink_records(sink, M.buf, len, c0, kout);
+    for (uint32_t l = tid; l < len; l += kClThreads) {
+        const uint2 x = M.buf[l];
+        kout[c0 + l] = x.x;
+        vout[c0 + l] = x.y;
     }
 }
 
@@ -577,13 +533,13 @@ static_assert(kSmallTile >= kSortTile / 2, "the digit counters are sized for til
 
 // Once per device: the opt-ins (shared memory, a cluster of more than eight blocks), and whether such a cluster can be
 // resident at all (a GPU's clusters are as large as its smallest partition of multiprocessors allows).
-template <class Src, class Sink>
+template <class Src>
 static bool cluster_sort_fits() {
     static std::atomic<unsigned long long> asked{0}, fits{0};
     int d = -1;
     if (cudaGetDevice(&d) != cudaSuccess || d < 0 || d >= 64) return false;
     if (!((asked.load(std::memory_order_acquire) >> d) & 1ull)) {
-        const void* fn = (const void*)sort_cluster_kernel<Src, Sink>;
+        const void* fn = (const void*)sort_cluster_kernel<Src>;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(kClBlocks);
         cfg.blockDim = dim3(kClThreads);
@@ -597,7 +553,7 @@ static bool cluster_sort_fits() {
         int clusters = 0;
         if (cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
             cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(ClusterSmem)) == cudaSuccess &&
-            cudaOccupancyMaxActiveClusters(&clusters, sort_cluster_kernel<Src, Sink>, &cfg) == cudaSuccess && clusters > 0)
+            cudaOccupancyMaxActiveClusters(&clusters, sort_cluster_kernel<Src>, &cfg) == cudaSuccess && clusters > 0)
             fits.fetch_or(1ull << d, std::memory_order_relaxed);
         cudaGetLastError();
         asked.fetch_or(1ull << d, std::memory_order_release);
@@ -629,23 +585,25 @@ static int sort_launch(ps_store* ps, const Src& src, const Sink& sink, uint32_t 
     P.zero_b = zero_me;
     P.st = ps->status;
     P.epoch = ps->epoch;
-    if (n <= kClusterSort && Sink::kPairs && cluster_sort_fits<Src, Sink>()) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(kClBlocks);
-        cfg.blockDim = dim3(kClThreads);
-        cfg.dynamicSmemBytes = sizeof(ClusterSmem);
-        cfg.stream = stream;
-        cudaLaunchAttribute attr;
-        attr.id = cudaLaunchAttributeClusterDimension;
-        attr.val.clusterDim.x = kClBlocks;
-        attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-        cfg.attrs = &attr;
-        cfg.numAttrs = 1;
-        if (ps->prof) prof_before(ps, "sort_cluster_kernel", stream);
-        cudaLaunchKernelEx(&cfg, sort_cluster_kernel<Src, Sink>, src, sink, P);
-        if (ps->prof) prof_after(ps, stream);
-        ps->launches++;
-        return (start + P.n_passes) & 1;
+    if constexpr (Sink::kPairs) {
+        if (n <= kClusterSort && cluster_sort_fits<Src>()) {
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(kClBlocks);
+            cfg.blockDim = dim3(kClThreads);
+            cfg.dynamicSmemBytes = sizeof(ClusterSmem);
+            cfg.stream = stream;
+            cudaLaunchAttribute attr;
+            attr.id = cudaLaunchAttributeClusterDimension;
+            attr.val.clusterDim.x = kClBlocks;
+            attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+            cfg.attrs = &attr;
+            cfg.numAttrs = 1;
+            if (ps->prof) prof_before(ps, "sort_cluster_kernel", stream);
+            cudaLaunchKernelEx(&cfg, sort_cluster_kernel<Src>, src, P);
+            if (ps->prof) prof_after(ps, stream);
+            ps->launches++;
+            return (start + P.n_passes) & 1;
+        }
     }
     if (ps->prof) prof_before(ps, "sort_all_kernel", stream);
     void* args[] = {(void*)&src, (void*)&sink, (void*)&P};

@@ -3,10 +3,11 @@
 // RESCAL: rescal.cu).  One warp handles one example (a matrix cell, a skip-gram
 // center word with its window): it looks the example's keys up in the location
 // table, gathers their rows with coalesced loads, forms dot products with warp
-// shuffles, and writes one additive update row per key occurrence plus that
-// occurrence's key.  The push stage (pull_push.cu) then sorts the occurrences
-// by key, sums them per key and applies them, so every read in here sees the
-// state from before the step.
+// shuffles, and writes one additive update row per key occurrence (skip-gram:
+// two rows and the occurrences' factors).  The push stage then sums them per key
+// and applies them: pull_push.cu on the sorted occurrences, small.cu for calls of
+// few, whose keys are written here too.  Every read sees the state from before the
+// step: a row is only updated here, in place, if its key occurs once in the batch.
 #include "ps_internal.cuh"
 
 namespace psb {
@@ -297,7 +298,7 @@ sgns_step_kernel(const uint32_t* tokens, uint64_t tok_first, uint64_t first_pos,
         return i == 0 ? tokens[q - tok_first] : negs[(z0 + j) * n_neg + (i - 1)];
     };
     // Words asked for ahead of their use: this lane's of the coming round and, in a center's last round, the next center's (the
-    // negatives come from memory: 265 -> 259 us for 32,768 centers of 300 values).
+    // negatives come from memory: 265 -> 259 us for 32,768 centers of 300 values, in a form compiled for that shape; 270 without it).
     uint32_t word_next = 0, wtok_next = 0;
     bool have = false;
     for (uint64_t cidx = warp; cidx < n_centers && !dead; cidx += n_warps) {
