@@ -720,6 +720,363 @@ __global__ void __launch_bounds__(256, Wide<kMaxNeg>::kPerSm) kge_wide_kernel(co
     }
 }
 
+// Rows of more than 128 dimensions whose data point fits a block's shared memory (13 rows of up to 2,176 dimensions): the
+// embeddings stay there from the first pass to the second.  A warp has chunks of 64 dimensions to itself (chunk
+// (s C + rank) warps + w of the row is the s-th of warp w), with their own places in shared memory and their own barrier
+// words: it asks for its part of the next data point's rows when it is done with this one's, and meets the others once per data
+// point, to add up the scores.  In kge_wide_kernel, which streams stretches of 256 dimensions through a block, the warps meet after every
+// stretch (a third of their stalls), a last stretch idles some of them, and the rows are read twice.  us per launch, streamed and
+// now: 4,000 data points of 200 dimensions with 10 negatives 148 and 90, 1,600 of 500 105 and 90, 800 of 1,000 98 and 89,
+// 1,500 of 300 with 20 negatives 171 and 94, 600 of 600 with 29 248 and 121, 8,000 of 141 with one 140 and 76.  Where a data point takes a cluster of two blocks
+// the streamed form is as good (2,048 of 4,000: 753 and 770) and keeps it.  Bound by the latency of its instructions at 16
+// warps per SM, which 128 registers fix.
+template <int kMaxNeg> struct Resident {
+    static constexpr uint32_t kNumbers = 3 + kMaxNeg <= 16 ? 16 : 32;                   // places per table of slots
+    __host__ __device__ static constexpr uint32_t pad(int kVec) { return kVec == 4 ? 64 : 68; }             // floats of a chunk of a row's Re or Im
+    static constexpr size_t smem(int kVec, uint32_t slots, uint32_t warps, uint32_t bufs, uint32_t C) {
+        return (size_t)warps * bufs * (slots * 2 * pad(kVec) * sizeof(float) + 8) + (size_t)2 * C * warps * (kMaxNeg + 1) * 8 +
+               (size_t)warps * 3 * kNumbers * 8 + 2 * 32 * 8 + 16;
+    }
+};
+
+template <int kMaxNeg, int kVec>
+__global__ void __launch_bounds__(512, 1) kge_resident_kernel(const KgeArgs A, const uint32_t n_str, const bool twice) {
+    constexpr int NP = kMaxNeg < 8 ? 8 : kMaxNeg < 16 ? 16 : 32;
+    constexpr uint32_t kPad = Resident<kMaxNeg>::pad(kVec), kNumbers = Resident<kMaxNeg>::kNumbers;
+    constexpr uint32_t kStep = kVec > 1 ? 1 : 32;               // a lane's two dimensions: neighbours, or 32 apart (odd d)
+    extern __shared__ __align__(128) float chunk_mem[];
+    const unsigned full = 0xffffffffu;
+    const uint32_t tid = threadIdx.x, lane = tid & 31, w = tid >> 5, n_warps = blockDim.x >> 5;
+    const uint32_t d = A.d, shift = kVec == 4 ? 0 : d & 3, n_neg = A.n_neg, n_slots = 3 + n_neg, n_bufs = twice ? 2 * n_str : n_str;
+    const bool slot = lane < n_slots;
+    const uint64_t L = 4 * (uint64_t)d, K = A.K;
+    uint32_t rank, C;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    asm("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(C));
+    float* const mine = chunk_mem + (size_t)w * n_bufs * n_slots * 2 * kPad;            // [buffer][slot][Re, Im][kPad]
+    double* const s_part = reinterpret_cast<double*>(chunk_mem + (size_t)n_warps * n_bufs * n_slots * 2 * kPad);  // [parity][rank][warp][1 + kMaxNeg]
+    double* const s_w = s_part + 2 * C * n_warps * (kMaxNeg + 1) + w * 3 * kNumbers;    // the warp's: coefficients, weights of a slot's directions
+    uint64_t* const s_off = reinterpret_cast<uint64_t*>(s_part + 2 * C * n_warps * (kMaxNeg + 1) + n_warps * 3 * kNumbers);   // [parity][slot]
+    uint64_t* const bars = s_off + 64 + w * n_bufs;
+    int* const s_dead = reinterpret_cast<int*>(s_off + 64 + n_warps * n_bufs);          // [parity]; then s_failed
+    if (lane < n_bufs) mbar_init(&bars[lane], 1);
+    if (tid < 3) s_dead[tid] = 0;
+    mbar_init_fence();
+    pdl_trigger();
+    pdl_wait();
+    __syncthreads();
+    if (C > 1) {                                                // (all blocks have started, their words are zero)
+        cluster_arrive();
+        cluster_wait();
+    }
+    if (A.single) {
+        bool failed = call_failed(A.st, A.epoch);
+        if (C > 1) {                                            // a block that started later may see more: one decision
+            if (tid == 0) s_dead[2] = failed;
+            cluster_arrive();
+            cluster_wait();
+            for (uint32_t r = 0; r < C; ++r) failed |= peer_i32(&s_dead[2], r) != 0;
+            cluster_arrive();
+            cluster_wait();
+        }
+        if (failed) return;
+    }
+    const uint64_t stride = gridDim.x / C;
+    // what a warp knows of a data point: lane u its slot u
+    struct Point {
+        uint64_t off;
+        uint32_t key;
+        int rep;
+        unsigned same, subj, reps, once;
+        bool bad;
+    };
+    auto look_up = [&](uint64_t t) {
+        Point P;
+        uint64_t key = K;
+        int side = 0;
+        bool bad = false;
+        if (slot) {
+            if (lane == 1) {
+                key = A.rel_base + A.tr[t];
+                bad = key >= K;
+            } else {
+                key = lane == 0 ? A.ts[t] : (lane == 2 ? A.to[t] : A.neg_ent[t * n_neg + (lane - 3)]);
+                bad = key >= A.rel_base;
+                if (lane >= 3) side = A.neg_side[t * n_neg + (lane - 3)] != 0;
+            }
+        }
+        P.bad = __any_sync(full, bad);
+        P.key = (uint32_t)key;
+        P.same = __match_any_sync(full, slot ? P.key : kSentinelPad);
+        P.rep = slot ? __ffs(P.same) - 1 : (int)lane;
+        const bool once = slot && !P.bad && A.single && P.rep == (int)lane && A.single[t * n_slots + lane];
+        P.off = (slot && !P.bad) ? phys_row(A.table[key], A.S) * L : 0;
+        P.subj = __ballot_sync(full, lane >= 3 && slot && side == 0) >> 3;
+        P.reps = __ballot_sync(full, slot && P.rep == (int)lane);
+        P.once = __ballot_sync(full, once);
+        return P;
+    };
+    // the first data point (from `from` on) whose indexes are all valid; marks the others (the same in every warp)
+    auto next_valid = [&](uint64_t from, Point& Q) {
+        for (; from < A.n; from += stride) {
+            Q = look_up(from);
+            if (A.keys_out && slot && w == 0 && rank == 0)
+                A.keys_out[from * n_slots + lane] = Q.bad ? kSentinelPad : Q.rep == (int)lane ? Q.key : (uint32_t)K;
+            if (!Q.bad) break;
+            if (tid == 0) latch_error(A.st, A.keys_out ? 0u : A.epoch, PS_ERR_KEY_RANGE);
+        }
+        return from;
+    };
+    // the lane's two dimensions at row + its first (the second may lie past the row: zero)
+    auto get = [&](const float* row, bool both) {
+        if constexpr (kVec > 1) return *reinterpret_cast<const float2*>(row);
+        else return make_float2(row[0], both ? row[32] : 0.f);
+    };
+    auto put = [&](float* row, bool both, float x, float y) {
+        if constexpr (kVec > 1) {
+            *reinterpret_cast<float2*>(row) = make_float2(x, y);
+        } else {
+            row[0] = x;
+            if (both) row[32] = y;
+        }
+    };
+    const uint32_t first = kVec > 1 ? 2 * lane : lane;
+    auto chunk_at = [&](uint32_t s) { return ((s * C + rank) * n_warps + w) * 64; };
+    auto buffer_of = [&](uint32_t j, uint32_t s) { return twice ? (j & 1) * n_str + s : s; };      // j: the block's j-th data point
+    auto parity_of = [&](uint32_t j) { return (twice ? j >> 1 : j) & 1; };
+    // lane u asks for the chunk of slot u's row (and has its accumulators brought to L2, where they are wanted)
+    auto ask = [&](const Point& Q, uint32_t j, uint32_t s) {
+        const uint32_t c0 = chunk_at(s);
+        if (c0 >= d) return;
+        const uint32_t len = tmin(64u, d - c0), buf = buffer_of(j, s);
+        const uint32_t re_bytes = ((len + 3) & ~3u) * 4, im_bytes = ((len + shift + 3) & ~3u) * 4;   // (Im may start between two 16-byte boundaries)
+        if (lane == 0) mbar_expect_tx(&bars[buf], n_slots * (re_bytes + im_bytes));
+        __syncwarp();
+        if (!slot) return;
+        float* to = mine + (size_t)(buf * n_slots + lane) * 2 * kPad;
+        const float* row = A.store + Q.off + c0;
+        bulk_g2s(to, row, re_bytes, &bars[buf]);
+        bulk_g2s(to + kPad, row + d - shift, im_bytes, &bars[buf]);
+        if ((Q.once >> lane) & 1u) {
+            const uint32_t at_re = (2 * d) & 3, at_im = (3 * d) & 3;
+            bulk_prefetch(row + 2 * d - at_re, ((len + at_re + 3) & ~3u) * 4);
+            bulk_prefetch(row + 3 * d - at_im, ((len + at_im + 3) & ~3u) * 4);
+        }
+    };
+    Point P = {}, N = {};
+    uint64_t t = next_valid(blockIdx.x / C, P);
+    double loss = 0;
+    if (t < A.n)
+        for (uint32_t s = 0; s < n_str; ++s) ask(P, 0, s);
+    uint32_t j = 0;
+    uint64_t tn = A.n;
+    bool dead = false;
+    for (; t < A.n; ++j) {
+        tn = next_valid(t + stride, N);
+        if (twice && tn < A.n) {
+            fence_async_smem();                                 // (the data point before this one has been read from there)
+            __syncwarp();
+            for (uint32_t s = 0; s < n_str; ++s) ask(N, j + 1, s);
+        }
+        const unsigned subj_mask = P.subj, rep_mask = P.reps, acc_mask = P.once;
+        const int rep_o = __shfl_sync(full, P.rep, 2);          // 0 if object == subject
+        // ---- pass A: scores of the 1 + n_neg triples over the warp's dimensions, two per lane at a time ----
+        double part[NP];
+#pragma unroll
+        for (int q = 0; q < NP; ++q) part[q] = 0.0;
+        for (uint32_t s = 0; s < n_str; ++s) {
+            const uint32_t c0 = chunk_at(s), buf = buffer_of(j, s);
+            if (c0 >= d) break;
+            if (!mbar_wait(&bars[buf], parity_of(j)) && !mbar_wait(&bars[buf], parity_of(j))) dead = true;
+            if (c0 + first >= d) continue;
+            const bool both = c0 + first + kStep < d;
+            const float *at = mine + (size_t)buf * n_slots * 2 * kPad + first, *at_im = at + kPad + shift;
+            auto re = [&](int u) { return get(at + u * 2 * kPad, both); };
+            auto im = [&](int u) { return get(at_im + u * 2 * kPad, both); };
+            const float2 av = re(0), bv = im(0), crv = re(1), civ = im(1), ev = re(2), fv = im(2);
+            double re_o[2], im_o[2], re_s[2], im_s[2];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const double a = i ? av.y : av.x, b = i ? bv.y : bv.x, cr = i ? crv.y : crv.x, ci = i ? civ.y : civ.x;
+                const double e = i ? ev.y : ev.x, f = i ? fv.y : fv.x;
+                part[0] += cr * (a * e + b * f) + ci * (a * f - b * e);
+                re_o[i] = cr * e + ci * f; im_o[i] = cr * f - ci * e;           // multiplies a negative in the subject's place
+                re_s[i] = cr * a - ci * b; im_s[i] = cr * b + ci * a;           // ... in the object's place
+            }
+#pragma unroll
+            for (int q = 0; q < kMaxNeg; ++q) {
+                if (q >= (int)n_neg) break;
+                const float2 na = re(3 + q), nb = im(3 + q);
+                if ((subj_mask >> q) & 1u)
+                    part[q + 1] += ((double)na.x * re_o[0] + (double)nb.x * im_o[0]) + ((double)na.y * re_o[1] + (double)nb.y * im_o[1]);
+                else
+                    part[q + 1] += ((double)na.x * re_s[0] + (double)nb.x * im_s[0]) + ((double)na.y * re_s[1] + (double)nb.y * im_s[1]);
+            }
+        }
+        // ---- the warps' sums meet in every block of the cluster, and are added in the order of the row ----
+        const uint32_t parity = j & 1;                          // (two data points on, all have met again: what is read below has been read)
+        {
+            const double sum = lane_sums<NP>(part, lane);
+            const uint32_t q = lane / (32 / NP);
+            double* const to = s_part + ((size_t)(parity * C + rank) * n_warps + w) * (kMaxNeg + 1) + q;
+            const bool writes = lane % (32 / NP) == 0 && q <= kMaxNeg;
+            if (w == 0) s_off[parity * 32 + lane] = P.off;
+            if (C == 1) {
+                if (writes) *to = sum;
+                if (dead) s_dead[parity] = 1;
+                __syncthreads();
+            } else {
+                for (uint32_t r = 0; r < C; ++r) {
+                    if (writes) asm volatile("st.shared::cluster.f64 [%0], %1;\n" ::"r"(peer_smem(to, r)), "d"(sum) : "memory");
+                    if (dead) asm volatile("st.shared::cluster.u32 [%0], %1;\n" ::"r"(peer_smem(&s_dead[parity], r)), "r"(1) : "memory");
+                }
+                cluster_arrive();
+                cluster_wait();
+            }
+        }
+        dead = *(volatile int*)&s_dead[parity] != 0;            // the same decision in every warp of the cluster
+        if (dead) break;
+        double coef = 0, loss_q = 0;                            // lane q + 1: negative q; lane 0: the triple
+        if (lane <= n_neg) {
+            const double* from = s_part + (size_t)parity * C * n_warps * (kMaxNeg + 1) + lane;
+            double phi = 0;
+            for (uint32_t i = 0; i < C * n_warps; ++i) phi += from[i * (kMaxNeg + 1)];
+            const double y = lane == 0 ? 1.0 : -1.0, z = -y * phi, ez = exp(-fabs(z));
+            loss_q = fmax(z, 0.0) + log1p(ez);
+            coef = -y * ((z >= 0.0 ? 1.0 : ez) / (1.0 + ez));
+        }
+        loss += loss_q;                                         // (lane q's share)
+        // ---- weights with which each entity slot receives the two "negative role" directions (see kge_short_kernel) ----
+        double *const cf = s_w, *const ws = s_w + kNumbers, *const wo = s_w + 2 * kNumbers;
+        if (lane >= 1 && lane <= n_neg) cf[lane - 1] = coef;
+        __syncwarp();
+        double wS = 0, wO = 0;
+        if (slot && P.rep == (int)lane) {
+            for (unsigned m = (P.same >> 3) & ((1u << n_neg) - 1u); m; m &= m - 1) {
+                const int q = __ffs(m) - 1;
+                if ((subj_mask >> q) & 1u) wS += cf[q]; else wO += cf[q];
+            }
+        }
+        if (lane < kNumbers) {
+            ws[lane] = wS;
+            wo[lane] = wO;
+        }
+        const double cf0 = __shfl_sync(full, coef, 0);
+        __syncwarp();
+        // ---- pass B: gradients ----
+        const uint32_t LU = 2 * d;                              // values per update row
+        float* const U = A.upd + t * n_slots * (uint64_t)LU;
+        const uint64_t* const off = s_off + parity * 32;
+        for (uint32_t s = 0; s < n_str; ++s) {
+            const uint32_t c0 = chunk_at(s), buf = buffer_of(j, s), at0 = c0 + first;
+            if (c0 >= d) break;
+            if (at0 < d) {
+                const bool both = at0 + kStep < d;
+                const float *at = mine + (size_t)buf * n_slots * 2 * kPad + first, *at_im = at + kPad + shift;
+                auto re = [&](int u) { return get(at + u * 2 * kPad, both); };
+                auto im = [&](int u) { return get(at_im + u * 2 * kPad, both); };
+                struct Acc { float2 re, im; };
+                // the accumulators of slot u, where they are needed
+                auto acc_of = [&](int u) {
+                    Acc G = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+                    if ((acc_mask >> u) & 1u) {
+                        const float* g = A.store + off[u] + 2 * d + at0;
+                        G.re = get(g, both);
+                        G.im = get(g + d, both);
+                    }
+                    return G;
+                };
+                auto out = [&](int u, const double (&gd)[4], const Acc& G) {    // gd: Re, Re, Im, Im
+                    const float g[4] = {(float)gd[0], (float)gd[1], (float)gd[2], (float)gd[3]};
+                    if (!((acc_mask >> u) & 1u)) {
+                        float* o = U + (uint64_t)u * LU + at0;
+                        put(o, both, g[0], g[1]);
+                        put(o + d, both, g[2], g[3]);
+                        return;
+                    }
+                    const float x[4] = {__fadd_rn(G.re.x, __fmul_rn(g[0], g[0])), __fadd_rn(G.re.y, __fmul_rn(g[1], g[1])),
+                                        __fadd_rn(G.im.x, __fmul_rn(g[2], g[2])), __fadd_rn(G.im.y, __fmul_rn(g[3], g[3]))};
+                    float step[4];
+                    adagrad_steps<4>(g, x, A.lr, A.eps, step);
+                    const float2 r = re(u), m = im(u);
+                    float* o = A.store + off[u] + at0;          // in place
+                    put(o, both, r.x + step[0], r.y + step[1]);
+                    put(o + d, both, m.x + step[2], m.y + step[3]);
+                    put(o + 2 * d, both, x[0], x[1]);
+                    put(o + 3 * d, both, x[2], x[3]);
+                };
+                const Acc G0 = acc_of(0), G1 = acc_of(1), G2 = acc_of(2);
+                Acc Ga = acc_of(tmin(3u, n_slots - 1)), Gb = acc_of(tmin(4u, n_slots - 1));
+                // the negatives' weighted sums: in the subject's place, in the object's
+                double A0[2] = {0.0, 0.0}, B0[2] = {0.0, 0.0}, A1[2] = {0.0, 0.0}, B1[2] = {0.0, 0.0};
+#pragma unroll
+                for (int q = 0; q < kMaxNeg; ++q) {
+                    if (q >= (int)n_neg) break;
+                    const float2 na = re(3 + q), nb = im(3 + q);
+                    const double wq = cf[q];
+                    if ((subj_mask >> q) & 1u) {
+                        A0[0] += wq * (double)na.x; A0[1] += wq * (double)na.y;
+                        B0[0] += wq * (double)nb.x; B0[1] += wq * (double)nb.y;
+                    } else {
+                        A1[0] += wq * (double)na.x; A1[1] += wq * (double)na.y;
+                        B1[0] += wq * (double)nb.x; B1[1] += wq * (double)nb.y;
+                    }
+                }
+                double dS[4], dO[4];                            // d phi / d subject (object = o), d phi / d object (subject = s)
+                {
+                    const float2 av = re(0), bv = im(0), crv = re(1), civ = im(1), ev = re(2), fv = im(2);
+                    double gs[4], gr[4], go[4];
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) {
+                        const double a = i ? av.y : av.x, b = i ? bv.y : bv.x, cr = i ? crv.y : crv.x, ci = i ? civ.y : civ.x;
+                        const double e = i ? ev.y : ev.x, f = i ? fv.y : fv.x;
+                        dS[i] = cr * e + ci * f; dS[2 + i] = cr * f - ci * e;
+                        dO[i] = cr * a - ci * b; dO[2 + i] = cr * b + ci * a;
+                        gr[i] = cf0 * (a * e + b * f) + (A0[i] * e + B0[i] * f) + (a * A1[i] + b * B1[i]);
+                        gr[2 + i] = cf0 * (a * f - b * e) + (A0[i] * f - B0[i] * e) + (a * B1[i] - b * A1[i]);
+                        // (negatives that coincide with the subject or the object: the slots' weights)
+                        go[i] = cf0 * dO[i] + (cr * A0[i] - ci * B0[i]) + ws[2] * dS[i] + wo[2] * dO[i];
+                        go[2 + i] = cf0 * dO[2 + i] + (cr * B0[i] + ci * A0[i]) + ws[2] * dS[2 + i] + wo[2] * dO[2 + i];
+                        gs[i] = cf0 * dS[i] + (cr * A1[i] + ci * B1[i]) + ws[0] * dS[i] + wo[0] * dO[i];
+                        gs[2 + i] = cf0 * dS[2 + i] + (cr * B1[i] - ci * A1[i]) + ws[0] * dS[2 + i] + wo[0] * dO[2 + i];
+                        if (rep_o == 0) { gs[i] += go[i]; gs[2 + i] += go[2 + i]; }
+                    }
+                    out(0, gs, G0);
+                    out(1, gr, G1);
+                    if (rep_o == 2) out(2, go, G2);
+                }
+                // one negative after the other, the accumulators of the next two on their way
+#pragma unroll 1
+                for (uint32_t u = 3; u < n_slots; ++u) {
+                    const Acc Gc = acc_of(tmin(u + 2, n_slots - 1));
+                    if ((rep_mask >> u) & 1u) {
+                        const double wSq = ws[u], wOq = wo[u];
+                        const double g[4] = {wSq * dS[0] + wOq * dO[0], wSq * dS[1] + wOq * dO[1], wSq * dS[2] + wOq * dO[2], wSq * dS[3] + wOq * dO[3]};
+                        out(u, g, Ga);
+                    }
+                    Ga = Gb;
+                    Gb = Gc;
+                }
+            }
+            if (!twice && tn < A.n) {
+                fence_async_smem();                             // (the rows have been read; the next ones come through the async proxy)
+                __syncwarp();
+                ask(N, j + 1, s);
+            }
+        }
+        P = N;
+        t = tn;
+    }
+    if (dead) {                                                 // a copy did not arrive: the call is given up
+        if (w == 0 && rank == 0) give_up(A, t, lane);
+        else if (tid == 0) latch_error(A.st, A.keys_out ? 0u : A.epoch, PS_ERR_CUDA);
+        if (twice && tn < A.n)                          // copies still on their way to this block
+            for (uint32_t s = 0; s < n_str && chunk_at(s) < d; ++s) mbar_wait(&bars[buffer_of(j + 1, s)], parity_of(j + 1));
+    }
+    loss = warp_sum_d(loss);
+    if (tid == 0) A.loss_partial[blockIdx.x] = rank == 0 ? loss : 0.0;
+}
+
 // Keys of the occurrence slots of each data point; a slot that repeats an earlier slot's key, and every
 // slot of a data point with an index out of range, gets the "no key" mark K.
 __global__ void __launch_bounds__(256)
@@ -787,6 +1144,77 @@ uint32_t launch_wide(ps_store* ps, const KgeArgs& A, cudaStream_t s) {
     return grid;
 }
 
+// 0: a data point does not fit one block.  The number of warps per block: as many warps per SM as 128 registers a thread allow (16), in blocks
+// whose chunks go evenly, several chunks per warp where that costs none (a warp's work per data point is about a quarter of
+// a chunk's).
+template <int kMaxNeg, int kVec>
+uint32_t launch_resident(ps_store* ps, const KgeArgs& A, cudaStream_t s) {
+    using R = Resident<kMaxNeg>;
+    const uint32_t chunks = (A.d + 63) / 64, slots = 3 + A.n_neg, sms = (uint32_t)ps->sm_count;
+    constexpr uint32_t kMost = 227 * 1024, kPerSm = 228 * 1024;
+    uint32_t warps = 0, n_str = 0, resident = 0, C = 1;
+    bool twice = false;
+    for (;; C *= 2) {
+        const uint32_t per = (chunks + C - 1) / C;
+        double best = 0;
+        for (uint32_t w = 1; w <= tmin(16u, per); ++w) {
+            const uint32_t str = (per + w - 1) / w;
+            const size_t once = R::smem(kVec, slots, w, str, C), both = R::smem(kVec, slots, w, 2 * str, C);
+            if (once > kMost || 2 * str > 32) continue;
+            const uint32_t blocks = tmin<uint32_t>(16 / w, (uint32_t)(kPerSm / (once + 1024)));
+            const double score = (double)blocks * per / str * (4 * str) / (4 * str + 1);
+            if (score > best) {
+                best = score;
+                warps = w;
+                n_str = str;
+                resident = blocks;
+                twice = both <= kMost && blocks * (both + 1024) <= kPerSm;
+            }
+        }
+        if (!warps) return 0;
+        // few data points: a cluster of two or four blocks for each, as long as none has to wait (16 data points of 600 dimensions
+        // and their reduction: 24 -> 20 us)
+        if (C == 4 || A.n * 2 * C > (uint64_t)sms * resident || chunks < 4 * C) break;
+    }
+    const void* fn = (const void*)kge_resident_kernel<kMaxNeg, kVec>;
+    const size_t smem = R::smem(kVec, slots, warps, twice ? 2 * n_str : n_str, C);
+    static std::atomic<unsigned long long> smem_set{0};
+    opt_in_smem(fn, kMost, &smem_set);
+    cudaLaunchConfig_t cfg = {};
+    cfg.blockDim = dim3(32 * warps);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = C;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    uint64_t places = (uint64_t)sms * resident;
+    if (C > 1) {                                                // clusters resident at once: asked once per shape
+        ClusterFit& f = ps->kge_fit;
+        if (f.fn != fn || f.smem != smem || f.threads != 32 * warps || f.blocks != C) {
+            int clusters = 0;
+            cfg.gridDim = dim3(C);
+            cfg.numAttrs = 1;
+            if (cudaOccupancyMaxActiveClusters(&clusters, fn, &cfg) != cudaSuccess) cudaGetLastError();
+            f.fn = fn; f.smem = smem; f.threads = 32 * warps; f.blocks = C;
+            f.clusters = (uint32_t)tmax(clusters, 0);
+        }
+        places = f.clusters;
+        if (places == 0) return 0;
+    }
+    const uint32_t grid = (uint32_t)tmin<uint64_t>(A.n, places) * C;
+    cfg.gridDim = dim3(grid);
+    cfg.numAttrs = A.keys_out ? 2 : 1;                          // (the pdl form: kernels of small calls)
+    if (ps->prof) prof_before(ps, "kge_resident_kernel", s);
+    cudaLaunchKernelEx(&cfg, kge_resident_kernel<kMaxNeg, kVec>, A, n_str, twice);
+    if (ps->prof) prof_after(ps, s);
+    ps->launches++;
+    return grid;
+}
+
 }  // namespace
 
 uint32_t launch_points_kge(ps_store* ps, const KgeBatch& B, const uint8_t* single, bool finished, uint32_t* keys_out, cudaStream_t s) {
@@ -814,6 +1242,16 @@ uint32_t launch_points_kge(ps_store* ps, const KgeBatch& B, const uint8_t* singl
         return grid;                                                                                             \
     } while (0)
     if (B.dim > 128) {
+        if (!finished) {
+#define KGE_RESIDENT(kMaxNeg)                                                                                     \
+            (B.dim % 4 == 0 ? launch_resident<kMaxNeg, 4>(ps, A, s) : B.dim % 2 == 0 ? launch_resident<kMaxNeg, 2>(ps, A, s) \
+                            : launch_resident<kMaxNeg, 1>(ps, A, s))
+            const uint32_t grid = B.n_neg <= 4    ? KGE_RESIDENT(4)
+                                  : B.n_neg <= 10 ? KGE_RESIDENT(10)
+                                  : B.n_neg <= 20 ? KGE_RESIDENT(20) : KGE_RESIDENT(29);
+#undef KGE_RESIDENT
+            if (grid) return grid;
+        }
 #define KGE_WIDE(kMaxNeg) return finished ? launch_wide<kMaxNeg, true>(ps, A, s) : launch_wide<kMaxNeg, false>(ps, A, s)
         if (B.n_neg <= 4) KGE_WIDE(4);
         if (B.n_neg <= 10) KGE_WIDE(10);

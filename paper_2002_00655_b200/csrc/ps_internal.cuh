@@ -45,6 +45,13 @@ struct DevStatus {
     unsigned long long loc_deferred;        // moved keys that had to wait for the call running beside the relocation
 };
 
+// clusters of a kernel that are resident at once, for the launch shape last asked about
+struct ClusterFit {
+    const void* fn;
+    size_t smem;
+    uint32_t threads, blocks, clusters;
+};
+
 static_assert(kSortSets <= 4, "one error-epoch word per call in flight");
 
 struct Profile;
@@ -140,6 +147,7 @@ struct ps_store {
     bool table_dirty[psb::kSideStreams];   // per side stream: the location table was rewritten since that stream last waited
                                     // for the caller's (a sort that reads the table must not start before the rewrite)
     unsigned long long capture_id;  // graph capture the caller's stream was in at the last step call (0 = none)
+    psb::ClusterFit kge_fit;
 };
 
 namespace psb {
@@ -561,6 +569,10 @@ __device__ __forceinline__ void tma_gather4(void* smem, const CUtensorMap* map, 
         "%5, %6}], [%7];\n" ::"r"(smem_addr(smem)),
         "l"(map), "r"(x), "r"(y0), "r"(y1), "r"(y2), "r"(y3), "r"(smem_addr(bar))
         : "memory");
+}
+// asks for `bytes` (a multiple of 16) from a 16-byte boundary on to be in L2
+__device__ __forceinline__ void bulk_prefetch(const void* gmem, unsigned bytes) {
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(gmem), "r"(bytes) : "memory");
 }
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;\n" ::: "memory"); }
 // until at most kPending of this thread's bulk groups still have to READ their source

@@ -1,0 +1,35 @@
+"""GPU parity of ComplEx on rows of more than 128 dimensions that stay in shared memory: chunks of 64 dimensions and their remainders, every
+alignment of a row's second half, one to 32 rows per data point, clusters for few data points, the last sizes that fit."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2002_00655_b200 as ps
+from tests.test_gpu_sorted import EPS, LR, ada_rows, check, check_no_op, on_gpu, triples
+from tests.util import make_pair
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("dim,n_neg", [(129, 10), (130, 0), (132, 20), (191, 29), (320, 10), (578, 13), (832, 29), (834, 29), (1001, 4), (1216, 20),
+                                       (2176, 10), (2178, 10)])
+@pytest.mark.parametrize("few", [2, 75, 0])
+def test_complex_rows_kept_in_shared_memory(dim, n_neg, few):
+    rng = np.random.default_rng(dim + few)
+    n = few or 8192 // (3 + n_neg) + 5                          # 0: as many as take a sort
+    E, R = (40, 3) if few else (n, 7)                           # (few entities: the same one in several places of a data point)
+    K = E + R
+    g, o = make_pair(K, 4 * dim, rows=ada_rows(rng, K, 4 * dim), max_batch_keys=(3 + n_neg) * n)
+    ps.ps_set_pipelining(g.h, True)
+    batches = [triples(rng, n, n_neg, E, R) for _ in range(2)]
+    gpu = [on_gpu(b) for b in batches]
+    torch.cuda.synchronize()
+    for b, d in zip(batches, gpu):
+        ps.ps_step_kge(g.h, *d, n_neg, E, dim, LR, EPS, g.loss)
+        o.step_kge(*b, E, dim, LR, EPS)
+    check(g, o, "complex")
+    bad = [x.copy() for x in batches[0]]
+    bad[2][-1] = E
+    d = on_gpu(bad)
+    torch.cuda.synchronize()
+    check_no_op(g, o, lambda: ps.ps_step_kge(g.h, *d, n_neg, E, dim, LR, EPS, g.loss), "an object out of range")
