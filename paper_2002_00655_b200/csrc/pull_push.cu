@@ -9,6 +9,8 @@
 //       cross tile borders; a second kernel adds those partials in tile order.
 //       The order of every sum is fixed by the sorted positions, so results
 //       are reproducible bit for bit.
+#include <type_traits>
+
 #include "ps_internal.cuh"
 
 namespace psb {
@@ -491,9 +493,13 @@ push_reduce_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restrict__
 // asked for at its start (prefetch_row) and read where they end.  Staged by bulk copies, a position at a time, the walk was
 // bound by its instructions (215 per position, issue slots 74 % used; now 85): 276 us for 1.04M positions of rows of 300
 // values, now 242 with two positions in flight at three blocks per SM (four at two blocks 287, three 297), bound by the
-// latency of its loads and the unit that widens values to fp64 (60 %).
+// latency of its loads and the unit that widens values to fp64 (60 %; an instruction of it takes as long for two lanes as for
+// 32).  So a row's last column block is spread over the lanes, kTail values each: 160 values are five per lane, not eight.
+// us per launch, with four throughout and now: 328,000 positions of 160 values 104 and 83, of 32 values 42 and 37, of 64
+// values 43 and 40, 164,000 of 300 values 59 and 52.
+// Tried without gain: four rows in flight as 16-byte asynchronous copies at 32 warps per SM; widening by integer operations.
 // skip_singles: keys that occur once have been updated by the gradient kernel.
-template <int kCh>
+template <int kCh, int kTail>
 __global__ void __launch_bounds__(256, kCh == 3 || kCh == 1 ? 3 : 2)
 scaled_reduce_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restrict__ sv, uint32_t n,
                      const float4* __restrict__ upd, const float* __restrict__ scales, uint32_t slots, uint32_t tile_len, bool skip_singles,
@@ -517,16 +523,42 @@ scaled_reduce_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restrict
     }
     const uint32_t L = L4 * 4;
     // (rows of more than 128 (kCh - 1) values: the dispatch's rule; only the last column block needs the comparison)
-    auto in_row = [&](int c) { return c + 1 < kCh || lane + 32 * c < L4; };
+    constexpr int kN = 4 * (kCh - 1) + kTail;                   // values of a row per lane
+    using Tail = typename std::conditional<kTail == 4, float4, typename std::conditional<kTail == 2, float2, float>::type>::type;
+    const bool in_tail = 128 * (kCh - 1) + kTail * lane < L;
+    // a row's values of this lane, from the row's first element on
+    auto get = [&](const float* row, float (&v)[kN]) {
+#pragma unroll
+        for (int c = 0; c + 1 < kCh; ++c) {
+            const float4 x = *reinterpret_cast<const float4*>(row + 128 * c + 4 * lane);
+            v[4 * c] = x.x; v[4 * c + 1] = x.y; v[4 * c + 2] = x.z; v[4 * c + 3] = x.w;
+        }
+        if (in_tail) {
+            const Tail x = *reinterpret_cast<const Tail*>(row + 128 * (kCh - 1) + kTail * lane);
+#pragma unroll
+            for (int i = 0; i < kTail; ++i) v[kN - kTail + i] = reinterpret_cast<const float*>(&x)[i];
+        }
+    };
+    auto put = [&](float* row, const float (&v)[kN]) {
+#pragma unroll
+        for (int c = 0; c + 1 < kCh; ++c)
+            *reinterpret_cast<float4*>(row + 128 * c + 4 * lane) = make_float4(v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]);
+        if (in_tail) {
+            Tail x;
+#pragma unroll
+            for (int i = 0; i < kTail; ++i) reinterpret_cast<float*>(&x)[i] = v[kN - kTail + i];
+            *reinterpret_cast<Tail*>(row + 128 * (kCh - 1) + kTail * lane) = x;
+        }
+    };
     constexpr int kG = kCh >= 3 ? 2 : 4;
-    d4 acc[kCh];
+    double acc[kN];
+    float u[kG][kN];                                            // (elements past the row are never loaded: zero throughout)
 #pragma unroll
-    for (int c = 0; c < kCh; ++c) acc[c] = d4{0.0, 0.0, 0.0, 0.0};
-    float4 u[kG][kCh];                                          // (elements past the row are never loaded: zero throughout)
+    for (int i = 0; i < kN; ++i) {
+        acc[i] = 0.0;
 #pragma unroll
-    for (int k = 0; k < kG; ++k)
-#pragma unroll
-        for (int c = 0; c < kCh; ++c) u[k][c] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int k = 0; k < kG; ++k) u[k][i] = 0.f;
+    }
     bool entered = true;                                        // no segment has begun in this tile so far
     for (uint32_t done = 0; done < tile_len; done += span) {
         const uint64_t base = (uint64_t)tile * tile_len + done;
@@ -570,10 +602,7 @@ scaled_reduce_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restrict
             for (int k = 0; k < kG; ++k) {
                 at[k] = todo ? __ffs(todo) - 1 : -1;
                 todo &= todo - 1;                                   // 0 stays 0
-                const float4* src = upd + (uint64_t)__shfl_sync(full, occ, at[k] & 31) * L4 + lane;
-#pragma unroll
-                for (int c = 0; c < kCh; ++c)
-                    if (in_row(c)) u[k][c] = __ldg(src + 32 * c);      // (past the last: some other row, not used)
+                get(reinterpret_cast<const float*>(upd + (uint64_t)__shfl_sync(full, occ, at[k] & 31) * L4), u[k]);    // (past the last: some other row, not used)
             }
 #pragma unroll
             for (int k = 0; k < kG; ++k) {
@@ -582,45 +611,38 @@ scaled_reduce_kernel(const uint32_t* __restrict__ sk, const uint32_t* __restrict
                 const float sc = __shfl_sync(full, scale, p);
                 const bool ends = (end_mask >> p) & 1u, whole = (fetch_mask >> p) & 1u;
                 if (whole && ((head_mask >> p) & 1u)) {             // one occurrence: a multiply-add rounds the exact sum once
-                    float4* to = store + __shfl_sync(full, row, p) * L4 + lane;
+                    float* to = reinterpret_cast<float*>(store + __shfl_sync(full, row, p) * L4);
+                    float v[kN] = {};
+                    get(to, v);
 #pragma unroll
-                    for (int c = 0; c < kCh; ++c) {
-                        if (!in_row(c)) continue;
-                        float4 v = to[32 * c];
-                        v.x = fmaf(sc, u[k][c].x, v.x); v.y = fmaf(sc, u[k][c].y, v.y);
-                        v.z = fmaf(sc, u[k][c].z, v.z); v.w = fmaf(sc, u[k][c].w, v.w);
-                        to[32 * c] = v;
-                    }
+                    for (int i = 0; i < kN; ++i) v[i] = fmaf(sc, u[k][i], v[i]);
+                    put(to, v);
                     continue;
                 }
                 const double d = (double)sc;
 #pragma unroll
-                for (int c = 0; c < kCh; ++c) {
-                    acc[c].x += d * (double)u[k][c].x; acc[c].y += d * (double)u[k][c].y;
-                    acc[c].z += d * (double)u[k][c].z; acc[c].w += d * (double)u[k][c].w;
-                }
+                for (int i = 0; i < kN; ++i) acc[i] += d * (double)u[k][i];
                 if (!ends) continue;
                 if (whole) {
-                    float4* to = store + __shfl_sync(full, row, p) * L4 + lane;
+                    float* to = reinterpret_cast<float*>(store + __shfl_sync(full, row, p) * L4);
+                    float v[kN] = {};
+                    get(to, v);
 #pragma unroll
-                    for (int c = 0; c < kCh; ++c) {
-                        if (!in_row(c)) continue;
-                        float4 v = to[32 * c];
-                        v.x = (float)((double)v.x + acc[c].x); v.y = (float)((double)v.y + acc[c].y);
-                        v.z = (float)((double)v.z + acc[c].z); v.w = (float)((double)v.w + acc[c].w);
-                        to[32 * c] = v;
-                    }
+                    for (int i = 0; i < kN; ++i) v[i] = (float)((double)v[i] + acc[i]);
+                    put(to, v);
                 } else {
-                    double* cs = carry + ((uint64_t)tile * 2 + ((uint32_t)p < first_head ? 0 : 1)) * L + (uint64_t)lane * 4;
+                    double* cs = carry + ((uint64_t)tile * 2 + ((uint32_t)p < first_head ? 0 : 1)) * L;
 #pragma unroll
-                    for (int c = 0; c < kCh; ++c) {
-                        if (!in_row(c)) continue;
-                        *(double2*)(cs + 128 * c) = make_double2(acc[c].x, acc[c].y);
-                        *(double2*)(cs + 128 * c + 2) = make_double2(acc[c].z, acc[c].w);
+                    for (int c = 0; c + 1 < kCh; ++c) {
+                        *(double2*)(cs + 128 * c + 4 * lane) = make_double2(acc[4 * c], acc[4 * c + 1]);
+                        *(double2*)(cs + 128 * c + 4 * lane + 2) = make_double2(acc[4 * c + 2], acc[4 * c + 3]);
                     }
+#pragma unroll
+                    for (int i = 0; i < kTail; ++i)
+                        if (in_tail) cs[128 * (kCh - 1) + kTail * lane + i] = acc[kN - kTail + i];
                 }
 #pragma unroll
-                for (int c = 0; c < kCh; ++c) acc[c] = d4{0.0, 0.0, 0.0, 0.0};
+                for (int i = 0; i < kN; ++i) acc[i] = 0.0;
             }
         }
     }
@@ -1337,20 +1359,28 @@ void run_push_reduce(ps_store* ps, uint32_t n, int which, const float* d_upd, do
         ps->launches++;                                                                                              \
     } while (0)
     if (d_scales) {
-#define SCALED_LAUNCH(kCh)                                                                                           \
+#define SCALED_LAUNCH_AS(kCh, kTail)                                                                                 \
     do {                                                                                                             \
         if (ps->prof) prof_before(ps, "scaled_reduce_kernel<" #kCh ">", s);                                          \
-        scaled_reduce_kernel<kCh><<<blocks, 256, 0, s>>>(sk, sv, n, (const float4*)d_upd, d_scales, slots,  \
+        scaled_reduce_kernel<kCh, kTail><<<blocks, 256, 0, s>>>(sk, sv, n, (const float4*)d_upd, d_scales, slots,  \
             tile_len, skip_singles, (float4*)ps->store, ps->table, ps->cfg.slots_per_part, (uint32_t)ps->cfg.num_keys, L4, ps->carry, \
             ps->starters, ps->starter_count, ps->group_done, ps->group_sum, ps->status, ps->epoch);                  \
         if (ps->prof) prof_after(ps, s);                                                                             \
         ps->launches++;                                                                                              \
+    } while (0)
+#define SCALED_LAUNCH(kCh)                                                                                           \
+    do {                                                                                                             \
+        const uint32_t rest = ps->cfg.row_len - 128 * ((kCh) - 1);                                                   \
+        if (rest <= 32) SCALED_LAUNCH_AS(kCh, 1);                                                                    \
+        else if (rest <= 64) SCALED_LAUNCH_AS(kCh, 2);                                                               \
+        else SCALED_LAUNCH_AS(kCh, 4);                                                                               \
     } while (0)
         if (L4 <= 32) SCALED_LAUNCH(1);
         else if (L4 <= 64) SCALED_LAUNCH(2);
         else if (L4 <= 96) SCALED_LAUNCH(3);
         else SCALED_LAUNCH(4);
 #undef SCALED_LAUNCH
+#undef SCALED_LAUNCH_AS
     } else {
         if (L4 <= 32) REDUCE_LAUNCH(1);
         else if (L4 <= 64) REDUCE_LAUNCH(2);

@@ -224,3 +224,17 @@ def test_complex_steps_replayed_from_a_graph(n, pipelined):
     torch.cuda.synchronize()
     assert a.sync() == g.sync() == ps.PS_OK
     assert torch.equal(a.export(table=False)[0], g.export(table=False)[0]) and loss_of(a) == loss_of(g)
+
+
+@pytest.mark.parametrize("row", [4, 32, 36, 64, 68, 160, 164, 192, 196, 288, 320, 416, 448, 452])
+def test_skip_gram_rows_whose_last_values_are_spread_over_the_lanes(row):
+    """The reduction's last column block holds one, two or four values per lane: around the limits of each."""
+    rng = np.random.default_rng(row)
+    window, n_neg, V = 2, 3, 300
+    n = SMALL // (1 + 2 * window * (1 + n_neg)) + 40
+    g, o = make_pair(2 * V, row, rows=rng.normal(0, 0.1, size=(2 * V, row)).astype(np.float32), max_batch_keys=n * (1 + 2 * window * (1 + n_neg)))
+    tok, neg = u32(rng.integers(0, V, size=n + 2 * window)), u32(rng.integers(0, V, size=(n * 2 * window, n_neg)))
+    d = on_gpu((tok, neg))
+    ps.ps_step_sgns(g.h, d[0], window, n, window, d[1], n_neg, V, 0.01, g.loss)
+    o.step_sgns(tok, window, n, window, neg, n_neg, V, 0.01)
+    check(g, o, "skip-gram")
