@@ -136,8 +136,8 @@ ps_status_t ps_localize(ps_store_t* ps, uint32_t worker, const uint64_t* d_keys,
  *   - every call made on the handle afterwards, on any stream, is ordered after the whole relocation.
  * The result (table, free stacks, rows) is that of ps_localize issued right after the most recent call.
  * If there is nothing to run beside (the most recent call was not a step or push, or was issued on `loc_stream`, or
- * had at most 8,192 key occurrences: such calls keep no sorted list of their keys), or the store has more than
- * 1024 partitions, the call is an ordinary ps_localize on `loc_stream` ordered after everything issued so far.  One such call per step; do not capture it into a CUDA graph. */
+ * was reduced without a sort: such calls, of at most 8,192 key occurrences, keep no sorted list of their keys), or the store has
+ * more than 1024 partitions, the call is an ordinary ps_localize on `loc_stream` ordered after everything issued so far.  One such call per step; do not capture it into a CUDA graph. */
 ps_status_t ps_localize_beside(ps_store_t* ps, uint32_t worker, const uint64_t* d_keys, uint64_t n,
                                void* loc_stream);
 

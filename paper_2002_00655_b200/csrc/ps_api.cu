@@ -605,7 +605,7 @@ ps_status_t ps_step_kge(ps_store_t* ps, const uint32_t* d_s, const uint32_t* d_r
     if (rel_key_base > ps->cfg.num_keys) return PS_ERR_INVALID_ARG;
     const uint32_t occ = (uint32_t)((3 + (uint64_t)n_neg) * n);
     const KgeBatch B = {d_s, d_r, d_o, d_neg_ent, d_neg_side, n, n_neg, rel_key_base, dim_complex, lr, eps};
-    if (small_call(occ)) {
+    if (small_step(occ, dim_complex)) {
         // (the reduction without a sort works on whole float4s: gradient rows where the halves of a row are)
         const bool finished = dim_complex % 2 != 0;
         const uint32_t lb = launch_points_kge(ps, B, nullptr, finished, begin_small(ps), s);
@@ -796,7 +796,7 @@ ps_status_t ps_step_sgns(ps_store_t* ps, const uint32_t* d_tokens, uint64_t firs
     uint64_t occ;
     const ps_status_t c = sgns_checks(ps, first_pos, n_centers, corpus_len, window, n_neg, out_key_base, &occ);
     if (c != PS_OK) return c;
-    if (small_call(occ)) {
+    if (small_step(occ, ps->cfg.row_len)) {
         sgns_small(ps, d_tokens, 0, first_pos, n_centers, corpus_len, window, d_negs, n_neg, out_key_base, lr, occ,
                    d_loss_accum, s);
         return after_launch();
@@ -954,7 +954,7 @@ ps_status_t ps_step_sgns_host(ps_store_t* ps, const uint32_t* h_tokens, uint64_t
     if (n_negs && cudaMemcpyAsync(d_negs, h_negs, n_negs * 4, cudaMemcpyHostToDevice, hb.cs) != cudaSuccess)
         return PS_ERR_CUDA;
     if (!host_batch_copied(ps, s, hb)) return PS_ERR_CUDA;
-    if (small_call(occ)) {
+    if (small_step(occ, ps->cfg.row_len)) {
         sgns_small(ps, d_tok, tok_first, first_pos, n_centers, corpus_len, window, d_negs, n_neg, out_key_base, lr, occ,
                    d_loss_accum, s);
         c = after_launch();

@@ -276,6 +276,15 @@ void run_mf_col(ps_store* ps, uint32_t n_cells, int which, float lr, float lambd
 // slots' keys in small_keys (num_keys: no key; kSentinelPad: index out of range) and its rows in ps->upd, as for the
 // sorted reductions.
 inline bool small_call(uint64_t n_occ) { return n_occ <= kSmallOcc; }
+// ComplEx (dim complex dimensions) and skip-gram (rows of dim values): no sort up to kSmallValues dimensions (values) of all
+// occurrences, either.  A sort costs 12 to 25 us however wide the rows are; without one every gradient is written out and read
+// again, with one most rows are updated in place and the reduction is tiled.  us per step on an ordered handle, without / with a
+// sort: ComplEx with ten negatives, 300 data points of 250 dimensions 40 / 51, 600 of 250 64 / 68, 300 of 500 69 / 63, 600 of 500
+// 116 / 90, 300 of 1,000 130 / 91, 600 of 1,000 218 / 128 (pipelined, calls back to back: 40 / 36, 64 / 52, 69 / 47, 116 / 73,
+// 130 / 74, 218 / 111); skip-gram, 4,100 occurrences of 300 values 35.5 / 35, 7,790 of 300 49 / 38, 7,790 of 512 59 / 42.
+// Pushes and matrix factorization gain nothing from a sort at any width (8,000 rows of 1,024 values: 64 / 87).
+constexpr uint64_t kSmallValues = 1600000;
+inline bool small_step(uint64_t n_occ, uint64_t dim) { return small_call(n_occ) && n_occ * dim <= kSmallValues; }
 uint32_t* small_keys(ps_store* ps);
 void run_small_push_keys(ps_store* ps, const uint64_t* d_keys, uint32_t n, const float* d_upd, cudaStream_t s);
 void run_small_reduce(ps_store* ps, uint32_t n, double* d_loss_accum, uint32_t loss_blocks, cudaStream_t s,

@@ -238,3 +238,33 @@ def test_skip_gram_rows_whose_last_values_are_spread_over_the_lanes(row):
     ps.ps_step_sgns(g.h, d[0], window, n, window, d[1], n_neg, V, 0.01, g.loss)
     o.step_sgns(tok, window, n, window, neg, n_neg, V, 0.01)
     check(g, o, "skip-gram")
+
+
+@pytest.mark.parametrize("pipelined", [False, True])
+@pytest.mark.parametrize("mode,dim,n", [("kge", 250, 492), ("kge", 250, 493), ("kge", 1001, 122), ("kge", 1001, 123), ("sgns", 300, 130),
+                                        ("sgns", 300, 131), ("sgns", 512, 150)])
+def test_wide_steps_on_either_side_of_the_sort(mode, dim, n, pipelined):
+    """Few occurrences of wide rows: with and without a sort (1,600,000 dimensions or values of all occurrences), calls of both kinds
+    one after the other."""
+    rng = np.random.default_rng(dim + n)
+    if mode == "kge":
+        E, R, q = 900, 5, 10
+        g, o = make_pair(E + R, 4 * dim, rows=ada_rows(rng, E + R, 4 * dim), max_batch_keys=(3 + q) * n)
+        ps.ps_set_pipelining(g.h, pipelined)
+        batches = [triples(rng, m, q, E, R) for m in (n, 9, n)]
+        gpu = [on_gpu(b) for b in batches]
+        torch.cuda.synchronize()
+        for b, d in zip(batches, gpu):
+            ps.ps_step_kge(g.h, *d, q, E, dim, LR, EPS, g.loss)
+            o.step_kge(*b, E, dim, LR, EPS)
+    else:
+        V, window, q = 900, 5, 3
+        g, o = make_pair(2 * V, dim, rows=rng.normal(0, 0.1, size=(2 * V, dim)).astype(np.float32), max_batch_keys=n * (1 + 2 * window * (1 + q)))
+        ps.ps_set_pipelining(g.h, pipelined)
+        batches = [(u32(rng.integers(0, V, size=m + 2 * window)), u32(rng.integers(0, V, size=(m * 2 * window, q))), m) for m in (n, 9, n)]
+        gpu = [on_gpu(b[:2]) for b in batches]
+        torch.cuda.synchronize()
+        for (tok, neg, m), d in zip(batches, gpu):
+            ps.ps_step_sgns(g.h, d[0], window, m, window, d[1], q, V, 0.01, g.loss)
+            o.step_sgns(tok, window, m, window, neg, q, V, 0.01)
+    check(g, o, mode)
