@@ -370,7 +370,8 @@ __global__ void __launch_bounds__(32 * kShortWarps, kMaxNeg <= 10 ? 4 : 2) kge_s
     }
 }
 
-// Rows of more than 128 complex dimensions: a block per data point (batches of few data points: a
+// Rows of more than 128 complex dimensions that kge_resident_kernel does not take (more than four blocks' shared memory; odd dimensions in
+// calls without a sort): a block per data point (batches of few data points: a
 // cluster of up to four, which meets to add up the scores), the rows streamed through shared memory in stretches of 256
 // dimensions as bulk copies, what the next job needs on its way while one is worked on, across the two passes and across
 // data points.  (With loads into registers, one stretch after the other, the memory system was idle three quarters of the
@@ -720,16 +721,18 @@ __global__ void __launch_bounds__(256, Wide<kMaxNeg>::kPerSm) kge_wide_kernel(co
     }
 }
 
-// Rows of more than 128 dimensions whose data point fits a block's shared memory (13 rows of up to 2,176 dimensions): the
-// embeddings stay there from the first pass to the second.  A warp has chunks of 64 dimensions to itself (chunk
-// (s C + rank) warps + w of the row is the s-th of warp w), with their own places in shared memory and their own barrier
-// words: it asks for its part of the next data point's rows when it is done with this one's, and meets the others once per data
-// point, to add up the scores.  In kge_wide_kernel, which streams stretches of 256 dimensions through a block, the warps meet after every
-// stretch (a third of their stalls), a last stretch idles some of them, and the rows are read twice.  us per launch, streamed and
-// now: 4,000 data points of 200 dimensions with 10 negatives 148 and 90, 1,600 of 500 105 and 90, 800 of 1,000 98 and 89,
-// 1,500 of 300 with 20 negatives 171 and 94, 600 of 600 with 29 248 and 121, 8,000 of 141 with one 140 and 76.  Where a data point takes a cluster of two blocks
-// the streamed form is as good (2,048 of 4,000: 753 and 770) and keeps it.  Bound by the latency of its instructions at 16
-// warps per SM, which 128 registers fix.
+// Rows of more than 128 dimensions (64, with more than ten negatives and rows updated in place) whose data point fits the shared memory of a block or of a
+// cluster of up to four (13 rows: 2,176 and 8,700 dimensions): the embeddings stay there from the first pass to the second.  A
+// warp has chunks of 64 dimensions to itself (chunk (s C + rank) warps + w of the row is the s-th of warp w), with their own
+// places in shared memory and their own barrier words: it asks for its part of the next data point's rows when it is done
+// with this one's, and meets the others once per data point, to add up the scores.  In kge_wide_kernel, which streams stretches
+// of 256 dimensions through a block, the warps meet after every stretch (a third of their stalls), a last stretch idles some
+// of them, and the rows are read twice.  us per launch, streamed and now: 4,000 data points of 200 dimensions with 10 negatives
+// 148 and 86, 1,600 of 500 105 and 86, 800 of 1,000 98 and 86, 1,500 of 300 with 20 negatives 171 and 92, 600 of 600 with 29 248 and
+// 121, 8,000 of 141 with one 140 and 76; clusters of two, 2,048 of 4,000 753 and 743.  On shorter rows the warp per data point of
+// kge_short_kernel is better, 89 and 115 us for 8,192 data points of 100 dimensions, but for its form for more than ten negatives
+// that updates rows in place (8 warps per SM; 6,000 of 70 with 20 negatives 123 and 102).  Bound by the latency of its
+// instructions at 16 warps per SM, which 128 registers fix (96 registers and 20 warps spill: 87 and 101 us at 500 dimensions).
 template <int kMaxNeg> struct Resident {
     static constexpr uint32_t kNumbers = 3 + kMaxNeg <= 16 ? 16 : 32;                   // places per table of slots
     __host__ __device__ static constexpr uint32_t pad(int kVec) { return kVec == 4 ? 64 : 68; }             // floats of a chunk of a row's Re or Im
@@ -858,9 +861,16 @@ __global__ void __launch_bounds__(512, 1) kge_resident_kernel(const KgeArgs A, c
         bulk_g2s(to, row, re_bytes, &bars[buf]);
         bulk_g2s(to + kPad, row + d - shift, im_bytes, &bars[buf]);
         if ((Q.once >> lane) & 1u) {
-            const uint32_t at_re = (2 * d) & 3, at_im = (3 * d) & 3;
-            bulk_prefetch(row + 2 * d - at_re, ((len + at_re + 3) & ~3u) * 4);
-            bulk_prefetch(row + 3 * d - at_im, ((len + at_im + 3) & ~3u) * 4);
+            // (as prefetches of lines: as bulk prefetches, each as dear as a copy, 3 % slower)
+            const float *g0 = row + 2 * d, *g1 = row + 3 * d;
+#pragma unroll
+            for (uint32_t o = 0; o < 64; o += 32)
+                if (o < len) {
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(g0 + o));
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(g1 + o));
+                }
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(g0 + len - 1));           // (a part need not start on a line)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(g1 + len - 1));
         }
     };
     Point P = {}, N = {};
@@ -1144,9 +1154,10 @@ uint32_t launch_wide(ps_store* ps, const KgeArgs& A, cudaStream_t s) {
     return grid;
 }
 
-// 0: a data point does not fit one block.  The number of warps per block: as many warps per SM as 128 registers a thread allow (16), in blocks
+// 0: a data point does not fit four blocks.  The number of warps per block: as many warps per SM as 128 registers a thread allow (16), in blocks
 // whose chunks go evenly, several chunks per warp where that costs none (a warp's work per data point is about a quarter of
-// a chunk's).
+// a chunk's); no blocks of one warp, whose waits nothing covers (9,000 data points of 170 dimensions with 4 negatives: 160 us a
+// step with those, 152).
 template <int kMaxNeg, int kVec>
 uint32_t launch_resident(ps_store* ps, const KgeArgs& A, cudaStream_t s) {
     using R = Resident<kMaxNeg>;
@@ -1157,7 +1168,7 @@ uint32_t launch_resident(ps_store* ps, const KgeArgs& A, cudaStream_t s) {
     for (;; C *= 2) {
         const uint32_t per = (chunks + C - 1) / C;
         double best = 0;
-        for (uint32_t w = 1; w <= tmin(16u, per); ++w) {
+        for (uint32_t w = tmin(2u, per); w <= tmin(16u, per); ++w) {
             const uint32_t str = (per + w - 1) / w;
             const size_t once = R::smem(kVec, slots, w, str, C), both = R::smem(kVec, slots, w, 2 * str, C);
             if (once > kMost || 2 * str > 32) continue;
@@ -1171,7 +1182,10 @@ uint32_t launch_resident(ps_store* ps, const KgeArgs& A, cudaStream_t s) {
                 twice = both <= kMost && blocks * (both + 1024) <= kPerSm;
             }
         }
-        if (!warps) return 0;
+        if (!warps) {
+            if (C == 4) return 0;
+            continue;
+        }
         // few data points: a cluster of two or four blocks for each, as long as none has to wait (16 data points of 600 dimensions
         // and their reduction: 24 -> 20 us)
         if (C == 4 || A.n * 2 * C > (uint64_t)sms * resident || chunks < 4 * C) break;
@@ -1241,17 +1255,17 @@ uint32_t launch_points_kge(ps_store* ps, const KgeBatch& B, const uint8_t* singl
         }                                                                                                        \
         return grid;                                                                                             \
     } while (0)
-    if (B.dim > 128) {
-        if (!finished) {
+    if (!finished && (B.dim > 128 || (B.dim > 64 && B.n_neg > 10 && single))) {
 #define KGE_RESIDENT(kMaxNeg)                                                                                     \
-            (B.dim % 4 == 0 ? launch_resident<kMaxNeg, 4>(ps, A, s) : B.dim % 2 == 0 ? launch_resident<kMaxNeg, 2>(ps, A, s) \
-                            : launch_resident<kMaxNeg, 1>(ps, A, s))
-            const uint32_t grid = B.n_neg <= 4    ? KGE_RESIDENT(4)
-                                  : B.n_neg <= 10 ? KGE_RESIDENT(10)
-                                  : B.n_neg <= 20 ? KGE_RESIDENT(20) : KGE_RESIDENT(29);
+    (B.dim % 4 == 0 ? launch_resident<kMaxNeg, 4>(ps, A, s) : B.dim % 2 == 0 ? launch_resident<kMaxNeg, 2>(ps, A, s) \
+                    : launch_resident<kMaxNeg, 1>(ps, A, s))
+        const uint32_t grid = B.n_neg <= 4    ? KGE_RESIDENT(4)
+                              : B.n_neg <= 10 ? KGE_RESIDENT(10)
+                              : B.n_neg <= 20 ? KGE_RESIDENT(20) : KGE_RESIDENT(29);
 #undef KGE_RESIDENT
-            if (grid) return grid;
-        }
+        if (grid) return grid;
+    }
+    if (B.dim > 128) {
 #define KGE_WIDE(kMaxNeg) return finished ? launch_wide<kMaxNeg, true>(ps, A, s) : launch_wide<kMaxNeg, false>(ps, A, s)
         if (B.n_neg <= 4) KGE_WIDE(4);
         if (B.n_neg <= 10) KGE_WIDE(10);

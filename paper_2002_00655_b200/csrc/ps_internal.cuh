@@ -579,10 +579,6 @@ __device__ __forceinline__ void tma_gather4(void* smem, const CUtensorMap* map, 
         "l"(map), "r"(x), "r"(y0), "r"(y1), "r"(y2), "r"(y3), "r"(smem_addr(bar))
         : "memory");
 }
-// asks for `bytes` (a multiple of 16) from a 16-byte boundary on to be in L2
-__device__ __forceinline__ void bulk_prefetch(const void* gmem, unsigned bytes) {
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(gmem), "r"(bytes) : "memory");
-}
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;\n" ::: "memory"); }
 // until at most kPending of this thread's bulk groups still have to READ their source
 template <int kPending>

@@ -1,5 +1,5 @@
-"""GPU parity of ComplEx on rows of more than 128 dimensions that stay in shared memory: chunks of 64 dimensions and their remainders, every
-alignment of a row's second half, one to 32 rows per data point, clusters for few data points, the last sizes that fit."""
+"""GPU parity of ComplEx on rows that stay in shared memory: chunks of 64 dimensions and their remainders, every alignment of a row's second
+half, one to 32 rows per data point, clusters for few data points and for wide rows, the last sizes that fit and what lies beyond."""
 import numpy as np
 import pytest
 import torch
@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("dim,n_neg", [(129, 10), (130, 0), (132, 20), (191, 29), (320, 10), (578, 13), (832, 29), (834, 29), (1001, 4), (1216, 20),
-                                       (2176, 10), (2178, 10)])
+                                       (2176, 10), (2178, 10), (66, 11), (100, 29), (127, 20), (2501, 20), (4098, 10), (8704, 10), (9000, 10)])
 @pytest.mark.parametrize("few", [2, 75, 0])
 def test_complex_rows_kept_in_shared_memory(dim, n_neg, few):
     rng = np.random.default_rng(dim + few)
