@@ -29,7 +29,7 @@
 // The d * d gradients of a data point never go through memory (335 MB per 8,192 data points of dimension 100 did, with
 // a sort of 112 keys per data point where 13 do now), and a relation's rows are read and written once per batch.
 // Before: a warp per data point with two passes over the matrix in L2, 292 us, and the matrix rows through the sorted
-// reduction, 278 us, of 577 us per step of 8,192 data points of dimension 100; now 125 + 105 us with the entities' reduction beside the latter, 237 us per step.
+// reduction, 278 us, of 577 us per step of 8,192 data points of dimension 100; now 122 + 105 us with the entities' reduction beside the latter, 235 us per step.
 // rescal_points_kernel is bound by the latency of its phases (16 warps per SM, issue slots 40 % used, tensor pipe 27 %),
 // rescal_matrix_kernel by instruction issue and the special-function unit.
 #include <string.h>
@@ -90,8 +90,7 @@ template <bool kSorted, int kWarps>
 __global__ void __launch_bounds__(32 * kWarps, 16 / kWarps) rescal_points_kernel(const RescalArgs A) {
     constexpr int kPointThreads = 32 * kWarps;
     extern __shared__ __align__(128) unsigned char dyn[];
-    __shared__ __align__(8) uint64_t bar;
-    __shared__ uint32_t s_t[kPoints];
+    __shared__ __align__(8) uint64_t bar, mat_bar;
     const unsigned full = 0xffffffffu;
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const uint32_t d = A.d, d4 = d / 4, ld = pad_ld(d), n_neg = A.n_neg, n_ent = 2 + n_neg;
@@ -103,7 +102,7 @@ __global__ void __launch_bounds__(32 * kWarps, 16 / kWarps) rescal_points_kernel
     double* const W = U + kPoints * ld;                         // R^T x_s
     float* const R = reinterpret_cast<float*>(W + kPoints * ld);        // [d][ld]
     float* const E = R + d * ld;                                // [points][n_ent][d]: the entities' rows
-    if (tid == 0) mbar_init(&bar, 1);
+    if (tid < 2) mbar_init(tid ? &mat_bar : &bar, 1);
     mbar_init_fence();
     pdl_trigger();
     pdl_wait();
@@ -150,36 +149,79 @@ __global__ void __launch_bounds__(32 * kWarps, 16 / kWarps) rescal_points_kernel
             if (col + 1 < len) o[ld] = acc[j][1];
         }
     };
-    for (uint32_t item = blockIdx.x; item < n_items; item += gridDim.x) {
-        uint32_t len = 1, pos = 0;
-        uint64_t rk;
-        if (kSorted) {
-            const uint2 it = A.L.pieces[item];
-            pos = it.x;
-            len = it.y;
-            rk = A.sk[pos];
-            if (tid < (int)len) s_t[tid] = A.sv[pos + tid] / n_slots;
-        } else {
-            rk = A.rel_base + (uint64_t)A.tr[item] * d;
-            if (tid == 0) s_t[0] = item;
-        }
-        if (tid == 0) mbar_expect_tx(&bar, (d + len * n_ent) * row_bytes);
+    // kSorted: look-ups of an item, a chain of four (piece, data points, their slots' keys, places of the rows).  With eight warps a
+    // link is asked for between the phases of the item before, and the matrix itself once that one's has been read (8,192 data
+    // points of dimension 100: 4 of an item's 24 us; the step 238 -> 235; blocks of four warps, of which more share an SM, lose 1 %).
+    constexpr bool kAhead = kSorted && kWarps == 8;
+    struct {
+        uint32_t pos, len, rk, t, key, side;
+        bool once;
+        uint2 entry, mat_entry;
+    } next = {};
+    auto find_piece = [&](uint32_t item) {
+        const uint2 it = item < n_items ? A.L.pieces[item] : make_uint2(0u, 0u);
+        next.pos = it.x;
+        next.len = it.y;
+    };
+    auto find_points = [&]() {
+        next.rk = next.len ? A.sk[next.pos] : 0u;
+        next.t = w < (int)next.len ? A.sv[next.pos + w] / n_slots : 0u;
+    };
+    auto key_of = [&](uint64_t t) -> uint32_t { return lane == 0 ? A.ts[t] : lane == 1 ? A.to[t] : A.neg_ent[t * n_neg + (lane - 2)]; };
+    auto find_keys = [&]() {
+        const bool mine = w < (int)next.len && slot;
+        next.key = mine ? key_of(next.t) : 0u;
+        next.side = mine && lane >= 2 ? A.neg_side[(uint64_t)next.t * n_neg + (lane - 2)] : 0u;
+        next.once = mine && A.L.single[(uint64_t)next.t * n_slots + lane];
+        next.mat_entry = next.len && tid < (int)d ? A.table[next.rk + tid] : make_uint2(0u, 0u);
+    };
+    auto find_rows = [&]() { next.entry = w < (int)next.len && slot ? A.table[next.key] : make_uint2(0u, 0u); };
+    auto announce_matrix = [&]() {
+        if (tid == 0 && next.len) mbar_expect_tx(&mat_bar, d * row_bytes);
+    };
+    auto ask_matrix = [&]() {                   // (after the block has met: nobody reads the matrix before)
+        if (next.len && tid < (int)d) bulk_g2s(R + tid * ld, A.store + phys_row(next.mat_entry, A.S) * L, row_bytes, &mat_bar);
+    };
+    auto look_up = [&](uint32_t item) {
+        find_piece(item);
+        find_points();
+        find_keys();
+        find_rows();
+        if (tid == 0 && next.len) mbar_expect_tx(&bar, next.len * n_ent * row_bytes);
+        announce_matrix();
         fence_async_smem();                     // (the rows of the item before have been read)
         __syncthreads();
+        ask_matrix();
+    };
+    if (kAhead) look_up(blockIdx.x);
+    for (uint32_t item = blockIdx.x; item < n_items; item += gridDim.x) {
+        if (kSorted && !kAhead) look_up(item);
+        const uint32_t len = kSorted ? next.len : 1;
+        const uint64_t rk = kSorted ? next.rk : A.rel_base + (uint64_t)A.tr[item] * d;
+        if (!kSorted) {
+            if (tid == 0) mbar_expect_tx(&bar, (d + n_ent) * row_bytes);
+            fence_async_smem();                 // (the rows of the item before have been read)
+            __syncthreads();
+        }
         // ---- the slots of the warp's data point: lane u holds slot u (subject, object, negatives) ----
         const bool mine = w < (int)len;
-        const uint64_t t = mine ? s_t[w] : 0;
+        const uint64_t t = !mine ? 0 : kSorted ? next.t : item;
         uint32_t key = 0, side = 0;
         int rep = lane;
         bool once = false, bad = !kSorted && rk + d > A.K;
         uint64_t erow = 0;
         if (mine) {
-            if (slot) key = lane == 0 ? A.ts[t] : (lane == 1 ? A.to[t] : A.neg_ent[t * n_neg + (lane - 2)]);
-            if (slot && lane >= 2) side = A.neg_side[t * n_neg + (lane - 2)];
-            if (!kSorted) bad |= slot && key >= A.rel_base;
+            if (kSorted) {
+                key = next.key;
+                side = next.side;
+            } else if (slot) {
+                key = key_of(t);
+                if (lane >= 2) side = A.neg_side[t * n_neg + (lane - 2)];
+                bad |= key >= A.rel_base;
+            }
             const unsigned same = __match_any_sync(full, slot ? key : kSentinelPad);
             if (slot) rep = __ffs(same) - 1;
-            if (kSorted && slot) once = rep == lane && A.L.single[t * n_slots + lane] != 0;
+            if (kSorted && slot) once = rep == lane && next.once;
         }
         if (!kSorted) {                         // (a call with a sort: checked and latched by its key kernel)
             uint32_t* ko = A.keys_out + (uint64_t)item * n_slots;
@@ -200,14 +242,16 @@ __global__ void __launch_bounds__(32 * kWarps, 16 / kWarps) rescal_points_kernel
             for (uint32_t a = tid; a < d; a += kPointThreads) ko[n_ent + a] = (uint32_t)(rk + a);
         }
         if (mine && slot) {
-            erow = phys_row(A.table[key], A.S);
+            erow = phys_row(kSorted ? next.entry : A.table[key], A.S);
             bulk_g2s(E + (w * n_ent + lane) * d, A.store + erow * L, row_bytes, &bar);
             if (once)                           // its accumulators are wanted at the end
                 for (uint32_t o = 0; o < row_bytes; o += 128)
                     asm volatile("prefetch.global.L2 [%0];" ::"l"((const char*)(A.store + erow * L + d) + o));
         }
-        if (tid < (int)d) bulk_g2s(R + tid * ld, A.store + phys_row(A.table[rk + tid], A.S) * L, row_bytes, &bar);
-        const bool ok = mbar_wait(&bar, parity) || mbar_wait(&bar, parity);
+        if (!kSorted && tid < (int)d) bulk_g2s(R + tid * ld, A.store + phys_row(A.table[rk + tid], A.S) * L, row_bytes, &bar);
+        if (kAhead) find_piece(item + gridDim.x);
+        const bool ok = (mbar_wait(&bar, parity) || mbar_wait(&bar, parity)) &&
+                        (!kSorted || mbar_wait(&mat_bar, parity) || mbar_wait(&mat_bar, parity));
         if (__syncthreads_or(!ok)) {
             if (tid == 0) {
                 latch_error(A.st, kSorted ? A.epoch : 0u, PS_ERR_CUDA);
@@ -229,9 +273,11 @@ __global__ void __launch_bounds__(32 * kWarps, 16 / kWarps) rescal_points_kernel
             x[0] = x_s.x; x[1] = x_s.y; x[2] = x_s.z; x[3] = x_s.w;
         }
         __syncthreads();
+        if (kAhead) find_points();
         products();
         store_products(U, W, len);
         __syncthreads();
+        if (kAhead) find_keys();
         // ---- scores, coefficients, a and b ----
         double coef = 0;                        // lane 1: the positive's, lane 2 + q: negative q's
         if (mine) {
@@ -249,7 +295,8 @@ __global__ void __launch_bounds__(32 * kWarps, 16 / kWarps) rescal_points_kernel
 #pragma unroll 4
                     for (uint32_t e = l8; e < d4; e += 8) {
                         const float4 v = row[e];
-                        s += (double)v.x * m[4 * e] + (double)v.y * m[4 * e + 1] + (double)v.z * m[4 * e + 2] + (double)v.w * m[4 * e + 3];
+                        const double2 m0 = *reinterpret_cast<const double2*>(m + 4 * e), m1 = *reinterpret_cast<const double2*>(m + 4 * e + 2);
+                        s += (double)v.x * m0.x + (double)v.y * m0.y + (double)v.z * m1.x + (double)v.w * m1.y;
                     }
                 }
                 s = sum8(s);
@@ -271,13 +318,14 @@ __global__ void __launch_bounds__(32 * kWarps, 16 / kWarps) rescal_points_kernel
             for (uint32_t z = 2; z < n_ent; ++z) {
                 const double c = __shfl_sync(full, coef, z);
                 const uint32_t sd = __shfl_sync(full, side, z);
-                const double ca = sd == 0 ? c : 0.0, cb = sd == 0 ? 0.0 : c;
                 const float4 v = act ? e4[z * d4 + lane] : make_float4(0.f, 0.f, 0.f, 0.f);
                 const double vv[4] = {v.x, v.y, v.z, v.w};
+                if (sd == 0) {
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    a[i] += ca * vv[i];
-                    b[i] += cb * vv[i];
+                    for (int i = 0; i < 4; ++i) a[i] += c * vv[i];
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) b[i] += c * vv[i];
                 }
             }
             if (act) {
@@ -300,8 +348,14 @@ __global__ void __launch_bounds__(32 * kWarps, 16 / kWarps) rescal_points_kernel
             }
         }
         __syncthreads();
+        if (kAhead) find_rows();
         products();
+        if (kAhead) {
+            fence_async_smem();
+            announce_matrix();
+        }
         __syncthreads();
+        if (kAhead) ask_matrix();
         store_products(Y, X, len);              // R b, R^T a
         __syncthreads();
         // ---- the entities' gradients, folded into the first slot of each key ----
@@ -328,6 +382,8 @@ __global__ void __launch_bounds__(32 * kWarps, 16 / kWarps) rescal_points_kernel
             }
             float* out = A.grad + t * n_slots * d;
             const unsigned reps = __ballot_sync(full, slot && rep == lane), in_place = __ballot_sync(full, once);
+            // negatives that are nothing else in the data point (nearly all): one number and one vector
+            const unsigned only3 = __ballot_sync(full, c1 == 0.0 && c2 == 0.0 && c4 == 0.0), only4 = __ballot_sync(full, c1 == 0.0 && c2 == 0.0 && c3 == 0.0);
             for (uint32_t v0 = 0; v0 < n_ent; v0 += 4) {        // four slots' accumulators asked for at a time
                 float4 G[4];
                 float* rows[4];
@@ -339,14 +395,21 @@ __global__ void __launch_bounds__(32 * kWarps, 16 / kWarps) rescal_points_kernel
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     const int v = v0 + i;
-                    const double f1 = __shfl_sync(full, c1, v & 31), f2 = __shfl_sync(full, c2, v & 31);
-                    const double f3 = __shfl_sync(full, c3, v & 31), f4 = __shfl_sync(full, c4, v & 31);
-                    if (v >= (int)n_ent || !((reps >> v) & 1u) || !act) continue;
+                    if (v >= (int)n_ent || !((reps >> v) & 1u)) continue;
+                    const double f3 = __shfl_sync(full, c3, v), f4 = __shfl_sync(full, c4, v);
                     float4 g;
-                    g.x = (float)(f1 * gs[0] + f2 * go[0] + f3 * u[0] + f4 * wv[0]);
-                    g.y = (float)(f1 * gs[1] + f2 * go[1] + f3 * u[1] + f4 * wv[1]);
-                    g.z = (float)(f1 * gs[2] + f2 * go[2] + f3 * u[2] + f4 * wv[2]);
-                    g.w = (float)(f1 * gs[3] + f2 * go[3] + f3 * u[3] + f4 * wv[3]);
+                    if ((only3 >> v) & 1u) {
+                        g = make_float4((float)(f3 * u[0]), (float)(f3 * u[1]), (float)(f3 * u[2]), (float)(f3 * u[3]));
+                    } else if ((only4 >> v) & 1u) {
+                        g = make_float4((float)(f4 * wv[0]), (float)(f4 * wv[1]), (float)(f4 * wv[2]), (float)(f4 * wv[3]));
+                    } else {
+                        const double f1 = __shfl_sync(full, c1, v), f2 = __shfl_sync(full, c2, v);
+                        g.x = (float)(f1 * gs[0] + f2 * go[0] + f3 * u[0] + f4 * wv[0]);
+                        g.y = (float)(f1 * gs[1] + f2 * go[1] + f3 * u[1] + f4 * wv[1]);
+                        g.z = (float)(f1 * gs[2] + f2 * go[2] + f3 * u[2] + f4 * wv[2]);
+                        g.w = (float)(f1 * gs[3] + f2 * go[3] + f3 * u[3] + f4 * wv[3]);
+                    }
+                    if (!act) continue;
                     if (kSorted && ((in_place >> v) & 1u)) {
                         const float4 s2 = make_float4(g.x * g.x, g.y * g.y, g.z * g.z, g.w * g.w);
                         float4 th = e4[v * d4 + lane], c = G[i];
@@ -375,6 +438,10 @@ __global__ void __launch_bounds__(32 * kWarps, 16 / kWarps) rescal_points_kernel
                 g.w = (float)(aa * xo[e + 3] + sa * b[e + 3]);
                 *reinterpret_cast<float4*>(out + (size_t)al * d + e) = g;
             }
+        }
+        if (kAhead) {
+            fence_async_smem();                 // (the rows have been read; the next ones come through the async proxy)
+            if (tid == 0 && next.len) mbar_expect_tx(&bar, next.len * n_ent * row_bytes);
         }
         __syncthreads();
     }

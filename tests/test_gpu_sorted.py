@@ -268,3 +268,20 @@ def test_wide_steps_on_either_side_of_the_sort(mode, dim, n, pipelined):
             ps.ps_step_sgns(g.h, d[0], window, m, window, d[1], q, V, 0.01, g.loss)
             o.step_sgns(tok, window, m, window, neg, q, V, 0.01)
     check(g, o, mode)
+
+
+@pytest.mark.parametrize("pipelined", [False, True])
+@pytest.mark.parametrize("d,n_neg", [(64, 3), (68, 0), (128, 5)])
+def test_rescal_blocks_that_take_several_pieces(d, n_neg, pipelined):
+    """More pieces of relations than blocks: a block looks the next one up while it works on one."""
+    rng = np.random.default_rng(d)
+    E, rels, n = 2_500, 11, 4_000
+    K = E + rels * d
+    g, o = make_pair(K, 2 * d, rows=ada_rows(rng, K, 2 * d), max_batch_keys=(2 + n_neg + d) * n)
+    ps.ps_set_pipelining(g.h, pipelined)
+    batch = triples(rng, n, n_neg, E, rels)
+    d_batch = on_gpu(batch)
+    torch.cuda.synchronize()
+    ps.ps_step_rescal(g.h, *d_batch, n_neg, E, d, 0.02, EPS, g.loss)
+    o.step_rescal(*batch, E, d, 0.02, EPS)
+    check(g, o, "RESCAL pieces")
