@@ -5,8 +5,8 @@
 // spends 20.  Here ONE launch does it.  Every block reads all keys of the call and keeps those of its hash bucket (a
 // dozen or two, in the order of the call: lane masks of the warps' shares, no sort), finds the first occurrence and the
 // number of occurrences of each in a table in shared memory, and a warp per distinct key adds its occurrences' rows in
-// the order of the call, in fp64, and rounds once, as the sorted reduction does.  A key with more than kShortRun
-// occurrences is shared by the block's warps (a range of the list each, partial sums added in range order).
+// the order of the call, in fp64, and rounds once, as the sorted reduction does.  Keys with more than kShortRun
+// occurrences are shared by four to sixteen of the block's warps (a range of the list each, partial sums added in range order).
 // Hot keys, which are a large part of the call, are shared by all blocks: 8,192 occurrences of one key took its block 118 us
 // at 128 values and 242 at 400, where a sort and the tiled reduction take 39 and 52.  Every block finds the same ones by itself
 // in a sample of kSample keys at jittered positions (hot_hits of one key make it hot: a key that is a quarter of the call is
@@ -31,6 +31,7 @@ namespace {
 constexpr int kThreads = 512;
 constexpr int kWarps = kThreads / 32;
 constexpr uint32_t kShortRun = 8;               // occurrences of one key that a warp adds alone
+__device__ __forceinline__ uint32_t long_warps(uint32_t occurrences) { return occurrences <= 16 ? 4 : occurrences <= 32 ? 8 : 16; }   // ... that add a longer one
 constexpr int kTableBits = 10, kTable = 1 << kTableBits;
 constexpr uint32_t kSample = 64;
 __host__ __device__ constexpr uint32_t hot_hits(int kCh) { return kCh == 1 ? 7 : 10; }   // (a warp has half as many rows of several column blocks in flight)
@@ -205,7 +206,8 @@ __global__ void __launch_bounds__(kThreads, kCh == 1 ? 2 : 1) small_push_kernel(
     __shared__ uint32_t t_key[kTable], t_first[kTable], t_count[kTable];
     __shared__ uint16_t s_firsts[kTable];
     __shared__ uint32_t s_cnt[kWarps], s_n_firsts, s_over;
-    __shared__ acc4 s_part[kWarps][32];
+    __shared__ acc4 s_part[kWarps * (kMode == kAdaGrad ? 2 : 1)][32];
+    __shared__ uint32_t s_n_longs;                          // keys with many occurrences: the last of s_firsts, backwards
     __shared__ __align__(16) uint32_t s_sample[kHot ? kSample : 4];
     __shared__ uint32_t s_hot[kMaxHot], s_hot_mask[kWarps], s_ticket;
     constexpr int kHalves = kMode == kAdaGrad ? 2 : 1;      // AdaGrad: sums for the parameters and for their accumulators
@@ -227,7 +229,7 @@ __global__ void __launch_bounds__(kThreads, kCh == 1 ? 2 : 1) small_push_kernel(
         t_key[i] = t_first[i] = kSentinelPad;
         t_count[i] = 0;
     }
-    if (tid == 0) s_n_firsts = s_over = 0;
+    if (tid == 0) s_n_firsts = s_n_longs = s_over = 0;
     pdl_wait();
     uint32_t sample = K;
     if constexpr (kHot) {
@@ -357,7 +359,13 @@ __global__ void __launch_bounds__(kThreads, kCh == 1 ? 2 : 1) small_push_kernel(
         const uint32_t k = s_key[i];
         uint32_t s = probe(k);
         while (t_key[s] != k) s = (s + 1) & (kTable - 1);
-        if (t_first[s] == i) s_firsts[atomicAdd(&s_n_firsts, 1u)] = (uint16_t)s;
+        if (t_first[s] != i) continue;
+        if (t_count[s] <= kShortRun) {
+            s_firsts[atomicAdd(&s_n_firsts, 1u)] = (uint16_t)s;
+            continue;
+        }
+        const uint32_t at = atomicAdd(&s_n_longs, 1u);
+        s_firsts[kTable - 1 - at] = (uint16_t)s;
     }
     __syncthreads();
     // ---- sums ----
@@ -497,42 +505,58 @@ __global__ void __launch_bounds__(kThreads, kCh == 1 ? 2 : 1) small_push_kernel(
         }
         return;
     }
-    const uint32_t n_firsts = s_n_firsts;
-    bool any_long = false;
-    for (uint32_t j = 0; j < n_firsts; ++j) {
-        const uint32_t s = s_firsts[j], count = t_count[s];
-        if (count > kShortRun) any_long = true;
-        else if (j % kWarps == (uint32_t)w) one_key(t_first[s], count);
-    }
-    if (!any_long) return;                      // the same decision in every warp
-    // ---- keys with many occurrences: the whole block on one at a time, a range of the list per warp ----
-    const uint32_t per = (m + kWarps - 1) / kWarps, lo = tmin<uint32_t>(w * per, m), hi = tmin<uint32_t>(lo + per, m);
-    for (uint32_t j = 0; j < n_firsts; ++j) {
+    const uint32_t n_firsts = s_n_firsts, n_longs = s_n_longs;
+    for (uint32_t j = w; j < n_firsts; j += kWarps) {
         const uint32_t s = s_firsts[j];
-        if (t_count[s] <= kShortRun) continue;
-        const uint32_t k = t_key[s];
-        float4* target = A.store + phys_row(A.table[k], A.S) * A.L4;
+        one_key(t_first[s], t_count[s]);
+    }
+    // ---- keys with many occurrences: a range of the list per warp, partial sums added in range order; up to four keys at a time ----
+    // (One after the other, all warps on each and a meeting of the block per half and column block, they took 3 to 6 us a key: the
+    // last 9 of 15 us in a push of 6,000 Zipf(0.9) keys, where every fifth block has one.  That push with its pull and relocation
+    // 26.6 -> 25.3 us, 8,000 of 256 values 40.2 -> 34.3, 4,000 cells of rank 64 20.8 -> 17.5, 600 ComplEx triples of 100 dimensions
+    // 38.6 -> 33.1.  Four warps for every such key: 256 triples 23.2 -> 26.6, the longer ones then take eight trips.  Their rows
+    // asked for ahead: no gain.)
+    for (uint32_t at = 0; at < n_longs;) {      // the same decisions in every warp
+        uint32_t used = 0, key_slot = kTable, first_warp = 0, warps = 0;
+        for (; at < n_longs; ++at) {            // (how a key's occurrences are grouped depends on their number alone)
+            const uint32_t s = s_firsts[kTable - 1 - at], r = long_warps(t_count[s]);
+            if (used + r > (uint32_t)kWarps) break;
+            if ((uint32_t)w >= used && (uint32_t)w < used + r) {
+                key_slot = s;
+                first_warp = used;
+                warps = r;
+            }
+            used += r;
+        }
+        float4* target = nullptr;
         float4 row[kHalves][kCh];
         acc4 a[kHalves][kCh];
-        load_row(target, row);
-        sum_range(k, lo, hi, a, row[kHalves - 1]);
+        if (warps) {
+            const uint32_t k = t_key[key_slot];
+            target = A.store + phys_row(A.table[k], A.S) * A.L4;
+            load_row(target, row);
+            const uint32_t per = (m + warps - 1) / warps, lo = tmin<uint32_t>((w - first_warp) * per, m);
+            sum_range(k, lo, tmin<uint32_t>(lo + per, m), a, row[kHalves - 1]);
+        }
 #pragma unroll
-        for (int h = 0; h < kHalves; ++h)
+        for (int c = 0; c < kCh; ++c) {
+            if (warps) {
 #pragma unroll
-            for (int c = 0; c < kCh; ++c) {
-                s_part[w][lane] = a[h][c];
-                __syncthreads();                // (every warp has read the row by now)
-                if (w == 0 && f0 + 32 * c < A.F4) {
-                    acc4 tot = s_part[0][lane];
-#pragma unroll
-                    for (int i = 1; i < kWarps; ++i) {
-                        tot.x += s_part[i][lane].x; tot.y += s_part[i][lane].y;
-                        tot.z += s_part[i][lane].z; tot.w += s_part[i][lane].w;
-                    }
-                    target[h * A.F4 + f0 + 32 * c] = finish(row[h][c], tot);
-                }
-                __syncthreads();
+                for (int h = 0; h < kHalves; ++h) s_part[w * kHalves + h][lane] = a[h][c];
             }
+            __syncthreads();                    // (every warp has read the row by now)
+            const uint32_t half = w - first_warp;
+            if (half < (uint32_t)kHalves && warps && f0 + 32 * c < A.F4) {      // a warp per half
+                acc4 tot = s_part[first_warp * kHalves + half][lane];
+                for (uint32_t i = 1; i < warps; ++i) {
+                    const acc4 x = s_part[(first_warp + i) * kHalves + half][lane];
+                    tot.x += x.x; tot.y += x.y; tot.z += x.z; tot.w += x.w;
+                }
+                float4* to = target + half * A.F4 + f0 + 32 * c;
+                *to = finish(kHalves == 2 && half ? row[kHalves - 1][c] : row[0][c], tot);
+            }
+            __syncthreads();
+        }
     }
 }
 

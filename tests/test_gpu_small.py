@@ -314,3 +314,26 @@ def test_small_calls_back_to_back(L, mode):
     assert torch.equal(g.loss, h.loss)
     o.set_rows(np.arange(K), g.export()[0].numpy())
     compare_state(g, o, exact_rows=True, what="tables and free lists")
+
+
+@pytest.mark.parametrize("L", [4, 128, 260, 520])
+@pytest.mark.parametrize("counts", [(8, 9, 16, 17, 32, 33), (9,) * 40, (33, 9, 64, 17, 9, 100, 12, 31, 40) * 3, (500, 9, 9, 300, 20)])
+def test_small_pushes_with_several_long_keys_per_block(counts, L):
+    """Keys of 4, 8 and 16 warps, several in one bucket of the call: sums exact on integers, and the same bits every time."""
+    rng = np.random.default_rng(len(counts) + L)
+    K = 3_000
+    keys = rng.permutation(np.concatenate([np.repeat(rng.choice(K, len(counts), replace=False), counts), rng.integers(0, K, size=20)]))
+    g, o = make_pair(K, L, rows=rng.integers(-50, 50, size=(K, L)).astype(np.float32))
+    upd = rng.integers(-9, 9, size=(len(keys), L)).astype(np.float32)
+    g.push(dev(keys), dev(upd))
+    o.push(keys, upd)
+    compare_state(g, o, exact_rows=True, what="integers")
+    upd = rng.normal(size=(len(keys), L)).astype(np.float32)
+    seen = []
+    for _ in range(3):
+        g.set_all_rows(torch.from_numpy(o.rows.copy()))
+        g.push(dev(keys), dev(upd))
+        seen.append(g.export(table=False)[0])
+    o.push(keys, upd)
+    compare_state(g, o, what="normal updates")
+    assert torch.equal(seen[0], seen[1]) and torch.equal(seen[0], seen[2])
