@@ -337,3 +337,17 @@ def test_small_pushes_with_several_long_keys_per_block(counts, L):
     o.push(keys, upd)
     compare_state(g, o, what="normal updates")
     assert torch.equal(seen[0], seen[1]) and torch.equal(seen[0], seen[2])
+
+
+@pytest.mark.parametrize("L,counts", [(516, (3, 700, 1_500)), (1024, (2_048, 2_047)), (4100, (1, 40, 511, 512))])
+def test_localize_of_wide_rows_around_the_limit_of_the_single_launch(L, counts):
+    """Rows that several warps move, a part each; calls of up to 8 MB of rows take the single launch."""
+    K, N = 2_500, 4
+    g, o = make_pair(K, L, N, K, max_batch_keys=2_500)
+    rng = np.random.default_rng(L)
+    for it, m in enumerate(counts):
+        keys = rng.integers(0, K, size=m)
+        g.localize(it % N, dev(keys))
+        o.localize(it % N, keys)
+        g.sync()
+        compare_state(g, o, exact_rows=True, what=f"localize of {m}")
