@@ -562,8 +562,17 @@ __global__ void __launch_bounds__(kThreads, kCh == 1 ? 2 : 1) small_push_kernel(
 
 template <int kMode, int kCh, bool kHot>
 void launch_kernel(ps_store* ps, const SmallArgs& a, uint32_t strips, cudaStream_t s) {
-    // about a dozen occurrences per block of 16 warps, two blocks per SM at most (more would only read the keys again)
-    const uint32_t buckets = tmax<uint32_t>(1u, tmin<uint32_t>(div_up_u32(a.n, 12), (uint32_t)ps->sm_count * 2 - 1));
+    // About a dozen occurrences per block of 16 warps, two blocks per SM at most (more would only read the keys again).  Up to 48 where
+    // the blocks of all stretches of columns would not be resident at once, as a second round of blocks reads the keys anew: 120
+    // ComplEx triples of 1,000 dimensions 47 -> 35 us, 240 of 500 58 -> 38, 200 of 66 25.8 -> 23.8; pull and push of 4,000 rows of
+    // 1,024 values 28 -> 23, 1,000 of them 14.1 -> 10.6.  Larger plain calls and small skip-gram steps have hot keys that want more
+    // blocks (with 48, Zipf(1): 8,000 rows of 400 values 35 -> 39, 3,000 of 512, one stretch, 21.8 -> 23.9, but 2,000 of them
+    // 18.2 -> 15.4; 100 centers of 300 values 34 -> 36.6): they keep the dozen.
+    const uint32_t wide = div_up_u32(strips, kCh), places = (uint32_t)ps->sm_count * (kCh == 1 ? 2 : 1) / wide;
+    const uint32_t dozens = div_up_u32(a.n, 12), limit = (uint32_t)ps->sm_count * 2 - 1;
+    const bool fewer = kMode == kAdaGrad || (kMode == kPlain && a.n <= (kCh == 4 && wide == 1 ? 2560u : 4096u));
+    const uint32_t fit = fewer ? tmax<uint32_t>(places > 1 ? places - 1 : 1u, div_up_u32(a.n, 48)) : limit;
+    const uint32_t buckets = tmax<uint32_t>(1u, tmin<uint32_t>(dozens, tmin<uint32_t>(fit, limit)));
     const size_t smem = ((size_t)a.n * 6 + 15) & ~(size_t)15;
     static std::atomic<unsigned long long> smem_set{0};
     opt_in_smem((const void*)small_push_kernel<kMode, kCh, kHot>, (size_t)kSmallOcc * 6, &smem_set);

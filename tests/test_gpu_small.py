@@ -125,6 +125,26 @@ def test_wide_complex_steps(n, dim, n_neg):
     test_small_complex_steps(n, dim, n_neg)
 
 
+@pytest.mark.parametrize("n,dim,n_neg", [(200, 66, 10), (300, 128, 10), (300, 250, 10), (120, 1000, 10), (45, 1001, 29), (3, 4000, 20)])
+def test_complex_steps_of_several_stretches_per_block(n, dim, n_neg):
+    """Reductions whose blocks of all stretches are resident at once: one to 48 occurrences of a bucket, one to 16 stretches."""
+    test_small_complex_steps(n, dim, n_neg)
+
+
+@pytest.mark.parametrize("n", [1, 13, 2559, 2560, 2561, 4095, 4096, 4097])
+@pytest.mark.parametrize("L", [200, 512, 700, 4100])
+def test_small_pushes_around_the_limits_of_the_buckets(n, L):
+    rng = np.random.default_rng(n + L)
+    g, o = make_pair(n + 50, L, rows=rng.integers(-4, 5, size=(n + 50, L)).astype(np.float32), max_batch_keys=n)
+    for share in (0.0, 0.5):
+        keys = np.where(rng.random(n) < share, rng.integers(0, 9, size=n), rng.integers(0, n + 50, size=n))
+        upd = rng.integers(-4, 5, size=(n, L)).astype(np.float32)
+        g.push(dev(keys), dev(upd))
+        o.push(keys, upd)
+    g.sync()
+    compare_state(g, o, exact_rows=True, what="pushes around the limits of the buckets")
+
+
 @pytest.mark.parametrize("N,L,counts", [(8, 128, (1, 7, 600, 2047, 2048, 2049)), (1500, 4, (5, 700, 2048, 2500, 4000)),
                                         (3, 256, (2048, 1, 2049, 1025)), (8, 64, (1151, 1152, 1153))])
 def test_localize_around_the_limit_of_the_single_launch(N, L, counts):
