@@ -1255,7 +1255,11 @@ uint32_t launch_points_kge(ps_store* ps, const KgeBatch& B, const uint8_t* singl
         }                                                                                                        \
         return grid;                                                                                             \
     } while (0)
-    if (!finished && (B.dim > 128 || (B.dim > 64 && B.n_neg > 10 && single))) {
+    // Up to 128 dimensions: with more than 10 negatives in calls with a sort; in calls without one with 5 to 10 negatives and more than
+    // 40 data points (us a step, streamed and now, 10 negatives: 307 of 100 dimensions 25.4 -> 23.2, 153 of 128 22.0 -> 19.9, 46 of
+    // 90 17.8 -> 17.3; 7 of 90 with 5 would lose, 11.7 -> 12.4, and so would 173 of 100 with 20, 26.1 -> 29.3).
+    const bool narrow = keys_out ? B.n_neg > 4 && B.n_neg <= 10 && B.n > 40 : B.n_neg > 10 && single;
+    if (!finished && (B.dim > 128 || (B.dim > 64 && narrow))) {
 #define KGE_RESIDENT(kMaxNeg)                                                                                     \
     (B.dim % 4 == 0 ? launch_resident<kMaxNeg, 4>(ps, A, s) : B.dim % 2 == 0 ? launch_resident<kMaxNeg, 2>(ps, A, s) \
                     : launch_resident<kMaxNeg, 1>(ps, A, s))

@@ -125,7 +125,7 @@ def test_wide_complex_steps(n, dim, n_neg):
     test_small_complex_steps(n, dim, n_neg)
 
 
-@pytest.mark.parametrize("n,dim,n_neg", [(200, 66, 10), (300, 128, 10), (300, 250, 10), (120, 1000, 10), (45, 1001, 29), (3, 4000, 20)])
+@pytest.mark.parametrize("n,dim,n_neg", [(200, 66, 10), (41, 100, 5), (300, 128, 10), (300, 250, 10), (120, 1000, 10), (45, 1001, 29), (3, 4000, 20)])
 def test_complex_steps_of_several_stretches_per_block(n, dim, n_neg):
     """Reductions whose blocks of all stretches are resident at once: one to 48 occurrences of a bucket, one to 16 stretches."""
     test_small_complex_steps(n, dim, n_neg)
