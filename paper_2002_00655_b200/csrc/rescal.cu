@@ -360,16 +360,16 @@ __global__ void __launch_bounds__(32 * kWarps, 16 / kWarps) rescal_points_kernel
         __syncthreads();
         // ---- the entities' gradients, folded into the first slot of each key ----
         if (mine) {
-            double c1 = 0, c2 = 0, c3 = 0, c4 = 0;      // lane v: the numbers of slot v
+            double c3 = 0, c4 = 0;              // lane v: the numbers of slot v
+            unsigned roles = 0;                 // ... and what it is: subject, object, negative in the subject's place, in the object's
             for (int z = 0; z < (int)n_ent; ++z) {
                 const int rz = __shfl_sync(full, rep, z);
                 const double cz = __shfl_sync(full, coef, z);
                 const uint32_t sz = __shfl_sync(full, side, z);
                 if (rz != lane) continue;
-                if (z == 0) c1 += 1.0;
-                else if (z == 1) c2 += 1.0;
-                else if (sz == 0u) c3 += cz;
-                else c4 += cz;
+                if (z >= 2 && sz == 0u) c3 += cz;
+                else if (z >= 2) c4 += cz;
+                roles |= z < 2 ? 1u << z : sz == 0u ? 4u : 8u;
             }
             double gs[4], go[4], u[4], wv[4];
 #pragma unroll
@@ -382,8 +382,10 @@ __global__ void __launch_bounds__(32 * kWarps, 16 / kWarps) rescal_points_kernel
             }
             float* out = A.grad + t * n_slots * d;
             const unsigned reps = __ballot_sync(full, slot && rep == lane), in_place = __ballot_sync(full, once);
-            // negatives that are nothing else in the data point (nearly all): one number and one vector
-            const unsigned only3 = __ballot_sync(full, c1 == 0.0 && c2 == 0.0 && c4 == 0.0), only4 = __ballot_sync(full, c1 == 0.0 && c2 == 0.0 && c3 == 0.0);
+            // A slot's gradient has the terms of its roles only, nearly always one (a number that is zero does not say that: the
+            // score that made it so may be infinite, and zero times that is no number).
+            const unsigned as_s = __ballot_sync(full, roles & 1u), as_o = __ballot_sync(full, roles & 2u);
+            const unsigned as_3 = __ballot_sync(full, roles & 4u), as_4 = __ballot_sync(full, roles & 8u);
             for (uint32_t v0 = 0; v0 < n_ent; v0 += 4) {        // four slots' accumulators asked for at a time
                 float4 G[4];
                 float* rows[4];
@@ -397,18 +399,17 @@ __global__ void __launch_bounds__(32 * kWarps, 16 / kWarps) rescal_points_kernel
                     const int v = v0 + i;
                     if (v >= (int)n_ent || !((reps >> v) & 1u)) continue;
                     const double f3 = __shfl_sync(full, c3, v), f4 = __shfl_sync(full, c4, v);
-                    float4 g;
-                    if ((only3 >> v) & 1u) {
-                        g = make_float4((float)(f3 * u[0]), (float)(f3 * u[1]), (float)(f3 * u[2]), (float)(f3 * u[3]));
-                    } else if ((only4 >> v) & 1u) {
-                        g = make_float4((float)(f4 * wv[0]), (float)(f4 * wv[1]), (float)(f4 * wv[2]), (float)(f4 * wv[3]));
-                    } else {
-                        const double f1 = __shfl_sync(full, c1, v), f2 = __shfl_sync(full, c2, v);
-                        g.x = (float)(f1 * gs[0] + f2 * go[0] + f3 * u[0] + f4 * wv[0]);
-                        g.y = (float)(f1 * gs[1] + f2 * go[1] + f3 * u[1] + f4 * wv[1]);
-                        g.z = (float)(f1 * gs[2] + f2 * go[2] + f3 * u[2] + f4 * wv[2]);
-                        g.w = (float)(f1 * gs[3] + f2 * go[3] + f3 * u[3] + f4 * wv[3]);
-                    }
+                    double x[4] = {0.0, 0.0, 0.0, 0.0};
+                    auto add = [&](unsigned has, double f, const double (&y)[4]) {
+                        if (!((has >> v) & 1u)) return;
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) x[k] += f * y[k];
+                    };
+                    add(as_s, 1.0, gs);
+                    add(as_o, 1.0, go);
+                    add(as_3, f3, u);
+                    add(as_4, f4, wv);
+                    const float4 g = make_float4((float)x[0], (float)x[1], (float)x[2], (float)x[3]);
                     if (!act) continue;
                     if (kSorted && ((in_place >> v) & 1u)) {
                         const float4 s2 = make_float4(g.x * g.x, g.y * g.y, g.z * g.z, g.w * g.w);

@@ -146,3 +146,33 @@ def test_rescal_pipelined_ordered_and_graph_replay_agree_bit_for_bit():
     for (e, l), what in zip(stores[1:], ("pipelined", "graph replay")):
         assert all((x == y).all() for x, y in zip(stores[0][0], e)), f"{what} differs from ordered calls"
         assert l == stores[0][1]
+
+
+@pytest.mark.parametrize("pipelined", [False, True])
+@pytest.mark.parametrize("d,n", [(16, 40), (100, 60), (100, 900), (28, 1300)])
+def test_rescal_with_infinite_values(d, n, pipelined):
+    """Entities with an infinite value, in every place of a data point, without and with a sort: scores of minus infinity, whose
+    coefficient is zero, times infinite vectors.  What is finite and what is not as in the oracle."""
+    E, R, n_neg = 3_000, 5, 6
+    rng = np.random.default_rng(d + n)
+    rows = np.abs(rng.normal(0, 0.3, size=(E + R * d, 2 * d))).astype(np.float32) + np.float32(0.05)
+    rows[E:, :d] *= -1
+    rows[:8, 0] = np.inf
+    s, t, ne = rng.integers(8, E, size=n), rng.integers(8, E, size=n), rng.integers(8, E, size=(n, n_neg))
+    s[:3], t[3:6], ne[6:8, 1] = (0, 1, 2), (3, 4, 5), (6, 7)
+    r, ns = rng.integers(1, R, size=n), rng.integers(0, 2, size=(n, n_neg))
+    r[:8], r[2], r[5] = 0, 1, 1
+    s, t, ne, r, ns = (x.astype(np.uint32) for x in (s, t, ne, r, ns))
+    ns = ns.astype(np.uint8)
+    g, o = make_pair(len(rows), 2 * d, rows=rows, max_batch_keys=(3 + n_neg + d) * n)
+    ps.ps_set_pipelining(g.h, pipelined)
+    a = [dev(x, torch.int32) for x in (s, r, t, ne)] + [dev(ns)]
+    torch.cuda.synchronize()
+    ps.ps_step_rescal(g.h, *a, n_neg, E, d, 0.1, 1e-8, g.loss)
+    o.step_rescal(s, r, t, ne, ns, E, d, 0.1, 1e-8)
+    g.sync()
+    got = g.export(table=False)[0].numpy()
+    ok = np.isfinite(o.rows)
+    assert 0 < (~ok).sum() < ok.size // 2
+    assert (np.isfinite(got) == ok).all()
+    assert close(got[ok], o.rows[ok]).all()
