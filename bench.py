@@ -542,7 +542,7 @@ class KGEWorkload:
         # updates in place (the accumulator half in, the row out); for the others it writes a gradient row of dim x 2
         # values, which the reduction reads before it read-modify-writes the keys' rows.
         grad = b * (12 + c.n_neg * 5) + occ * (8 + rb // 2) + once * (rb // 2 + rb) + (occ - once) * (rb // 2)
-        for name in ("kge_short_kernel", "kge_wide_kernel"):
+        for name in ("kge_short_kernel", "kge_resident_kernel", "kge_wide_kernel"):
             kb[name] = grad
         kb["segment_adagrad_kernel"] = (occ - once) * (8 + rb // 2) + (u - once) * (8 + 2 * rb)
         return kb

@@ -70,3 +70,19 @@ def test_gpus_flag_without_a_launcher_starts_the_ranks_itself():
     assert len(lines) == 1
     line = json.loads(lines[0])
     assert line["impl"] == "reference" and line["n_gpus"] == 2
+
+
+def test_every_gradient_kernel_of_complex_has_its_bytes():
+    """A kernel without bytes drops out of the line's roofline, which then names a smaller one."""
+    import re
+
+    import bench
+    from synth import workloads as W
+    with open(os.path.join(ROOT, "paper_2002_00655_b200", "csrc", "complex.cu")) as f:
+        launched = set(re.findall(r'"(kge_\w+_kernel)', f.read()))
+    assert len(launched) >= 3
+    wl = bench.KGEWorkload(W.KGE_TINY)
+    wl.row_bytes = 4 * W.KGE_TINY.row_len
+    wl.s, wl.r, wl.o, wl.neg, wl.side = W.kge_triples(W.KGE_TINY, 0, 2 * W.KGE_TINY.batch, "cpu")
+    kb = wl.kernel_bytes(1)
+    assert all(kb.get(name) for name in launched), launched
