@@ -250,9 +250,10 @@ __global__ void __launch_bounds__(32 * kWarps, 16 / kWarps) rescal_points_kernel
         }
         if (!kSorted && tid < (int)d) bulk_g2s(R + tid * ld, A.store + phys_row(A.table[rk + tid], A.S) * L, row_bytes, &bar);
         if (kAhead) find_piece(item + gridDim.x);
-        const bool ok = (mbar_wait(&bar, parity) || mbar_wait(&bar, parity)) &&
-                        (!kSorted || mbar_wait(&mat_bar, parity) || mbar_wait(&mat_bar, parity));
-        if (__syncthreads_or(!ok)) {
+        // (both are waited for, also where one does not come: a block that gives up has no copy on its way)
+        const bool rows_in = mbar_wait(&bar, parity) || mbar_wait(&bar, parity);
+        const bool matrix_in = !kSorted || mbar_wait(&mat_bar, parity) || mbar_wait(&mat_bar, parity);
+        if (__syncthreads_or(!rows_in || !matrix_in)) {
             if (tid == 0) {
                 latch_error(A.st, kSorted ? A.epoch : 0u, PS_ERR_CUDA);
                 if (!kSorted) A.keys_out[(uint64_t)item * n_slots] = kSentinelPad;      // (the reduction then does nothing)
