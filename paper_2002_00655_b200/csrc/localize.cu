@@ -465,27 +465,24 @@ loc_fused_kernel(const uint32_t* __restrict__ sk, uint32_t n, uint32_t span, uin
 }
 
 // ------------------------------------------------------------------------------------------------
-// Few keys and rows (loc_small_limit, loc_small_bytes): the whole call, sort included, as ONE launch of one cluster
-// of sixteen blocks, or eight where such a cluster does not fit.  With the cooperative sort and the launch above, 600 keys took 30 us of which nearly all was grid
+// Few keys and rows (localize_is_small): the whole call, sort included, as ONE launch of one cluster
+// of sixteen blocks.  With the cooperative sort and the launch above, 600 keys took 30 us of which nearly all was grid
 // barriers and launches; here the blocks meet once, at the cluster's own barrier.
 // Every block reads all keys, drops repeats with a hash table in shared memory and looks the others up; no order is needed
 // beyond what counting gives: a moving key's place among the moving keys (= its slot from the top of the requester's
 // stack) is the number of smaller moving keys, its place on its old owner's stack the number of smaller ones
 // with that owner.  A block counts for its share of the keys, kLocSmallThreads / share threads per key; the n^2 / 16
 // comparisons per block are what limits it.  us per call with eight blocks / sixteen / sort and launch above: 600 keys of 128 values
-// 8.9 / 6.8 / 22, 1,100 17.6 / 10.6 / 22, 1,500 of 4 33 / 12.9 / 22.7, 2,048 of 256 41.5 / 20.1 / 20.7; by bytes, 1,500 of 1,024
-// 21.1 with sixteen, 22.7 sorted, 600 of 2,048 16 and 34.
+// 8.9 / 6.8 / 22, 1,100 17.6 / 10.6 / 22, 1,500 of 4 33 / 12.9 / 22.7, 2,048 of 256 41.5 / 20.1 / 20.7.
 // Nothing is written before every block has read what it needs (cluster barrier), and each block then moves its own keys.
 constexpr int kLocSmallThreads = 1024;
 constexpr uint32_t kLocSmallBlocks = 16;
-constexpr uint32_t kLocSmallKeys = 2048;            // places in shared memory: the largest limit, to a multiple of the threads
-constexpr uint32_t loc_small_limit(uint32_t blocks) { return blocks == 16 ? kLocSmallKeys : 1152; }
-constexpr uint64_t loc_small_bytes(uint32_t blocks) { return blocks == 16 ? 8u << 20 : 2u << 20; }     // more is better spread over the chip
+constexpr uint32_t kLocSmallKeys = 2048;            // keys at most, and places in shared memory: a multiple of the threads
+constexpr uint64_t kLocSmallBytes = 8u << 20;       // by bytes: 1,500 keys of 1,024 values 21.1 us here, 22.7 sorted, 600 of 2,048 16 and 34
 constexpr int kLocTableBits = 12;
 constexpr size_t kLocSmallSmem = ((size_t)kLocSmallKeys * 2 + ((size_t)2 << kLocTableBits)) * 4;
 
-template <uint32_t kBlocks>
-__global__ void __cluster_dims__(kBlocks, 1, 1) __launch_bounds__(kLocSmallThreads)
+__global__ void __cluster_dims__(kLocSmallBlocks, 1, 1) __launch_bounds__(kLocSmallThreads)
 loc_small_kernel(const uint64_t* keys, uint32_t n, uint2* table, uint32_t worker, uint64_t S, uint32_t K,
                  unsigned long long* tops, uint32_t* stacks, float4* store, uint32_t L4, uint32_t part_size, DevStatus* st) {
     constexpr uint32_t kSlots = 1u << kLocTableBits, kPer = kLocSmallKeys / kLocSmallThreads;
@@ -494,7 +491,7 @@ loc_small_kernel(const uint64_t* keys, uint32_t n, uint2* table, uint32_t worker
     uint32_t* const s_own = s_key + kLocSmallKeys;          // ... and its old owner
     uint32_t* const t_key = s_own + kLocSmallKeys;
     uint32_t* const t_first = t_key + kSlots;
-    __shared__ uint32_t s_src[kLocSmallKeys / kBlocks][2], s_dst[kLocSmallKeys / kBlocks];
+    __shared__ uint32_t s_src[kLocSmallKeys / kLocSmallBlocks][2], s_dst[kLocSmallKeys / kLocSmallBlocks];
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const uint32_t b = blockIdx.x;
     for (uint32_t i = tid; i < kSlots; i += kLocSmallThreads) t_key[i] = t_first[i] = kSentinelPad;
@@ -547,7 +544,7 @@ loc_small_kernel(const uint64_t* keys, uint32_t n, uint2* table, uint32_t worker
         return;
     }
     // ---- the block's share of the positions, T neighbouring lanes per position ----
-    const uint32_t share = (n + kBlocks - 1) / kBlocks;
+    const uint32_t share = (n + kLocSmallBlocks - 1) / kLocSmallBlocks;
     uint32_t T = 1;
     while (T < 32 && share * T * 2 <= kLocSmallThreads) T <<= 1;
     const uint32_t mine = tid / T, sub = tid % T, i = b * share + mine;
@@ -618,7 +615,7 @@ static bool loc_cluster_fits() {
     int d = -1;
     if (cudaGetDevice(&d) != cudaSuccess || d < 0 || d >= 64) return false;
     if (!((asked.load(std::memory_order_acquire) >> d) & 1ull)) {
-        const void* fn = (const void*)loc_small_kernel<kLocSmallBlocks>;
+        const void* fn = (const void*)loc_small_kernel;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(kLocSmallBlocks);
         cfg.blockDim = dim3(kLocSmallThreads);
@@ -626,7 +623,7 @@ static bool loc_cluster_fits() {
         int clusters = 0;
         if (cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
             cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLocSmallSmem) == cudaSuccess &&
-            cudaOccupancyMaxActiveClusters(&clusters, loc_small_kernel<kLocSmallBlocks>, &cfg) == cudaSuccess && clusters > 0)
+            cudaOccupancyMaxActiveClusters(&clusters, loc_small_kernel, &cfg) == cudaSuccess && clusters > 0)
             fits.fetch_or(1ull << d, std::memory_order_relaxed);
         cudaGetLastError();
         asked.fetch_or(1ull << d, std::memory_order_release);
@@ -634,23 +631,13 @@ static bool loc_cluster_fits() {
     return (fits.load(std::memory_order_relaxed) >> d) & 1ull;
 }
 bool localize_is_small(const ps_store* ps, uint64_t n) {
-    const uint32_t blocks = loc_cluster_fits() ? kLocSmallBlocks : 8;
-    return n <= loc_small_limit(blocks) && n * ps->cfg.row_len * 4 <= loc_small_bytes(blocks);
+    return n <= kLocSmallKeys && n * ps->cfg.row_len * 4 <= kLocSmallBytes && loc_cluster_fits();
 }
 
 void run_localize_small(ps_store* ps, uint32_t worker, const uint64_t* d_keys, uint32_t n, cudaStream_t s) {
-#define LOC_SMALL(kBlocks)                                                                                                              \
-    PS_LAUNCH_PDL(ps, "loc_small_kernel", loc_small_kernel<kBlocks>, dim3(kBlocks), dim3(kLocSmallThreads), kLocSmallSmem, s, d_keys, n, \
-                  ps->table, worker, ps->cfg.slots_per_part, (uint32_t)ps->cfg.num_keys, ps->tops, ps->stacks, (float4*)ps->store,       \
-                  ps->cfg.row_len / 4, div_up_u32(ps->cfg.num_keys, ps->cfg.num_workers), ps->status)
-    if (loc_cluster_fits()) {
-        LOC_SMALL(kLocSmallBlocks);
-        return;
-    }
-    static std::atomic<unsigned long long> smem_set{0};
-    opt_in_smem((const void*)loc_small_kernel<8>, kLocSmallSmem, &smem_set);
-    LOC_SMALL(8);
-#undef LOC_SMALL
+    PS_LAUNCH_PDL(ps, "loc_small_kernel", loc_small_kernel, dim3(kLocSmallBlocks), dim3(kLocSmallThreads), kLocSmallSmem, s,
+                  d_keys, n, ps->table, worker, ps->cfg.slots_per_part, (uint32_t)ps->cfg.num_keys, ps->tops, ps->stacks,
+                  (float4*)ps->store, ps->cfg.row_len / 4, div_up_u32(ps->cfg.num_keys, ps->cfg.num_workers), ps->status);
 }
 
 // Second half of a relocation that ran beside another call: the moving keys that call touched (flag[m] = 1) get
