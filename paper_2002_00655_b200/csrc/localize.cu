@@ -478,7 +478,6 @@ loc_fused_kernel(const uint32_t* __restrict__ sk, uint32_t n, uint32_t span, uin
 constexpr int kLocSmallThreads = 1024;
 constexpr uint32_t kLocSmallBlocks = 16;
 constexpr uint32_t kLocSmallKeys = 2048;            // keys at most, and places in shared memory: a multiple of the threads
-constexpr uint64_t kLocSmallBytes = 8u << 20;       // by bytes: 1,500 keys of 1,024 values 21.1 us here, 22.7 sorted, 600 of 2,048 16 and 34
 constexpr int kLocTableBits = 12;
 constexpr size_t kLocSmallSmem = ((size_t)kLocSmallKeys * 2 + ((size_t)2 << kLocTableBits)) * 4;
 
@@ -630,8 +629,15 @@ static bool loc_cluster_fits() {
     }
     return (fits.load(std::memory_order_relaxed) >> d) & 1ull;
 }
+// Up to 1,600 keys and 8 MB of rows; of more keys 3.5 MB, or 8 of rows of more than 1,024 values.  us of a pull, push and
+// relocation of n keys, with this launch / with the sort and the launch above, which spreads the rows over the whole chip: 1,500 keys of
+// 1,024 values 32.1 / 34.3, 1,600 of 512 27.9 / 31.2, of 1,024 34.5 / 34.1; 1,700 of 512 29.1 / 31.1, of 700 34.4 / 33.9, of 1,024
+// 36.0 / 34.5; 2,048 of 300 31.1 / 31.1, of 400 32.5 / 32.0, of 600 39.1 / 33.5, of 1,024 42.5 / 36.3.  On wider rows that launch
+// takes longer: 1,700 of 1,200 51.6 / 59.2, 1,000 of 2,048 48.9 / 66.1, 125 of 16,384 122 / 233.  More than 8 MB has not been measured.
 bool localize_is_small(const ps_store* ps, uint64_t n) {
-    return n <= kLocSmallKeys && n * ps->cfg.row_len * 4 <= kLocSmallBytes && loc_cluster_fits();
+    const uint32_t L = ps->cfg.row_len;
+    const uint64_t bytes = n <= 1600 || L > 1024 ? 8u << 20 : 7u << 19;
+    return n <= kLocSmallKeys && n * L * 4 <= bytes && loc_cluster_fits();
 }
 
 void run_localize_small(ps_store* ps, uint32_t worker, const uint64_t* d_keys, uint32_t n, cudaStream_t s) {

@@ -359,9 +359,10 @@ def test_small_pushes_with_several_long_keys_per_block(counts, L):
     assert torch.equal(seen[0], seen[1]) and torch.equal(seen[0], seen[2])
 
 
-@pytest.mark.parametrize("L,counts", [(516, (3, 700, 1_500)), (1024, (2_048, 2_047)), (4100, (1, 40, 511, 512))])
+@pytest.mark.parametrize("L,counts", [(516, (3, 700, 1_500)), (1024, (2_048, 2_047)), (4100, (1, 40, 511, 512)), (448, (2_048, 2_049)),
+                                      (452, (2_029, 2_030)), (1024, (1_600, 1_601)), (1028, (1_601, 2_040, 2_041))])
 def test_localize_of_wide_rows_around_the_limit_of_the_single_launch(L, counts):
-    """Rows that several warps move, a part each; calls of up to 8 MB of rows take the single launch."""
+    """Rows that several warps move, a part each; both sides of each limit of the single launch: 1,600 keys, 3.5 MB and 8 MB of rows."""
     K, N = 2_500, 4
     g, o = make_pair(K, L, N, K, max_batch_keys=2_500)
     rng = np.random.default_rng(L)
