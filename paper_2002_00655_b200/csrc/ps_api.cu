@@ -796,7 +796,7 @@ ps_status_t ps_step_sgns(ps_store_t* ps, const uint32_t* d_tokens, uint64_t firs
     uint64_t occ;
     const ps_status_t c = sgns_checks(ps, first_pos, n_centers, corpus_len, window, n_neg, out_key_base, &occ);
     if (c != PS_OK) return c;
-    if (small_step(occ, ps->cfg.row_len)) {
+    if (small_sgns(occ, ps->cfg.row_len, occ / n_centers)) {
         sgns_small(ps, d_tokens, 0, first_pos, n_centers, corpus_len, window, d_negs, n_neg, out_key_base, lr, occ,
                    d_loss_accum, s);
         return after_launch();
@@ -954,7 +954,7 @@ ps_status_t ps_step_sgns_host(ps_store_t* ps, const uint32_t* h_tokens, uint64_t
     if (n_negs && cudaMemcpyAsync(d_negs, h_negs, n_negs * 4, cudaMemcpyHostToDevice, hb.cs) != cudaSuccess)
         return PS_ERR_CUDA;
     if (!host_batch_copied(ps, s, hb)) return PS_ERR_CUDA;
-    if (small_step(occ, ps->cfg.row_len)) {
+    if (small_sgns(occ, ps->cfg.row_len, occ / n_centers)) {
         sgns_small(ps, d_tok, tok_first, first_pos, n_centers, corpus_len, window, d_negs, n_neg, out_key_base, lr, occ,
                    d_loss_accum, s);
         c = after_launch();

@@ -276,15 +276,27 @@ void run_mf_col(ps_store* ps, uint32_t n_cells, int which, float lr, float lambd
 // slots' keys in small_keys (num_keys: no key; kSentinelPad: index out of range) and its rows in ps->upd, as for the
 // sorted reductions.
 inline bool small_call(uint64_t n_occ) { return n_occ <= kSmallOcc; }
-// ComplEx (dim complex dimensions) and skip-gram (rows of dim values): no sort up to kSmallValues dimensions (values) of all
-// occurrences, either.  A sort costs 12 to 25 us however wide the rows are; without one every gradient is written out and read
-// again, with one most rows are updated in place and the reduction is tiled.  us per step on an ordered handle, without / with a
-// sort: ComplEx with ten negatives, 300 data points of 250 dimensions 40 / 51, 600 of 250 64 / 68, 300 of 500 69 / 63, 600 of 500
-// 116 / 90, 300 of 1,000 130 / 91, 600 of 1,000 218 / 128 (pipelined, calls back to back: 40 / 36, 64 / 52, 69 / 47, 116 / 73,
-// 130 / 74, 218 / 111); skip-gram, 4,100 occurrences of 300 values 35.5 / 35, 7,790 of 300 49 / 38, 7,790 of 512 59 / 42.
-// Pushes and matrix factorization gain nothing from a sort at any width (8,000 rows of 1,024 values: 64 / 87).
+// ComplEx and skip-gram on wide rows sort even fewer occurrences than that: a sort costs 12 to 25 us however wide the rows are; without
+// one every gradient is written out and read again, with one most rows are updated in place and the reduction is tiled.  One limit for
+// ordered and pipelined handles, whose results are the same bits, and it lies where a pipelined handle, whose sorts run beside
+// other calls, breaks even (between 1.5 and 2.0M; an ordered one would at about 3M).
+// ComplEx (dim complex dimensions): no sort up to kSmallValues dimensions of all occurrences.  us per step, ordered without and with a sort,
+// pipelined without and with, 10 negatives: 476 data points of 250 dimensions (1.55M) 39.0 56.3, 39.1 39.0, 615 of 250 (2.0M) 52.3 66.4,
+// 52.0 49.8; 238 of 500 37.1 57.4, 37.2 43.9, 307 of 500 48.9 61.4, 48.7 46.3, 461 of 500 (3.0M) 66.2 71.1, 66.1 55.9; 119 of 1,000
+// 34.7 50.1, 34.8 37.6, 153 of 1,000 48.3 59.3, 48.4 45.8.  Odd dimensions, whose gradients are written out as finished steps: 297 of
+// 401 (1.55M) 55.2 60.6, 55.0 45.7, 383 of 401 (2.0M) 82.0 64.8, 81.8 49.2.
+// Pushes and matrix factorization gain nothing from a sort (8,000 rows of 1,024 values: 64 / 87).
 constexpr uint64_t kSmallValues = 1600000;
 inline bool small_step(uint64_t n_occ, uint64_t dim) { return small_call(n_occ) && n_occ * dim <= kSmallValues; }
+// Skip-gram (rows of row_len values, slots per center): a sort from 5,001 occurrences and kSmallValues values on, if a center has 26 to
+// 48 slots.  With fewer the gradient kernel is too short to cover a sort, with more it is most of the step either way.  us per step as
+// above: rows of 512 values, 13 slots (window 2, 2 negatives): 7,000 occurrences 34 41, 34 37; 25 slots 39 36, 39 37; 31 slots 47 40, 47
+// 42; 41 slots (window 5, 3 negatives) 4,900 occurrences 45 42, 44 44, 7,000 53 44, 53 46; 61 slots 54 53, 53 57; 113 slots 71 72,
+// 71 78.  Rows of 300: 41 slots 4,000 occurrences 31 34, 31 37, 6,600 41 36, 41 38.
+constexpr uint64_t kSgnsSortOcc = 5000, kSgnsSortFrom = 26, kSgnsSortTo = 48;
+inline bool small_sgns(uint64_t n_occ, uint64_t row_len, uint64_t slots) {
+    return small_step(n_occ, row_len) || (small_call(n_occ) && (n_occ <= kSgnsSortOcc || slots < kSgnsSortFrom || slots > kSgnsSortTo));
+}
 uint32_t* small_keys(ps_store* ps);
 void run_small_push_keys(ps_store* ps, const uint64_t* d_keys, uint32_t n, const float* d_upd, cudaStream_t s);
 void run_small_reduce(ps_store* ps, uint32_t n, double* d_loss_accum, uint32_t loss_blocks, cudaStream_t s,

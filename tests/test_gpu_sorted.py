@@ -270,6 +270,28 @@ def test_wide_steps_on_either_side_of_the_sort(mode, dim, n, pipelined):
     check(g, o, mode)
 
 
+@pytest.mark.parametrize("row,window,n_neg,n", [(400, 5, 3, 121), (400, 5, 3, 122), (512, 2, 2, 600), (300, 2, 5, 300), (320, 3, 3, 208), (260, 6, 3, 160),
+                                                (512, 7, 7, 70)])
+def test_wide_skip_gram_steps_by_slots_of_a_center(row, window, n_neg, n):
+    """5,000 occurrences on either side, and centers of 13 to 113 slots: ordered and pipelined handles leave the oracle's rows, and
+    the same bits."""
+    rng = np.random.default_rng(row + n)
+    V = 900
+    rows = rng.normal(0, 0.1, size=(2 * V, row)).astype(np.float32)
+    (g, o), (h, _) = (make_pair(2 * V, row, rows=rows, max_batch_keys=n * (1 + 2 * window * (1 + n_neg))) for _ in range(2))
+    ps.ps_set_pipelining(h.h, True)
+    for m in (n, 5, n):
+        tok, neg = u32(rng.integers(0, V, size=m + 2 * window)), u32(rng.integers(0, V, size=(m * 2 * window, n_neg)))
+        d = on_gpu((tok, neg))
+        torch.cuda.synchronize()
+        for s in (g, h):
+            ps.ps_step_sgns(s.h, d[0], window, m, window, d[1], n_neg, V, 0.01, s.loss)
+        o.step_sgns(tok, window, m, window, neg, n_neg, V, 0.01)
+    check(g, o, "skip-gram")
+    h.sync()
+    assert torch.equal(g.export(table=False)[0], h.export(table=False)[0]) and loss_of(g) == loss_of(h)
+
+
 @pytest.mark.parametrize("pipelined", [False, True])
 @pytest.mark.parametrize("d,n_neg", [(64, 3), (68, 0), (128, 5)])
 def test_rescal_blocks_that_take_several_pieces(d, n_neg, pipelined):
