@@ -1154,10 +1154,18 @@ uint32_t launch_wide(ps_store* ps, const KgeArgs& A, cudaStream_t s) {
     return grid;
 }
 
-// 0: a data point does not fit four blocks.  The number of warps per block: as many warps per SM as 128 registers a thread allow (16), in blocks
-// whose chunks go evenly, several chunks per warp where that costs none (a warp's work per data point is about a quarter of
-// a chunk's); no blocks of one warp, whose waits nothing covers (9,000 data points of 170 dimensions with 4 negatives: 160 us a
-// step with those, 152).
+// 0: not with this kernel (a data point does not fit four blocks, or only in blocks of few warps).  The number of warps per block: as many
+// warps per SM as 128 registers a thread allow (16), in blocks whose chunks go evenly, several chunks per warp where that costs none (a
+// warp's work per data point is about a quarter of a chunk's); no blocks of one warp, whose waits nothing covers (9,000 data points of 170
+// dimensions with 4 negatives: 160 us a step with those, 152).
+// Near the most that fits, the only blocks may be a few warps with many chunks each (2,000 dimensions with 11 negatives: two warps of 16),
+// and an SM with so few waits most of the time.  A wider cluster, or in the end kge_wide_kernel, is better from `least` warps per SM on:
+// us per step with any number of warps, with these limits, with kge_wide_kernel: 300 data points of 2,000 dimensions with 11 negatives 403,
+// 122, 225; 148 of 3,902 with 10 170, 113, 94; 300 of 1,102 with 20 259, 130, 176; 111 of 4,102 with 20 338, 183, 183; 60 of 13,900 with
+// 5 136, 96, 96.  In clusters of four there is only kge_wide_kernel left to take, which is slow with more than ten negatives: 60 of 15,900
+// with 4 (seven warps) 108, 93, 93; 60 of 7,001 with 11 (seven) 108, 108, 125; 60 of 2,902 with 29 (six) 111, 111, 152; 60 of 3,700 with
+// 25 (five) 135, 135, 172; 60 of 5,800 with 15 (four) 155, 120, 120; and where every data point has its cluster at once: 30 of 15,900
+// with 4 58, 58, 76, 30 of 13,900 with 5 (five) 74, 74, 78, 30 of 5,800 with 15 86, 86, 106.
 template <int kMaxNeg, int kVec>
 uint32_t launch_resident(ps_store* ps, const KgeArgs& A, cudaStream_t s) {
     using R = Resident<kMaxNeg>;
@@ -1171,7 +1179,7 @@ uint32_t launch_resident(ps_store* ps, const KgeArgs& A, cudaStream_t s) {
         for (uint32_t w = tmin(2u, per); w <= tmin(16u, per); ++w) {
             const uint32_t str = (per + w - 1) / w;
             const size_t once = R::smem(kVec, slots, w, str, C), both = R::smem(kVec, slots, w, 2 * str, C);
-            if (once > kMost || 2 * str > 32) continue;
+            if (once > kMost || 2 * str > 32) continue;        // (32 barrier words per warp; so many chunks go with few warps)
             const uint32_t blocks = tmin<uint32_t>(16 / w, (uint32_t)(kPerSm / (once + 1024)));
             const double score = (double)blocks * per / str * (4 * str) / (4 * str + 1);
             if (score > best) {
@@ -1182,8 +1190,11 @@ uint32_t launch_resident(ps_store* ps, const KgeArgs& A, cudaStream_t s) {
                 twice = both <= kMost && blocks * (both + 1024) <= kPerSm;
             }
         }
-        if (!warps) {
+        const bool at_once = A.n * C <= (uint64_t)sms * resident;
+        const uint32_t least = C < 4 ? 7 : A.n_neg <= 10 ? (at_once ? 5 : 8) : (at_once ? 4 : 5);
+        if (warps * resident < least) {
             if (C == 4) return 0;
+            warps = 0;
             continue;
         }
         // few data points: a cluster of two or four blocks for each, as long as none has to wait (16 data points of 600 dimensions

@@ -1,5 +1,6 @@
 """GPU parity of ComplEx on rows that stay in shared memory: chunks of 64 dimensions and their remainders, every alignment of a row's second
-half, one to 32 rows per data point, clusters for few data points and for wide rows, the last sizes that fit and what lies beyond."""
+half, one to 32 rows per data point, clusters for few data points and for wide rows; both sides of the last sizes that fit a block, a
+cluster of two and one of four, and the streamed kernel beyond them."""
 import numpy as np
 import pytest
 import torch
@@ -33,3 +34,16 @@ def test_complex_rows_kept_in_shared_memory(dim, n_neg, few):
     d = on_gpu(bad)
     torch.cuda.synchronize()
     check_no_op(g, o, lambda: ps.ps_step_kge(g.h, *d, n_neg, E, dim, LR, EPS, g.loss), "an object out of range")
+
+
+# The last dimension that a block, a cluster of two and one of four take, and the next, by the number of negatives (launch_resident's sums
+# for 227 KB of shared memory and the fewest warps per SM); beyond the last the rows are streamed.
+@pytest.mark.parametrize("dim,n_neg", [(2112, 10), (2116, 10), (4224, 10), (4228, 10), (8448, 10), (8452, 10), (2047, 10), (2049, 10), (3838, 10),
+                                       (3842, 10), (7679, 10), (7681, 10), (7682, 10), (1152, 20), (1156, 20), (2304, 20), (2308, 20), (4608, 20),
+                                       (4612, 20), (4095, 20), (4097, 20), (4102, 20), (832, 29), (836, 29), (1536, 29), (1540, 29), (3072, 29),
+                                       (3076, 29), (3071, 29), (3074, 29), (3077, 29), (4032, 4), (4036, 4), (8064, 4), (8068, 4), (15360, 4),
+                                       (15364, 4), (14335, 4), (14337, 4), (14338, 4), (1920, 11), (1924, 11), (7180, 11), (3702, 25)])
+@pytest.mark.parametrize("n", [2, 75])
+def test_complex_rows_around_the_last_sizes_that_fit(dim, n_neg, n):
+    """Two data points: no sort (odd dimensions: finished rows, streamed); 75: with a sort and rows updated in place."""
+    test_complex_rows_kept_in_shared_memory(dim, n_neg, n)
