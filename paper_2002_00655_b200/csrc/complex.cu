@@ -1158,6 +1158,9 @@ uint32_t launch_wide(ps_store* ps, const KgeArgs& A, cudaStream_t s) {
 // warps per SM as 128 registers a thread allow (16), in blocks whose chunks go evenly, several chunks per warp where that costs none (a
 // warp's work per data point is about a quarter of a chunk's); no blocks of one warp, whose waits nothing covers (9,000 data points of 170
 // dimensions with 4 negatives: 160 us a step with those, 152).
+// Few data points have an SM to themselves: what counts then are the warps of one block, and its rows may take all the shared memory
+// (us per step, ordered, in blocks that could share an SM / so / kge_wide_kernel: 12 data points of 3,000 dimensions with one negative
+// 20.3, 13.8, 16.3, 12 of 1,000 with 4 15.8, 13.2, 14.0, 30 of 900 with 4 19.4, 15.9, 15.9, 90 of 130 with 20 28.3, 24.3, 25.4).
 // Near the most that fits, the only blocks may be a few warps with many chunks each (2,000 dimensions with 11 negatives: two warps of 16),
 // and an SM with so few waits most of the time.  A wider cluster, or in the end kge_wide_kernel, is better from `least` warps per SM on:
 // us per step with any number of warps, with these limits, with kge_wide_kernel: 300 data points of 2,000 dimensions with 11 negatives 403,
@@ -1175,24 +1178,27 @@ uint32_t launch_resident(ps_store* ps, const KgeArgs& A, cudaStream_t s) {
     bool twice = false;
     for (;; C *= 2) {
         const uint32_t per = (chunks + C - 1) / C;
+        const bool alone = A.n * C * 8 <= (uint64_t)sms * 7;    // (clusters do not come by all SMs)
+        uint32_t most = 0;                                      // warps that an SM has room for
         double best = 0;
         for (uint32_t w = tmin(2u, per); w <= tmin(16u, per); ++w) {
             const uint32_t str = (per + w - 1) / w;
             const size_t once = R::smem(kVec, slots, w, str, C), both = R::smem(kVec, slots, w, 2 * str, C);
             if (once > kMost || 2 * str > 32) continue;        // (32 barrier words per warp; so many chunks go with few warps)
-            const uint32_t blocks = tmin<uint32_t>(16 / w, (uint32_t)(kPerSm / (once + 1024)));
+            const uint32_t fit = tmin<uint32_t>(16 / w, (uint32_t)(kPerSm / (once + 1024))), blocks = alone ? 1 : fit;
             const double score = (double)blocks * per / str * (4 * str) / (4 * str + 1);
             if (score > best) {
                 best = score;
                 warps = w;
                 n_str = str;
                 resident = blocks;
+                most = w * fit;
                 twice = both <= kMost && blocks * (both + 1024) <= kPerSm;
             }
         }
-        const bool at_once = A.n * C <= (uint64_t)sms * resident;
+        const bool at_once = A.n * C <= (uint64_t)sms * (most / tmax(warps, 1u));
         const uint32_t least = C < 4 ? 7 : A.n_neg <= 10 ? (at_once ? 5 : 8) : (at_once ? 4 : 5);
-        if (warps * resident < least) {
+        if (most < least) {
             if (C == 4) return 0;
             warps = 0;
             continue;
