@@ -370,12 +370,13 @@ __global__ void __launch_bounds__(32 * kShortWarps, kMaxNeg <= 10 ? 4 : 2) kge_s
     }
 }
 
-// Rows of more than 128 complex dimensions that kge_resident_kernel does not take (more than four blocks' shared memory; odd dimensions in
-// calls without a sort): a block per data point (batches of few data points: a
+// Rows of more than 128 complex dimensions that kge_resident_kernel does not take (launch_resident; odd dimensions in calls without a
+// sort): a block per data point (batches of few data points: a
 // cluster of up to four, which meets to add up the scores), the rows streamed through shared memory in stretches of 256
 // dimensions as bulk copies, what the next job needs on its way while one is worked on, across the two passes and across
-// data points.  (With loads into registers, one stretch after the other, the memory system was idle three quarters of the
-// time: 1,199 us for 2,048 data points of 4,000 dimensions whose rows take 440 us; streamed 808 us; with two stretches per job
+// data points.  (Measured on 2,048 data points of 4,000 dimensions with 10 negatives, whose rows take 440 us; they go to
+// kge_resident_kernel now, 743.  With loads into registers, one stretch after the other, the memory system was idle three quarters
+// of the time: 1,199 us; streamed 808 us; with two stretches per job
 // in the first pass, which has little to do on them and waits for their arrival, and the two kinds of update row compiled
 // apart, 747.)  It is bound by the second pass's instructions (1,300 per warp and stretch, half of them AdaGrad's, issued at
 // 16 warps per SM in chains) and by those arrivals.  Filling a stage when its last reader leaves, without a barrier per
@@ -386,7 +387,8 @@ __global__ void __launch_bounds__(32 * kShortWarps, kMaxNeg <= 10 ? 4 : 2) kge_s
 // kGroups = 2 (more than ten negatives): a stretch is 128 dimensions, and the block's halves share the negatives, so that a
 // thread's score sums stay in registers and two blocks' stages fit an SM (up to 20 negatives).  The first half, which also
 // has the subject, the relation and the object, gets fewer of them; the second hands it its weighted sums.  1,000 data points
-// of 400 dimensions with 20 negatives: 287 us with a block per data point and loads into registers at 8 warps per SM, now 146.
+// of 400 dimensions with 20 negatives, which this kernel had then: 287 us with a block per data point and loads into registers at 8
+// warps per SM, so 146.
 template <int kMaxNeg>
 struct Wide {
     static constexpr int kGroups = kMaxNeg > 10 ? 2 : 1, kSlots = 3 + kMaxNeg;
@@ -721,8 +723,9 @@ __global__ void __launch_bounds__(256, Wide<kMaxNeg>::kPerSm) kge_wide_kernel(co
     }
 }
 
-// Rows of more than 128 dimensions (64, with more than ten negatives and rows updated in place) whose data point fits the shared memory of a block or of a
-// cluster of up to four (13 rows: 2,176 and 8,700 dimensions): the embeddings stay there from the first pass to the second.  A
+// Rows of more than 128 dimensions, and some of 65 to 128 (launch_points_kge), whose data point fits the shared memory of a block or of a
+// cluster of two or four (13 rows: 2,112, 4,224 and 8,448 dimensions, 2,047, 3,839 and 7,679 where they are no multiple of four;
+// launch_resident): the embeddings stay there from the first pass to the second.  A
 // warp has chunks of 64 dimensions to itself (chunk (s C + rank) warps + w of the row is the s-th of warp w), with their own
 // places in shared memory and their own barrier words: it asks for its part of the next data point's rows when it is done
 // with this one's, and meets the others once per data point, to add up the scores.  In kge_wide_kernel, which streams stretches
@@ -730,8 +733,8 @@ __global__ void __launch_bounds__(256, Wide<kMaxNeg>::kPerSm) kge_wide_kernel(co
 // of them, and the rows are read twice.  us per launch, streamed and now: 4,000 data points of 200 dimensions with 10 negatives
 // 148 and 86, 1,600 of 500 105 and 86, 800 of 1,000 98 and 86, 1,500 of 300 with 20 negatives 171 and 92, 600 of 600 with 29 248 and
 // 121, 8,000 of 141 with one 140 and 76; clusters of two, 2,048 of 4,000 753 and 743.  On shorter rows the warp per data point of
-// kge_short_kernel is better, 89 and 115 us for 8,192 data points of 100 dimensions, but for its form for more than ten negatives
-// that updates rows in place (8 warps per SM; 6,000 of 70 with 20 negatives 123 and 102).  Bound by the latency of its
+// kge_short_kernel is better in large calls, 89 and 115 us for 8,192 data points of 100 dimensions, but for its form for more than ten
+// negatives that updates rows in place (8 warps per SM; 6,000 of 70 with 20 negatives 123 and 102).  Bound by the latency of its
 // instructions at 16 warps per SM, which 128 registers fix (96 registers and 20 warps spill: 87 and 101 us at 500 dimensions).
 template <int kMaxNeg> struct Resident {
     static constexpr uint32_t kNumbers = 3 + kMaxNeg <= 16 ? 16 : 32;                   // places per table of slots
@@ -1223,7 +1226,7 @@ uint32_t launch_resident(ps_store* ps, const KgeArgs& A, cudaStream_t s) {
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     uint64_t places = (uint64_t)sms * resident;
-    if (C > 1) {                                                // clusters resident at once: asked once per shape
+    if (C > 1) {                                                // clusters resident at once: asked for when the shape is not the last one (shapes in turn: no slower)
         ClusterFit& f = ps->kge_fit;
         if (f.fn != fn || f.smem != smem || f.threads != 32 * warps || f.blocks != C) {
             int clusters = 0;
@@ -1272,9 +1275,12 @@ uint32_t launch_points_kge(ps_store* ps, const KgeBatch& B, const uint8_t* singl
         }                                                                                                        \
         return grid;                                                                                             \
     } while (0)
-    // Up to 128 dimensions: with more than 10 negatives in calls with a sort; in calls without one with 5 to 10 negatives and more than
-    // 40 data points (us a step, streamed and now, 10 negatives: 307 of 100 dimensions 25.4 -> 23.2, 153 of 128 22.0 -> 19.9, 46 of
-    // 90 17.8 -> 17.3; 7 of 90 with 5 would lose, 11.7 -> 12.4, and so would 173 of 100 with 20, 26.1 -> 29.3).
+    // 65 to 128 dimensions: with more than 10 negatives in calls with a sort; in calls without one with 5 to 10 negatives and more than
+    // 40 data points.  A step with kge_resident_kernel over one with kge_short_kernel, 8 dimensions from 66 to 128 by 10 numbers of data
+    // points from 7 to 500: 10 negatives 1.01 to 1.04 at 7 and 16 data points, 0.98 to 1.03 at 30 and 41, 0.87 to 0.98 from 60 on; 8
+    // negatives 0.93 to 1.03 from 41 on; 5 and 6 negatives 1.00 to 1.06 up to 30, 0.96 to 1.04 from 41 to 100 (a limit of 100 for 5 to 7:
+    // 0.2 % slower over 270 sizes), 0.92 to 0.99 from 160 on; with few relations single sizes up to 1.10.  Outside: 4 negatives 0.92 to
+    // 1.06, 1 and 3 0.95 to 1.10, 11 to 20 up to 1.13.
     const bool narrow = keys_out ? B.n_neg > 4 && B.n_neg <= 10 && B.n > 40 : B.n_neg > 10 && single;
     if (!finished && (B.dim > 128 || (B.dim > 64 && narrow))) {
 #define KGE_RESIDENT(kMaxNeg)                                                                                     \

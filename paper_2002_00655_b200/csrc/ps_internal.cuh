@@ -21,7 +21,7 @@ constexpr int kReduceTile = 32;                  // sorted occurrences per warp 
 constexpr uint32_t kTiledRow = 512;              // ... rows up to this many values: 8 to 128 (reduce_tile)
 constexpr uint32_t kMidTiles = 4096;             // shorter tiles than 32 positions that a call has at most
 constexpr int kMaxLossBlocks = 4096;
-constexpr uint32_t kSmallOcc = 8192;             // calls of at most this many key occurrences are reduced without a sort (small.cu)
+constexpr uint32_t kSmallOcc = 8192;             // calls of at most this many key occurrences are reduced without a sort (small.cu; steps on wide rows: small_step, small_sgns)
 constexpr uint32_t kMaxHot = 8;                  // keys of such a call that all blocks share, at most
 constexpr uint32_t kHotStretches = 128;          // ... on rows of at most this many stretches of columns
 constexpr int kHostStages = 3;                   // staging areas for batches that arrive from host memory

@@ -2,8 +2,8 @@
 //
 // A push of a few thousand rows is a microsecond or two of memory traffic; sorted, it is a fork to another stream, a
 // cooperative sort with a grid barrier per pass, a reduction and a fix-up launch: 27 us for 13 rows, of which the host
-// spends 20.  Here ONE launch does it.  Every block reads all keys of the call and keeps those of its hash bucket (a
-// dozen or two, in the order of the call: lane masks of the warps' shares, no sort), finds the first occurrence and the
+// spends 20.  Here ONE launch does it.  Every block reads all keys of the call and keeps those of its hash bucket (one to
+// four dozen, in the order of the call: lane masks of the warps' shares, no sort), finds the first occurrence and the
 // number of occurrences of each in a table in shared memory, and a warp per distinct key adds its occurrences' rows in
 // the order of the call, in fp64, and rounds once, as the sorted reduction does.  Keys with more than kShortRun
 // occurrences are shared by four to sixteen of the block's warps (a range of the list each, partial sums added in range order).
@@ -518,7 +518,7 @@ __global__ void __launch_bounds__(kThreads, kCh == 1 ? 2 : 1) small_push_kernel(
     // asked for ahead: no gain.)
     for (uint32_t at = 0; at < n_longs;) {      // the same decisions in every warp
         uint32_t used = 0, key_slot = kTable, first_warp = 0, warps = 0;
-        for (; at < n_longs; ++at) {            // (how a key's occurrences are grouped depends on their number alone)
+        for (; at < n_longs; ++at) {            // (how many warps depends on the key's count alone; what each adds also on the bucket's list: the same in every such call)
             const uint32_t s = s_firsts[kTable - 1 - at], r = long_warps(t_count[s]);
             if (used + r > (uint32_t)kWarps) break;
             if ((uint32_t)w >= used && (uint32_t)w < used + r) {
@@ -564,10 +564,12 @@ template <int kMode, int kCh, bool kHot>
 void launch_kernel(ps_store* ps, const SmallArgs& a, uint32_t strips, cudaStream_t s) {
     // About a dozen occurrences per block of 16 warps, two blocks per SM at most (more would only read the keys again).  Up to 48 where
     // the blocks of all stretches of columns would not be resident at once, as a second round of blocks reads the keys anew: 120
-    // ComplEx triples of 1,000 dimensions 47 -> 35 us, 240 of 500 58 -> 38, 200 of 66 25.8 -> 23.8; pull and push of 4,000 rows of
-    // 1,024 values 28 -> 23, 1,000 of them 14.1 -> 10.6.  Larger plain calls and small skip-gram steps have hot keys that want more
-    // blocks (with 48, Zipf(1): 8,000 rows of 400 values 35 -> 39, 3,000 of 512, one stretch, 21.8 -> 23.9, but 2,000 of them
-    // 18.2 -> 15.4; 100 centers of 300 values 34 -> 36.6): they keep the dozen.
+    // ComplEx triples of 1,000 dimensions 47 -> 35 us, 240 of 500 58 -> 38; pull and push of 4,000 rows of 1,024 values 28 -> 23.  Larger
+    // plain calls and small skip-gram steps have hot keys that want more blocks (100 centers of 300 values 34 -> 36.6): they keep
+    // the dozen.  Time with 48 over time with a dozen, pulls and pushes of 500 to 8,192 rows of 132 to 4,096 values (378 sizes): up to 4,096
+    // rows 0.57 to 1.04 with uniform and Zipf(0.6) keys, 0.77 to 1.12 (median 0.89) with Zipf(1); above 0.71 to 1.07 and 0.84 to 1.11
+    // (median 1.00); one stretch of 388 to 512 values above 2,560 rows 0.73 to 1.03, and 1.02 to 1.09 with Zipf(1); ComplEx steps
+    // 0.69 to 1.07.
     const uint32_t wide = div_up_u32(strips, kCh), places = (uint32_t)ps->sm_count * (kCh == 1 ? 2 : 1) / wide;
     const uint32_t dozens = div_up_u32(a.n, 12), limit = (uint32_t)ps->sm_count * 2 - 1;
     const bool fewer = kMode == kAdaGrad || (kMode == kPlain && a.n <= (kCh == 4 && wide == 1 ? 2560u : 4096u));
