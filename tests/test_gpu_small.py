@@ -119,9 +119,9 @@ def test_small_complex_steps(n, dim, n_neg):
 @pytest.mark.parametrize("n,dim,n_neg", [(1, 129, 2), (74, 256, 4), (75, 257, 10), (148, 515, 3), (149, 512, 10), (33, 1028, 9),
                                          (700, 514, 10), (2, 130, 11), (50, 385, 20), (80, 260, 21), (160, 131, 29), (400, 258, 20)])
 def test_wide_complex_steps(n, dim, n_neg):
-    """Clusters of four, two and one block per data point, stretches that do and do not divide among them and among the
-    jobs of a pass, rows whose parts start off a 16-byte boundary, negatives shared by the halves of a block; the largest of
-    each form with a sort and rows updated in place."""
+    """Even dimensions: rows kept in shared memory.  Odd ones without a sort: streamed as finished rows, in clusters of four, two and one
+    block per data point, stretches that do and do not divide among them and among the jobs of a pass, parts that start off a
+    16-byte boundary, negatives shared by the halves of a block.  (Streamed gradients and rows updated in place: test_gpu_resident.)"""
     test_small_complex_steps(n, dim, n_neg)
 
 

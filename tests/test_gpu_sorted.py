@@ -307,3 +307,30 @@ def test_rescal_blocks_that_take_several_pieces(d, n_neg, pipelined):
     ps.ps_step_rescal(g.h, *d_batch, n_neg, E, d, 0.02, EPS, g.loss)
     o.step_rescal(*batch, E, d, 0.02, EPS)
     check(g, o, "RESCAL pieces")
+
+
+@pytest.mark.parametrize("pipelined", [False, True])
+def test_wide_skip_gram_steps_replayed_from_a_graph(pipelined):
+    """Fewer than 8,192 occurrences, sorted for their width: captured once, replayed twice, against the same calls one by one."""
+    rng = np.random.default_rng(5)
+    V, row, window, n_neg, n = 700, 400, 5, 3, 130
+    rows = rng.normal(0, 0.1, size=(2 * V, row)).astype(np.float32)
+    (a, _), (g, _) = (make_pair(2 * V, row, rows=rows, max_batch_keys=n * (1 + 2 * window * (1 + n_neg))) for _ in range(2))
+    d = on_gpu((u32(rng.integers(0, V, size=n + 2 * window)), u32(rng.integers(0, V, size=(n * 2 * window, n_neg)))))
+    for s in (a, g):
+        ps.ps_set_pipelining(s.h, pipelined)
+    step = lambda s: ps.ps_step_sgns(s.h, d[0], window, n, window, d[1], n_neg, V, 0.01, s.loss)
+    step(a); step(g)
+    torch.cuda.synchronize()
+    graph, stream = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        graph.capture_begin(capture_error_mode="thread_local")
+        step(g)
+        step(g)
+        graph.capture_end()
+    for _ in range(2):
+        graph.replay()
+        step(a); step(a)
+    torch.cuda.synchronize()
+    assert a.sync() == g.sync() == ps.PS_OK
+    assert torch.equal(a.export(table=False)[0], g.export(table=False)[0]) and loss_of(a) == loss_of(g)
