@@ -112,6 +112,21 @@ def test_a_wait_that_runs_out_is_reported_and_the_handle_stays_usable():
         compare_state(g, o, exact_rows=True, what=f"after the wait ran out, round {round_}")
 
 
+@pytest.mark.parametrize("L", [1028, 1156, 2048, 4100, 16384])
+@pytest.mark.parametrize("n", [1, 4, 31, 33, 260, 2500])
+def test_pulls_of_wide_rows_shared_by_blocks(n, L):
+    """One share of a row per block to one block for 32 whole rows; a key out of range among them leaves zeros."""
+    import paper_2002_00655_b200 as ps
+    K = 300
+    g, o = make_pair(K, L)
+    keys = np.random.default_rng(n).integers(0, K, size=n)
+    assert (g.pull(dev(keys)).cpu().numpy() == o.pull(keys)).all()
+    keys[-1] = K
+    out = g.pull(dev(keys)).cpu().numpy()
+    assert g.sync(check=False) == ps.PS_ERR_KEY_RANGE
+    assert (out[-1] == 0).all() and (out[:-1] == o.pull(keys[:-1])).all()
+
+
 def test_push_and_pull_reject_bad_keys_without_touching_the_store():
     import paper_2002_00655_b200 as ps
     K, L = 500, 12
